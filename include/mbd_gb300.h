@@ -51,12 +51,14 @@ extern "C" {
  * subtraction and all sums stay in FP64 with compensation.  Gradients use Z.  In the same
  * modes the screening matrices are factored in FP32 (tensor-core TF32x3 updates) and each
  * solution is refined once against the FP64 matrix. */
-#define MBD_PREC_FP64 0           /* plain FP64 throughout                           */
+#define MBD_PREC_FP64 0           /* FP64 throughout; the Newton-Schulz products are formed on the
+                                     bf16 tensor cores from exact residues, with less rounding
+                                     than an FP64 sum                                 */
 #define MBD_PREC_TF32 1           /* TF32 tensor-core products, FP64 correction      */
 #define MBD_PREC_BF16X3 2         /* bf16 hi/lo split products (3 per GEMM), FP64 correction */
 #define MBD_PREC_TF32X3 3         /* TF32 hi/lo split products (3 per GEMM), FP64 correction */
-#define MBD_PREC_FP64_SPLIT 4     /* as FP64, the Newton-Schulz products FP64-accurate on the TF32
-                                     tensor cores by error-free splitting (finite systems) */
+#define MBD_PREC_FP64_SPLIT 4     /* as FP64, whose products are FP64-accurate on the tensor cores too;
+                                     finite systems only                              */
 
 typedef struct mbd_ctx mbd_ctx;
 

@@ -70,6 +70,50 @@ size_t gemm_f64_split_work_bytes(int M, int N, int K);
 cudaError_t gemm_f64_split(int trans_b, int mode, int M, int N, int K, double alpha, const double *A, long long lda,
                            const double *B, long long ldb, double beta, const double *D, long long ldd, double *C,
                            long long ldc, void *work, int *err, cudaStream_t s);
+// FP64-accurate products on the bf16 tensor cores by residues (k_crt.cu, crt64.cuh).  An operand
+// is an array of rows along K: A's rows, or the columns of B (the rows of B^T).  crt_rows turns it into
+// residue planes in caller memory of crt_operand_bytes; crt_multiply forms
+// C = alpha A B + beta D from two operands through crt_bytes_bytes of scratch.  Row pitches are
+// even and rows 16-byte aligned; K any.  Complex operands have planar parts: the left
+// one's are [Ar | Ai], the right one's (right = true) the columns of B as rows, which for conj =
+// true are read from the rows of a Hermitian B.
+struct CrtShape {
+    int rows, K, batch;
+    bool complex, right;
+    int half, second, out_rows;   // complex: entries to the imaginary half, rows to the second set
+    long long pitch;              // entries of a plane's row
+};
+struct CrtOperand {
+    CrtShape shape;
+    __nv_bfloat16 *planes;
+    int *exps;
+};
+struct CrtResult {
+    double alpha, beta;
+    const double *D;         // may be C
+    double *C, *T;           // T: also the transpose (or null; not with sym)
+    long long ldd, ldc, ldt, sD, sC, sT;   // pitches and batch strides
+    long long im_off;        // complex: from a real plane to its imaginary one (D, C, T)
+    int col0;                // the product's first column in D, C and T
+    bool sym;                // square results known to be symmetric (Hermitian): entries on or above the
+                             // diagonal, mirrored exactly
+};
+CrtShape crt_shape(int rows, int K, int batch, bool complex, bool right);
+size_t crt_operand_bytes(const CrtShape &s);
+size_t crt_bytes_bytes(int M, int N, int batch);
+CrtOperand crt_rows(const CrtShape &s, const double *re, const double *im, long long ld, long long stride, bool conj,
+                    void *mem, cudaStream_t st);
+cudaError_t crt_multiply(const CrtOperand &A, const CrtOperand &B, const CrtResult &r, void *bytes, int *err,
+                         cudaStream_t st);
+// C = alpha A B + beta D for real operands of any size through crt_gemm_bytes of scratch, in panels
+// of columns and of K when they are long.  Bt: the rows of B^T.
+// Columns and K of one panel: the planes of a matrix of order n then take at most 30 n kCrtBlock
+// bytes, and all of the scratch 17 GB at n = 41000, the largest order that fits the card.
+constexpr int kCrtBlock = 8192;
+size_t crt_gemm_bytes(int M, int N, int K);
+cudaError_t crt_gemm(const double *A, long long lda, const double *Bt, long long ldb, int M, int N, int K,
+                     const CrtResult &r, void *work, int *err, cudaStream_t st);
+
 // Mixed-precision helpers: Y = scale Q (FP32 and, if Yh, bf16 hi/lo) and Z = I;
 // Z = a I + b P; Zd = scale Zf in FP64; and the variational energy
 // E = (1/4)(3 Tr V - sum V o W) - 3/2 sum omega (work: 608 doubles).

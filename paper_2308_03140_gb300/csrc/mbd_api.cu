@@ -53,8 +53,7 @@ constexpr double kMixedFloor = 1e-7;
 // mirrored, imaginary part mirrored with a sign change), a third fewer flops per step.
 constexpr bool kHermitianNs = true;
 constexpr int kLF = MBD_LEARNED_FEATURES;   // inputs of the learned screening model
-// The FP64 path (screening, bounds, Newton-Schulz, gradients in FP64), with its Newton-Schulz
-// products on the DMMA pipe (MBD_PREC_FP64) or FP64-accurate on the TF32 tensor cores.
+// The FP64 path (screening, bounds, Newton-Schulz, gradients in FP64).
 inline bool fp64_path(int precision) { return precision == MBD_PREC_FP64 || precision == MBD_PREC_FP64_SPLIT; }
 }  // namespace
 
@@ -140,7 +139,11 @@ struct mbd_ctx {
     CellGeom cell{};
     std::vector<double> hkq, hG;
     std::vector<int> hglist, hgcount;
-    void *dsplit = nullptr;   // slices of the split FP64 GEMM (MBD_PREC_FP64_SPLIT)
+    // FP64 path: residue planes of three operands and the bytes of a product (k_crt.cu), or the
+    // scratch of products taken in panels; dPT: the transpose of P.  Null when they did not fit:
+    // the products then run on the FP64 pipe.
+    char *crt = nullptr;
+    double *dPT = nullptr;
     double *dkq = nullptr, *dG = nullptr, *dcoef = nullptr, *dlzw = nullptr, *dgA = nullptr, *dgAout = nullptr,
            *dgApart = nullptr, *dgc = nullptr, *dtsg = nullptr;
     int *dglist = nullptr, *dgcount = nullptr;
@@ -303,6 +306,64 @@ int ensure_learned(mbd_ctx *ctx) {
     return MBD_OK;
 }
 
+// Scratch of the FP64 path's products for matrices of order n: three operands' residue planes and a
+// product's bytes while a matrix is one panel, else that of products in panels.
+size_t crt_ns_bytes(int n) {
+    if (n > kCrtBlock) return crt_gemm_bytes(n, n, n);
+    return 3 * crt_operand_bytes(crt_shape(n, n, 1, false, false)) + crt_bytes_bytes(n, n, 1);
+}
+
+// The products of a coupled Newton-Schulz step on the tensor cores (k_crt.cu).  All operands are
+// rows: Y and Z are symmetric, and P's columns are the rows of its transpose, which P's own
+// product writes beside it.  Each matrix becomes residue planes once a step.
+struct CrtProducts {
+    mbd_ctx *ctx;
+    cudaStream_t s;
+    CrtShape shape;
+    char *slot[3], *bytes;
+    CrtOperand oY{}, oZ{};
+    CrtProducts(mbd_ctx *c, cudaStream_t st) : ctx(c), s(st), shape(crt_shape(c->n, c->n, 1, false, false)) {
+        const size_t b = crt_operand_bytes(shape);
+        for (int k = 0; k < 3; ++k) slot[k] = c->crt + k * b;
+        bytes = c->crt + 3 * b;
+    }
+    bool panels() const { return ctx->n > kCrtBlock; }
+    CrtOperand rows(const double *X, int k) { return crt_rows(shape, X, nullptr, ctx->ld, 0, false, slot[k], s); }
+    CrtResult result(double *C, double *T, double alpha, double beta, const double *D, bool sym) const {
+        const long long ld = ctx->ld;
+        return CrtResult{alpha, beta, D, C, T, ld, ld, ld, 0, 0, 0, 0, 0, sym};
+    }
+    cudaError_t whole(const double *A, const double *Bt, const CrtResult &r) {
+        return crt_gemm(A, ctx->ld, Bt, ctx->ld, ctx->n, ctx->n, ctx->n, r, ctx->crt, ctx->dstatus, s);
+    }
+    // P = Z Y and its transpose
+    cudaError_t product(const double *Z, const double *Y, double *P, double *PT) {
+        const CrtResult r = result(P, PT, 1.0, 0.0, nullptr, false);
+        if (panels()) return whole(Z, Y, r);
+        oZ = rows(Z, 0);
+        oY = rows(Y, 1);
+        return crt_multiply(oZ, oY, r, bytes, ctx->dstatus, s);
+    }
+    // Y2 = c1 Y + c3 Y P, Z2 = c1 Z + c3 P Z, after product()
+    cudaError_t step(const double *Y, const double *Z, const double *P, const double *PT, double *Y2, double *Z2,
+                     double c1, double c3) {
+        const CrtResult ry = result(Y2, nullptr, c3, c1, Y, true), rz = result(Z2, nullptr, c3, c1, Z, true);
+        if (panels()) {
+            const cudaError_t e = whole(Y, PT, ry);
+            return e == cudaSuccess ? whole(P, Z, rz) : e;
+        }
+        const cudaError_t e = crt_multiply(oY, rows(PT, 2), ry, bytes, ctx->dstatus, s);
+        return e == cudaSuccess ? crt_multiply(rows(P, 1), oZ, rz, bytes, ctx->dstatus, s) : e;
+    }
+    // Y2 = c1 Y + c3 Y Y
+    cudaError_t first_step(const double *Y, double *Y2, double c1, double c3) {
+        const CrtResult r = result(Y2, nullptr, c3, c1, Y, true);
+        if (panels()) return whole(Y, Y, r);
+        oY = rows(Y, 1);
+        return crt_multiply(oY, oY, r, bytes, ctx->dstatus, s);
+    }
+};
+
 // Carves the workspace out of one allocation (256-byte aligned pieces).
 int allocate(mbd_ctx *ctx) {
     const long long ld = ctx->ld, N = ctx->N, nf1 = ctx->nf1, nb = ctx->nb;
@@ -351,11 +412,6 @@ int allocate(mbd_ctx *ctx) {
     const size_t emat = sizeof(double) * static_cast<size_t>(ctx->lde) * ctx->lde;
     const bool embed = ctx->periodic && !fp64_path(prec);
     if (embed) bytes += 5 * emat;
-    const size_t split_work = prec == MBD_PREC_FP64_SPLIT ? al(gemm_f64_split_work_bytes(static_cast<int>(ld),
-                                                                                          static_cast<int>(ld),
-                                                                                          static_cast<int>(ld)))
-                                                          : 0;
-    bytes += split_work;
     bytes += 12 * split_mat;
     // FP32 screening factors, their diagonal-block inverses and solve workspace
     const size_t panel_words = 2 * nf1 * static_cast<size_t>(ld) * kScsPanel;
@@ -366,15 +422,28 @@ int allocate(mbd_ctx *ctx) {
                                    al(sizeof(float) * grad32)
                              : 0;
     bytes += scs32;
+    const size_t crt_work = fp64_path(prec) && !ctx->periodic ? al(crt_ns_bytes(ctx->n)) + mat : 0;
     // A slab large enough for the new size is re-carved in place (systems of varying size in
     // a batch then reuse one allocation); otherwise it is replaced.
     cudaError_t e = cudaSuccess;
-    if (!ctx->slab || ctx->slab_bytes < bytes) {
+    if (!ctx->slab || ctx->slab_bytes < bytes + crt_work) {
         release(ctx);
-        e = cudaMalloc(&ctx->slab, bytes);
-        if (e != cudaSuccess) return cuda_fail(ctx, "mbd_set_geometry", e);
-        ctx->slab_bytes = bytes;
+        size_t want = bytes + crt_work;
+        e = cudaMalloc(&ctx->slab, want);
+        if (e != cudaSuccess && crt_work) {   // without the tensor-core products' scratch
+            cudaGetLastError();
+            want = bytes;
+            e = cudaMalloc(&ctx->slab, want);
+        }
+        if (e != cudaSuccess) {
+            ctx->slab = nullptr;
+            return cuda_fail(ctx, "mbd_set_geometry", e);
+        }
+        ctx->slab_bytes = want;
     }
+    const bool crt = crt_work && ctx->slab_bytes >= bytes + crt_work;
+    ctx->dPT = crt ? reinterpret_cast<double *>(static_cast<char *>(ctx->slab) + bytes) : nullptr;
+    ctx->crt = crt ? static_cast<char *>(ctx->slab) + bytes + mat : nullptr;
     char *p = static_cast<char *>(ctx->slab);
     for (auto &q : plan) {
         *q.first = reinterpret_cast<double *>(p);
@@ -388,10 +457,6 @@ int allocate(mbd_ctx *ctx) {
     for (auto m : mats) {
         *m = reinterpret_cast<double *>(p);
         p += matq;
-    }
-    if (split_work) {
-        ctx->dsplit = p;
-        p += split_work;
     }
     if (!fp64_path(prec)) {
         float **f32[6] = {&ctx->fY, &ctx->fZ, &ctx->fY2, &ctx->fZ2, &ctx->fP, &ctx->fPT};
@@ -1057,18 +1122,11 @@ int run(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &out, bool
     const long long launches0 = launch_count();
     cudaEvent_t e_start = nullptr, e_scs = nullptr, e_ns = nullptr, e_grad = nullptr, e_corr = nullptr;
     std::vector<Span> gemms, tc_spans;
-    cudaError_t split_err = cudaSuccess;   // first launch error of the split FP64 GEMM
     auto timed_gemm = [&](const GemmArgs &g, double flops) {
         Span sp;
         sp.flops = flops;
         mark(ctx, s, sp.a);
-        if (ctx->opt.precision == MBD_PREC_FP64_SPLIT) {
-            const cudaError_t e = gemm_f64_split(g.trans_b, g.mode, g.M, g.N, g.K, g.alpha, g.A, g.lda, g.B, g.ldb,
-                                                 g.beta, g.D, g.ldd, g.C, g.ldc, ctx->dsplit, ctx->dstatus, s);
-            if (e != cudaSuccess && split_err == cudaSuccess) split_err = e;
-        } else {
-            gemm_f64(g, s);
-        }
+        gemm_f64(g, s);
         mark(ctx, s, sp.b);
         if (ctx->profiling) gemms.push_back(sp);
     };
@@ -1173,6 +1231,8 @@ int run(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &out, bool
         scale_matrix(Y, ld, 1.0 / sc, s);
         set_identity(Z, ld, s);
         const int M = static_cast<int>(ld);
+        CrtProducts crt(ctx, s);
+        cudaError_t ce = cudaSuccess;
         bool converged = false;
         double resid = 0.0;
         int it = 0;
@@ -1180,8 +1240,18 @@ int run(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &out, bool
             // P = Z Y (not symmetric once rounding separates Z and Y; computed in full)
             const double *Pk = Y;   // Z_0 = I: P_0 = Y_0
             if (it > 0) {
-                GemmArgs g{Z, Y, nullptr, P, ld, ld, 0, ld, 0, 0, 0, 0, M, M, M, 1, 1.0, 0.0, 0, 0};
-                timed_gemm(g, flops_full);
+                if (ctx->crt) {
+                    Span sp;
+                    sp.flops = flops_full;
+                    mark(ctx, s, sp.a);
+                    ce = crt.product(Z, Y, P, ctx->dPT);
+                    mark(ctx, s, sp.b);
+                    if (ctx->profiling) gemms.push_back(sp);
+                    if (ce != cudaSuccess) return cuda_fail(ctx, "newton_schulz", ce);
+                } else {
+                    GemmArgs g{Z, Y, nullptr, P, ld, ld, 0, ld, 0, 0, 0, 0, M, M, M, 1, 1.0, 0.0, 0, 0};
+                    timed_gemm(g, flops_full);
+                }
                 Pk = P;
             }
             frob_dev_identity(Pk, ld, n, ctx->dscal + 2, s);
@@ -1204,14 +1274,23 @@ int run(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &out, bool
             // Z Y Z are symmetric for any symmetric Y, Z, so only their upper tiles are
             // computed.  (Using P^T in place of P, i.e. Y Y Z, breaks the coupling and makes
             // rounding errors grow by about sqrt(cond Q)/2 per step.)
-            GemmArgs gy{Y, Pk, Y, Y2, ld, ld, ld, ld, 0, 0, 0, 0, M, M, M, 1, c3, c1, 2, 0};
-            timed_gemm(gy, flops_sym);
-            if (it == 0) {
-                axpby_identity(Z2, Pk, ld, c1, c3, s);
+            if (ctx->crt) {
+                Span sp;
+                sp.flops = it == 0 ? flops_sym : 2.0 * flops_sym;
+                mark(ctx, s, sp.a);
+                ce = it == 0 ? crt.first_step(Y, Y2, c1, c3) : crt.step(Y, Z, P, ctx->dPT, Y2, Z2, c1, c3);
+                mark(ctx, s, sp.b);
+                if (ctx->profiling) gemms.push_back(sp);
+                if (ce != cudaSuccess) return cuda_fail(ctx, "newton_schulz", ce);
             } else {
-                GemmArgs gz{Pk, Z, Z, Z2, ld, ld, ld, ld, 0, 0, 0, 0, M, M, M, 1, c3, c1, 2, 0};
-                timed_gemm(gz, flops_sym);
+                GemmArgs gy{Y, Pk, Y, Y2, ld, ld, ld, ld, 0, 0, 0, 0, M, M, M, 1, c3, c1, 2, 0};
+                timed_gemm(gy, flops_sym);
+                if (it > 0) {
+                    GemmArgs gz{Pk, Z, Z, Z2, ld, ld, ld, ld, 0, 0, 0, 0, M, M, M, 1, c3, c1, 2, 0};
+                    timed_gemm(gz, flops_sym);
+                }
             }
+            if (it == 0) axpby_identity(Z2, Pk, ld, c1, c3, s);
             std::swap(Y, Y2);
             std::swap(Z, Z2);
             if (last) {
@@ -1222,12 +1301,11 @@ int run(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &out, bool
         }
         ctx->ns_iter = it;
         ctx->ns_resid = resid;
-        if (split_err != cudaSuccess) return cuda_fail(ctx, "newton_schulz_split", split_err);
-        if (ctx->opt.precision == MBD_PREC_FP64_SPLIT) {   // tensor-core waits are bounded: check them
+        if (ctx->crt) {   // tensor-core waits are bounded: check them
             int st = 0;
             MBD_CUDA(cudaMemcpyAsync(&st, ctx->dstatus, sizeof(int), cudaMemcpyDeviceToHost, s), "newton_schulz");
             MBD_CUDA(cudaStreamSynchronize(s), "newton_schulz");
-            if (st & ST_TC_TIMEOUT) return fail(ctx, MBD_ERR_CUDA, "newton_schulz_split", "tensor-core GEMM wait timed out");
+            if (st & ST_TC_TIMEOUT) return fail(ctx, MBD_ERR_CUDA, "newton_schulz", "tensor-core GEMM wait timed out");
         }
         if (!converged)
             return fail(ctx, MBD_ERR_NOT_CONVERGED, "newton_schulz", "iteration cap reached");
