@@ -159,10 +159,10 @@ __host__ __device__ __forceinline__ float stored(float r, float m, float inv, fl
 
 // From the stored residues to the integer: sum_i y_i / m_i is x.y / P up to an integer.  It is summed
 // in units of 2^-96 in three words (the products below 2^40, their sums below 2^44), of which the
-// upper 64 bits as a signed fraction times P are the result; what is cut off is below P 2^-64, less
-// than the rounding of the rows left.
+// upper 64 bits as a signed fraction times P are the result, rounded to P 2^-64, which is less than
+// the rounding of the rows left.
 struct Words {
-    unsigned long long s0, s1, s2;
+    unsigned long long s0 = 1ull << 31, s1 = 0, s2 = 0;   // (the first rounds: a cut would bias every entry alike)
 };
 template <int I>
 __host__ __device__ __forceinline__ void accumulate(Words &w, uint32_t y) {

@@ -85,7 +85,9 @@ struct CrtShape {
 };
 struct CrtOperand {
     CrtShape shape;
-    __nv_bfloat16 *planes;
+    long long plane;         // entries of a plane
+    long long exp_stride;    // exponents of a batch item
+    __nv_bfloat16 *planes;   // [batch][moduli][rows][pitch]
     int *exps;
 };
 struct CrtResult {
@@ -95,14 +97,17 @@ struct CrtResult {
     long long ldd, ldc, ldt, sD, sC, sT;   // pitches and batch strides
     long long im_off;        // complex: from a real plane to its imaginary one (D, C, T)
     int col0;                // the product's first column in D, C and T
-    bool sym;                // square results known to be symmetric (Hermitian): entries on or above the
-                             // diagonal, mirrored exactly
+    int sym;                 // square results: 1 symmetric (Hermitian) ones, the entries on or above the diagonal,
+                             // mirrored exactly; 2 the entries on or below it only
 };
 CrtShape crt_shape(int rows, int K, int batch, bool complex, bool right);
 size_t crt_operand_bytes(const CrtShape &s);
 size_t crt_bytes_bytes(int M, int N, int batch);
 CrtOperand crt_rows(const CrtShape &s, const double *re, const double *im, long long ld, long long stride, bool conj,
                     void *mem, cudaStream_t st);
+// The products' residues alone, [batch][moduli][M][N up to 16], half as sym (whole tiles).
+cudaError_t crt_products(const CrtOperand &A, const CrtOperand &B, int M, int half, void *bytes, int *err,
+                         cudaStream_t st);
 cudaError_t crt_multiply(const CrtOperand &A, const CrtOperand &B, const CrtResult &r, void *bytes, int *err,
                          cudaStream_t st);
 // C = alpha A B + beta D for real operands of any size through crt_gemm_bytes of scratch, in panels

@@ -6,12 +6,12 @@
 //   k_crt_gemm    the products of the planes, each reduced by its modulus to one byte per entry
 //   k_crt_result  bytes -> FP64, with alpha, beta D, and the mirrored or transposed copies
 #include <algorithm>
+#include <atomic>
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
-#include <math_constants.h>
 
-#include "crt64.cuh"
+#include "crt_dev.cuh"
 #include "internal.h"
 #include "tc_ops.cuh"
 
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(128) k_crt_rows(RowsArgs g) {
 }
 
 // ---- products -------------------------------------------------------------------------------
-// Work item: (batch item, modulus, tile of 256 x 256 entries).  A cluster of two CTAs computes it
+// Work item: (batch item, modulus, tile of 256 x kN entries).  The wide form, kN = 256:  a cluster of two CTAs computes it
 // with tcgen05.mma.cta_group::2 (M = 256, N = 256): CTA r stages rows 128 r .. 128 r + 127 of A's and of B's
 // 256 (32 KB per stage of 64 entries, six stages), so the two together load 64 KB for 512 cycles of
 // MMA, and holds rows 128 r .. of the tile in its tensor memory, in two buffers of 256 columns.
@@ -188,11 +188,15 @@ __global__ void __launch_bounds__(128) k_crt_rows(RowsArgs g) {
 // neighbouring tiles in L2.  Barriers as in the CTA-pair GEMM (k_tc.cu): full, cfree on the even CTA; empty,
 // cfull, done in both.  Every wait is bounded; on a timeout the kernel raises ST_TC_TIMEOUT,
 // waits (bounded) for its copies and MMAs, frees its tensor memory and returns.
-constexpr int kTileM = 256, kTileN = 256;
+// Narrow tiles (256 x 64) serve the Cholesky factorisation's 64-column blocks and small matrices.
+constexpr int kTileM = 256;
 constexpr int kHalfBytes = 128 * 128;              // 128 rows of 64 bf16
-constexpr int kStageBytes = 2 * kHalfBytes;        // per CTA
-constexpr int kStages = 6;
-constexpr int kSmem = kStages * kStageBytes + 1024 + 256;
+template <int kN>
+struct Tile {
+    static constexpr int kStageBytes = kHalfBytes + kN / 2 * 128;   // per CTA
+    static constexpr int kStages = kN == 256 ? 6 : 8;
+    static constexpr int kSmem = kStages * kStageBytes + 1024 + 256;
+};
 constexpr int kWarps = 10;                         // 8 epilogue, TMA, MMA
 
 __constant__ float c_m[kMod] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197};
@@ -205,7 +209,7 @@ __constant__ float c_back[kMod] = {
 struct GemmCrt {
     int M, N, K;             // K: entries of a plane's row (a multiple of 8; the tail reads as zeros)
     int batch, tiles_m, tiles_n, tiles;
-    int upper;               // tiles on or above the diagonal only
+    int half;                // 1: tiles on or above the diagonal only, 2: on or below it
     uint8_t *Y;              // [batch][kMod][M][ldy]
     long long ldy;
     int *err;
@@ -247,9 +251,10 @@ __device__ __forceinline__ void tma_load_3d_pair(void *dst, const CUtensorMap *m
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
-// bf16 operands, FP32 accumulator, both K-major, M = 256 (two CTAs), N = 256.
+// bf16 operands, FP32 accumulator, both K-major, M = 256 (two CTAs), N = kN.
+template <int kN>
 __device__ __forceinline__ void mma_pair(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc) {
-    constexpr uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(kTileN >> 3) << 17) |
+    constexpr uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(kN >> 3) << 17) |
                             (static_cast<uint32_t>(kTileM >> 4) << 24);
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
@@ -260,15 +265,15 @@ __device__ __forceinline__ void commit_pair(uint32_t cluster_addr) {
                  : "memory");
 }
 
-// Tile t of the walk: columns of tiles in groups of eight rows, or (upper) column by column down to the
-// diagonal.
+// Tile t of the walk: columns of tiles in groups of eight rows, or the triangle's columns (rows).
 __device__ __forceinline__ void crt_tile(const GemmCrt &g, int t, int &tm, int &tn) {
-    if (g.upper) {
+    if (g.half) {
         int c = static_cast<int>((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
         while ((c + 1) * (c + 2) / 2 <= t) ++c;
         while (c * (c + 1) / 2 > t) --c;
-        tn = c;
-        tm = t - c * (c + 1) / 2;
+        const int r = t - c * (c + 1) / 2;   // r <= c
+        tm = g.half == 1 ? r : c;
+        tn = g.half == 1 ? c : r;
         return;
     }
     const int group = t / (8 * g.tiles_n), first = group * 8, rows = min(8, g.tiles_m - first);
@@ -277,8 +282,10 @@ __device__ __forceinline__ void crt_tile(const GemmCrt &g, int t, int &tm, int &
     tn = l / rows;
 }
 
+template <int kN>
 __global__ void __launch_bounds__(32 * kWarps, 1)
     k_crt_gemm(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, GemmCrt g) {
+    constexpr int kStages = Tile<kN>::kStages, kStageBytes = Tile<kN>::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes);
@@ -310,7 +317,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(su32(tmem_slot)),
-                     "r"(2 * kTileN));
+                     "r"(2 * kN));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n");
     }
     fence_before();
@@ -330,7 +337,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
                 const int z = w / g.tiles;   // (batch item, modulus)
                 int tm, tn;
                 crt_tile(g, w - z * g.tiles, tm, tn);
-                const int ya = tm * kTileM + static_cast<int>(rank) * 128, yb = tn * kTileN + static_cast<int>(rank) * 128;
+                const int ya = tm * kTileM + static_cast<int>(rank) * 128, yb = tn * kN + static_cast<int>(rank) * (kN / 2);
                 for (int kt = 0; kt < nk && !*abort_flag; ++kt, ++kg) {
                     const int s = kg % kStages;
                     if (kg >= kStages && !mbar_wait_cl(&empty[s], ((kg / kStages) & 1) ^ 1, g.err)) {
@@ -372,10 +379,10 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
                         break;
                     }
                     fence_after();
-                    const uint32_t base = su32(smem + s * kStageBytes), dt = tmem + static_cast<uint32_t>(buf * kTileN);
+                    const uint32_t base = su32(smem + s * kStageBytes), dt = tmem + static_cast<uint32_t>(buf * kN);
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        mma_pair(dt, sdesc(base + k * 32), sdesc(base + kHalfBytes + k * 32), (in | k) != 0 ? 1u : 0u);
+                        mma_pair<kN>(dt, sdesc(base + k * 32), sdesc(base + kHalfBytes + k * 32), (in | k) != 0 ? 1u : 0u);
                     commit_pair(su32(&empty[s]));
                     commit_pair(peer_addr(su32(&empty[s]), 1));
                     if (in == crt::kChunk - 1 || kt == nk - 1) {
@@ -389,6 +396,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
         }
     } else {
         // ---- epilogue: lane quarter q of this CTA's 128 rows, column half h; thread = row ----
+        constexpr int kHalf = kN / 2;   // columns of a thread
         const int q = warp & 3, h = warp >> 2;
         const uint32_t cfree_pair = lead ? su32(&cfree[0]) : peer_addr(su32(&cfree[0]), 0);
         bool ok = true;
@@ -398,9 +406,9 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
             int tm, tn;
             crt_tile(g, w - z * g.tiles, tm, tn);
             const float m = c_m[z % kMod], back = c_back[z % kMod], inv = 1.0f / m;
-            float acc[128];
+            float acc[kHalf];
 #pragma unroll
-            for (int j = 0; j < 128; ++j) acc[j] = 0.f;
+            for (int j = 0; j < kHalf; ++j) acc[j] = 0.f;
             for (int c = 0; c < nchunks; ++c) {
                 const int buf = (cg + c) & 1;
                 ok = mbar_wait_cl(&cfull[buf], ((cg + c) >> 1) & 1, g.err) && !*abort_flag;
@@ -410,9 +418,9 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
                     break;
                 }
                 fence_after();
-                const uint32_t tb = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(buf * kTileN + h * 128);
+                const uint32_t tb = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(buf * kN + h * kHalf);
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {
+                for (int p = 0; p < kHalf / 32; ++p) {
                     uint32_t r[32];
                     tmem_ld32(tb + p * 32, r);
 #pragma unroll
@@ -428,9 +436,9 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
             const long long row = static_cast<long long>(tm) * kTileM + rank * 128 + q * 32 + lane;
             if (!ok) break;
             uint8_t *y = g.Y + (static_cast<long long>(z) * g.M + row) * g.ldy;
-            const int n0 = tn * kTileN + h * 128;
+            const int n0 = tn * kN + h * kHalf;
 #pragma unroll
-            for (int p = 0; p < 8; ++p) {
+            for (int p = 0; p < kHalf / 16; ++p) {
                 if (row >= g.M || n0 + 16 * p >= g.N) continue;   // ldy is a multiple of 16 not below N
                 uint32_t v[4];
 #pragma unroll
@@ -453,7 +461,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
         if (lane == 0) mbar_wait_cl(done, 0, g.err);
         __syncwarp();
         fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(2 * kTileN));
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(2 * kN));
     }
     __syncthreads();
     cluster_sync();
@@ -467,8 +475,8 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
 struct ResultArgs {
     const uint8_t *Y;
     long long ldy;
-    const int *ea, *eb;      // [batch][a_rows], [batch][N]
-    int a_rows, M, N, batch, n;      // n: columns of one part (N, or the complex product's half)
+    const int *ea, *eb;      // [batch][a_rows], [batch][b_rows]
+    int a_rows, b_rows, M, batch, n;      // n: columns of one part (all, or the complex product's half)
     int second;              // complex: first column of the imaginary part (0: real)
     double alpha, beta;
     const double *D;         // C and D: real plane, the imaginary one im_off further on
@@ -476,36 +484,30 @@ struct ResultArgs {
     long long ldd, ldc, ldt, sD, sC, sT, im_off;
     int col0;                // first column of C that this product covers
     int sym;                 // 0: all entries; 1: those on or above the diagonal, mirrored (the imaginary
-                             // part with its sign changed)
+                             // part with its sign changed); 2: those on or below it, not mirrored
 };
 
-// v 2^-(ea + eb): the exponent field directly while the result stays a normal number.
-__device__ __forceinline__ double scaled_down(double v, int ea, int eb) {
-    if (ea == crt::kBadRow || eb == crt::kBadRow) return CUDART_NAN;
-    const int e = ea + eb, hi = __double2hiint(v), f = (hi >> 20) & 0x7ff, to = f - e;
-    if (f > 0 && f < 2047 && to > 0 && to < 2047) return __hiloint2double(hi - (e << 20), __double2loint(v));
-    return v == 0.0 ? v : scalbn(v, -e);
-}
+__device__ __forceinline__ bool kept(int sym, int r, int c) { return sym == 0 || (sym == 1 ? c >= r : c <= r); }
 
 __global__ void __launch_bounds__(256) k_crt_result(ResultArgs g, int tiles_c) {
     __shared__ double tile[32][129];
     const long long b = blockIdx.z;
     const int part = blockIdx.y;   // 0 real, 1 imaginary
     const int r0 = (blockIdx.x / tiles_c) * 32, c0 = (blockIdx.x % tiles_c) * 128;
-    if (g.sym && g.col0 + c0 + 127 < r0) return;
+    if (g.sym == 1 ? g.col0 + c0 + 127 < r0 : g.sym && g.col0 + c0 > r0 + 31) return;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int c = c0 + 4 * tx, gc = g.col0 + c;
     double *C = g.C + b * g.sC + part * g.im_off;
     int eb[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) eb[j] = c + j < g.n ? g.eb[b * g.N + part * g.second + c + j] : 0;
+    for (int j = 0; j < 4; ++j) eb[j] = c + j < g.n ? g.eb[b * g.b_rows + part * g.second + c + j] : 0;
     const double unit = g.alpha * crt::kProduct;
     for (int i = ty; i < 32; i += 8) {
         const int r = r0 + i;
         double v[4] = {0.0, 0.0, 0.0, 0.0};
         if (r < g.M && c < g.n) {
             const uint8_t *y = g.Y + (b * kMod * g.M + r) * g.ldy + part * g.second + c;
-            crt::Words s[4] = {};
+            crt::Words s[4];
             crt::each_modulus([&](auto I) {
                 constexpr int k = decltype(I)::value;
                 const uint32_t p = *reinterpret_cast<const uint32_t *>(y + k * g.M * g.ldy);
@@ -515,27 +517,27 @@ __global__ void __launch_bounds__(256) k_crt_result(ResultArgs g, int tiles_c) {
             const int e = g.ea[b * g.a_rows + r];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                v[j] = scaled_down(static_cast<double>(crt::fraction(s[j])) * unit, e, eb[j]);
-                if (g.beta != 0.0 && c + j < g.n && (!g.sym || gc + j >= r))
+                v[j] = crt::scaled_down(static_cast<double>(crt::fraction(s[j])) * unit, e, eb[j]);
+                if (g.beta != 0.0 && c + j < g.n && kept(g.sym, r, gc + j))
                     v[j] += g.beta * g.D[b * g.sD + part * g.im_off + r * g.ldd + gc + j];
                 if (g.sym && part && gc + j == r) v[j] = 0.0;   // a Hermitian result's diagonal is real
             }
             double *out = C + r * g.ldc + gc;
-            if (c + 3 < g.n && (!g.sym || gc >= r)) {
+            if (c + 3 < g.n && kept(g.sym, r, gc) && kept(g.sym, r, gc + 3)) {
                 reinterpret_cast<double2 *>(out)[0] = make_double2(v[0], v[1]);
                 reinterpret_cast<double2 *>(out)[1] = make_double2(v[2], v[3]);
             } else {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    if (c + j < g.n && (!g.sym || gc + j >= r)) out[j] = v[j];
+                    if (c + j < g.n && kept(g.sym, r, gc + j)) out[j] = v[j];
             }
         }
-        if (g.sym || g.T) {
+        if (g.sym == 1 || g.T) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) tile[i][4 * tx + j] = v[j];
         }
     }
-    if (!g.sym && !g.T) return;
+    if (g.sym != 1 && !g.T) return;
     __syncthreads();
     const double sign = g.sym && part ? -1.0 : 1.0;
     double *out = g.sym ? C : g.T + b * g.sT + part * g.im_off;
@@ -559,14 +561,14 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-// Planes [z][rows][pitch] of bf16, boxes of 128 rows by 64 entries of one plane, 128-byte swizzle.
+// Planes [z][rows][pitch] of bf16, boxes of box_rows rows by 64 entries of one plane, 128-byte swizzle.
 bool plane_map(CUtensorMap *m, const void *base, long long K, long long rows, long long z, long long pitch,
-               long long plane) {
+               long long plane, int box_rows) {
     auto fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(K), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(z)};
     cuuint64_t strides[2] = {static_cast<cuuint64_t>(2 * pitch), static_cast<cuuint64_t>(2 * plane)};
-    cuuint32_t box[3] = {crt::kStageK, 128, 1};
+    cuuint32_t box[3] = {crt::kStageK, static_cast<cuuint32_t>(box_rows), 1};
     cuuint32_t es[3] = {1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, es,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -599,9 +601,9 @@ size_t crt_bytes_bytes(int M, int N, int batch) { return static_cast<size_t>(up(
 
 CrtOperand crt_rows(const CrtShape &s, const double *re, const double *im, long long ld, long long stride, bool conj,
                     void *mem, cudaStream_t st) {
-    CrtOperand o{s, static_cast<__nv_bfloat16 *>(mem),
-                 reinterpret_cast<int *>(static_cast<char *>(mem) + up(2LL * kMod * s.batch * s.out_rows * s.pitch, 256))};
     const long long plane = s.out_rows * s.pitch;
+    CrtOperand o{s, plane, s.out_rows, static_cast<__nv_bfloat16 *>(mem),
+                 reinterpret_cast<int *>(static_cast<char *>(mem) + up(2LL * kMod * s.batch * plane, 256))};
     RowsArgs g{re, s.complex ? im : nullptr, ld, stride, s.rows, s.K, s.right, conj, s.half, s.second, o.planes, s.pitch,
                plane, kMod * plane, o.exps, s.out_rows};
     count_launches(1);
@@ -611,66 +613,89 @@ CrtOperand crt_rows(const CrtShape &s, const double *re, const double *im, long 
     return o;
 }
 
-cudaError_t crt_multiply(const CrtOperand &A, const CrtOperand &B, const CrtResult &r, void *bytes, int *err,
-                         cudaStream_t st) {
+namespace {
+
+template <int kN>
+cudaError_t launch_gemm(const CrtOperand &A, const CrtOperand &B, GemmCrt &g, cudaStream_t st) {
     const CrtShape &a = A.shape, &b = B.shape;
-    if (a.pitch != b.pitch || a.batch != b.batch || a.complex != b.complex || (a.complex && (a.right || !b.right)))
-        return cudaErrorInvalidValue;
-    // a symmetric result needs the rows above its last column only
-    const int M = r.sym ? std::min(a.rows, r.col0 + b.rows) : a.rows, N = b.out_rows;
     CUtensorMap ma, mb;
     const long long z = static_cast<long long>(kMod) * a.batch;
-    if (!plane_map(&ma, A.planes, a.pitch, a.out_rows, z, a.pitch, a.out_rows * a.pitch) ||
-        !plane_map(&mb, B.planes, b.pitch, b.out_rows, z, b.pitch, b.out_rows * b.pitch))
+    if (!plane_map(&ma, A.planes, g.K, a.out_rows, z, a.pitch, A.plane, 128) ||
+        !plane_map(&mb, B.planes, g.K, b.out_rows, z, b.pitch, B.plane, kN / 2))
         return cudaErrorInvalidValue;
-    GemmCrt g{};
-    g.M = M;
-    g.N = N;
-    g.K = static_cast<int>(a.pitch);
-    g.batch = a.batch;
-    g.tiles_m = (M + kTileM - 1) / kTileM;
-    g.tiles_n = (N + kTileN - 1) / kTileN;
-    g.upper = r.sym && !a.complex && M == N && r.col0 == 0;
-    g.tiles = g.upper ? g.tiles_n * (g.tiles_n + 1) / 2 : g.tiles_m * g.tiles_n;
-    g.Y = static_cast<uint8_t *>(bytes);
-    g.ldy = up(N, 16);
-    g.err = err;
-    static int max_clusters = 0;   // the same for every device of this kind
+    g.tiles_m = (g.M + kTileM - 1) / kTileM;
+    g.tiles_n = (g.N + kN - 1) / kN;
+    g.tiles = g.half ? g.tiles_n * (g.tiles_n + 1) / 2 : g.tiles_m * g.tiles_n;
+    static std::atomic<int> resident{0};   // clusters at one time, the same for every device of this kind
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.blockDim = dim3(32 * kWarps);
-    cfg.dynamicSmemBytes = kSmem;
+    cfg.dynamicSmemBytes = Tile<kN>::kSmem;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaFuncSetAttribute(k_crt_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    cudaError_t e = cudaFuncSetAttribute(k_crt_gemm<kN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<kN>::kSmem);
     if (e != cudaSuccess) return e;
-    if (!max_clusters) {
-        int dev = 0, sms = 0, n = 0;
+    int most = resident.load();
+    if (!most) {
+        int dev = 0, sms = 0;
         e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cfg.gridDim = dim3(static_cast<unsigned>(sms & ~1));
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_crt_gemm, &cfg);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&most, k_crt_gemm<kN>, &cfg);
         if (e != cudaSuccess) return e;
-        if (n < 1) return cudaErrorInvalidConfiguration;
-        max_clusters = n;
+        if (most < 1) return cudaErrorInvalidConfiguration;
+        resident.store(most);
     }
     const long long items = static_cast<long long>(g.tiles) * kMod * a.batch;
-    cfg.gridDim = dim3(static_cast<unsigned>(2 * std::min<long long>(items, max_clusters)));
+    cfg.gridDim = dim3(static_cast<unsigned>(2 * std::min<long long>(items, most)));
     count_launches(1);
-    e = cudaLaunchKernelEx(&cfg, k_crt_gemm, ma, mb, g);
+    return cudaLaunchKernelEx(&cfg, k_crt_gemm<kN>, ma, mb, g);
+}
+
+}  // namespace
+
+cudaError_t crt_products(const CrtOperand &A, const CrtOperand &B, int M, int half, void *bytes, int *err,
+                         cudaStream_t st) {
+    GemmCrt g{};
+    g.M = M;
+    g.N = B.shape.out_rows;
+    g.K = static_cast<int>(A.shape.K);
+    if (A.shape.complex) g.K = static_cast<int>(A.shape.pitch);
+    g.batch = A.shape.batch;
+    g.half = half;
+    g.Y = static_cast<uint8_t *>(bytes);
+    g.ldy = up(g.N, 16);
+    g.err = err;
+    // narrow tiles where wide ones would be mostly padding, or too few to go round
+    if (g.N <= 128) {
+        g.half = 0;
+        return launch_gemm<64>(A, B, g, st);
+    }
+    return launch_gemm<256>(A, B, g, st);
+}
+
+cudaError_t crt_multiply(const CrtOperand &A, const CrtOperand &B, const CrtResult &r, void *bytes, int *err,
+                         cudaStream_t st) {
+    const CrtShape &a = A.shape, &b = B.shape;
+    if (a.K != b.K || a.batch != b.batch || a.complex != b.complex || (a.complex && (a.right || !b.right)))
+        return cudaErrorInvalidValue;
+    // a symmetric result's upper half needs the rows above its last column only
+    const int M = r.sym == 1 ? std::min(a.rows, r.col0 + b.rows) : a.rows, N = b.out_rows;
+    const bool square = !a.complex && M == N && r.col0 == 0;
+    const cudaError_t e = crt_products(A, B, M, square ? r.sym : 0, bytes, err, st);
     if (e != cudaSuccess) return e;
     ResultArgs o{};
-    o.Y = g.Y;
-    o.ldy = g.ldy;
+    o.Y = static_cast<const uint8_t *>(bytes);
+    o.ldy = up(N, 16);
     o.ea = A.exps;
-    o.a_rows = a.out_rows;
     o.eb = B.exps;
+    o.a_rows = A.exp_stride;
+    o.b_rows = B.exp_stride;
     o.M = M;
-    o.N = N;
     o.batch = a.batch;
     o.n = b.rows;
     o.second = b.second;

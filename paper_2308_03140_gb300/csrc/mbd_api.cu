@@ -331,7 +331,7 @@ struct CrtProducts {
     CrtOperand rows(const double *X, int k) { return crt_rows(shape, X, nullptr, ctx->ld, 0, false, slot[k], s); }
     CrtResult result(double *C, double *T, double alpha, double beta, const double *D, bool sym) const {
         const long long ld = ctx->ld;
-        return CrtResult{alpha, beta, D, C, T, ld, ld, ld, 0, 0, 0, 0, 0, sym};
+        return CrtResult{alpha, beta, D, C, T, ld, ld, ld, 0, 0, 0, 0, 0, sym ? 1 : 0};
     }
     cudaError_t whole(const double *A, const double *Bt, const CrtResult &r) {
         return crt_gemm(A, ctx->ld, Bt, ctx->ld, ctx->n, ctx->n, ctx->n, r, ctx->crt, ctx->dstatus, s);
@@ -363,6 +363,40 @@ struct CrtProducts {
         return crt_multiply(oY, oY, r, bytes, ctx->dstatus, s);
     }
 };
+
+// Bloch vectors per complex product, and its scratch: as many as 2 GiB hold, which at order 768 is
+// 16, 48 times the chip in tiles (the full grid at once gains nothing and costs 7 GB).
+int crt_cell_group(int n, int nk) {
+    const size_t one = crt_operand_bytes(crt_shape(n, n, 1, true, false)) +
+                       crt_operand_bytes(crt_shape(n, n, 1, true, true)) +
+                       crt_bytes_bytes(n, crt_shape(n, n, 1, true, true).out_rows, 1);
+    return static_cast<int>(std::min<size_t>(nk, std::max<size_t>(1, (size_t{2} << 30) / one)));
+}
+size_t crt_cell_bytes(int n, int nk) {
+    const int g = crt_cell_group(n, nk);
+    return crt_operand_bytes(crt_shape(n, n, g, true, false)) + crt_operand_bytes(crt_shape(n, n, g, true, true)) +
+           crt_bytes_bytes(n, crt_shape(n, n, g, true, true).out_rows, g);
+}
+
+// C = alpha A B + beta D for the planar complex matrices of every Bloch vector, B from the rows of B^T
+// (conj: from the rows of a Hermitian B); T: also the transpose; sym: Hermitian results.
+cudaError_t crt_cell_product(mbd_ctx *ctx, const double *A, const double *Bt, bool conj, const double *D, double *C,
+                             double *T, double alpha, double beta, bool sym, cudaStream_t s) {
+    const int n = ctx->n, group = crt_cell_group(n, ctx->nk);
+    const long long ld = ctx->ld, m2 = ld * ld, st = 2 * m2;
+    for (int k0 = 0; k0 < ctx->nk; k0 += group) {
+        const int g = std::min(group, ctx->nk - k0);
+        const CrtShape sa = crt_shape(n, n, g, true, false), sb = crt_shape(n, n, g, true, true);
+        char *pb = ctx->crt + crt_operand_bytes(sa);
+        const CrtOperand a = crt_rows(sa, A + k0 * st, A + k0 * st + m2, ld, st, false, ctx->crt, s);
+        const CrtOperand b = crt_rows(sb, Bt + k0 * st, Bt + k0 * st + m2, ld, st, conj, pb, s);
+        const CrtResult r{alpha, beta, D ? D + k0 * st : nullptr, C + k0 * st, T ? T + k0 * st : nullptr,
+                          ld, ld, ld, st, st, st, m2, 0, sym ? 1 : 0};
+        const cudaError_t e = crt_multiply(a, b, r, pb + crt_operand_bytes(sb), ctx->dstatus, s);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
 
 // Carves the workspace out of one allocation (256-byte aligned pieces).
 int allocate(mbd_ctx *ctx) {
@@ -422,7 +456,8 @@ int allocate(mbd_ctx *ctx) {
                                    al(sizeof(float) * grad32)
                              : 0;
     bytes += scs32;
-    const size_t crt_work = fp64_path(prec) && !ctx->periodic ? al(crt_ns_bytes(ctx->n)) + mat : 0;
+    const size_t crt_work =
+        fp64_path(prec) ? al(ctx->periodic ? crt_cell_bytes(ctx->n, static_cast<int>(nk)) : crt_ns_bytes(ctx->n)) + matq : 0;
     // A slab large enough for the new size is re-carved in place (systems of varying size in
     // a batch then reuse one allocation); otherwise it is replaced.
     cudaError_t e = cudaSuccess;
@@ -443,7 +478,7 @@ int allocate(mbd_ctx *ctx) {
     }
     const bool crt = crt_work && ctx->slab_bytes >= bytes + crt_work;
     ctx->dPT = crt ? reinterpret_cast<double *>(static_cast<char *>(ctx->slab) + bytes) : nullptr;
-    ctx->crt = crt ? static_cast<char *>(ctx->slab) + bytes + mat : nullptr;
+    ctx->crt = crt ? static_cast<char *>(ctx->slab) + bytes + matq : nullptr;
     char *p = static_cast<char *>(ctx->slab);
     for (auto &q : plan) {
         *q.first = reinterpret_cast<double *>(p);
@@ -897,13 +932,20 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
     std::vector<Span> gemms;
     const double nd = static_cast<double>(n);
     const double flops_cplx = 8.0 * nd * nd * nd * nk;   // one complex product per Bloch vector
-    // herm: Hermitian result, upper tiles only (about half the work)
-    auto timed_cgemm = [&](const double *A, const double *B, const double *D, double *C, double alpha, double bt,
-                           bool herm) {
+    cudaError_t crt_err = cudaSuccess;   // first launch error of the tensor-core products
+    // herm: Hermitian result, of which one triangle is formed (about half the work on the FP64 pipe).
+    // Bt, conj: the rows of B^T for the tensor cores; T: also the transpose (there only).
+    auto timed_cgemm = [&](const double *A, const double *B, const double *Bt, bool conj, const double *D, double *C,
+                           double *T, double alpha, double bt, bool herm) {
         Span sp;
         sp.flops = herm ? 4.0 * nd * nd * (nd + 1.0) * nk : flops_cplx;
         mark(ctx, s, sp.a);
-        cgemm_f64(A, B, D, C, ld, nk, alpha, bt, herm, s);
+        if (ctx->crt) {
+            const cudaError_t e = crt_cell_product(ctx, A, Bt, conj, D, C, T, alpha, bt, herm, s);
+            if (crt_err == cudaSuccess) crt_err = e;
+        } else {
+            cgemm_f64(A, B, D, C, ld, nk, alpha, bt, herm, s);
+        }
         mark(ctx, s, sp.b);
         if (ctx->profiling) gemms.push_back(sp);
     };
@@ -1040,7 +1082,7 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
     for (; it < ctx->opt.ns_max_iter; ++it) {
         const double *Pk = Y;
         if (it > 0) {
-            timed_cgemm(Z, Y, nullptr, P, 1.0, 0.0, false);   // P = Z Y: not Hermitian in floating point
+            timed_cgemm(Z, Y, Y, true, nullptr, P, ctx->dPT, 1.0, 0.0, false);   // P = Z Y: not Hermitian in floating point
             Pk = P;
         }
         cfrob_dev_identity(Pk, ld, n, nk, ctx->dscal + 2, s);
@@ -1057,9 +1099,11 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
         const bool last = resid < ctx->opt.ns_tol;
         const ns::Coeffs cf = ns::step(lbound, ubound, last);
         const double c1 = cf.c1, c3 = cf.c3;
-        timed_cgemm(Y, Pk, Y, Y2, c3, c1, kHermitianNs);   // Y' = c1 Y + c3 Y P (Hermitian: Y Z Y)
+        // Y' = c1 Y + c3 Y P (Hermitian: Y Z Y; P_0 = Y_0)
+        timed_cgemm(Y, Pk, it == 0 ? Y : ctx->dPT, it == 0, Y, Y2, nullptr, c3, c1, kHermitianNs);
         if (it == 0) caxpby_identity(Z2, Pk, ld, nk, c1, c3, s);
-        else timed_cgemm(Pk, Z, Z, Z2, c3, c1, kHermitianNs);   // Z' = c1 Z + c3 P Z (Hermitian: Z Y Z)
+        else timed_cgemm(Pk, Z, Z, true, Z, Z2, nullptr, c3, c1, kHermitianNs);   // Z' = c1 Z + c3 P Z (Hermitian: Z Y Z)
+        if (crt_err != cudaSuccess) return cuda_fail(ctx, "newton_schulz", crt_err);
         std::swap(Y, Y2);
         std::swap(Z, Z2);
         if (last) {
@@ -1070,6 +1114,12 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
     }
     ctx->ns_iter = it;
     ctx->ns_resid = resid;
+    if (ctx->crt) {   // tensor-core waits are bounded: check them
+        int st = 0;
+        MBD_CUDA(cudaMemcpyAsync(&st, ctx->dstatus, sizeof(int), cudaMemcpyDeviceToHost, s), "newton_schulz");
+        MBD_CUDA(cudaStreamSynchronize(s), "newton_schulz");
+        if (st & ST_TC_TIMEOUT) return fail(ctx, MBD_ERR_CUDA, "newton_schulz", "tensor-core GEMM wait timed out");
+    }
     if (!converged) return fail(ctx, MBD_ERR_NOT_CONVERGED, "newton_schulz", "iteration cap reached");
     energy_trace_periodic(Y, ld, n, nk, ctx->dombar, N, ss, energy_out, s);
     ctx->Zlast = Z;
@@ -1087,7 +1137,7 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
     ctx->prof.launches = static_cast<int>(launch_count() - launches0);
     if (ctx->profiling) {
         mbd_profile &p = ctx->prof;
-        p.gemm_launches = 4 * static_cast<int>(gemms.size());
+        p.gemm_launches = (ctx->crt ? 1 : 4) * static_cast<int>(gemms.size());
         for (const Span &sp : gemms) {
             p.gemm_ms += span_ms(sp.a, sp.b);
             p.gemm_flops += sp.flops;

@@ -8,7 +8,7 @@ extern "C" size_t crt_real_bytes(int M, int N, int K) { return crt_gemm_bytes(M,
 extern "C" int crt_real(const double *A, long long lda, const double *Bt, long long ldb, int M, int N, int K, double alpha,
                         double beta, const double *D, long long ldd, double *C, long long ldc, double *T, long long ldt,
                         int sym, void *work, int *err) {
-    CrtResult r{alpha, beta, D, C, T, ldd, ldc, ldt, 0, 0, 0, 0, 0, sym != 0};
+    CrtResult r{alpha, beta, D, C, T, ldd, ldc, ldt, 0, 0, 0, 0, 0, sym};
     return static_cast<int>(crt_gemm(A, lda, Bt, ldb, M, N, K, r, work, err, nullptr));
 }
 
@@ -26,6 +26,6 @@ extern "C" int crt_complex(const double *A, const double *B, int conj, int n, lo
     p += crt_operand_bytes(sa);
     const CrtOperand b = crt_rows(sb, B, B + m2, ld, 2 * m2, conj != 0, p, nullptr);
     p += crt_operand_bytes(sb);
-    CrtResult r{alpha, beta, D, C, T, ld, ld, ld, 2 * m2, 2 * m2, 2 * m2, m2, 0, sym != 0};
+    CrtResult r{alpha, beta, D, C, T, ld, ld, ld, 2 * m2, 2 * m2, 2 * m2, m2, 0, sym};
     return static_cast<int>(crt_multiply(a, b, r, p, err, nullptr));
 }

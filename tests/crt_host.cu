@@ -33,7 +33,7 @@ extern "C" void crt_stored(int i, const float *r, int n, float *y) {
 }
 extern "C" double crt_result(const unsigned char *y, int n, long long *frac) {
     for (int j = 0; j < n; ++j) {
-        crt::Words w = {};
+        crt::Words w;
         crt::each_modulus([&](auto I) { crt::accumulate<decltype(I)::value>(w, y[decltype(I)::value * n + j]); });
         frac[j] = crt::fraction(w);
     }
