@@ -174,6 +174,12 @@ void axpby_identity(double *Z, const double *P, long long ld, double a, double b
 void cholesky_f64(double *A, long long ld, long long mstride, int batch, double *dinv,
                   int *status, cudaStream_t s);
 
+// The same factorisation with its products on the tensor cores (k_chol.cu), through
+// cholesky_crt_bytes of scratch; tensor-core timeouts set ST_TC_TIMEOUT in *status.  ld a multiple of 128.
+size_t cholesky_crt_bytes(long long ld, int batch);
+cudaError_t cholesky_crt(double *A, long long ld, long long mstride, int batch, double *dinv, void *work, int *status,
+                         cudaStream_t s);
+
 // Batched triangular solves with 3 right-hand sides, in place on X [b][ld][3]:
 // forward L y = x, then backward L^T z = y (L from cholesky_f64).  work: same shape
 // as X (the intermediate y).

@@ -398,6 +398,17 @@ cudaError_t crt_cell_product(mbd_ctx *ctx, const double *A, const double *Bt, bo
     return cudaSuccess;
 }
 
+// FP64 factors of a batch of matrices: on the tensor cores where their scratch is there.
+int factorise(mbd_ctx *ctx, double *A, int batch, cudaStream_t s, const char *origin) {
+    const long long ld = ctx->ld;
+    if (!ctx->crt) {
+        cholesky_f64(A, ld, ld * ld, batch, ctx->ddinv, ctx->dstatus, s);
+        return MBD_OK;
+    }
+    MBD_CUDA(cholesky_crt(A, ld, ld * ld, batch, ctx->ddinv, ctx->crt, ctx->dstatus, s), origin);
+    return MBD_OK;
+}
+
 // Carves the workspace out of one allocation (256-byte aligned pieces).
 int allocate(mbd_ctx *ctx) {
     const long long ld = ctx->ld, N = ctx->N, nf1 = ctx->nf1, nb = ctx->nb;
@@ -457,7 +468,9 @@ int allocate(mbd_ctx *ctx) {
                              : 0;
     bytes += scs32;
     const size_t crt_work =
-        fp64_path(prec) ? al(ctx->periodic ? crt_cell_bytes(ctx->n, static_cast<int>(nk)) : crt_ns_bytes(ctx->n)) + matq : 0;
+        fp64_path(prec) ? std::max(al(cholesky_crt_bytes(ld, static_cast<int>(nf1))),
+                                   al(ctx->periodic ? crt_cell_bytes(ctx->n, static_cast<int>(nk)) : crt_ns_bytes(ctx->n))) + matq
+                        : 0;
     // A slab large enough for the new size is re-carved in place (systems of varying size in
     // a batch then reuse one allocation); otherwise it is replaced.
     cudaError_t e = cudaSuccess;
@@ -686,6 +699,7 @@ int read_status(mbd_ctx *ctx, cudaStream_t s, const char *origin) {
     MBD_CUDA(cudaStreamSynchronize(s), origin);
     MBD_CUDA(cudaGetLastError(), origin);
     if (st & ST_INPUT) return fail(ctx, MBD_ERR_INPUT, origin, "non-finite or non-positive input, or coincident atoms");
+    if (st & ST_TC_TIMEOUT) return fail(ctx, MBD_ERR_CUDA, origin, "tensor-core GEMM wait timed out");
     if (st & ST_SCS_NOT_PD)
         return fail(ctx, MBD_ERR_SCS_NOT_PD, origin, "screening matrix alpha^-1 + T^scs is not positive definite");
     if (st & ST_NEG_ALPHA)
@@ -963,7 +977,7 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
         prepare_atoms(b, ctx->dstatus, s);
         structure_factors(b, pb, s);
         build_scs_periodic(b, ctx->cell, beta, a, ctx->dM, ld, mat, ctx->dstatus, s);
-        cholesky_f64(ctx->dM, ld, mat, nf1, ctx->ddinv, ctx->dstatus, s);
+        if (const int rf = factorise(ctx, ctx->dM, nf1, s, "screening")) return rf;
         init_rhs_identity(ctx->dX, ld, n, nf1, xs, s);
         chol_solve3_f64(ctx->dM, ld, mat, nf1, ctx->ddinv, ctx->dX, ctx->dB, xs, s);
         contract_screen(b, ctx->dX, ld, xs, ctx->dstatus, s);
@@ -1211,7 +1225,7 @@ int run(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &out, bool
         prepare_atoms(b, ctx->dstatus, s);
         build_scs(b, beta, a, ctx->dM, ld, mat, ctx->dstatus, s);
         if (fp64_path(ctx->opt.precision)) {
-            cholesky_f64(ctx->dM, ld, mat, nf1, ctx->ddinv, ctx->dstatus, s);
+            if (const int rf = factorise(ctx, ctx->dM, nf1, s, "screening")) return rf;
             init_rhs_identity(ctx->dX, ld, n, nf1, xs, s);
             chol_solve3_f64(ctx->dM, ld, mat, nf1, ctx->ddinv, ctx->dX, ctx->dB, xs, s);
         } else {   // FP32 factors, FP64-refined solutions
@@ -1713,7 +1727,7 @@ int mbd_screen(mbd_ctx *ctx, double *alpha_iu, double *alpha_free_iu, double *c6
     if (ctx->periodic) build_scs_periodic(b, ctx->cell, ctx->opt.beta, ctx->opt.a, ctx->dM, ld, mat, ctx->dstatus, s);
     else build_scs(b, ctx->opt.beta, ctx->opt.a, ctx->dM, ld, mat, ctx->dstatus, s);
     if (fp64_path(ctx->opt.precision) || ctx->periodic) {
-        cholesky_f64(ctx->dM, ld, mat, nf1, ctx->ddinv, ctx->dstatus, s);
+        if (const int rf = factorise(ctx, ctx->dM, nf1, s, "mbd_screen")) return rf;
         init_rhs_identity(ctx->dX, ld, n, nf1, xs, s);
         chol_solve3_f64(ctx->dM, ld, mat, nf1, ctx->ddinv, ctx->dX, ctx->dB, xs, s);
     } else {
@@ -1835,7 +1849,7 @@ int mbd_log_energy(mbd_ctx *ctx, int max_order, double *energy, double *orders) 
         }
     }
     add_identity_batch(A, ld, mat, nf, s);
-    cholesky_f64(A, ld, mat, nf, ctx->ddinv, ctx->dstatus, s);
+    if (const int rf = factorise(ctx, A, nf, s, "mbd_log_energy")) return rf;
     logdiag_batch(A, ld, mat, nf, sums, ctx->dstatus, s);
     std::vector<double> h(4 * nf);
     MBD_CUDA(cudaMemcpyAsync(h.data(), sums, sizeof(double) * 4 * nf, cudaMemcpyDeviceToHost, s), "mbd_log_energy");

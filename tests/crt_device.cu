@@ -29,3 +29,8 @@ extern "C" int crt_complex(const double *A, const double *B, int conj, int n, lo
     CrtResult r{alpha, beta, D, C, T, ld, ld, ld, 2 * m2, 2 * m2, 2 * m2, m2, 0, sym};
     return static_cast<int>(crt_multiply(a, b, r, p, err, nullptr));
 }
+
+extern "C" size_t crt_cholesky_bytes(long long ld, int batch) { return cholesky_crt_bytes(ld, batch); }
+extern "C" int crt_cholesky(double *A, long long ld, int batch, double *dinv, void *work, int *status) {
+    return static_cast<int>(cholesky_crt(A, ld, ld * ld, batch, dinv, work, status, nullptr));
+}

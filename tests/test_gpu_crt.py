@@ -214,3 +214,54 @@ def test_complex_products(dev, n, batch):
     torch.cuda.synchronize()
     near(back(c), H @ H, H, H, -2.0 * D)
     assert np.array_equal(back(c), np.conj(back(c).transpose(0, 2, 1))) and int(err.item()) == 0
+
+
+def _factor(L, A):
+    import torch
+    batch, ld = A.shape[:2]
+    a = _cuda(A)
+    dinv = torch.full((batch, ld // 64, 64, 64), float("nan"), dtype=torch.float64, device="cuda:0")
+    work = torch.empty(int(L.crt_cholesky_bytes(C.c_longlong(ld), batch)), dtype=torch.uint8, device="cuda:0")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda:0")
+    assert L.crt_cholesky(_p(a), C.c_longlong(ld), batch, _p(dinv), _p(work), _p(status)) == 0
+    torch.cuda.synchronize()
+    return np.tril(a.cpu().numpy()), dinv.cpu().numpy(), int(status.item())
+
+
+@pytest.mark.parametrize("ld,batch", [(128, 1), (256, 3), (512, 2), (640, 16), (1280, 2)])
+def test_cholesky_factors(dev, ld, batch):
+    # one and several panels, rows of very different size, poisoned upper halves.  A backward-stable
+    # factorisation leaves |A - L L^T|_ij <= (ld + 2) 2^-53 sqrt(A_ii A_jj) and some
+    rng = np.random.default_rng(ld)
+    dev.crt_cholesky_bytes.restype = C.c_size_t
+    A = np.zeros((batch, ld, ld))
+    for b in range(batch):
+        X = rng.normal(size=(ld, ld)) / np.sqrt(ld)
+        d = np.exp(rng.uniform(-4, 4, ld)) if b else np.ones(ld)
+        A[b] = (X @ X.T + np.diag(rng.uniform(1e-3, 1.0, ld))) * np.outer(d, d)
+    got, dinv, status = _factor(dev, np.where(np.tri(ld, dtype=bool), A, np.nan))
+    assert status == 0
+    size = np.sqrt(np.einsum("bi,bj->bij", A.diagonal(axis1=1, axis2=2), A.diagonal(axis1=1, axis2=2)))
+    back = got @ got.transpose(0, 2, 1)
+    assert np.all(np.abs(back - A) <= 2 * (ld + 2) * 2.0 ** -53 * size)
+    for b in range(batch):
+        for j in range(ld // 64):
+            blk = got[b, 64 * j:64 * j + 64, 64 * j:64 * j + 64]
+            tol = 8 * 64 * 2.0 ** -53 * (np.abs(dinv[b, j]) @ np.abs(blk))
+            assert np.all(np.abs(dinv[b, j] @ blk - np.eye(64)) <= tol + 1e-300)
+            assert np.all(np.triu(dinv[b, j], 1) == 0.0)
+
+
+def test_cholesky_flags_what_is_not_positive_definite(dev):
+    dev.crt_cholesky_bytes.restype = C.c_size_t
+    rng = np.random.default_rng(9)
+    X = rng.normal(size=(640, 640))
+    good = X @ X.T + np.eye(640)
+    for where in (0, 100, 600):
+        for value in (-1.0, 0.0, np.nan):
+            A = np.stack([good, good])
+            A[1, where, where] = value
+            assert _factor(dev, A)[2] == 2   # ST_SCS_NOT_PD
+    A = np.stack([good, good])
+    A[0, 630, 10] = A[0, 10, 630] = 1e6      # positive diagonal, negative eigenvalue
+    assert _factor(dev, A)[2] == 2
