@@ -6,8 +6,8 @@
 // A row a of the left operand is scaled by a power of two and rounded to integers x = rint(a 2^e)
 // with |x|_2 < sqrt(P/2), P the product of the moduli; likewise a column b of the right one.
 // Then |x.y| < P/2, so x.y is known from its residues: for each modulus m the tensor cores
-// sum products of residues in [-m/2 - 1, m/2 + 1] (exact in bf16: 8 bits), 512 of them at a time, so that
-// every partial sum is an integer below 2^23 + m and exact in FP32.  What is lost is only the rounding of x
+// sum products of residues in [-128, 128] (exact in bf16: 8 bits), 1024 of them at a time, so that
+// every partial sum is an integer of at most 2^24 and exact in FP32.  What is lost is only the rounding of x
 // and y: an error of about 0.4 2^-kRowBits |a| |b| in a.b, against about 0.2 2^-52 |a| |b| for an
 // FP64 sum of random terms, whose roundings grow with their number.
 #pragma once
@@ -29,7 +29,7 @@ constexpr int kMod = 15;   // P = 2^117.78; with 14 moduli (2^110.2) the small e
 constexpr int kModuli[kMod] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197};
 constexpr int kRowBits = 58;   // scaled rows have |x|_2 <= 0.65 * 2^(kRowBits + 1) < sqrt(P/2) = 2^58.39
 constexpr int kStageK = 64;    // K per shared-memory stage (128 bytes of bf16)
-constexpr int kChunk = 8;      // stages per FP32 accumulation: 512 products of at most 2^14
+constexpr int kChunk = 16;     // stages per FP32 accumulation: 1024 products of at most 2^14
 
 constexpr int mod_pow2(int k, int m) {   // 2^k mod m in [-m/2, m/2]
     int r = 1 % m;

@@ -182,8 +182,13 @@ __global__ void __launch_bounds__(128) k_crt_rows(RowsArgs g) {
 // 256 (32 KB per stage of 64 entries, six stages), so the two together load 64 KB for 512 cycles of
 // MMA, and holds rows 128 r .. of the tile in its tensor memory, in two buffers of 256 columns.
 // A single CTA on 128 x 256 tiles would load 48 KB in the same time, more than an SM takes in.
-// Every 512 products the eight epilogue warps add the buffer (exact integers) to their 128 sums a
-// thread and reduce them by the modulus, four FP32 operations an entry, while the other buffer fills.
+// Every 1024 products the eight epilogue warps reduce the buffer (exact integers) by the modulus and
+// add it to their 128 sums a thread, four FP32 operations an entry, while the other buffer fills.
+// The TMA and MMA warps run uniformly and issue from an elected lane: from a branch on the lane each MMA
+// took about 200 cycles to issue, more than its 128 to run (a whole product of order 6016 with its
+// conversions: 6.98 ms, 4.54 so, 4.30 with sums of 1024 products instead of 512; order 3000 1.06, then
+// 0.92, 0.90, and 0.71 with rows on 128-byte lines).  The MMAs alone run for 2.76 ms of the 3.3 ms of this
+// kernel at order 6016, the loads alone for 3.0 (17 TB/s out of L2), which bound it.
 // Clusters are persistent and walk the items in order, so that those in flight share a modulus and
 // neighbouring tiles in L2.  Barriers as in the CTA-pair GEMM (k_tc.cu): full, cfree on the even CTA; empty,
 // cfull, done in both.  Every wait is bounded; on a timeout the kernel raises ST_TC_TIMEOUT,
@@ -260,9 +265,13 @@ __device__ __forceinline__ void mma_pair(uint32_t tmem, uint64_t a, uint64_t b, 
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
         "l"(a), "l"(b), "r"(id), "r"(acc));
 }
-__device__ __forceinline__ void commit_pair(uint32_t cluster_addr) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(cluster_addr)
-                 : "memory");
+// Arrival on the barrier at this shared-memory address in both CTAs of the pair, once the MMAs so far
+// are done.
+__device__ __forceinline__ void commit_both(uint32_t addr) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n" ::"r"(addr),
+        "h"(static_cast<unsigned short>(3))
+        : "memory");
 }
 
 // Tile t of the walk: columns of tiles in groups of eight rows, or the triangle's columns (rows).
@@ -328,71 +337,72 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
     const int nk = (g.K + crt::kStageK - 1) / crt::kStageK;
     const int nchunks = (nk + crt::kChunk - 1) / crt::kChunk;
 
+    // A wait of the whole warp, and whether it may go on: every lane gets the same answer.
+    auto warp_wait = [&](uint64_t *bar, uint32_t parity) {
+        const bool ok = __all_sync(0xffffffffu, mbar_wait_cl(bar, parity, g.err) && !*abort_flag);
+        if (!ok) *abort_flag = 1;
+        return ok;
+    };
     if (warp == 8) {
         // ---- TMA: this CTA's rows of both operands, counted on the even CTA's full[s] ----
-        if (lane == 0) {
-            int issued = 0, kg = 0;
-            const uint32_t full_pair = peer_addr(su32(&full[0]), 0);
-            for (int w = cl; w < items && !*abort_flag; w += ncl) {
-                const int z = w / g.tiles;   // (batch item, modulus)
-                int tm, tn;
-                crt_tile(g, w - z * g.tiles, tm, tn);
-                const int ya = tm * kTileM + static_cast<int>(rank) * 128, yb = tn * kN + static_cast<int>(rank) * (kN / 2);
-                for (int kt = 0; kt < nk && !*abort_flag; ++kt, ++kg) {
-                    const int s = kg % kStages;
-                    if (kg >= kStages && !mbar_wait_cl(&empty[s], ((kg / kStages) & 1) ^ 1, g.err)) {
-                        *abort_flag = 1;
-                        break;
-                    }
+        const bool one = elected();
+        bool ok = true;
+        int issued = 0, kg = 0;
+        const uint32_t full_pair = peer_addr(su32(&full[0]), 0);
+        for (int w = cl; w < items && ok; w += ncl) {
+            const int z = w / g.tiles;   // (batch item, modulus)
+            int tm, tn;
+            crt_tile(g, w - z * g.tiles, tm, tn);
+            const int ya = tm * kTileM + static_cast<int>(rank) * 128, yb = tn * kN + static_cast<int>(rank) * (kN / 2);
+            for (int kt = 0; kt < nk; ++kt, ++kg) {
+                const int s = kg % kStages;
+                if (kg >= kStages && !(ok = warp_wait(&empty[s], ((kg / kStages) & 1) ^ 1))) break;
+                if (one) {
                     uint8_t *st = smem + s * kStageBytes;
                     if (lead) mbar_expect_tx(&full[s], 2 * kStageBytes);
                     const uint32_t fb = full_pair + static_cast<uint32_t>(s) * 8u;
                     tma_load_3d_pair(st, &mA, kt * crt::kStageK, ya, z, fb);
                     tma_load_3d_pair(st + kHalfBytes, &mB, kt * crt::kStageK, yb, z, fb);
-                    issued = kg + 1;
                 }
+                __syncwarp();
+                issued = kg + 1;
             }
-            if (*abort_flag) {   // let the copies land before shared memory is released (as in k_tc.cu)
-                if (lead) {
-                    for (int k = (issued > kStages ? issued - kStages : 0); k < issued; ++k)
-                        mbar_wait_cl(&full[k % kStages], (k / kStages) & 1, g.err, kSpinCycles / 8);
-                } else {
-                    const long long t0 = clock64();
-                    while (clock64() - t0 < 2000000LL) {
-                    }
+        }
+        if (!ok) {   // let the copies land before shared memory is released (as in k_tc.cu)
+            if (lead) {
+                for (int k = (issued > kStages ? issued - kStages : 0); k < issued; ++k)
+                    mbar_wait_cl(&full[k % kStages], (k / kStages) & 1, g.err, kSpinCycles / 8);
+            } else {
+                const long long t0 = clock64();
+                while (clock64() - t0 < 2000000LL) {
                 }
             }
         }
     } else if (warp == 9) {
-        if (lane == 0 && lead) {
+        if (lead) {
+            const bool one = elected();
+            bool ok = true;
             int kg = 0, cg = 0;
-            for (int w = cl; w < items && !*abort_flag; w += ncl, cg += nchunks) {
-                for (int kt = 0; kt < nk && !*abort_flag; ++kt, ++kg) {
-                    const int in = kt % crt::kChunk, c = cg + kt / crt::kChunk, buf = c & 1;
-                    if (in == 0 && c >= 2 && !mbar_wait_cl(&cfree[buf], ((c >> 1) - 1) & 1, g.err)) {
-                        *abort_flag = 1;
-                        break;
-                    }
-                    const int s = kg % kStages;
-                    if (!mbar_wait_cl(&full[s], (kg / kStages) & 1, g.err)) {
-                        *abort_flag = 1;
-                        break;
-                    }
+            for (int w = cl; w < items && ok; w += ncl, cg += nchunks) {
+                for (int kt = 0; kt < nk; ++kt, ++kg) {
+                    const int in = kt % crt::kChunk, c = cg + kt / crt::kChunk, buf = c & 1, s = kg % kStages;
+                    if (in == 0 && c >= 2 && !(ok = warp_wait(&cfree[buf], ((c >> 1) - 1) & 1))) break;
+                    if (!(ok = warp_wait(&full[s], (kg / kStages) & 1))) break;
                     fence_after();
                     const uint32_t base = su32(smem + s * kStageBytes), dt = tmem + static_cast<uint32_t>(buf * kN);
+                    if (one) {
+                        const uint64_t da = sdesc(base), db = sdesc(base + kHalfBytes);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        mma_pair<kN>(dt, sdesc(base + k * 32), sdesc(base + kHalfBytes + k * 32), (in | k) != 0 ? 1u : 0u);
-                    commit_pair(su32(&empty[s]));
-                    commit_pair(peer_addr(su32(&empty[s]), 1));
-                    if (in == crt::kChunk - 1 || kt == nk - 1) {
-                        commit_pair(su32(&cfull[buf]));
-                        commit_pair(peer_addr(su32(&cfull[buf]), 1));
+                        for (int k = 0; k < 4; ++k)   // 32 bytes of K: two 16-byte units of the descriptor
+                            mma_pair<kN>(dt, da + 2 * k, db + 2 * k, (in | k) != 0 ? 1u : 0u);
+                        commit_both(su32(&empty[s]));
+                        if (in == crt::kChunk - 1 || kt == nk - 1) commit_both(su32(&cfull[buf]));
                     }
+                    __syncwarp();
                 }
             }
-            commit_pair(su32(done));
-            commit_pair(peer_addr(su32(done), 1));
+            if (one) commit_both(su32(done));
+            __syncwarp();
         }
     } else {
         // ---- epilogue: lane quarter q of this CTA's 128 rows, column half h; thread = row ----
@@ -424,7 +434,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
                     uint32_t r[32];
                     tmem_ld32(tb + p * 32, r);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) acc[p * 32 + j] = crt::reduce(acc[p * 32 + j] + __uint_as_float(r[j]), m, inv);
+                    for (int j = 0; j < 32; ++j) acc[p * 32 + j] += crt::reduce(__uint_as_float(r[j]), m, inv);
                 }
                 fence_before();
                 __syncwarp();
@@ -446,7 +456,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
                     uint32_t b4[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
-                        b4[j] = __float_as_uint(crt::stored(acc[16 * p + 4 * u + j], m, inv, back) + 8388608.0f);
+                        b4[j] = __float_as_uint(crt::stored(crt::reduce(acc[16 * p + 4 * u + j], m, inv), m, inv, back) + 8388608.0f);
                     v[u] = __byte_perm(__byte_perm(b4[0], b4[1], 0x0040), __byte_perm(b4[2], b4[3], 0x0040), 0x5410);
                 }
                 *reinterpret_cast<uint4 *>(y + n0 + 16 * p) = make_uint4(v[0], v[1], v[2], v[3]);
@@ -585,7 +595,7 @@ CrtShape crt_shape(int rows, int K, int batch, bool complex, bool right) {
     s.rows = rows;
     s.K = K;
     s.batch = batch;
-    s.half = static_cast<int>(up(K, 8));
+    s.half = static_cast<int>(up(K, 64));   // rows on 128-byte lines
     s.second = complex && right ? static_cast<int>(up(rows, 16)) : 0;
     s.out_rows = rows + s.second;
     s.pitch = complex ? 2LL * s.half : s.half;

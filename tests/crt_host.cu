@@ -20,10 +20,10 @@ extern "C" void crt_residues(const long long *x, int n, float *r) {
     }
 }
 
-// One step of the products' running residue: (acc + v) mod m_i, as k_crt_gemm reduces a chunk's sum v.
-extern "C" void crt_reduce(int i, const float *acc, const float *v, int n, float *out) {
+// An accumulation's sum v mod m_i, as k_crt_gemm reduces it.
+extern "C" void crt_reduce(int i, const float *v, int n, float *out) {
     const float m = static_cast<float>(crt::kModuli[i]), inv = 1.0f / m;
-    for (int j = 0; j < n; ++j) out[j] = crt::reduce(acc[j] + v[j], m, inv);
+    for (int j = 0; j < n; ++j) out[j] = crt::reduce(v[j], m, inv);
 }
 
 // The stored byte of a residue, and the result from the bytes y [kMod][n]: x.y / P 2^64.
