@@ -120,8 +120,7 @@ cudaError_t crt_gemm(const double *A, long long lda, const double *Bt, long long
                      const CrtResult &r, void *work, int *err, cudaStream_t st);
 
 // Mixed-precision helpers: Y = scale Q (FP32 and, if Yh, bf16 hi/lo) and Z = I;
-// Z = a I + b P; Zd = scale Zf in FP64; and the variational energy
-// E = (1/4)(3 Tr V - sum V o W) - 3/2 sum omega (work: 608 doubles).
+// Z = a I + b P; Zd = scale Zf in FP64.
 void mixed_init(int kind, const double *Q, long long ld, double scale, float *Yf, void *Yh, void *Yl, float *Zf,
                 void *Zh, void *Zl, cudaStream_t s);
 void mixed_axpby_identity(int kind, const float *P, long long ld, float a, float b, float *Zf, void *Zh, void *Zl,
@@ -140,12 +139,10 @@ void diag_scale_rows_f64(const double *A, const float *B, long long ld, double s
 void diag_scale_rows_f32(const float *A, const double *B, long long ld, double *Out, cudaStream_t s);
 void split_tf32_f64_t(const double *A, long long ld, double scale, void *H, void *L, cudaStream_t s);   // of A^T
 // Energy of the mixed modes from T1 = Tr(scale Q Z) (FP64 dot), T2 = sum V o W:
-// E = (sqrt_s/4)(3 T1 - T2) - 3/2 sum omega; resid = |I - W|_F (work: 912 doubles).
+// E = (sqrt_s/4)(3 T1 - T2) - 3/2 sum omega; resid = |I - W|_F (work: 1824 doubles).
 void energy_correction(const double *Q, double scale, const float *Z, const double *V, const double *W, long long ld,
                        int n, double sqrt_s, const double *ombar, int N, double *work, double *out, double *resid,
                        cudaStream_t s);
-void energy_variational(const double *V, const double *W, long long ld, int n, const double *ombar, int N,
-                        double *work, double *out, cudaStream_t s);
 
 // ---- dense FP64 (k_dense.cu) ----------------------------------------------------
 // C[b] = alpha * A[b] op(B[b]) + beta * D[b] on 64x64 tiles, FP64 DMMA (mma.sync m8n8k4).

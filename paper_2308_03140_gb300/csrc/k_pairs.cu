@@ -15,6 +15,7 @@
 // The dipole tensors are written T_ab = P delta_ab + W r_a r_b with radial P, W.
 // Pair loops keep one CTA per "row" atom and stride over partner atoms, so every
 // per-atom sum is a fixed-order block reduction (deterministic, no atomics).
+#include "comp_sum.cuh"
 #include "internal.h"
 #include "pair_math.cuh"
 
@@ -258,39 +259,15 @@ __global__ void k_pad_q(double *Q, long long ld, int n, const double *ombar) {
     }
 }
 
-// E = 1/2 sqrt(s) Tr Y - 3/2 sum omega_bar, Neumaier-compensated, one CTA.
-__device__ __forceinline__ void two_sum(double a, double b, double &s, double &e) {
-    s = a + b;
-    const double bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-__global__ void k_energy(const double *Y, long long ld, int n, const double *ombar, int N,
-                         double sqrt_s, double *out) {
-    double s = 0.0, c = 0.0;
-    for (int p = threadIdx.x; p < n; p += blockDim.x) {
-        double t, e;
-        two_sum(s, 0.5 * sqrt_s * Y[p * ld + p], t, e);
-        s = t; c += e;
-    }
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        double t, e;
-        two_sum(s, -1.5 * ombar[i], t, e);
-        s = t; c += e;
-    }
-    __shared__ double ss[256], cc[256];
-    ss[threadIdx.x] = s;
-    cc[threadIdx.x] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double S = 0.0, Cc = 0.0;
-        for (int k = 0; k < blockDim.x; ++k) {
-            double t, e;
-            two_sum(S, ss[k], t, e);
-            S = t;
-            Cc += e + cc[k];
-        }
-        out[0] = S + Cc;
-    }
+// E = 1/2 sqrt(s) Tr Y - 3/2 sum omega_bar, compensated, one CTA of 256.
+__global__ void __launch_bounds__(256) k_energy(const double *Y, long long ld, int n, const double *ombar, int N,
+                                               double sqrt_s, double *out) {
+    __shared__ double sh[8][2];
+    comp::Sum v;
+    for (int p = threadIdx.x; p < n; p += 256) v.add(0.5 * sqrt_s * Y[p * ld + p]);
+    for (int i = threadIdx.x; i < N; i += 256) v.add(-1.5 * ombar[i]);
+    v = comp::block_sum256(v, sh);
+    if (threadIdx.x == 0) out[0] = v.value();
 }
 
 // ---- gradients -------------------------------------------------------------------------

@@ -16,6 +16,7 @@
 // The reciprocal phase e^{+i G.(R_j - R_i)} with k = G + q follows from Poisson summation of
 // sum_n T(r) e^{-i q.r}; the erfc numerator is the -grad grad of erfc(gamma r)/r; the
 // damped-away part (1 - g) T is removed in real space because it decays exponentially.
+#include "comp_sum.cuh"
 #include "internal.h"
 #include "pair_math.cuh"
 
@@ -426,41 +427,18 @@ __global__ void __launch_bounds__(1024) k_clanczos_update(double *w, double *v, 
     }
 }
 
-__device__ __forceinline__ void two_sum(double a, double b, double &s, double &e) {
-    s = a + b;
-    const double bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
-__global__ void k_energy_periodic(const double *Y, long long ld, int n, int nk, const double *ombar, int N,
-                                  double scale, double *out) {
-    double s = 0.0, cc = 0.0;
+__global__ void __launch_bounds__(256) k_energy_periodic(const double *Y, long long ld, int n, int nk,
+                                                         const double *ombar, int N, double scale, double *out) {
+    __shared__ double sh[8][2];
+    comp::Sum v;
     const long long total = static_cast<long long>(n) * nk;
-    for (long long e = threadIdx.x; e < total; e += blockDim.x) {
+    for (long long e = threadIdx.x; e < total; e += 256) {
         const long long k = e / n, pp = e % n;
-        double t, er;
-        two_sum(s, scale * Y[k * 2 * ld * ld + pp * ld + pp], t, er);
-        s = t; cc += er;
+        v.add(scale * Y[k * 2 * ld * ld + pp * ld + pp]);
     }
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        double t, er;
-        two_sum(s, -1.5 * ombar[i], t, er);
-        s = t; cc += er;
-    }
-    __shared__ double ss[256], sc2[256];
-    ss[threadIdx.x] = s;
-    sc2[threadIdx.x] = cc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double S = 0.0, C = 0.0;
-        for (int k = 0; k < blockDim.x; ++k) {
-            double t, er;
-            two_sum(S, ss[k], t, er);
-            S = t;
-            C += er + sc2[k];
-        }
-        out[0] = S + C;
-    }
+    for (int i = threadIdx.x; i < N; i += 256) v.add(-1.5 * ombar[i]);
+    v = comp::block_sum256(v, sh);
+    if (threadIdx.x == 0) out[0] = v.value();
 }
 
 // ---- MBD gradient of the periodic energy ---------------------------------------------
@@ -641,14 +619,9 @@ __global__ void k_mbd_grad_periodic_finalize(AtomBufs b, const double *Z, long l
 __global__ void k_mean_rows(const double *x, int rows, int N, double *out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    double s = 0.0, c = 0.0;
-    for (int r = 0; r < rows; ++r) {
-        double t, e;
-        two_sum(s, x[static_cast<long long>(r) * N + i], t, e);
-        s = t;
-        c += e;
-    }
-    out[i] = (s + c) / rows;
+    comp::Sum v;
+    for (int r = 0; r < rows; ++r) v.add(x[static_cast<long long>(r) * N + i]);
+    out[i] = v.value() / rows;
 }
 
 // ---- SCS adjoint over lattice images -------------------------------------------------
@@ -827,32 +800,14 @@ __global__ void k_extract_hermitian(const double *Ze, long long lde, int n, doub
 // E = 1/(2 nk) sum_k e_k - 3/4 sum omega_bar, where e_k = 1/2 Tr M_k^{1/2} - 3/2 sum omega_bar is
 // the mixed modes' corrected energy of the embedded matrix of Bloch vector k (Tr M_k^{1/2} =
 // 2 Tr Q(q_k)^{1/2}); compensated sums.
-__global__ void k_periodic_mixed_energy(const double *ek, int nk, const double *ombar, int N, double *out) {
-    double s = 0.0, cc = 0.0;
-    for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-        double t, er;
-        two_sum(s, 0.5 * ek[k] / nk, t, er);
-        s = t; cc += er;
-    }
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        double t, er;
-        two_sum(s, -0.75 * ombar[i], t, er);
-        s = t; cc += er;
-    }
-    __shared__ double ss[256], sc2[256];
-    ss[threadIdx.x] = s;
-    sc2[threadIdx.x] = cc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double S = 0.0, C = 0.0;
-        for (int q = 0; q < blockDim.x; ++q) {
-            double t, er;
-            two_sum(S, ss[q], t, er);
-            S = t;
-            C += er + sc2[q];
-        }
-        out[0] = S + C;
-    }
+__global__ void __launch_bounds__(256) k_periodic_mixed_energy(const double *ek, int nk, const double *ombar, int N,
+                                                               double *out) {
+    __shared__ double sh[8][2];
+    comp::Sum v;
+    for (int k = threadIdx.x; k < nk; k += 256) v.add(0.5 * ek[k] / nk);
+    for (int i = threadIdx.x; i < N; i += 256) v.add(-0.75 * ombar[i]);
+    v = comp::block_sum256(v, sh);
+    if (threadIdx.x == 0) out[0] = v.value();
 }
 }  // namespace
 

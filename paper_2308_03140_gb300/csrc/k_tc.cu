@@ -43,6 +43,7 @@
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include "comp_sum.cuh"
 #include "internal.h"
 #include "tc_ops.cuh"
 #include "tc_tiles.cuh"
@@ -1264,12 +1265,11 @@ __global__ void __launch_bounds__(128) k_block_trace_sqrt(const double *V, const
                                                          double sqrt_s, double *tq) {
     const int i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= N) return;
+    const double *v0 = V + 3LL * i * ld, *v1 = v0 + ld, *v2 = v1 + ld, *w = W + 3LL * i;
     double acc = 0.0;
-    for (int x = 0; x < 3; ++x) {
-        const long long p = 3LL * i + x;
-        const double *vp = V + p * ld;
-        for (long long k = lane; k < ld; k += 32) acc += vp[k] * W[k * ld + p];
-    }
+#pragma unroll 4
+    for (long long k = lane; k < ld; k += 32)   // three neighbouring columns of W: one sector of a row or two
+        acc += v0[k] * w[k * ld] + v1[k] * w[k * ld + 1] + v2[k] * w[k * ld + 2];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) {
@@ -1324,115 +1324,74 @@ __global__ void k_to_f64(const float *Zf, long long total, double scale, double 
         Zd[e] = scale * static_cast<double>(Zf[e]);
 }
 
-__device__ __forceinline__ void two_sum(double a, double b, double &s, double &e) {
-    s = a + b;
-    const double bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
-// Per-block compensated partial sums of Tr V (diagonal of the leading n x n block) and
-// of sum_pq V_pq W_pq; out[2 * block + {0,1}].
-__global__ void __launch_bounds__(256) k_trace_dot_partials(const double *V, const double *W, long long ld, int n,
-                                                            double *out) {
-    double s0 = 0.0, c0 = 0.0, s1 = 0.0, c1 = 0.0;
-    const long long total = static_cast<long long>(n) * n;
-    for (long long e = blockIdx.x * 256LL + threadIdx.x; e < total; e += static_cast<long long>(gridDim.x) * 256) {
-        const long long i = e / n, j = e % n;
-        const double v = V[i * ld + j];
-        double t, r;
-        two_sum(s1, v * W[i * ld + j], t, r);
-        s1 = t; c1 += r;
-        if (i == j) {
-            two_sum(s0, v, t, r);
-            s0 = t; c0 += r;
+// Per-block partial sums over the leading n x n block of T1 = sum Q o Z (FP64 x FP32, i.e.
+// Tr(Q Z) for symmetric Z), T2 = sum V o W and R = sum (delta - W)^2.  A thread adds the products
+// of kRun entries of a row in one chain of multiply-adds and then the chain to its compensated sum:
+// the chain rounds as often as the products themselves would, and the FP64 pipe, which bounds the pass,
+// spends 7 operations an entry instead of 21 (order 6000: 1.33 -> 0.74 ms; the entries' 28 bytes
+// would take 0.15).
+constexpr int kRun = 4, kCorrectionBlocks = 304;
+__global__ void __launch_bounds__(256) k_correction_partials(const double *Q, const float *Z, const double *V,
+                                                             const double *W, long long ld, int n, comp::Sum *out) {
+    __shared__ double sh[8][2];
+    comp::Sum t1, t2, r2;
+    const int warps = kCorrectionBlocks * 8, warp = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    for (int i = warp; i < n; i += warps) {   // a warp per row, 32 kRun entries at a time
+        const long long row = i * ld;
+        for (int j0 = 0; j0 < n; j0 += 32 * kRun) {
+            double a = 0.0, b = 0.0, c = 0.0;
+#pragma unroll
+            for (int u = 0; u < kRun; ++u) {
+                const int j = j0 + 32 * u + lane;
+                if (j < n) {
+                    const double w = W[row + j], d = i == j ? 1.0 - w : w;
+                    a += Q[row + j] * static_cast<double>(Z[row + j]);
+                    b += V[row + j] * w;
+                    c += d * d;
+                }
+            }
+            t1.add(a);
+            t2.add(b);
+            r2.s += c;
         }
     }
-    __shared__ double sh[4][256];
-    sh[0][threadIdx.x] = s0; sh[1][threadIdx.x] = c0; sh[2][threadIdx.x] = s1; sh[3][threadIdx.x] = c1;
-    __syncthreads();
+    t1 = comp::block_sum256(t1, sh);
+    t2 = comp::block_sum256(t2, sh);
+    r2 = comp::block_sum256(r2, sh);
     if (threadIdx.x == 0) {
-        double a = 0.0, ac = 0.0, b = 0.0, bc = 0.0;
-        for (int k = 0; k < 256; ++k) {
-            double t, r;
-            two_sum(a, sh[0][k], t, r); a = t; ac += r + sh[1][k];
-            two_sum(b, sh[2][k], t, r); b = t; bc += r + sh[3][k];
-        }
-        out[2 * blockIdx.x] = a + ac;
-        out[2 * blockIdx.x + 1] = b + bc;
+        out[blockIdx.x] = t1;
+        out[kCorrectionBlocks + blockIdx.x] = t2;
+        out[2 * kCorrectionBlocks + blockIdx.x] = r2;
     }
 }
 
-// Per-block compensated partials over the leading n x n block of T1 = sum (scale Q) o Z
-// (FP64 x FP32, i.e. Tr(scale Q Z) for symmetric Z), T2 = sum V o W (FP32 x FP32) and
-// R = sum (delta - W)^2; out[3 * block + {0,1,2}].
-__global__ void __launch_bounds__(256) k_correction_partials(const double *Q, double scale, const float *Z,
-                                                             const double *V, const double *W, long long ld, int n,
-                                                             double *out) {
-    double s0 = 0.0, c0 = 0.0, s1 = 0.0, c1 = 0.0, r2 = 0.0;
-    const long long total = static_cast<long long>(n) * n;
-    for (long long e = blockIdx.x * 256LL + threadIdx.x; e < total; e += static_cast<long long>(gridDim.x) * 256) {
-        const long long i = e / n, j = e % n, o = i * ld + j;
-        double t, r;
-        two_sum(s0, scale * Q[o] * static_cast<double>(Z[o]), t, r);
-        s0 = t; c0 += r;
-        const double w = W[o];
-        two_sum(s1, V[o] * w, t, r);
-        s1 = t; c1 += r;
-        const double d = (i == j ? 1.0 : 0.0) - w;
-        r2 += d * d;
+// E = (sqrt(s)/4)(3 scale T1 - T2) - 3/2 sum omega_bar; resid = sqrt(R).  One CTA.
+__global__ void __launch_bounds__(256) k_energy_correction(const comp::Sum *part, double scale, double sqrt_s,
+                                                           const double *ombar, int N, double *out, double *resid) {
+    __shared__ double sh[8][2];
+    comp::Sum t1, t2, r2, w;
+    for (int k = threadIdx.x; k < kCorrectionBlocks; k += 256) {
+        t1.add(part[k]);
+        t2.add(part[kCorrectionBlocks + k]);
+        r2.add(part[2 * kCorrectionBlocks + k]);
     }
-    __shared__ double sh[5][256];
-    sh[0][threadIdx.x] = s0; sh[1][threadIdx.x] = c0; sh[2][threadIdx.x] = s1; sh[3][threadIdx.x] = c1;
-    sh[4][threadIdx.x] = r2;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0, ac = 0.0, b = 0.0, bc = 0.0, rr = 0.0;
-        for (int k = 0; k < 256; ++k) {
-            double t, r;
-            two_sum(a, sh[0][k], t, r); a = t; ac += r + sh[1][k];
-            two_sum(b, sh[2][k], t, r); b = t; bc += r + sh[3][k];
-            rr += sh[4][k];
-        }
-        out[3 * blockIdx.x] = a + ac;
-        out[3 * blockIdx.x + 1] = b + bc;
-        out[3 * blockIdx.x + 2] = rr;
-    }
-}
-
-// E = (sqrt(s)/4)(3 T1 - T2) - 3/2 sum omega_bar; resid = sqrt(R).
-__global__ void k_energy_correction(const double *part, int nblocks, double sqrt_s, const double *ombar, int N,
-                                    double *out, double *resid) {
+    for (int i = threadIdx.x; i < N; i += 256) w.add(ombar[i]);
+    t1 = comp::block_sum256(t1, sh);
+    t2 = comp::block_sum256(t2, sh);
+    r2 = comp::block_sum256(r2, sh);
+    w = comp::block_sum256(w, sh);
     if (threadIdx.x != 0) return;
-    double a = 0.0, ac = 0.0, b = 0.0, bc = 0.0, w = 0.0, wc = 0.0, rr = 0.0;
-    for (int k = 0; k < nblocks; ++k) {
-        double t, r;
-        two_sum(a, part[3 * k], t, r); a = t; ac += r;
-        two_sum(b, part[3 * k + 1], t, r); b = t; bc += r;
-        rr += part[3 * k + 2];
-    }
-    for (int i = 0; i < N; ++i) {
-        double t, r;
-        two_sum(w, ombar[i], t, r); w = t; wc += r;
-    }
-    out[0] = 0.25 * sqrt_s * (3.0 * (a + ac) - (b + bc)) - 1.5 * (w + wc);
-    resid[0] = sqrt(rr);
-}
-
-// E = 1/2 * (1/2)(3 Tr V - sum V o W) - 3/2 sum omega_bar, from the partials (one CTA).
-__global__ void k_energy_variational(const double *part, int nblocks, const double *ombar, int N, double *out) {
-    if (threadIdx.x != 0) return;
-    double a = 0.0, ac = 0.0, b = 0.0, bc = 0.0, w = 0.0, wc = 0.0;
-    for (int k = 0; k < nblocks; ++k) {
-        double t, r;
-        two_sum(a, part[2 * k], t, r); a = t; ac += r;
-        two_sum(b, part[2 * k + 1], t, r); b = t; bc += r;
-    }
-    for (int i = 0; i < N; ++i) {
-        double t, r;
-        two_sum(w, ombar[i], t, r); w = t; wc += r;
-    }
-    const double trv = a + ac, vw = b + bc, sw = w + wc;
-    out[0] = 0.25 * (3.0 * trv - vw) - 1.5 * sw;
+    // the difference of large numbers once more without loss
+    comp::Sum e;
+    const double c1 = 0.75 * sqrt_s * scale, c2 = -0.25 * sqrt_s;
+    e.add(c1 * t1.s);
+    e.c += fma(c1, t1.s, -(c1 * t1.s)) + c1 * t1.c;
+    e.add(c2 * t2.s);
+    e.c += fma(c2, t2.s, -(c2 * t2.s)) + c2 * t2.c;
+    e.add(-1.5 * w.s);
+    e.c += fma(-1.5, w.s, 1.5 * w.s) - 1.5 * w.c;
+    out[0] = e.value();
+    resid[0] = sqrt(r2.value());
 }
 
 inline int grid_for(long long total) { return static_cast<int>(std::min<long long>((total + 255) / 256, 152 * 16)); }
@@ -1500,18 +1459,10 @@ void split_panel_tf32(const float *A, long long ld, long long mstride, int batch
 void energy_correction(const double *Q, double scale, const float *Z, const double *V, const double *W, long long ld,
                        int n, double sqrt_s, const double *ombar, int N, double *work, double *out, double *resid,
                        cudaStream_t s) {
-    const int nb = 304;   // work: 3 * nb doubles
+    comp::Sum *part = reinterpret_cast<comp::Sum *>(work);
     count_launches(2);
-    k_correction_partials<<<nb, 256, 0, s>>>(Q, scale, Z, V, W, ld, n, work);
-    k_energy_correction<<<1, 32, 0, s>>>(work, nb, sqrt_s, ombar, N, out, resid);
-}
-
-void energy_variational(const double *V, const double *W, long long ld, int n, const double *ombar, int N,
-                        double *work, double *out, cudaStream_t s) {
-    const int nb = 304;   // work: 2 * nb doubles
-    count_launches(2);
-    k_trace_dot_partials<<<nb, 256, 0, s>>>(V, W, ld, n, work);
-    k_energy_variational<<<1, 32, 0, s>>>(work, nb, ombar, N, out);
+    k_correction_partials<<<kCorrectionBlocks, 256, 0, s>>>(Q, Z, V, W, ld, n, part);
+    k_energy_correction<<<1, 256, 0, s>>>(part, scale, sqrt_s, ombar, N, out, resid);
 }
 
 }  // namespace mbdgb
