@@ -271,23 +271,24 @@ __global__ void k_f64_to_f32(const double *A, long long total, float *B) {
         B[e] = static_cast<float>(A[e]);
 }
 
-__device__ double block_sum1024(double v, double *sh) {
-    v = warp_sum(v);
+// Sum over the block (1024 threads), the same in every thread; sh: 33 entries not in use by a sum
+// before.  `active`: whether this warp has any terms (a warp's FP64 addition takes the pipe for 64 cycles
+// whatever it adds up).
+__device__ __forceinline__ double block_sum1024(double v, double *sh, bool active) {
+    if (active) v = warp_sum(v);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
-    double t = (threadIdx.x < 32) ? sh[threadIdx.x] : 0.0;
-    if (threadIdx.x < 32) t = warp_sum(t);
+    if (threadIdx.x < 32) {
+        const double t = warp_sum(sh[threadIdx.x]);
+        if (threadIdx.x == 0) sh[32] = t;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) sh[0] = t;
-    __syncthreads();
-    const double r = sh[0];
-    __syncthreads();
-    return r;
+    return sh[32];
 }
 
 // v = a fixed pseudo-random unit vector, vprev = 0; v32 (if given) = (float) v.
 __global__ void __launch_bounds__(1024) k_lanczos_init(double *v, double *vprev, float *v32, long long ld) {
-    __shared__ double sh[32];
+    __shared__ double sh[33];
     double ss = 0.0;
     for (long long p = threadIdx.x; p < ld; p += 1024) {
         const double x = sin(0.7548776662 * static_cast<double>(p) + 0.5698402910) + 0.25;
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(1024) k_lanczos_init(double *v, double *vprev,
         vprev[p] = 0.0;
         ss += x * x;
     }
-    const double nrm = sqrt(block_sum1024(ss, sh));
+    const double nrm = sqrt(block_sum1024(ss, sh, true));
     for (long long p = threadIdx.x; p < ld; p += 1024) {
         v[p] /= nrm;
         if (v32) v32[p] = static_cast<float>(v[p]);
@@ -304,26 +305,68 @@ __global__ void __launch_bounds__(1024) k_lanczos_init(double *v, double *vprev,
 
 // One Lanczos step after w = A v: alpha = w.v; w -= alpha v + beta_prev vprev;
 // beta = |w|; vprev = v; v = w / beta (and v32 = (float) v if given).  coef[2j] = alpha,
-// coef[2j+1] = beta.
+// coef[2j+1] = beta.  kPer > 0: the vectors (ld <= 1024 kPer) stay in registers between the sums.  Latency
+// and the FP64 additions of its 32 warps bound it: with three passes over the vectors, and warps without
+// terms adding zeros, it took 10.6 us at order 128 and 11.5 at 768, so 5.2 and 9.9; longer vectors gain nothing
+// from registers (20.6 us at 6016 either way).
+template <int kPer>
 __global__ void __launch_bounds__(1024) k_lanczos_update(double *w, double *v, double *vprev, float *v32, long long ld,
                                                          double *coef, int j) {
-    __shared__ double sh[32];
-    double d = 0.0;
-    for (long long p = threadIdx.x; p < ld; p += 1024) d += w[p] * v[p];
-    const double alpha = block_sum1024(d, sh);
+    __shared__ double sh[2][33];
+    constexpr int kHeld = kPer > 0 ? kPer : 1;
+    double rw[kHeld], rv[kHeld], rp[kHeld];
+    const bool active = (threadIdx.x & ~31) < ld;
     const double bprev = j > 0 ? coef[2 * j - 1] : 0.0;
-    double ss = 0.0;
-    for (long long p = threadIdx.x; p < ld; p += 1024) {
-        const double x = w[p] - alpha * v[p] - bprev * vprev[p];
-        w[p] = x;
-        ss += x * x;
+    double d = 0.0, ss = 0.0;
+    if constexpr (kPer > 0) {
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const long long p = threadIdx.x + 1024LL * u;
+            if (p >= ld) break;
+            rw[u] = w[p];
+            rv[u] = v[p];
+            rp[u] = vprev[p];
+            d += rw[u] * rv[u];
+        }
+    } else {
+        for (long long p = threadIdx.x; p < ld; p += 1024) d += w[p] * v[p];
     }
-    const double beta = sqrt(block_sum1024(ss, sh));
+    const double alpha = block_sum1024(d, sh[0], active);
+    if constexpr (kPer > 0) {
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            if (threadIdx.x + 1024LL * u >= ld) break;
+            const double x = rw[u] - alpha * rv[u] - bprev * rp[u];
+            rw[u] = x;
+            ss += x * x;
+        }
+    } else {
+        for (long long p = threadIdx.x; p < ld; p += 1024) {
+            const double x = w[p] - alpha * v[p] - bprev * vprev[p];
+            w[p] = x;
+            ss += x * x;
+        }
+    }
+    const double ss2 = block_sum1024(ss, sh[1], active);
+    if (!active) return;
+    const double beta = sqrt(ss2);
     const double inv = beta > 1e-300 ? 1.0 / beta : 0.0;
-    for (long long p = threadIdx.x; p < ld; p += 1024) {
-        vprev[p] = v[p];
-        v[p] = w[p] * inv;
-        if (v32) v32[p] = static_cast<float>(v[p]);
+    if constexpr (kPer > 0) {
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const long long p = threadIdx.x + 1024LL * u;
+            if (p >= ld) break;
+            const double x = rw[u] * inv;
+            vprev[p] = rv[u];
+            v[p] = x;
+            if (v32) v32[p] = static_cast<float>(x);
+        }
+    } else {
+        for (long long p = threadIdx.x; p < ld; p += 1024) {
+            vprev[p] = v[p];
+            v[p] = w[p] * inv;
+            if (v32) v32[p] = static_cast<float>(v[p]);
+        }
     }
     if (threadIdx.x == 0) {
         coef[2 * j] = alpha;
@@ -344,7 +387,8 @@ void lanczos_run(const T *A, long long ld, int steps, double *work, double *coef
     for (int j = 0; j < steps; ++j) {
         count_launches(2);
         k_gemv<T><<<static_cast<int>((ld + 7) / 8), 256, 0, s>>>(A, ld, x, w);
-        k_lanczos_update<<<1, 1024, 0, s>>>(w, v, vprev, v32, ld, coef, j);
+        if (ld <= 1024) k_lanczos_update<1><<<1, 1024, 0, s>>>(w, v, vprev, v32, ld, coef, j);
+        else k_lanczos_update<0><<<1, 1024, 0, s>>>(w, v, vprev, v32, ld, coef, j);
     }
 }
 
