@@ -10,6 +10,8 @@
 //
 // Layout as in k_dense.cu: batch of row-major ld x ld matrices, ld a multiple of 64,
 // right-hand sides [batch][ld][3].
+#include <type_traits>
+
 #include "internal.h"
 
 namespace mbdgb {
@@ -80,10 +82,12 @@ __global__ void __launch_bounds__(256) k_sgemm_nt(const float *A, const float *B
 }
 
 // FP32 Cholesky of a 64x64 diagonal block plus the inverse of its factor, one CTA per
-// matrix.  The factorisation is blocked by 16: warp 0 factors each 16x16 diagonal block
-// (warp-synchronous, one lane per row), one thread per row solves the rows below it, and
-// all threads apply the 16-term trailing update (3 block barriers per 16 columns).  The
-// inverse is blocked by 16 as well: the diagonal blocks by forward substitution in
+// matrix.  Latency bounds it: the chain of 64 square roots and divisions.  The block stays in registers
+// (thread (ty, tx): rows ty + 16 a, columns tx + 16 c), and a column costs one barrier: the warp that holds
+// the next column updates it first, takes its pivot's root, divides and stores the column before the rest of
+// its update.  Each entry still sees the same operations in the same order as a column-by-column
+// factorisation.  (With a warp factoring 16x16 blocks through shared memory the kernel took 60 us, so 35.)
+// The inverse is blocked by 16: the diagonal blocks by forward substitution in
 // registers, the blocks below them by two small block products per block row.
 __global__ void __launch_bounds__(256) k_spotrf_diag(float *A, long long ld, long long mstride, float *dinv,
                                                      long long dstride, int *status) {
@@ -93,56 +97,59 @@ __global__ void __launch_bounds__(256) k_spotrf_diag(float *A, long long ld, lon
     __shared__ int bad;
     float *Ab = A + static_cast<long long>(blockIdx.x) * mstride;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int ty = t & 15, tx = t >> 4;   // a warp holds the rows of two columns
     if (t == 0) bad = 0;
-    for (int e = t; e < 4096; e += 256) {
-        const int r = e >> 6, c = e & 63;
-        S[r][c] = (c <= r) ? Ab[r * ld + c] : 0.f;
-    }
-    __syncthreads();
-    for (int j0 = 0; j0 < 64; j0 += 16) {
-        if (warp == 0) {   // 16x16 diagonal block, lane = row j0 + lane
-            for (int j = 0; j < 16; ++j) {
-                const int jj = j0 + j;
-                float d = S[jj][jj];
-                if (!(d > 0.f)) {
-                    if (lane == 0) bad = 1;
-                    d = 1.f;
-                }
-                d = sqrtf(d);
-                __syncwarp();
-                if (lane == 0) S[jj][jj] = d;
-                if (lane > j && lane < 16) S[j0 + lane][jj] /= d;
-                __syncwarp();
-                if (lane > j && lane < 16) {
-                    const int i = j0 + lane;
-                    const float lij = S[i][jj];
-                    for (int k = jj + 1; k <= i; ++k) S[i][k] -= lij * S[k][jj];
-                }
-                __syncwarp();
-            }
-        }
-        __syncthreads();
-        for (int i = j0 + 16 + t; i < 64; i += 256) {   // rows below: L21 = A21 L11^{-T}
-            for (int c = 0; c < 16; ++c) {
-                float v = S[i][j0 + c];
-                for (int k = 0; k < c; ++k) v -= S[i][j0 + k] * S[j0 + c][j0 + k];
-                S[i][j0 + c] = v / S[j0 + c][j0 + c];
-            }
-        }
-        __syncthreads();
-        const int r0 = j0 + 16;   // trailing lower triangle [r0, 64)^2 -= L21 L21^T
-        if (r0 < 64) {
-            const int ty = t >> 4, tx = t & 15;
-            for (int i = r0 + ty; i < 64; i += 16)
-                for (int k = r0 + tx; k <= i; k += 16) {
-                    float v = S[i][k];
+    float a[4][4];   // a[i][c]: row ty + 16 i, column tx + 16 c, c <= i
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) v -= S[i][j0 + c] * S[k][j0 + c];
-                    S[i][k] = v;
-                }
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c <= i; ++c) a[i][c] = (tx + 16 * c <= ty + 16 * i) ? Ab[(ty + 16 * i) * ld + tx + 16 * c] : 0.f;
+    __syncthreads();   // bad
+    // Column j = 16 cb + jx of the factor from its owners (half a warp) to shared memory.
+    auto publish = [&](auto CB, int jx) {
+        constexpr int cb = decltype(CB)::value;
+        float d = __shfl_sync(0xffffffffu, a[cb][cb], (t & 16) | jx);
+        if (tx != jx) return;
+        if (!(d > 0.f)) {
+            if (ty == jx) bad = 1;
+            d = 1.f;
         }
-        __syncthreads();
-    }
+        d = sqrtf(d);
+        const int j = 16 * cb + jx;
+        if (ty == jx) S[j][j] = d;
+#pragma unroll
+        for (int i = cb; i < 4; ++i)
+            if (i > cb || ty > jx) S[ty + 16 * i][j] = a[i][cb] / d;
+    };
+    auto columns = [&](auto CB) {   // 16 cb .. 16 cb + 15
+        constexpr int cb = decltype(CB)::value;
+        for (int jx = 0; jx < 16; ++jx) {
+            const int j = 16 * cb + jx;
+            __syncthreads();   // column j is there
+            float x[4], w[4];
+#pragma unroll
+            for (int i = cb; i < 4; ++i) {
+                x[i] = ty + 16 * i > j ? S[ty + 16 * i][j] : 0.f;
+                w[i] = tx + 16 * i > j ? S[tx + 16 * i][j] : 0.f;
+            }
+#pragma unroll
+            for (int i = cb; i < 4; ++i) a[i][cb] -= x[i] * w[cb];
+            if (jx < 15 && tx >> 1 == (jx + 1) >> 1) publish(CB, jx + 1);
+#pragma unroll
+            for (int c = cb + 1; c < 4; ++c)
+#pragma unroll
+                for (int i = c; i < 4; ++i) a[i][c] -= x[i] * w[c];
+            if constexpr (cb < 3) {
+                if (jx == 15 && tx < 2) publish(std::integral_constant<int, cb + 1>{}, 0);
+            }
+        }
+    };
+    if (tx < 2) publish(std::integral_constant<int, 0>{}, 0);
+    columns(std::integral_constant<int, 0>{});
+    columns(std::integral_constant<int, 1>{});
+    columns(std::integral_constant<int, 2>{});
+    columns(std::integral_constant<int, 3>{});
+    __syncthreads();
     // V = L^{-1} by 16x16 blocks.  Diagonal blocks: warp w < 4 inverts block w, lane c < 16
     // holding column c in registers (forward substitution).  Block rows I = 1..3 then follow
     // from V_IJ = -V_II sum_{K=J}^{I-1} L_IK V_KJ (J < I), every element in parallel.
@@ -166,6 +173,7 @@ __global__ void __launch_bounds__(256) k_spotrf_diag(float *A, long long ld, lon
             const int J = e >> 8, r = (e >> 4) & 15, cc = e & 15;
             const int i = 16 * I + r, j = 16 * J + cc;
             float sum = 0.f;
+#pragma unroll 16
             for (int k = 16 * J; k < 16 * I; ++k) sum += S[i][k] * V[k][j];
             Tp[J][r][cc] = sum;
         }
