@@ -130,6 +130,14 @@ __global__ void __launch_bounds__(256) k_solve(double *A, long long ld, long lon
     put2(v[0], v[1], row_scale(e), pp, planes + b * kMod * pp + r * pitch + kcol + 2 * lane);
 }
 
+// 1 / d to about an ulp, d a normal number: two Newton steps from the hardware's approximation.
+__device__ __forceinline__ double reciprocal(double d) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(d));
+    y = fma(y, fma(-d, y, 1.0), y);
+    return fma(y, fma(-d, y, 1.0), y);
+}
+
 // Factor and inverse of a 64 x 64 diagonal block.  A cluster of four CTAs takes one matrix: each
 // factors the block by itself (its 45e3 multiply-adds take 11 us of an SM's FP64 pipe, exchanging columns
 // would take longer) and inverts every fourth column, so that the inverse, as much work again,
@@ -157,25 +165,30 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256)
         for (int c = 0; c <= i; ++c) a[i][c] = (tx + 16 * c <= ty + 16 * i) ? Ab[(ty + 16 * i) * ld + tx + 16 * c] : 0.0;
     // every CTA of the cluster has read the block before one writes its factor
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-    // Column j = 16 cb + jx (its owners are half a warp) to shared memory, with its pivot's reciprocal.
-    auto publish = [&](auto CB, int jx) {
+    // The pivot of column j = 16 cb + jx and its reciprocal, in the warp that holds the column; then the
+    // column itself to shared memory, by its owners (half the warp).
+    auto pivot = [&](auto CB, int jx, double &r) {
         constexpr int cb = decltype(CB)::value;
-        const int j = 16 * cb + jx;
-        double d = __shfl_sync(0xffffffffu, a[cb][cb], (threadIdx.x & 16) | jx);
-        if (tx != jx) return;
-        if (!(d > 0.0)) {
-            if (ty == jx) bad = 1;
-            d = 1.0;
+        double d = __shfl_sync(0xffffffffu, a[cb][cb], (t & 16) | jx);
+        const bool ok = d > 0.0;
+        d = ok ? d : 1.0;
+        r = reciprocal(d);
+        if (tx == jx && ty == jx) {
+            if (!ok) bad = 1;
+            piv[16 * cb + jx] = d;
         }
-        const double r = 1.0 / d;
+    };
+    auto publish = [&](auto CB, int jx, double r) {
+        constexpr int cb = decltype(CB)::value;
+        const int p = jx & 1;   // the parity of j
+        if (tx != jx) return;
 #pragma unroll
         for (int i = cb; i < 4; ++i) {
             if (i > cb || ty > jx) {
-                col[j & 1][ty + 16 * i] = a[i][cb];
-                row[j & 1][ty + 16 * i] = a[i][cb] * r;
+                col[p][ty + 16 * i] = a[i][cb];
+                row[p][ty + 16 * i] = a[i][cb] * r;
             }
         }
-        if (ty == jx) piv[j] = d;
     };
     auto blocks = [&](auto CB) {   // columns 16 cb .. 16 cb + 15
         constexpr int cb = decltype(CB)::value;
@@ -188,22 +201,32 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256)
                 x[i] = ty + 16 * i > j ? col[p][ty + 16 * i] : 0.0;
                 w[i] = tx + 16 * i > j ? row[p][tx + 16 * i] : 0.0;
             }
-            // the block column of the next pivot first
+            // the next pivot first, then its column: every FP64 instruction of the warp that holds them is
+            // 64 cycles of the chain
+            a[cb][cb] -= x[cb] * w[cb];
+            const bool owner = jx < 15 && tx >> 1 == (jx + 1) >> 1;
+            double r = 0.0;
+            if (owner) pivot(CB, jx + 1, r);
 #pragma unroll
-            for (int i = cb; i < 4; ++i) a[i][cb] -= x[i] * w[cb];
-            if (jx < 15) {
-                if (tx >> 1 == (jx + 1) >> 1) publish(CB, jx + 1);
-            }
+            for (int i = cb + 1; i < 4; ++i) a[i][cb] -= x[i] * w[cb];
+            if (owner) publish(CB, jx + 1, r);
 #pragma unroll
             for (int c = cb + 1; c < 4; ++c)
 #pragma unroll
                 for (int i = c; i < 4; ++i) a[i][c] -= x[i] * w[c];
             if constexpr (cb < 3) {
-                if (jx == 15 && tx < 2) publish(std::integral_constant<int, cb + 1>{}, 0);
+                if (jx == 15 && tx < 2) {
+                    pivot(std::integral_constant<int, cb + 1>{}, 0, r);
+                    publish(std::integral_constant<int, cb + 1>{}, 0, r);
+                }
             }
         }
     };
-    if (tx < 2) publish(std::integral_constant<int, 0>{}, 0);
+    if (tx < 2) {
+        double r;
+        pivot(std::integral_constant<int, 0>{}, 0, r);
+        publish(std::integral_constant<int, 0>{}, 0, r);
+    }
     blocks(std::integral_constant<int, 0>{});
     blocks(std::integral_constant<int, 1>{});
     blocks(std::integral_constant<int, 2>{});

@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
 }
 
 // ---- results --------------------------------------------------------------------------------
-// A block of 256 threads takes 32 rows x 128 columns: a thread reads four neighbouring bytes of
+// A block of 256 threads takes kRows rows x 128 columns: a thread reads four neighbouring bytes of
 // each of the 15 planes and sums them in three words (45 wide multiply-adds an entry, the FP64 pipe being
 // the scarcer one: one conversion, three products).  Mirrored and transposed copies leave
 // through shared memory, so that every store is a run of 256 bytes.
@@ -499,12 +499,13 @@ struct ResultArgs {
 
 __device__ __forceinline__ bool kept(int sym, int r, int c) { return sym == 0 || (sym == 1 ? c >= r : c <= r); }
 
+template <int kRows>
 __global__ void __launch_bounds__(256) k_crt_result(ResultArgs g, int tiles_c) {
-    __shared__ double tile[32][129];
+    __shared__ double tile[kRows][129];
     const long long b = blockIdx.z;
     const int part = blockIdx.y;   // 0 real, 1 imaginary
-    const int r0 = (blockIdx.x / tiles_c) * 32, c0 = (blockIdx.x % tiles_c) * 128;
-    if (g.sym == 1 ? g.col0 + c0 + 127 < r0 : g.sym && g.col0 + c0 > r0 + 31) return;
+    const int r0 = (blockIdx.x / tiles_c) * kRows, c0 = (blockIdx.x % tiles_c) * 128;
+    if (g.sym == 1 ? g.col0 + c0 + 127 < r0 : g.sym && g.col0 + c0 > r0 + kRows - 1) return;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int c = c0 + 4 * tx, gc = g.col0 + c;
     double *C = g.C + b * g.sC + part * g.im_off;
@@ -512,7 +513,7 @@ __global__ void __launch_bounds__(256) k_crt_result(ResultArgs g, int tiles_c) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) eb[j] = c + j < g.n ? g.eb[b * g.b_rows + part * g.second + c + j] : 0;
     const double unit = g.alpha * crt::kProduct;
-    for (int i = ty; i < 32; i += 8) {
+    for (int i = ty; i < kRows; i += 8) {
         const int r = r0 + i;
         double v[4] = {0.0, 0.0, 0.0, 0.0};
         if (r < g.M && c < g.n) {
@@ -552,10 +553,11 @@ __global__ void __launch_bounds__(256) k_crt_result(ResultArgs g, int tiles_c) {
     const double sign = g.sym && part ? -1.0 : 1.0;
     double *out = g.sym ? C : g.T + b * g.sT + part * g.im_off;
     const long long ldo = g.sym ? g.ldc : g.ldt;
-    const int r = r0 + tx;
-    for (int k = ty; k < 128; k += 8) {
+    constexpr int kGroups = 256 / kRows;   // columns of the tile at a time
+    const int i = threadIdx.x % kRows, r = r0 + i;
+    for (int k = threadIdx.x / kRows; k < 128; k += kGroups) {
         const int cc = g.col0 + c0 + k;
-        if (r < g.M && c0 + k < g.n && (!g.sym || r < cc)) out[cc * ldo + r] = sign * tile[tx][k];
+        if (r < g.M && c0 + k < g.n && (!g.sym || r < cc)) out[cc * ldo + r] = sign * tile[i][k];
     }
 }
 
@@ -723,9 +725,15 @@ cudaError_t crt_multiply(const CrtOperand &A, const CrtOperand &B, const CrtResu
     o.im_off = r.im_off;
     o.col0 = r.col0;
     o.sym = r.sym;
-    const int tr = (M + 31) / 32, tc = (o.n + 127) / 128;
+    const int tc = (o.n + 127) / 128, z = (a.complex ? 2 : 1) * a.batch;
+    const dim3 rest(1, a.complex ? 2 : 1, a.batch);
     count_launches(1);
-    k_crt_result<<<dim3(tr * tc, a.complex ? 2 : 1, a.batch), 256, 0, st>>>(o, tc);
+    // blocks of 8 rows, one a warp, until they fill the chip twice (order 96: 15.6 us with 32 rows, 6.1 with 8)
+    if ((M + 31) / 32 * tc * z >= 2 * 152) {
+        k_crt_result<32><<<dim3((M + 31) / 32 * tc, rest.y, rest.z), 256, 0, st>>>(o, tc);
+    } else {
+        k_crt_result<8><<<dim3((M + 7) / 8 * tc, rest.y, rest.z), 256, 0, st>>>(o, tc);
+    }
     return cudaGetLastError();
 }
 
