@@ -326,10 +326,11 @@ struct CellGeom {
 // Bloch vectors and reciprocal lattice: kq [nk][3] (Cartesian q), G [nG][3] (every G
 // with |G + q| < kc for some q), glist [nk][maxG] indices into G of the vectors with
 // 0 < |G + q_k| < kc (gcount[k] of them), S [nG][N] structure factors e^{i G.R_i}.
+// Of a grid of nkt Bloch vectors nk are kept, with weights kw [nk] whose sum is nkt.
 struct PeriodicBufs {
     CellGeom cell;
-    int nk, nG, maxG;
-    const double *kq, *G;
+    int nk, nkt, nG, maxG;
+    const double *kq, *kw, *G;
     const int *glist, *gcount;
     double2 *S;
 };
@@ -347,7 +348,7 @@ void build_q_periodic(const AtomBufs &b, const PeriodicBufs &p, double beta, dou
 void cscale(double *Y, long long ld, int nk, double scale, cudaStream_t s);
 void cset_identity(double *Z, long long ld, int nk, cudaStream_t s);
 void caxpby_identity(double *Z, const double *P, long long ld, int nk, double a, double b, cudaStream_t s);
-void cfrob_dev_identity(const double *P, long long ld, int n, int nk, double *out, cudaStream_t s);
+void cfrob_dev_identity(const double *P, long long ld, int n, int nk, const double *kw, double *out, cudaStream_t s);
 void cmax_abs_rowsum(const double *Q, long long ld, int nk, double *out, cudaStream_t s);
 // C = alpha A B + beta D for nk planar complex matrices (4 real FP64 GEMMs; D may be C).
 // herm: the result is Hermitian (as Y Z Y, Z Y Z for Hermitian Y, Z): upper tiles only,
@@ -364,8 +365,8 @@ void clanczos_coefficients(const double *Q, long long ld, int nk, int steps, dou
 void embed_hermitian(const double *Q, long long ld, int n, int k, double *M, long long lde, cudaStream_t s);
 void extract_hermitian(const double *Ze, long long lde, int n, double *Z, long long ld, int k, cudaStream_t s);
 void periodic_mixed_energy(const double *ek, int nk, const double *ombar, int N, double *out, cudaStream_t s);
-// E = sqrt_s/(2 nk) sum_k Re Tr Y_k - 3/2 sum omega_bar (compensated).
-void energy_trace_periodic(const double *Y, long long ld, int n, int nk, const double *ombar, int N,
+// E = sqrt_s/(2 nkt) sum_k kw_k Re Tr Y_k - 3/2 sum omega_bar (compensated).
+void energy_trace_periodic(const double *Y, long long ld, int n, const PeriodicBufs &p, const double *ombar, int N,
                            double sqrt_s, double *out, cudaStream_t s);
 // MBD gradient of the periodic energy from Z_k (Q(q_k)^{-1/2} = zscale Z_k): per atom
 // g_ombar, g_abar0, g_rbar, gR (o), and dE/dA accumulated into gA [9].  work: 2N doubles.
@@ -379,10 +380,11 @@ void periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double beta, do
 // out[i] = (1/rows) sum_r x[r][i] for a rows x N array (compensated).
 void mean_rows(const double *x, int rows, int N, double *out, cudaStream_t s);
 // SCS adjoint pair pass over lattice images (as scs_grad_pass), with the lattice part
-// accumulated into gA [9].  gA_part: N x 9 doubles of workspace.
+// accumulated into gA [9].  work: scs_grad_periodic_words doubles.
+long long scs_grad_periodic_words(int N, int nf1);
 void scs_grad_periodic(const AtomBufs &b, const CellGeom &c, double beta, double a, const double *X,
                        const double *V, long long xstride, double *g_a0, double *g_om, double *g_rv, double *gR,
-                       double *gA_part, double *gA, cudaStream_t s);
+                       double *work, double *gA, cudaStream_t s);
 
 // Periodic TS dispersion (k_ts_periodic.cu; the sum of Eq. ts-ewald minus the damped-away
 // part) of the TS-scaled oscillators, from the structure factors p.S of the current

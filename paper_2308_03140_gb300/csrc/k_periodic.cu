@@ -65,49 +65,68 @@ __global__ void k_structure_factors(const double *R, int N, const double *G, int
 }
 
 // ---- Gamma-point screening matrices ------------------------------------------------
-// Thread (i, j), j <= i, writes block (i, j) of every frequency's matrix and its mirror:
-// delta_ij I / alpha_i + sum over images r = R_j - R_i + n A (0 < |r| < rc) of (1 - f) T^GG.
-__global__ void k_build_scs_periodic(AtomBufs b, CellGeom c, double beta, double a, double *M, long long ld,
-                                     long long mstride, int *status) {
+// Thread (i, j), j <= i, writes block (i, j) of kScsFreq frequencies' matrices (blockIdx.z) and their
+// mirrors: delta_ij I / alpha_i + sum over images r = R_j - R_i + n A (0 < |r| < rc) of (1 - f) T^GG.
+// FP64 arithmetic bounds it: about 100 operations an image and frequency, after 60 an image for the
+// distance and the damping, which the frequencies of a thread share; dividing them over the grid fills the
+// chip with small cells (96 atoms: 36 blocks and 11.1 ms with all frequencies in a thread, one after
+// the other, 1.36 ms so).
+constexpr int kScsFreq = 4;
+__global__ void __launch_bounds__(128) k_build_scs_periodic(AtomBufs b, CellGeom c, double beta, double a, double *M,
+                                                            long long ld, long long mstride, int *status) {
     const int j = blockIdx.x * 32 + threadIdx.x;
-    const int i = blockIdx.y * 8 + threadIdx.y;
+    const int i = blockIdx.y * 4 + threadIdx.y;
     if (i >= b.N || j > i) return;
     const double x[3] = {b.R[3 * j] - b.R[3 * i], b.R[3 * j + 1] - b.R[3 * i + 1], b.R[3 * j + 2] - b.R[3 * i + 2]};
     int lo[3], hi[3];
     image_box(c, x, lo, hi);
     const double S = b.rv[i] + b.rv[j];
-    for (int k = 0; k < b.nf1; ++k) {
-        const double si = b.sig_u[k * b.N + i], sj = b.sig_u[k * b.N + j], s = sqrt(si * si + sj * sj);
-        double acc[6] = {0, 0, 0, 0, 0, 0};
-        bool bad = false;
-        for (int n0 = lo[0]; n0 <= hi[0]; ++n0)
-            for (int n1 = lo[1]; n1 <= hi[1]; ++n1)
-                for (int n2 = lo[2]; n2 <= hi[2]; ++n2) {
-                    double r[3];
-                    for (int e = 0; e < 3; ++e) r[e] = x[e] + n0 * c.A[e] + n1 * c.A[3 + e] + n2 * c.A[6 + e];
-                    const double rho2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-                    if (rho2 >= c.rc * c.rc) continue;
-                    if (rho2 < 1e-16) {
-                        if (i != j || n0 || n1 || n2) bad = true;
-                        continue;
-                    }
-                    const double rho = sqrt(rho2);
-                    const Fermi f = fermi(rho, S, beta, a);
-                    const Radial t = tgg_radial(rho, s);
-                    const double sr = 1.0 - f.f;
-                    acc[0] += sr * (t.P + t.W * r[0] * r[0]);
-                    acc[1] += sr * (t.P + t.W * r[1] * r[1]);
-                    acc[2] += sr * (t.P + t.W * r[2] * r[2]);
-                    acc[3] += sr * t.W * r[0] * r[1];
-                    acc[4] += sr * t.W * r[0] * r[2];
-                    acc[5] += sr * t.W * r[1] * r[2];
+    const int k0 = blockIdx.z * kScsFreq;
+    double s[kScsFreq], acc[kScsFreq][6];
+#pragma unroll
+    for (int f = 0; f < kScsFreq; ++f) {
+        const int k = min(k0 + f, b.nf1 - 1);
+        const double si = b.sig_u[k * b.N + i], sj = b.sig_u[k * b.N + j];
+        s[f] = sqrt(si * si + sj * sj);
+#pragma unroll
+        for (int e = 0; e < 6; ++e) acc[f][e] = 0.0;
+    }
+    bool bad = false;
+    for (int n0 = lo[0]; n0 <= hi[0]; ++n0)
+        for (int n1 = lo[1]; n1 <= hi[1]; ++n1)
+            for (int n2 = lo[2]; n2 <= hi[2]; ++n2) {
+                double r[3];
+                for (int e = 0; e < 3; ++e) r[e] = x[e] + n0 * c.A[e] + n1 * c.A[3 + e] + n2 * c.A[6 + e];
+                const double rho2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
+                if (rho2 >= c.rc * c.rc) continue;
+                if (rho2 < 1e-16) {
+                    if (i != j || n0 || n1 || n2) bad = true;
+                    continue;
                 }
-        if (bad) atomicOr(status, ST_INPUT);
+                const double rho = sqrt(rho2);
+                const double sr = 1.0 - fermi(rho, S, beta, a).f;
+                if (sr == 0.0) continue;   // damped away to the last bit
+#pragma unroll
+                for (int f = 0; f < kScsFreq; ++f) {
+                    const Radial t = tgg_radial(rho, s[f]);
+                    acc[f][0] += sr * (t.P + t.W * r[0] * r[0]);
+                    acc[f][1] += sr * (t.P + t.W * r[1] * r[1]);
+                    acc[f][2] += sr * (t.P + t.W * r[2] * r[2]);
+                    acc[f][3] += sr * t.W * r[0] * r[1];
+                    acc[f][4] += sr * t.W * r[0] * r[2];
+                    acc[f][5] += sr * t.W * r[1] * r[2];
+                }
+            }
+    if (bad) atomicOr(status, ST_INPUT);
+#pragma unroll
+    for (int f = 0; f < kScsFreq; ++f) {
+        const int k = k0 + f;
+        if (k >= b.nf1) break;
         if (i == j) {
             const double d = 1.0 / b.al_u[k * b.N + i];
-            acc[0] += d; acc[1] += d; acc[2] += d;
+            acc[f][0] += d; acc[f][1] += d; acc[f][2] += d;
         }
-        const double blk[9] = {acc[0], acc[3], acc[4], acc[3], acc[1], acc[5], acc[4], acc[5], acc[2]};
+        const double blk[9] = {acc[f][0], acc[f][3], acc[f][4], acc[f][3], acc[f][1], acc[f][5], acc[f][4], acc[f][5], acc[f][2]};
         double *Mk = M + k * mstride;
         for (int xx = 0; xx < 3; ++xx)
             for (int y = 0; y < 3; ++y) {
@@ -309,9 +328,9 @@ __device__ __forceinline__ double block_sum256(double v, double *sh) {
     return t;
 }
 
-// out[0] += sum_k sum_{p,q < n} |P_k - I|^2 (both planes)
+// out[0] += sum_k kw_k sum_{p,q < n} |P_k - I|^2 (both planes)
 __global__ void __launch_bounds__(256) k_cfrob_dev_identity(const double *P, long long ld, int n, int nk,
-                                                            double *out) {
+                                                            const double *kw, double *out) {
     __shared__ double sh[8];
     const long long per = static_cast<long long>(n) * n, total = per * nk;
     double acc = 0.0;
@@ -319,7 +338,7 @@ __global__ void __launch_bounds__(256) k_cfrob_dev_identity(const double *P, lon
         const long long k = e / per, w = e % per, r = w / n, cidx = w % n;
         const double *Pr = P + k * 2 * ld * ld;
         const double vr = Pr[r * ld + cidx] - (r == cidx ? 1.0 : 0.0), vi = Pr[ld * ld + r * ld + cidx];
-        acc += vr * vr + vi * vi;
+        acc += kw[k] * (vr * vr + vi * vi);
     }
     const double t = block_sum256(acc, sh);
     if (threadIdx.x == 0) atomicAdd(out, t);
@@ -427,14 +446,14 @@ __global__ void __launch_bounds__(1024) k_clanczos_update(double *w, double *v, 
     }
 }
 
-__global__ void __launch_bounds__(256) k_energy_periodic(const double *Y, long long ld, int n, int nk,
+__global__ void __launch_bounds__(256) k_energy_periodic(const double *Y, long long ld, int n, int nk, const double *kw,
                                                          const double *ombar, int N, double scale, double *out) {
     __shared__ double sh[8][2];
     comp::Sum v;
     const long long total = static_cast<long long>(n) * nk;
     for (long long e = threadIdx.x; e < total; e += 256) {
         const long long k = e / n, pp = e % n;
-        v.add(scale * Y[k * 2 * ld * ld + pp * ld + pp]);
+        v.add(kw[k] * scale * Y[k * 2 * ld * ld + pp * ld + pp]);
     }
     for (int i = threadIdx.x; i < N; i += 256) v.add(-1.5 * ombar[i]);
     v = comp::block_sum256(v, sh);
@@ -442,7 +461,7 @@ __global__ void __launch_bounds__(256) k_energy_periodic(const double *Y, long l
 }
 
 // ---- MBD gradient of the periodic energy ---------------------------------------------
-// Thread (i <= j) of tile (I, J) at Bloch vector k: with z = w_ij Z_k[i, j] (w_ij = zscale/(4 nk),
+// Thread (i <= j) of tile (I, J) at Bloch vector k: with z = w_ij Z_k[i, j] (w_ij = kw_k zscale/(4 nkt),
 // doubled for i != j, which folds in block (j, i)), only the symmetric part zs of the
 // block meets the (symmetric) tensors.  Accumulates
 //   zT = Re <conj zs, T^lr> (the self term included for i = j), zS = Re <conj zs, dT^lr/dS>, zx = Re <conj zs, dT^lr/dx>,
@@ -468,7 +487,7 @@ __global__ void __launch_bounds__(256) k_mbd_grad_periodic(AtomBufs b, PeriodicB
     double zT = 0.0, zS = 0.0, zx[3] = {0, 0, 0}, zA[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     double su = 0.0, M1[3] = {0, 0, 0}, M2[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (valid) {
-        const double w = 0.25 * zscale / p.nk * (i == j ? 1.0 : 2.0);
+        const double w = 0.25 * zscale / p.nkt * p.kw[kq] * (i == j ? 1.0 : 2.0);
         const double *Zr = Z + static_cast<long long>(kq) * 2 * ld * ld, *Zi = Zr + ld * ld;
         const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
         for (int e = 0; e < 6; ++e) {
@@ -596,22 +615,22 @@ __global__ void __launch_bounds__(256) k_mbd_grad_periodic(AtomBufs b, PeriodicB
     for (int e = 0; e < 9; ++e) atomicAdd(&gA[e], cij * zA[e]);
 }
 
-// g_ombar = zscale/(4 nk) sum_k Re Tr Z_k[i,i] 2 omega_bar_i - 3/2 + g_c sqrt(abar0), or, with tq_i
+// g_ombar = zscale/4 (zscale here over nkt) sum_k kw_k Re Tr Z_k[i,i] 2 omega_bar_i - 3/2 + g_c sqrt(abar0), or, with tq_i
 // = (1/nk) sum_k Re Tr (Q(q_k)^{1/2})_ii given, the same derivative as tq_i / (2 omega_bar_i) - 3/2
 // (the diagonal and coupling terms of dQ/d omega_bar_i together, second order in the error of Z);
 // g_abar0 = g_c omega_bar / (2 sqrt(abar0)).
-__global__ void k_mbd_grad_periodic_finalize(AtomBufs b, const double *Z, long long ld, int nk, double zscale,
-                                             const double *g_c, MbdGradOut o, const double *tq) {
+__global__ void k_mbd_grad_periodic_finalize(AtomBufs b, const double *Z, long long ld, int nk, const double *kw,
+                                             double zscale, const double *g_c, MbdGradOut o, const double *tq) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= b.N) return;
     double d = 0.0;
     for (int k = 0; k < nk; ++k) {
         const double *Zr = Z + static_cast<long long>(k) * 2 * ld * ld;
-        for (int xx = 0; xx < 3; ++xx) d += Zr[(3LL * i + xx) * ld + 3 * i + xx];
+        for (int xx = 0; xx < 3; ++xx) d += kw[k] * Zr[(3LL * i + xx) * ld + 3 * i + xx];
     }
     const double sa = sqrt(b.abar0[i]);
     o.g_ombar[i] = tq ? tq[i] / (2.0 * b.ombar[i]) - 1.5
-                      : 0.25 * zscale / nk * d * 2.0 * b.ombar[i] - 1.5 + g_c[i] * sa;
+                      : 0.25 * zscale * d * 2.0 * b.ombar[i] - 1.5 + g_c[i] * sa;
     o.g_abar0[i] = g_c[i] * b.ombar[i] / (2.0 * sa);
 }
 
@@ -625,103 +644,120 @@ __global__ void k_mean_rows(const double *x, int rows, int N, double *out) {
 }
 
 // ---- SCS adjoint over lattice images -------------------------------------------------
-// One CTA (128 threads) per atom i; partners j = 0..N-1 including j = i (its images).
 // With Ws = V_i X_j^T + X_i V_j^T per frequency (blocks (i,j) and (j,i) folded), every
 // term of the finite pass is summed over the images r = R_j - R_i + n A, and
 // dE/dA_cd += 1/2 (-1/3) n_c <Ws, dB/dr_d> (each unordered pair is visited from both ends).
+// One CTA (128 threads) per atom i and kGradFreq frequencies; its units are partners j = 0..N-1 including
+// j = i (its images), each partner's images dealt out to kScsSplit units.  Bound by FP64 arithmetic as the
+// matrix build; one CTA per atom with all frequencies left two thirds of the chip idle with 96
+// atoms (11.2 ms, 5.8 so).  Partial sums per CTA: part[group][atom] = (g_rv, gR, gA), gal[k][atom].
+constexpr int kGradFreq = 2, kScsSplit = 4, kScsPart = 13;
 __global__ void __launch_bounds__(128) k_scs_grad_periodic(AtomBufs b, CellGeom c, double beta, double a,
                                                            const double *X, const double *V, long long xstride,
-                                                           double *g_a0, double *g_om, double *g_rv, double *gR,
-                                                           double *gA_part) {
-    extern __shared__ double gal_s[];   // [nf1][128]
-    const int i = blockIdx.x, t = threadIdx.x;
-    for (int k = 0; k < b.nf1; ++k) gal_s[k * 128 + t] = 0.0;
-    double acc[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // g_rv, gR x3, gA x9
-    for (int j = t; j < b.N; j += 128) {
+                                                           double *part, double *gal_out) {
+    const int i = blockIdx.x, t = threadIdx.x, k0 = blockIdx.y * kGradFreq;
+    double acc[kScsPart + kGradFreq];   // g_rv, gR x3, gA x9, then dE/d alpha_i(u) of the frequencies
+#pragma unroll
+    for (int e = 0; e < kScsPart + kGradFreq; ++e) acc[e] = 0.0;
+    for (int unit = t; unit < b.N * kScsSplit; unit += 128) {
+        const int j = unit / kScsSplit, part_of = unit % kScsSplit;
         const double x[3] = {b.R[3 * j] - b.R[3 * i], b.R[3 * j + 1] - b.R[3 * i + 1], b.R[3 * j + 2] - b.R[3 * i + 2]};
         int lo[3], hi[3];
         image_box(c, x, lo, hi);
+        const int d1 = hi[1] - lo[1] + 1, d2 = hi[2] - lo[2] + 1, boxes = (hi[0] - lo[0] + 1) * d1 * d2;
         const double S = b.rv[i] + b.rv[j];
-        for (int k = 0; k < b.nf1; ++k) {
+        double Ws[kGradFreq][9], s[kGradFreq], dsda[kGradFreq];
+#pragma unroll
+        for (int f = 0; f < kGradFreq; ++f) {
+            const int k = min(k0 + f, b.nf1 - 1);
             const double *Vk = V + k * xstride, *Xk = X + k * xstride;
-            double Ws[9];
             for (int xx = 0; xx < 3; ++xx)
                 for (int y = 0; y < 3; ++y) {
                     double w = 0.0;
                     for (int cc = 0; cc < 3; ++cc)
                         w += Vk[9LL * i + 3 * xx + cc] * Xk[9LL * j + 3 * y + cc] +
                              Xk[9LL * i + 3 * xx + cc] * Vk[9LL * j + 3 * y + cc];
-                    Ws[3 * xx + y] = w;
+                    Ws[f][3 * xx + y] = k0 + f < b.nf1 ? w : 0.0;
                 }
-            const double tr = Ws[0] + Ws[4] + Ws[8];
-            const double si = b.sig_u[k * b.N + i], sj = b.sig_u[k * b.N + j], s = sqrt(si * si + sj * sj);
-            const double dsda = si * si / (3.0 * s * b.al_u[k * b.N + i]);
-            double gal = 0.0;
-            for (int n0 = lo[0]; n0 <= hi[0]; ++n0)
-                for (int n1 = lo[1]; n1 <= hi[1]; ++n1)
-                    for (int n2 = lo[2]; n2 <= hi[2]; ++n2) {
-                        const int nn[3] = {n0, n1, n2};
-                        double r[3];
-                        for (int e = 0; e < 3; ++e) r[e] = x[e] + n0 * c.A[e] + n1 * c.A[3 + e] + n2 * c.A[6 + e];
-                        const double rho2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-                        if (rho2 >= c.rc * c.rc || rho2 < 1e-16) continue;
-                        const double rho = sqrt(rho2), ir = 1.0 / rho;
-                        const Fermi f = fermi(rho, S, beta, a);
-                        const double sr = 1.0 - f.f;
-                        if (sr == 0.0 && f.df_drho == 0.0 && f.df_dS == 0.0) continue;   // exact zeros
-                        double Wr[3], Wtr[3];
-                        for (int xx = 0; xx < 3; ++xx) {
-                            Wr[xx] = Ws[3 * xx] * r[0] + Ws[3 * xx + 1] * r[1] + Ws[3 * xx + 2] * r[2];
-                            Wtr[xx] = Ws[xx] * r[0] + Ws[3 + xx] * r[1] + Ws[6 + xx] * r[2];
-                        }
-                        const double rWr = r[0] * Wr[0] + r[1] * Wr[1] + r[2] * Wr[2];
-                        const Radial qd = tgg_radial(rho, s);
-                        const double WT = qd.P * tr + qd.W * rWr;
-                        const double WTs = qd.dPs * tr + qd.dWs * rWr;
-                        gal += -1.0 / 3.0 * sr * WTs * dsda;
-                        acc[0] += -1.0 / 3.0 * (-f.df_dS) * WT;
-                        for (int cc = 0; cc < 3; ++cc) {
-                            const double WdT = (qd.dP * tr + qd.dW * rWr) * r[cc] * ir + qd.W * (Wr[cc] + Wtr[cc]);
-                            const double dB = sr * WdT - f.df_drho * r[cc] * ir * WT;   // <Ws, dB/dr_cc>
-                            if (j != i) acc[1 + cc] += 1.0 / 3.0 * dB;
-                            for (int kk = 0; kk < 3; ++kk) acc[4 + 3 * kk + cc] += -1.0 / 6.0 * nn[kk] * dB;
-                        }
-                    }
-            gal_s[k * 128 + t] += gal;
+            const double si = b.sig_u[k * b.N + i], sj = b.sig_u[k * b.N + j];
+            s[f] = sqrt(si * si + sj * sj);
+            dsda[f] = si * si / (3.0 * s[f] * b.al_u[k * b.N + i]);
+        }
+        for (int box = part_of; box < boxes; box += kScsSplit) {
+            const int nn[3] = {lo[0] + box / (d1 * d2), lo[1] + box / d2 % d1, lo[2] + box % d2};
+            double r[3];
+            for (int e = 0; e < 3; ++e) r[e] = x[e] + nn[0] * c.A[e] + nn[1] * c.A[3 + e] + nn[2] * c.A[6 + e];
+            const double rho2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
+            if (rho2 >= c.rc * c.rc || rho2 < 1e-16) continue;
+            const double rho = sqrt(rho2), ir = 1.0 / rho;
+            const Fermi f = fermi(rho, S, beta, a);
+            const double sr = 1.0 - f.f;
+            if (sr == 0.0 && f.df_drho == 0.0 && f.df_dS == 0.0) continue;   // exact zeros
+            double dBs[3] = {0.0, 0.0, 0.0}, wts = 0.0;
+#pragma unroll
+            for (int q = 0; q < kGradFreq; ++q) {
+                double Wr[3], Wtr[3];
+                for (int xx = 0; xx < 3; ++xx) {
+                    Wr[xx] = Ws[q][3 * xx] * r[0] + Ws[q][3 * xx + 1] * r[1] + Ws[q][3 * xx + 2] * r[2];
+                    Wtr[xx] = Ws[q][xx] * r[0] + Ws[q][3 + xx] * r[1] + Ws[q][6 + xx] * r[2];
+                }
+                const double tr = Ws[q][0] + Ws[q][4] + Ws[q][8];
+                const double rWr = r[0] * Wr[0] + r[1] * Wr[1] + r[2] * Wr[2];
+                const Radial qd = tgg_radial(rho, s[q]);
+                const double WT = qd.P * tr + qd.W * rWr;
+                const double WTs = qd.dPs * tr + qd.dWs * rWr;
+                acc[kScsPart + q] += -1.0 / 3.0 * sr * WTs * dsda[q];
+                wts += WT;
+                for (int cc = 0; cc < 3; ++cc) {
+                    const double WdT = (qd.dP * tr + qd.dW * rWr) * r[cc] * ir + qd.W * (Wr[cc] + Wtr[cc]);
+                    dBs[cc] += sr * WdT - f.df_drho * r[cc] * ir * WT;   // <Ws, dB/dr_cc>
+                }
+            }
+            acc[0] += 1.0 / 3.0 * f.df_dS * wts;
+            for (int cc = 0; cc < 3; ++cc) {
+                if (j != i) acc[1 + cc] += 1.0 / 3.0 * dBs[cc];
+                for (int kk = 0; kk < 3; ++kk) acc[4 + 3 * kk + cc] += -1.0 / 6.0 * nn[kk] * dBs[cc];
+            }
         }
     }
-    __syncthreads();
-    __shared__ double scratch[4 * 13];
-    block_sum128<13>(acc, scratch);
-    if (t < b.nf1) {
-        const int k = t;
-        double sacc = 0.0;
-        for (int e = 0; e < 128; ++e) sacc += gal_s[k * 128 + e];
+    __shared__ double scratch[4 * (kScsPart + kGradFreq)];
+    block_sum128<kScsPart + kGradFreq>(acc, scratch);
+    if (t != 0) return;
+    for (int e = 0; e < kScsPart; ++e) part[(static_cast<long long>(blockIdx.y) * b.N + i) * kScsPart + e] = acc[e];
+#pragma unroll
+    for (int q = 0; q < kGradFreq; ++q) {
+        const int k = k0 + q;
+        if (k >= b.nf1) break;
+        // the diagonal block
         const double *Vk = V + k * xstride, *Xk = X + k * xstride;
         double wd = 0.0;
         for (int e = 0; e < 9; ++e) wd += Vk[9LL * i + e] * Xk[9LL * i + e];
         const double al = b.al_u[k * b.N + i];
-        sacc += -1.0 / 3.0 * wd * (-1.0 / (al * al));
-        gal_s[k * 128] = sacc;
+        gal_out[k * b.N + i] = acc[kScsPart + q] - 1.0 / 3.0 * wd * (-1.0 / (al * al));
     }
-    __syncthreads();
-    if (t == 0) {
-        double ga0 = 0.0, gom = 0.0;
-        const double a0 = b.a0[i], om = b.om[i];
-        for (int k = 0; k < b.nf1; ++k) {
-            const double u = b.u[k], qq = 1.0 + u * u / (om * om);
-            const double gl = gal_s[k * 128];
-            ga0 += gl / qq;
-            gom += gl * a0 * 2.0 * u * u / (om * om * om) / (qq * qq);
-        }
-        g_a0[i] += ga0;
-        g_om[i] += gom;
-        g_rv[i] += acc[0];
-        gR[3 * i] += acc[1];
-        gR[3 * i + 1] += acc[2];
-        gR[3 * i + 2] += acc[3];
-        for (int e = 0; e < 9; ++e) gA_part[9LL * i + e] = acc[4 + e];
+}
+
+// Sums of the partial results of atom i, in a fixed order; the chain from alpha_i(u) to (alpha0, omega).
+__global__ void k_scs_grad_periodic_sum(AtomBufs b, const double *part, int groups, const double *gal, double *g_a0,
+                                        double *g_om, double *g_rv, double *gR, double *gA_part) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= b.N) return;
+    double acc[kScsPart];
+    for (int e = 0; e < kScsPart; ++e) acc[e] = 0.0;
+    for (int g = 0; g < groups; ++g)
+        for (int e = 0; e < kScsPart; ++e) acc[e] += part[(static_cast<long long>(g) * b.N + i) * kScsPart + e];
+    double ga0 = 0.0, gom = 0.0;
+    const double a0 = b.a0[i], om = b.om[i];
+    for (int k = 0; k < b.nf1; ++k) {
+        const double u = b.u[k], qq = 1.0 + u * u / (om * om), gl = gal[k * b.N + i];
+        ga0 += gl / qq;
+        gom += gl * a0 * 2.0 * u * u / (om * om * om) / (qq * qq);
     }
+    g_a0[i] += ga0;
+    g_om[i] += gom;
+    g_rv[i] += acc[0];
+    for (int e = 0; e < 3; ++e) gR[3 * i + e] += acc[1 + e];
+    for (int e = 0; e < 9; ++e) gA_part[9LL * i + e] = acc[4 + e];
 }
 
 // gA[e] += sum_i part[i][e] (fixed order).
@@ -746,8 +782,8 @@ void structure_factors(const AtomBufs &b, const PeriodicBufs &p, cudaStream_t s)
 void build_scs_periodic(const AtomBufs &b, const CellGeom &c, double beta, double a, double *M, long long ld,
                         long long mstride, int *status, cudaStream_t s) {
     count_launches(1);
-    k_build_scs_periodic<<<dim3(cdiv(b.N, 32), cdiv(b.N, 8)), dim3(32, 8), 0, s>>>(b, c, beta, a, M, ld, mstride,
-                                                                                    status);
+    k_build_scs_periodic<<<dim3(cdiv(b.N, 32), cdiv(b.N, 4), cdiv(b.nf1, kScsFreq)), dim3(32, 4), 0, s>>>(
+        b, c, beta, a, M, ld, mstride, status);
     pad_identity(M, ld, 3 * b.N, b.nf1, mstride, s);
 }
 
@@ -841,10 +877,10 @@ void caxpby_identity(double *Z, const double *P, long long ld, int nk, double a,
     k_caxpby_identity<<<1216, 256, 0, s>>>(Z, P, ld, static_cast<long long>(nk) * 2 * ld * ld, a, b);
 }
 
-void cfrob_dev_identity(const double *P, long long ld, int n, int nk, double *out, cudaStream_t s) {
+void cfrob_dev_identity(const double *P, long long ld, int n, int nk, const double *kw, double *out, cudaStream_t s) {
     cudaMemsetAsync(out, 0, sizeof(double), s);
     count_launches(1);
-    k_cfrob_dev_identity<<<1216, 256, 0, s>>>(P, ld, n, nk, out);
+    k_cfrob_dev_identity<<<1216, 256, 0, s>>>(P, ld, n, nk, kw, out);
 }
 
 void cmax_abs_rowsum(const double *Q, long long ld, int nk, double *out, cudaStream_t s) {
@@ -884,10 +920,10 @@ void clanczos_coefficients(const double *Q, long long ld, int nk, int steps, dou
     }
 }
 
-void energy_trace_periodic(const double *Y, long long ld, int n, int nk, const double *ombar, int N,
+void energy_trace_periodic(const double *Y, long long ld, int n, const PeriodicBufs &p, const double *ombar, int N,
                            double sqrt_s, double *out, cudaStream_t s) {
     count_launches(1);
-    k_energy_periodic<<<1, 256, 0, s>>>(Y, ld, n, nk, ombar, N, 0.5 * sqrt_s / nk, out);
+    k_energy_periodic<<<1, 256, 0, s>>>(Y, ld, n, p.nk, p.kw, ombar, N, 0.5 * sqrt_s / p.nkt, out);
 }
 
 void mean_rows(const double *x, int rows, int N, double *out, cudaStream_t s) {
@@ -910,15 +946,21 @@ void periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double beta, do
         k_mbd_grad_periodic<float><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, g_c, o.g_rbar, o.gR, gA);
     else
         k_mbd_grad_periodic<double><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, g_c, o.g_rbar, o.gR, gA);
-    k_mbd_grad_periodic_finalize<<<cdiv(b.N, 128), 128, 0, s>>>(b, Z, ld, p.nk, zscale, g_c, o, tq);
+    k_mbd_grad_periodic_finalize<<<cdiv(b.N, 128), 128, 0, s>>>(b, Z, ld, p.nk, p.kw, zscale / p.nkt, g_c, o, tq);
+}
+
+long long scs_grad_periodic_words(int N, int nf1) {
+    return static_cast<long long>(N) * (9 + kScsPart * cdiv(nf1, kGradFreq) + nf1);
 }
 
 void scs_grad_periodic(const AtomBufs &b, const CellGeom &c, double beta, double a, const double *X,
                        const double *V, long long xstride, double *g_a0, double *g_om, double *g_rv, double *gR,
-                       double *gA_part, double *gA, cudaStream_t s) {
-    count_launches(2);
-    k_scs_grad_periodic<<<b.N, 128, sizeof(double) * b.nf1 * 128, s>>>(b, c, beta, a, X, V, xstride, g_a0, g_om,
-                                                                       g_rv, gR, gA_part);
+                       double *work, double *gA, cudaStream_t s) {
+    const int groups = cdiv(b.nf1, kGradFreq);
+    double *gA_part = work, *gal = gA_part + 9LL * b.N, *part = gal + static_cast<long long>(b.nf1) * b.N;
+    count_launches(3);
+    k_scs_grad_periodic<<<dim3(b.N, groups), 128, 0, s>>>(b, c, beta, a, X, V, xstride, part, gal);
+    k_scs_grad_periodic_sum<<<cdiv(b.N, 64), 64, 0, s>>>(b, part, groups, gal, g_a0, g_om, g_rv, gR, gA_part);
     k_reduce_lattice<<<1, 32, 0, s>>>(gA_part, b.N, gA);
 }
 

@@ -136,15 +136,16 @@ struct mbd_ctx {
     // periodic systems: cell, Bloch vectors and reciprocal lattice (host lists, device copies)
     bool periodic = false;
     int nk = 1, nG = 0, maxG = 0;
+    int nkt = 1;   // Bloch vectors of the whole grid, of which nk are kept (with weights hkw, the sum nkt)
     CellGeom cell{};
-    std::vector<double> hkq, hG;
+    std::vector<double> hkq, hkw, hG;
     std::vector<int> hglist, hgcount;
     // FP64 path: residue planes of three operands and the bytes of a product (k_crt.cu), or the
     // scratch of products taken in panels; dPT: the transpose of P.  Null when they did not fit:
     // the products then run on the FP64 pipe.
     char *crt = nullptr;
     double *dPT = nullptr;
-    double *dkq = nullptr, *dG = nullptr, *dcoef = nullptr, *dlzw = nullptr, *dgA = nullptr, *dgAout = nullptr,
+    double *dkq = nullptr, *dkw = nullptr, *dG = nullptr, *dcoef = nullptr, *dlzw = nullptr, *dgA = nullptr, *dgAout = nullptr,
            *dgApart = nullptr, *dgc = nullptr, *dtsg = nullptr;
     int *dglist = nullptr, *dgcount = nullptr;
     double2 *dS = nullptr;
@@ -426,12 +427,13 @@ int allocate(mbd_ctx *ctx) {
     const long long nk = ctx->nk;
     if (ctx->periodic) {
         plan.push_back({&ctx->dkq, 3 * nk});
+        plan.push_back({&ctx->dkw, nk});
         plan.push_back({&ctx->dG, 3LL * ctx->nG});
         plan.push_back({&ctx->dcoef, nk * 2 * kLanczosSteps});
         plan.push_back({&ctx->dlzw, 3 * nk * 2 * ld});
         plan.push_back({&ctx->dgA, 9});
         plan.push_back({&ctx->dgAout, 9});
-        plan.push_back({&ctx->dgApart, 9 * N});
+        plan.push_back({&ctx->dgApart, scs_grad_periodic_words(static_cast<int>(N), static_cast<int>(nf1))});
         plan.push_back({&ctx->dgc, N});
         plan.push_back({&ctx->dtsg, 2LL * ctx->nG});
         plan.push_back({reinterpret_cast<double **>(&ctx->dS), 2LL * ctx->nG * N});
@@ -554,6 +556,7 @@ int allocate(mbd_ctx *ctx) {
 // Uploads the Bloch vectors and reciprocal-vector lists of a periodic geometry.
 int upload_periodic(mbd_ctx *ctx) {
     cudaError_t e = cudaMemcpy(ctx->dkq, ctx->hkq.data(), sizeof(double) * ctx->hkq.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(ctx->dkw, ctx->hkw.data(), sizeof(double) * ctx->hkw.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(ctx->dG, ctx->hG.data(), sizeof(double) * ctx->hG.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(ctx->dglist, ctx->hglist.data(), sizeof(int) * ctx->hglist.size(), cudaMemcpyHostToDevice);
@@ -564,15 +567,15 @@ int upload_periodic(mbd_ctx *ctx) {
 }
 
 PeriodicBufs periodic_bufs(mbd_ctx *ctx) {
-    return PeriodicBufs{ctx->cell, ctx->nk, ctx->nG, ctx->maxG, ctx->dkq, ctx->dG, ctx->dglist, ctx->dgcount, ctx->dS};
+    return PeriodicBufs{ctx->cell, ctx->nk, ctx->nkt, ctx->nG, ctx->maxG, ctx->dkq, ctx->dkw, ctx->dG, ctx->dglist, ctx->dgcount, ctx->dS};
 }
 
 // Host preparation of a periodic geometry: cell inverse and reciprocal vectors, Ewald
 // parameters, Monkhorst-Pack Bloch vectors and the reciprocal vectors of each.
 struct PeriodicSetup {
     CellGeom cell{};
-    int nk = 0, nG = 0, maxG = 0;
-    std::vector<double> kq, G;
+    int nk = 0, nkt = 0, nG = 0, maxG = 0;
+    std::vector<double> kq, kw, G;
     std::vector<int> glist, gcount;
     std::string msg;
 };
@@ -603,12 +606,20 @@ int periodic_setup(const mbd_options &o, const double *A, const int *grid, Perio
     c.rc = rc;
     c.kc = kc;
     auto norm = [](const double *v) { return std::sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]); };
-    // Monkhorst-Pack: kappa_c = (2m - n_c - 1)/(2 n_c), q = kappa B
-    ps.nk = grid[0] * grid[1] * grid[2];
+    // Monkhorst-Pack: kappa_c = (2m - n_c - 1)/(2 n_c), q = kappa B.  The grid holds -q with every q, and
+    // Q(-q) is the conjugate of Q(q), with the same spectrum and the conjugate inverse root: the FP64 path keeps
+    // one of the two with weight 2.  (The mixed modes' rounding differs between the two; they keep
+    // the whole grid.)
+    const bool pairs = fp64_path(o.precision);
+    ps.nkt = grid[0] * grid[1] * grid[2];
     double qmax = 0.0;
     for (int m0 = 1; m0 <= grid[0]; ++m0)
         for (int m1 = 1; m1 <= grid[1]; ++m1)
             for (int m2 = 1; m2 <= grid[2]; ++m2) {
+                const int t[3] = {2 * m0 - grid[0] - 1, 2 * m1 - grid[1] - 1, 2 * m2 - grid[2] - 1};
+                const int sign = t[0] ? t[0] : (t[1] ? t[1] : t[2]);
+                if (pairs && sign < 0) continue;
+                ps.kw.push_back(pairs && sign > 0 ? 2.0 : 1.0);
                 const double kap[3] = {(2.0 * m0 - grid[0] - 1) / (2.0 * grid[0]),
                                        (2.0 * m1 - grid[1] - 1) / (2.0 * grid[1]),
                                        (2.0 * m2 - grid[2] - 1) / (2.0 * grid[2])};
@@ -617,6 +628,7 @@ int periodic_setup(const mbd_options &o, const double *A, const int *grid, Perio
                 for (int e = 0; e < 3; ++e) ps.kq.push_back(q[e]);
                 qmax = std::max(qmax, norm(q));
             }
+    ps.nk = static_cast<int>(ps.kw.size());
     // every G = m B with |G + q| < kc for some q: |G| < kc + qmax, |m_c| <= (kc + qmax)|a_c|/(2 pi)
     const double gr = kc + qmax;
     int mm[3];
@@ -1099,12 +1111,12 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
             timed_cgemm(Z, Y, Y, true, nullptr, P, ctx->dPT, 1.0, 0.0, false);   // P = Z Y: not Hermitian in floating point
             Pk = P;
         }
-        cfrob_dev_identity(Pk, ld, n, nk, ctx->dscal + 2, s);
+        cfrob_dev_identity(Pk, ld, n, nk, ctx->dkw, ctx->dscal + 2, s);
         double r2 = 0.0;
         MBD_CUDA(cudaMemcpyAsync(&r2, ctx->dscal + 2, sizeof(double), cudaMemcpyDeviceToHost, s), "newton_schulz");
         MBD_CUDA(cudaStreamSynchronize(s), "newton_schulz");
         resid = std::sqrt(r2);
-        if (!std::isfinite(resid) || resid > 2.0 * std::sqrt(nd * nk) + 1.0) {
+        if (!std::isfinite(resid) || resid > 2.0 * std::sqrt(nd * ctx->nkt) + 1.0) {
             ctx->ns_iter = it;
             ctx->ns_resid = resid;
             return fail(ctx, MBD_ERR_NEG_EIGENVALUE, "newton_schulz",
@@ -1135,7 +1147,7 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
         if (st & ST_TC_TIMEOUT) return fail(ctx, MBD_ERR_CUDA, "newton_schulz", "tensor-core GEMM wait timed out");
     }
     if (!converged) return fail(ctx, MBD_ERR_NOT_CONVERGED, "newton_schulz", "iteration cap reached");
-    energy_trace_periodic(Y, ld, n, nk, ctx->dombar, N, ss, energy_out, s);
+    energy_trace_periodic(Y, ld, n, periodic_bufs(ctx), ctx->dombar, N, ss, energy_out, s);
     ctx->Zlast = Z;
     ctx->zscale = 1.0 / ss;
     }
@@ -1555,6 +1567,8 @@ int mbd_set_geometry(mbd_ctx *ctx, int n_atoms, const double *coords, const doub
     if (periodic) {
         ctx->cell = ps.cell;
         ctx->nk = ps.nk;
+        ctx->nkt = ps.nkt;
+        ctx->hkw = ps.kw;
         ctx->nG = ps.nG;
         ctx->maxG = ps.maxG;
         ctx->hkq = ps.kq;
@@ -1562,7 +1576,7 @@ int mbd_set_geometry(mbd_ctx *ctx, int n_atoms, const double *coords, const doub
         ctx->hglist = ps.glist;
         ctx->hgcount = ps.gcount;
     } else {
-        ctx->nk = 1;
+        ctx->nk = ctx->nkt = 1;
         ctx->nG = ctx->maxG = 0;
     }
     ctx->have_lattice_grad = false;
