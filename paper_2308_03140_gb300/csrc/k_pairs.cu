@@ -474,44 +474,89 @@ __global__ void k_scs_grad_inputs_f32(const double *X, const double *V, const do
     }
 }
 
-// TS pairwise dispersion (Secs. 2.6 and 2.7, Eq. pairwise with the TS oscillators of Eq. ts-scaling and
-// the damping of Eq. fermi-damping, steepness 20): one CTA per atom i, threads over j.  For
-// the pair (i, j) the energy is -C6_ij h(r), h = f/r^6, C6_ij = 3/2 a_i a_j w_i w_j / (w_i + w_j)
-// (the two ordered terms of -1/2 sum_{i != j}).  Per atom: eatom[i] = -1/2 sum_j C6_ij h_ij;
-// dE/dR_i = sum_j C6_ij h'(r) r_hat (r = R_j - R_i); dE/d a_i, dE/d w_i, dE/d R_vdW,i of the
-// TS-scaled oscillators (b.a0, b.om, b.rv) into ga0, gom, grv.
-__global__ void __launch_bounds__(128) k_ts_pairs(AtomBufs b, double s_r, double *eatom, double *gR, double *ga0,
-                                                  double *gom, double *grv) {
-    const int i = blockIdx.x;
-    const double ai = b.a0[i], wi = b.om[i], rvi = b.rv[i];
-    const double Ri[3] = {b.R[3 * i], b.R[3 * i + 1], b.R[3 * i + 2]};
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};   // e, gR x3, ga0, gom, grv
-    for (int j = threadIdx.x; j < b.N; j += 128) {
-        if (j == i) continue;
-        const double r[3] = {b.R[3 * j] - Ri[0], b.R[3 * j + 1] - Ri[1], b.R[3 * j + 2] - Ri[2]};
-        const double rho2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2], rho = sqrt(rho2);
-        const double aj = b.a0[j], wj = b.om[j];
-        const double c6 = 1.5 * ai * aj * wi * wj / (wi + wj);
-        const Fermi f = fermi(rho, rvi + b.rv[j], s_r, 20.0);
-        const double ir6 = 1.0 / (rho2 * rho2 * rho2);
-        const double h = f.f * ir6, dh = f.df_drho * ir6 - 6.0 * h / rho, dhS = f.df_dS * ir6;
-        acc[0] += -0.5 * c6 * h;
-        for (int c = 0; c < 3; ++c) acc[1 + c] += c6 * dh * r[c] / rho;
-        acc[4] += -h * c6 / ai;
-        acc[5] += -h * c6 * (1.0 / wi - 1.0 / (wi + wj));
-        acc[6] += -c6 * dhS;
+// TS pairwise energy and gradients: a CTA takes the pairs of two tiles of 32 atoms, every unordered pair
+// once (i in tile I, j in tile J, i < j), and writes both ends' sums of the tile pair to
+// part[other tile][7][atom]; k_ts_sum adds them up in a fixed order.  Bound by FP64 arithmetic: four
+// divisions, a square root and an exponential a pair of about 150 operations (each ordered pair for itself with a
+// division wherever the formula has one, 250 operations: 1.36 ms for 2000 atoms, RESULT).
+constexpr int kTsTile = 32, kTsVals = 7;   // e, gR x3, ga0, gom, grv
+__global__ void __launch_bounds__(256) k_ts_pairs(AtomBufs b, double s_r, int tiles, double *part) {
+    int J = static_cast<int>((sqrtf(8.0f * blockIdx.x + 1.0f) - 1.0f) * 0.5f);
+    while ((J + 1) * (J + 2) / 2 <= static_cast<int>(blockIdx.x)) ++J;
+    while (J * (J + 1) / 2 > static_cast<int>(blockIdx.x)) --J;
+    const int I = static_cast<int>(blockIdx.x) - J * (J + 1) / 2;   // I <= J
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, j = J * kTsTile + tx;
+    __shared__ double sj[8][kTsVals][kTsTile];   // the warps' sums for the atoms j
+    double aj = 1.0, wj = 1.0, rvj = 1.0, iaj = 1.0, iwj = 1.0, Rj[3] = {0.0, 0.0, 0.0};
+    if (j < b.N) {
+        aj = b.a0[j];
+        wj = b.om[j];
+        rvj = b.rv[j];
+        iaj = 1.0 / aj;
+        iwj = 1.0 / wj;
+        for (int c = 0; c < 3; ++c) Rj[c] = b.R[3 * j + c];
     }
-    __shared__ double scratch[4 * 7];
-    block_sum128<7>(acc, scratch);
-    if (threadIdx.x == 0) {
-        eatom[i] = acc[0];
-        gR[3 * i] = acc[1];
-        gR[3 * i + 1] = acc[2];
-        gR[3 * i + 2] = acc[3];
-        ga0[i] = acc[4];
-        gom[i] = acc[5];
-        grv[i] = acc[6];
+    double accj[kTsVals] = {0, 0, 0, 0, 0, 0, 0};
+    for (int u = 0; u < kTsTile / 8; ++u) {   // a warp's rows: ty, ty + 8, ...
+        const int i = I * kTsTile + ty + 8 * u;
+        if (i >= b.N) continue;   // the same for the whole warp
+        double acc[kTsVals] = {0, 0, 0, 0, 0, 0, 0};
+        if (j < b.N && i < j) {
+            const double ai = b.a0[i], wi = b.om[i];
+            const double r[3] = {Rj[0] - b.R[3 * i], Rj[1] - b.R[3 * i + 1], Rj[2] - b.R[3 * i + 2]};
+            const double rho = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]), ir = 1.0 / rho, ir2 = ir * ir;
+            const double iw = 1.0 / (wi + wj), c6 = 1.5 * ai * aj * wi * wj * iw;
+            // Fermi damping of steepness 20 and its derivatives (pair_math.cuh)
+            const double iS = 1.0 / (s_r * (b.rv[i] + rvj)), x = rho * iS;
+            const double f = 1.0 / (1.0 + exp(-20.0 * (x - 1.0))), df = 20.0 * f * (1.0 - f);
+            const double ir6 = ir2 * ir2 * ir2, h = f * ir6, hc = h * c6;
+            const double dh = (df * iS * ir6 - 6.0 * h * ir) * c6 * ir;
+            acc[0] = -0.5 * hc;
+            for (int c = 0; c < 3; ++c) acc[1 + c] = dh * r[c];
+            acc[6] = c6 * ir6 * df * x * s_r * iS;   // -c6 dh/dS
+            accj[0] += acc[0];
+            for (int c = 0; c < 3; ++c) accj[1 + c] -= acc[1 + c];
+            accj[4] -= hc * iaj;
+            accj[5] -= hc * (iwj - iw);
+            accj[6] += acc[6];
+            acc[4] = -hc;             // over alpha_i and with 1/omega_i below
+            acc[5] = hc * iw;
+        }
+#pragma unroll
+        for (int e = 0; e < kTsVals; ++e) acc[e] = warp_sum(acc[e]);
+        if (tx == 0) {
+            const double hc = -acc[4];
+            acc[5] -= hc / b.om[i];
+            acc[4] = -hc / b.a0[i];
+            double *p = part + static_cast<long long>(J) * kTsVals * b.N + i;
+            // (the diagonal tile's other ends are added below)
+            for (int e = 0; e < kTsVals; ++e) p[static_cast<long long>(e) * b.N] = acc[e];
+        }
     }
+#pragma unroll
+    for (int e = 0; e < kTsVals; ++e) sj[ty][e][tx] = accj[e];
+    __syncthreads();
+    if (ty < kTsVals && j < b.N) {
+        double s = 0.0;
+        for (int w = 0; w < 8; ++w) s += sj[w][ty][tx];
+        double *p = part + (static_cast<long long>(I) * kTsVals + ty) * b.N + j;
+        *p = I == J ? *p + s : s;
+    }
+}
+
+// Sums over the partner tiles, a warp per atom and value.
+__global__ void __launch_bounds__(256) k_ts_sum(int N, int tiles, const double *part, double *eatom, double *gR,
+                                                double *ga0, double *gom, double *grv) {
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31), e = threadIdx.x >> 5;
+    if (i >= N || e >= kTsVals) return;
+    double s = 0.0;
+#pragma unroll 8
+    for (int t = 0; t < tiles; ++t) s += part[(static_cast<long long>(t) * kTsVals + e) * N + i];
+    if (e == 0) eatom[i] = s;
+    else if (e < 4) gR[3 * i + e - 1] = s;
+    else if (e == 4) ga0[i] = s;
+    else if (e == 5) gom[i] = s;
+    else grv[i] = s;
 }
 
 __global__ void k_ts_chain(AtomBufs b, const double *g_a0, const double *g_om, const double *g_rv,
@@ -637,9 +682,11 @@ void nl_chain(const AtomBufs &b, const MbdGradOut &o, const double *scale, doubl
 }
 
 void ts_pairs(const AtomBufs &b, double s_r, double *eatom, double *gR, double *ga0, double *gom, double *grv,
-              cudaStream_t s) {
-    count_launches(1);
-    k_ts_pairs<<<b.N, 128, 0, s>>>(b, s_r, eatom, gR, ga0, gom, grv);
+              double *work, cudaStream_t s) {
+    const int tiles = (b.N + kTsTile - 1) / kTsTile;
+    count_launches(2);
+    k_ts_pairs<<<tiles * (tiles + 1) / 2, 256, 0, s>>>(b, s_r, tiles, work);
+    k_ts_sum<<<tiles, 256, 0, s>>>(b.N, tiles, work, eatom, gR, ga0, gom, grv);
 }
 
 void ts_chain(const AtomBufs &b, const double *g_a0, const double *g_om, const double *g_rv,

@@ -1801,7 +1801,7 @@ int mbd_ts_energy(mbd_ctx *ctx, double s_r, double *energy, double *grad_coords,
     MBD_CUDA(cudaMemsetAsync(ctx->dstatus, 0, sizeof(int), s), "mbd_ts_energy");
     const AtomBufs b = atom_bufs(ctx, Inputs{ctx->dR, ctx->da0ref, ctx->dc6ref, ctx->drref, ctx->dratio});
     prepare_atoms(b, ctx->dstatus, s);   // TS-scaled oscillators (Eq. ts-scaling) and input checks
-    // scratch: per-atom energies in dh, dE/d(a0, om, rv) in dga0, dgom, dgrv (and for a cell
+    // scratch: partial sums in dM, per-atom energies in dh, dE/d(a0, om, rv) in dga0, dgom, dgrv (and for a cell
     // the lattice parts in dgApart, their sum in dgA); the next evaluation rewrites all of
     // them before use
     if (ctx->periodic) {
@@ -1810,7 +1810,7 @@ int mbd_ts_energy(mbd_ctx *ctx, double s_r, double *energy, double *grad_coords,
         ts_periodic(b, pb, s_r, ctx->dtsg, ctx->dh, ctx->dgR, ctx->dga0, ctx->dgom, ctx->dgrv, ctx->dgApart,
                     ctx->dgA, ctx->dstatus, s);
     } else {
-        ts_pairs(b, s_r, ctx->dh, ctx->dgR, ctx->dga0, ctx->dgom, ctx->dgrv, s);
+        ts_pairs(b, s_r, ctx->dh, ctx->dgR, ctx->dga0, ctx->dgom, ctx->dgrv, ctx->dM, s);   // (dM: 144 N^2 doubles)
     }
     if (grad_params) ts_chain(b, ctx->dga0, ctx->dgom, ctx->dgrv, nullptr, ctx->dgp, s);
     std::vector<double> ea(N);
