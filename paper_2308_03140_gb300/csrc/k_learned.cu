@@ -474,7 +474,9 @@ __global__ void k_dyson_forces(int n, int n_sys, const int *offsets, const doubl
     }
 }
 
-// Shared layout of the MLP kernels: weights (FP16), standardised inputs, two hidden layers.
+// Shared layout of the parameter-gradient kernel: weights (FP16), and the standardised inputs and two hidden
+// layers of the CTA's kTA atoms, atom by atom along a row ([unit][atom], rows of kTS words).
+constexpr int kTS = kTA + 4;
 struct MlpSmem {
     __half *W;
     float *Xs, *h1, *h2;
@@ -483,25 +485,15 @@ __device__ __forceinline__ MlpSmem mlp_smem(char *base) {
     MlpSmem m;
     m.W = reinterpret_cast<__half *>(base);
     m.Xs = reinterpret_cast<float *>(base + ((kParams * 2 + 15) / 16) * 16);
-    m.h1 = m.Xs + kTA * kF;
-    m.h2 = m.h1 + kTA * kH;
+    m.h1 = m.Xs + kTS * kF;
+    m.h2 = m.h1 + kTS * kH;
     return m;
 }
-constexpr size_t kMlpSmem = ((kParams * 2 + 15) / 16) * 16 + sizeof(float) * (kTA * kF + 2 * kTA * kH);
-
-__device__ __forceinline__ void load_params_and_inputs(const MlpSmem &m, const __half *P, const float *X,
-                                                       const float *mean, const float *stdv, int a0, int B) {
-    const int t = threadIdx.x;
-    for (int e = t; e < kParams; e += blockDim.x) m.W[e] = P[e];
-    for (int e = t; e < kTA * kF; e += blockDim.x) {
-        const int a = e / kF, k = e % kF, atom = a0 + a;
-        m.Xs[e] = atom < B ? (X[static_cast<long long>(atom) * kF + k] - mean[k]) / stdv[k] : 0.0f;
-    }
-    __syncthreads();
-}
+static_assert(kParams % 8 == 0 && oW2 % 8 == 0, "weights are read 16 bytes at a time");
+constexpr size_t kMlpSmem = ((kParams * 2 + 15) / 16) * 16 + sizeof(float) * kTS * (kF + 2 * kH);
 
 // ---- MLP forward on the tensor cores (tcgen05, kind::tf32) ---------------------------------
-// One CTA of 128 threads per 128 atoms and ensemble member; thread t owns atom a0 + t, which is
+// One CTA of 256 threads per 128 atoms and ensemble member; threads t and t + 128 own atom a0 + t, which is
 // TMEM lane t of the accumulator.  Each layer Z = H W + b (M = 128 atoms, K = 128 inputs, the
 // 122 features padded with zeros, N = 128 or 16) is one chain of tcgen05.mma: the FP32
 // activations as TF32 hi + lo parts (hi = rna(h), lo = rna(h - hi)) against the weights,
@@ -509,6 +501,7 @@ __device__ __forceinline__ void load_params_and_inputs(const MlpSmem &m, const _
 // written to shared memory by the threads in the K-major 128-byte-swizzled layout: element
 // (row r, k) in slab k / 32 (r x 128 bytes each), 16-byte chunk ((k % 32) / 4) xor (r % 8).
 constexpr int kMT = 128;                 // atoms per CTA
+constexpr int kMThreads = 256;           // two threads an atom, each with half of a layer's units
 constexpr int kSlab = kMT * 128;         // bytes of one 32-element K slab of a 128-row operand
 constexpr size_t kMlpTcSmem = 3 * 4 * static_cast<size_t>(kSlab) + 1024 + 64;
 static_assert(kF <= 128 && kH == 128 && kO == 16, "layer shapes of the tensor-core MLP");
@@ -526,19 +519,52 @@ __device__ __forceinline__ void mlp_mma(uint32_t tmem, uint64_t a, uint64_t b, u
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
         "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
-__device__ __forceinline__ void put_split(uint8_t *hi, uint8_t *lo, int r, int k, float v) {
-    uint32_t h, l;
-    asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(h) : "f"(v));
-    asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(l) : "f"(v - __uint_as_float(h)));
-    *reinterpret_cast<uint32_t *>(hi + swz(r, k)) = h;
-    *reinterpret_cast<uint32_t *>(lo + swz(r, k)) = l;
+__device__ __forceinline__ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+// Four neighbouring floats, in one access where the array starts on 16 bytes (vec).
+__device__ __forceinline__ void store4(float *p, const float (&v)[4], bool vec) {
+    if (vec) {
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p[j] = v[j];
+    }
 }
-// B operand of a layer: row n = output unit, K = input (W is stored [in][out]); rows n < nout.
-__device__ __forceinline__ void put_weights(uint8_t *Bs, const __half *W, int nin, int nout) {
-    for (int e = threadIdx.x; e < nout * 128; e += blockDim.x) {
-        const int k = e / nout, n = e % nout;   // consecutive threads: consecutive outputs of one input
-        const float w = k < nin ? __half2float(W[k * nout + n]) : 0.0f;
-        *reinterpret_cast<float *>(Bs + swz(n, k)) = w;
+__device__ __forceinline__ void load4(const float *p, float (&v)[4], bool vec) {
+    if (vec) {
+        const float4 f = *reinterpret_cast<const float4 *>(p);
+        v[0] = f.x;
+        v[1] = f.y;
+        v[2] = f.z;
+        v[3] = f.w;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = p[j];
+    }
+}
+// Four neighbouring entries of a row (k a multiple of 4) as TF32 hi + lo parts: one 16-byte chunk each.
+__device__ __forceinline__ void put_split4(uint8_t *hi, uint8_t *lo, int r, int k, const float (&v)[4]) {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(h[j]) : "f"(v[j]));
+        asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(l[j]) : "f"(v[j] - __uint_as_float(h[j])));
+    }
+    *reinterpret_cast<uint4 *>(hi + swz(r, k)) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4 *>(lo + swz(r, k)) = make_uint4(l[0], l[1], l[2], l[3]);
+}
+// B operand of a layer: row n = output unit, K = input (W is stored [in][out]); rows n < nout, a power of
+// two.  The staging loops of these kernels are a chain of L2 latencies unless several loads are in
+// flight: a thread takes four inputs of an output, eight times over (with one entry at a time the
+// forward of 4096 atoms spent 150 of its 190 us here and in the features).
+template <int nout>
+__device__ __forceinline__ void put_weights(uint8_t *Bs, const __half *W, int nin) {
+#pragma unroll 8
+    for (int e = threadIdx.x; e < nout * 32; e += kMThreads) {
+        const int k = e / nout * 4, n = e % nout;   // consecutive threads: consecutive outputs of one input
+        float w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = k + j < nin ? __half2float(W[(k + j) * nout + n]) : 0.0f;
+        *reinterpret_cast<float4 *>(Bs + swz(n, k)) = make_float4(w[0], w[1], w[2], w[3]);
     }
 }
 // The six B operands of the tensor-core MLP of each member in their shared-memory layout
@@ -614,10 +640,10 @@ __device__ __forceinline__ bool mlp_layer(uint32_t tmem, uint8_t *Ahi, uint8_t *
     return __syncthreads_and(ok) != 0;   // uniform over the CTA: every later barrier is reached by all
 }
 
-// grid (ceil(B / 128), members), 128 threads.  Y [member][B][16]; optional cache
+// grid (ceil(B / 128), members), 256 threads.  Y [member][B][16]; optional cache
 // z [member][2][B][128] (pre-activations of both hidden layers).  A wait that times out raises
 // ST_TC_TIMEOUT in *err and leaves NaN outputs.
-__global__ void __launch_bounds__(128, 1) k_mlp_forward_tc(int B, const float *X, const float *mean,
+__global__ void __launch_bounds__(kMThreads, 1) k_mlp_forward_tc(int B, const float *X, const float *mean,
                                                            const float *stdv, const __half *params, float *Y,
                                                            float *zcache, const float *packed, int *err) {
     extern __shared__ uint8_t smem_raw[];
@@ -626,7 +652,8 @@ __global__ void __launch_bounds__(128, 1) k_mlp_forward_tc(int B, const float *X
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + 12 * kSlab);
     WeightLoad wl{bar + 1, 0, false};
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar + 2);
-    const int member = blockIdx.y, t = threadIdx.x, warp = t >> 5, a = blockIdx.x * kMT + t;
+    const int member = blockIdx.y, t = threadIdx.x, warp = t >> 5, row_t = t & 127, half = t >> 7;
+    const int a = blockIdx.x * kMT + row_t;   // this thread's atom; units 64 half .. 64 half + 63
     const __half *P = params + static_cast<long long>(member) * kParams;
     const float *img = packed ? packed + static_cast<long long>(member) * 6 * kImgFloats : nullptr;
     if (t == 0) {
@@ -644,18 +671,31 @@ __global__ void __launch_bounds__(128, 1) k_mlp_forward_tc(int B, const float *X
     // layer 1 operands: the standardised features of the CTA's atoms (read row by row, the
     // threads along the features), W1
     const int a0 = blockIdx.x * kMT;
-    for (int e = t; e < kMT * 128; e += kMT) {
-        const int row = e >> 7, k = e & 127, ar = a0 + row;
-        const float x = (ar < B && k < kF) ? (X[static_cast<long long>(ar) * kF + k] - mean[k]) / stdv[k] : 0.0f;
-        put_split(Ahi, Alo, row, k, x);
+    {
+        const int k = (t & 31) * 4;   // this thread's features, of every eighth atom
+        float mu[4], sd[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            mu[j] = k + j < kF ? mean[k + j] : 0.0f;
+            sd[j] = k + j < kF ? stdv[k + j] : 1.0f;
+        }
+#pragma unroll 8
+        for (int row = warp; row < kMT; row += kMThreads / 32) {
+            const int ar = a0 + row;
+            float x[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                x[j] = (ar < B && k + j < kF) ? (X[static_cast<long long>(ar) * kF + k + j] - mu[j]) / sd[j] : 0.0f;
+            put_split4(Ahi, Alo, row, k, x);
+        }
     }
     bool ok = true;
     if (img) ok = weights_wait(wl, err);
-    else put_weights(Bs, P + oW1, kF, kH);
+    else put_weights<kH>(Bs, P + oW1, kF);
     fence_before();
     ok = __syncthreads_and(ok) != 0;
     fence_after();
-    const uint32_t tmem = *tmem_slot + (static_cast<uint32_t>(warp * 32) << 16);
+    const uint32_t tmem = *tmem_slot + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     float *z1 = zcache ? zcache + static_cast<long long>(member) * 2 * B * kH : nullptr;
     float *z2 = zcache ? z1 + static_cast<long long>(B) * kH : nullptr;
     uint32_t phase = 0;
@@ -665,21 +705,26 @@ __global__ void __launch_bounds__(128, 1) k_mlp_forward_tc(int B, const float *X
     for (int layer = 0; layer < 2 && ok; ++layer) {
         const __half *bias = P + (layer == 0 ? ob1 : ob2);
         float *zc = layer == 0 ? z1 : z2;
-        for (int c0 = 0; c0 < kH; c0 += 32) {
+        for (int c0 = 64 * half; c0 < 64 * half + 64; c0 += 32) {
             uint32_t r[32];
             tmem_ld32(tmem + c0, r);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const float z = __uint_as_float(r[j]) + __half2float(bias[c0 + j]);
-                if (zc && a < B) zc[static_cast<long long>(a) * kH + c0 + j] = z;
-                put_split(Ahi, Alo, t, c0 + j, a < B ? silu(z) : 0.0f);
+            for (int j = 0; j < 32; j += 4) {
+                float z[4], hs[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    z[u] = __uint_as_float(r[j + u]) + __half2float(bias[c0 + j + u]);
+                    hs[u] = a < B ? silu(z[u]) : 0.0f;
+                }
+                if (zc && a < B) store4(zc + static_cast<long long>(a) * kH + c0 + j, z, aligned16(zcache));
+                put_split4(Ahi, Alo, row_t, c0 + j, hs);
             }
         }
         fence_before();
         __syncthreads();   // every thread's reads of TMEM and of the weights are done
         if (img) ok = weights_wait(wl, err);
-        else if (layer == 0) put_weights(Bs, P + oW2, kH, kH);
-        else put_weights(Bs, P + oW3, kH, kO);
+        else if (layer == 0) put_weights<kH>(Bs, P + oW2, kH);
+        else put_weights<kO>(Bs, P + oW3, kH);
         ok = __syncthreads_and(ok) != 0;
         phase ^= 1;
         if (ok) ok = mlp_layer(*tmem_slot, Ahi, Alo, Bs, layer == 0 ? kH : kO, bar, phase, err);
@@ -689,7 +734,7 @@ __global__ void __launch_bounds__(128, 1) k_mlp_forward_tc(int B, const float *X
     // takes part (ok is uniform over the CTA), only the rows of real atoms are stored.
     uint32_t r[32];
     if (ok) tmem_ld32(tmem, r);   // columns 16..31 are not part of the product
-    if (a < B) {
+    if (a < B && half == 0) {
         float *y = Y + (static_cast<long long>(member) * B + a) * kO;
         for (int o = 0; o < kO; ++o) y[o] = ok ? __uint_as_float(r[o]) + __half2float(P[ob3 + o]) : __int_as_float(0x7fc00000);
     }
@@ -706,10 +751,13 @@ __global__ void __launch_bounds__(128, 1) k_mlp_forward_tc(int B, const float *X
 // B operand of a backward product: W used as stored ([in][out], row n = input unit), rows
 // n < nin, K = the outputs k < nout (zero beyond).
 __device__ __forceinline__ void put_weights_rows(uint8_t *Bs, const __half *W, int nin, int nout) {
-    for (int e = threadIdx.x; e < 128 * 128; e += blockDim.x) {
-        const int n = e >> 7, k = e & 127;   // consecutive threads: consecutive outputs of one row
-        const float w = (n < nin && k < nout) ? __half2float(W[n * nout + k]) : 0.0f;
-        *reinterpret_cast<float *>(Bs + swz(n, k)) = w;
+#pragma unroll 8
+    for (int e = threadIdx.x; e < 128 * 32; e += kMThreads) {
+        const int n = e >> 5, k = (e & 31) * 4;   // consecutive threads: consecutive outputs of one row
+        float w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = (n < nin && k + j < nout) ? __half2float(W[n * nout + k + j]) : 0.0f;
+        *reinterpret_cast<float4 *>(Bs + swz(n, k)) = make_float4(w[0], w[1], w[2], w[3]);
     }
 }
 
@@ -717,9 +765,9 @@ __device__ __forceinline__ void put_weights_rows(uint8_t *Bs, const __half *W, i
 // path of the backward, without parameter gradients): dh2 = dY W3^T, dz2 = dh2 silu'(z2),
 // dh1 = dz2 W2^T, dz1 = dh1 silu'(z1), dX = (dz1 W1^T) / std, each product as in the forward
 // (TF32 hi/lo parts of the FP32 left factor against the exact weights, FP32 accumulation in
-// TMEM).  grid (ceil(B / 128), members), 128 threads; zcache from the forward; a wait that
+// TMEM).  grid (ceil(B / 128), members), 256 threads; zcache from the forward; a wait that
 // times out raises ST_TC_TIMEOUT in *err and leaves NaN in dX.
-__global__ void __launch_bounds__(128, 1) k_mlp_backward_dx_tc(int B, const float *stdv, const __half *params,
+__global__ void __launch_bounds__(kMThreads, 1) k_mlp_backward_dx_tc(int B, const float *stdv, const __half *params,
                                                                const float *zcache, const float *dY, float *dX,
                                                                const float *packed, int *err) {
     extern __shared__ uint8_t smem_raw[];
@@ -728,7 +776,8 @@ __global__ void __launch_bounds__(128, 1) k_mlp_backward_dx_tc(int B, const floa
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + 12 * kSlab);
     WeightLoad wl{bar + 1, 0, false};
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar + 2);
-    const int member = blockIdx.y, t = threadIdx.x, warp = t >> 5, a0 = blockIdx.x * kMT, a = a0 + t;
+    const int member = blockIdx.y, t = threadIdx.x, warp = t >> 5, row_t = t & 127, half = t >> 7;
+    const int a0 = blockIdx.x * kMT, a = a0 + row_t;
     const __half *P = params + static_cast<long long>(member) * kParams;
     const float *img = packed ? packed + (static_cast<long long>(member) * 6 + 3) * kImgFloats : nullptr;
     const float *z1 = zcache + static_cast<long long>(member) * 2 * B * kH, *z2 = z1 + static_cast<long long>(B) * kH;
@@ -745,10 +794,14 @@ __global__ void __launch_bounds__(128, 1) k_mlp_backward_dx_tc(int B, const floa
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
     }
     // dY rows of the CTA's atoms (K = the 16 outputs), W3 by rows
-    for (int e = t; e < kMT * 128; e += kMT) {
-        const int row = e >> 7, k = e & 127, ar = a0 + row;
-        const float v = (ar < B && k < kO) ? dY[(static_cast<long long>(member) * B + ar) * kO + k] : 0.0f;
-        put_split(Ahi, Alo, row, k, v);
+#pragma unroll 8
+    for (int row = warp; row < kMT; row += kMThreads / 32) {
+        const int k = (t & 31) * 4, ar = a0 + row;
+        float v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            v[j] = (ar < B && k + j < kO) ? dY[(static_cast<long long>(member) * B + ar) * kO + k + j] : 0.0f;
+        put_split4(Ahi, Alo, row, k, v);
     }
     bool ok = true;
     if (img) ok = weights_wait(wl, err);
@@ -756,19 +809,22 @@ __global__ void __launch_bounds__(128, 1) k_mlp_backward_dx_tc(int B, const floa
     fence_before();
     ok = __syncthreads_and(ok) != 0;
     fence_after();
-    const uint32_t tmem = *tmem_slot + (static_cast<uint32_t>(warp * 32) << 16);
+    const uint32_t tmem = *tmem_slot + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     uint32_t phase = 0;
     if (ok) ok = mlp_layer(*tmem_slot, Ahi, Alo, Bs, kH, bar, phase, err);
     if (ok && img) weights_issue(Bs, img + kImgFloats, wl);   // W2 under the epilogue
     for (int layer = 0; layer < 2 && ok; ++layer) {   // dz2 from dh2, then dz1 from dh1
         const float *zc = layer == 0 ? z2 : z1;
-        for (int c0 = 0; c0 < kH; c0 += 32) {
+        for (int c0 = 64 * half; c0 < 64 * half + 64; c0 += 32) {
             uint32_t r[32];
             tmem_ld32(tmem + c0, r);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const float dz = a < B ? __uint_as_float(r[j]) * dsilu(zc[static_cast<long long>(a) * kH + c0 + j]) : 0.0f;
-                put_split(Ahi, Alo, t, c0 + j, dz);
+            for (int j = 0; j < 32; j += 4) {
+                float zv[4] = {0.0f, 0.0f, 0.0f, 0.0f}, dz[4];
+                if (a < B) load4(zc + static_cast<long long>(a) * kH + c0 + j, zv, aligned16(zcache));
+#pragma unroll
+                for (int u = 0; u < 4; ++u) dz[u] = a < B ? __uint_as_float(r[j + u]) * dsilu(zv[u]) : 0.0f;
+                put_split4(Ahi, Alo, row_t, c0 + j, dz);
             }
         }
         fence_before();
@@ -782,7 +838,7 @@ __global__ void __launch_bounds__(128, 1) k_mlp_backward_dx_tc(int B, const floa
         if (ok && img && layer == 0) weights_issue(Bs, img + 2 * kImgFloats, wl);   // W1 under the epilogue
     }
     // dX = acc / std over the 122 features (TMEM loads on every lane, stores for real atoms)
-    for (int c0 = 0; c0 < kH; c0 += 32) {
+    for (int c0 = 64 * half; c0 < 64 * half + 64; c0 += 32) {
         uint32_t r[32];
         if (ok) tmem_ld32(tmem + c0, r);
         if (a < B)
@@ -803,36 +859,77 @@ __global__ void __launch_bounds__(128, 1) k_mlp_backward_dx_tc(int B, const floa
     }
 }
 
+// sum over the CTA's atoms of row[a] dz[a], in order.
+__device__ __forceinline__ float atom_dot(const float *row, const float (&dz)[kTA]) {
+    float s = 0.0f;
+#pragma unroll
+    for (int a = 0; a < kTA; a += 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(row + a);
+        s += v.x * dz[a];
+        s += v.y * dz[a + 1];
+        s += v.z * dz[a + 2];
+        s += v.w * dz[a + 3];
+    }
+    return s;
+}
+// acc[a] += row[a] w.
+__device__ __forceinline__ void atom_axpy(const float *row, float w, float (&acc)[kTA]) {
+#pragma unroll
+    for (int a = 0; a < kTA; a += 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(row + a);
+        acc[a] += v.x * w;
+        acc[a + 1] += v.y * w;
+        acc[a + 2] += v.z * w;
+        acc[a + 3] += v.w * w;
+    }
+}
+
 // Backward of sum(dY * Y): grid (ceil(B / 32), members), 128 threads.  Needs the cache of the
-// forward pass.  dX (optional) [member][B][74]: gradient with respect to the raw features.
+// forward pass.  dX (optional) [member][B][122]: gradient with respect to the raw features.
 // grad (optional) [member][kParams] FP32, accumulated (atomic adds of per-CTA sums).
+// Bound by shared-memory reads: thread t holds one unit's 32 atoms in registers, and a read of four atoms
+// of another unit, the same for the whole warp, feeds four multiply-adds; a weight is read once for all
+// atoms.  (One word per multiply-add, and a row of weights per thread with all threads on one bank:
+// 169 us for 4096 atoms of a member, 98 so.)
 __global__ void __launch_bounds__(128) k_mlp_backward(int B, const float *X, const float *mean, const float *stdv,
                                                       const __half *params, const float *zcache, const float *dY,
                                                       float *dX, float *grad) {
     extern __shared__ __align__(16) char smem[];
     const MlpSmem m = mlp_smem(smem);
     const int member = blockIdx.y, a0 = blockIdx.x * kTA, t = threadIdx.x;
-    load_params_and_inputs(m, params + static_cast<long long>(member) * kParams, X, mean, stdv, a0, B);
+    const __half *P = params + static_cast<long long>(member) * kParams;
+    if (aligned16(P)) {
+#pragma unroll 8
+        for (int e = t; e < kParams / 8; e += 128)
+            reinterpret_cast<uint4 *>(m.W)[e] = reinterpret_cast<const uint4 *>(P)[e];
+    } else {
+        for (int e = t; e < kParams; e += 128) m.W[e] = P[e];
+    }
     const float *z1 = zcache + static_cast<long long>(member) * 2 * B * kH, *z2 = z1 + static_cast<long long>(B) * kH;
     __shared__ float dy_s[kTA * kO];
     for (int e = t; e < kTA * kO; e += 128) {
         const int a = e / kO, o = e % kO;
         dy_s[e] = a0 + a < B ? dY[(static_cast<long long>(member) * B + a0 + a) * kO + o] : 0.0f;
     }
-    // h1, h2 from the cached pre-activations (padding atoms: zero)
-    for (int e = t; e < kTA * kH; e += 128) {
-        const int a = e / kH, k = e % kH;
+    // inputs and h1, h2 from the cached pre-activations (padding atoms: zero); thread t: unit t
+    const float mu = t < kF ? mean[t] : 0.0f, sd = t < kF ? stdv[t] : 1.0f;
+#pragma unroll 8
+    for (int a = 0; a < kTA; ++a) {
         const bool ok = a0 + a < B;
-        m.h1[e] = ok ? silu(z1[static_cast<long long>(a0 + a) * kH + k]) : 0.0f;
-        m.h2[e] = ok ? silu(z2[static_cast<long long>(a0 + a) * kH + k]) : 0.0f;
+        const long long row = a0 + a;
+        if (t < kF) m.Xs[t * kTS + a] = ok ? (X[row * kF + t] - mu) / sd : 0.0f;
+        m.h1[t * kTS + a] = ok ? silu(z1[row * kH + t]) : 0.0f;
+        m.h2[t * kTS + a] = ok ? silu(z2[row * kH + t]) : 0.0f;
     }
     __syncthreads();
     float *g = grad ? grad + static_cast<long long>(member) * kParams : nullptr;
+    const int first = static_cast<int>(blockIdx.x * 37u) & (kH - 1);   // the CTAs' atomics start at different rows
     if (g) {   // output layer: gW3[k][o] = sum_a h2[a][k] dy[a][o], gb3[o] = sum_a dy[a][o]
         for (int e = t; e < kH * kO; e += 128) {
             const int k = e / kO, o = e % kO;
             float s = 0.0f;
-            for (int a = 0; a < kTA; ++a) s += m.h2[a * kH + k] * dy_s[a * kO + o];
+#pragma unroll
+            for (int a = 0; a < kTA; ++a) s += m.h2[k * kTS + a] * dy_s[a * kO + o];
             atomicAdd(&g[oW3 + e], s);
         }
         if (t < kO) {
@@ -842,54 +939,74 @@ __global__ void __launch_bounds__(128) k_mlp_backward(int B, const float *X, con
         }
     }
     // dz2[a][t] = (sum_o dy[a][o] W3[t][o]) dsilu(z2[a][t]); kept in registers
-    float dz[kTA];
+    float dz[kTA], w3[kO];
+#pragma unroll
+    for (int o = 0; o < kO; ++o) w3[o] = __half2float(m.W[oW3 + t * kO + o]);
+#pragma unroll
     for (int a = 0; a < kTA; ++a) {
         float s = 0.0f;
 #pragma unroll
-        for (int o = 0; o < kO; ++o) s += dy_s[a * kO + o] * __half2float(m.W[oW3 + t * kO + o]);
+        for (int o = 0; o < kO; ++o) s += dy_s[a * kO + o] * w3[o];
         dz[a] = a0 + a < B ? s * dsilu(z2[static_cast<long long>(a0 + a) * kH + t]) : 0.0f;
     }
     if (g) {   // gW2[k][t] = sum_a h1[a][k] dz2[a][t]; gb2[t]
         float sb = 0.0f;
+#pragma unroll
         for (int a = 0; a < kTA; ++a) sb += dz[a];
         atomicAdd(&g[ob2 + t], sb);
-        for (int k = 0; k < kH; ++k) {
-            float s = 0.0f;
-#pragma unroll
-            for (int a = 0; a < kTA; ++a) s += m.h1[a * kH + k] * dz[a];
-            atomicAdd(&g[oW2 + k * kH + t], s);
+#pragma unroll 4
+        for (int u = 0; u < kH; ++u) {
+            const int k = (u + first) & (kH - 1);
+            atomicAdd(&g[oW2 + k * kH + t], atom_dot(m.h1 + k * kTS, dz));
         }
     }
     __syncthreads();   // h2 is no longer needed: reuse it for dz2
-    for (int a = 0; a < kTA; ++a) m.h2[a * kH + t] = dz[a];
+#pragma unroll
+    for (int a = 0; a < kTA; ++a) {
+        m.h2[t * kTS + a] = dz[a];
+        dz[a] = 0.0f;
+    }
     __syncthreads();
     // dz1[a][t] = (sum_k dz2[a][k] W2[t][k]) dsilu(z1[a][t])
-    for (int a = 0; a < kTA; ++a) {
-        float s = 0.0f;
-        for (int k = 0; k < kH; ++k) s += m.h2[a * kH + k] * __half2float(m.W[oW2 + t * kH + k]);
-        dz[a] = a0 + a < B ? s * dsilu(z1[static_cast<long long>(a0 + a) * kH + t]) : 0.0f;
+#pragma unroll 1
+    for (int k = 0; k < kH; k += 8) {
+        const uint4 w = *reinterpret_cast<const uint4 *>(m.W + oW2 + t * kH + k);
+        const __half *wh = reinterpret_cast<const __half *>(&w);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) atom_axpy(m.h2 + (k + u) * kTS, __half2float(wh[u]), dz);
     }
+#pragma unroll
+    for (int a = 0; a < kTA; ++a) dz[a] = a0 + a < B ? dz[a] * dsilu(z1[static_cast<long long>(a0 + a) * kH + t]) : 0.0f;
     if (g) {   // gW1[k][t] = sum_a Xs[a][k] dz1[a][t]; gb1[t]
         float sb = 0.0f;
+#pragma unroll
         for (int a = 0; a < kTA; ++a) sb += dz[a];
         atomicAdd(&g[ob1 + t], sb);
-        for (int k = 0; k < kF; ++k) {
-            float s = 0.0f;
-#pragma unroll
-            for (int a = 0; a < kTA; ++a) s += m.Xs[a * kF + k] * dz[a];
-            atomicAdd(&g[oW1 + k * kH + t], s);
+#pragma unroll 4
+        for (int u = 0; u < kH; ++u) {
+            const int k = (u + first) & (kH - 1);
+            if (k < kF) atomicAdd(&g[oW1 + k * kH + t], atom_dot(m.Xs + k * kTS, dz));
         }
     }
     if (dX) {
         __syncthreads();
-        for (int a = 0; a < kTA; ++a) m.h1[a * kH + t] = dz[a];
+#pragma unroll
+        for (int a = 0; a < kTA; ++a) {
+            m.h1[t * kTS + a] = dz[a];
+            dz[a] = 0.0f;
+        }
         __syncthreads();
-        for (int e = t; e < kTA * kF; e += 128) {
-            const int a = e / kF, k = e % kF;
-            if (a0 + a >= B) continue;
-            float s = 0.0f;
-            for (int j = 0; j < kH; ++j) s += m.h1[a * kH + j] * __half2float(m.W[oW1 + k * kH + j]);
-            dX[(static_cast<long long>(member) * B + a0 + a) * kF + k] = s / stdv[k];
+        if (t < kF) {   // dX[a][t] = (sum_j dz1[a][j] W1[t][j]) / std
+#pragma unroll 1
+            for (int j = 0; j < kH; j += 8) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(m.W + oW1 + t * kH + j);
+                const __half *wh = reinterpret_cast<const __half *>(&w);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) atom_axpy(m.h1 + (j + u) * kTS, __half2float(wh[u]), dz);
+            }
+#pragma unroll
+            for (int a = 0; a < kTA; ++a)
+                if (a0 + a < B) dX[(static_cast<long long>(member) * B + a0 + a) * kF + t] = dz[a] / sd;
         }
     }
 }
@@ -1207,7 +1324,7 @@ cudaError_t mlp_forward(int B, int members, const float *X, const float *mean, c
                                          static_cast<int>(kMlpTcSmem));
     if (e != cudaSuccess) return e;
     count_launches(1);
-    k_mlp_forward_tc<<<dim3(cdiv(B, kMT), members), 128, kMlpTcSmem, s>>>(
+    k_mlp_forward_tc<<<dim3(cdiv(B, kMT), members), kMThreads, kMlpTcSmem, s>>>(
         B, X, mean, stdv, static_cast<const __half *>(params16), Y, zcache, packed, err);
     return cudaGetLastError();
 }
@@ -1227,7 +1344,7 @@ cudaError_t mlp_backward(int B, int members, const float *X, const float *mean, 
                                              static_cast<int>(kMlpTcSmem));
         if (e != cudaSuccess) return e;
         count_launches(1);
-        k_mlp_backward_dx_tc<<<dim3(cdiv(B, kMT), members), 128, kMlpTcSmem, s>>>(
+        k_mlp_backward_dx_tc<<<dim3(cdiv(B, kMT), members), kMThreads, kMlpTcSmem, s>>>(
             B, stdv, static_cast<const __half *>(params16), zcache, dY, dX, packed, own_err);
         return cudaGetLastError();
     }

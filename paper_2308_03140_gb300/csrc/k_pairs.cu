@@ -478,7 +478,7 @@ __global__ void k_scs_grad_inputs_f32(const double *X, const double *V, const do
 // once (i in tile I, j in tile J, i < j), and writes both ends' sums of the tile pair to
 // part[other tile][7][atom]; k_ts_sum adds them up in a fixed order.  Bound by FP64 arithmetic: four
 // divisions, a square root and an exponential a pair of about 150 operations (each ordered pair for itself with a
-// division wherever the formula has one, 250 operations: 1.36 ms for 2000 atoms, RESULT).
+// division wherever the formula has one, 250 operations: 1.36 ms for 2000 atoms, 0.61 so).
 constexpr int kTsTile = 32, kTsVals = 7;   // e, gR x3, ga0, gom, grv
 __global__ void __launch_bounds__(256) k_ts_pairs(AtomBufs b, double s_r, int tiles, double *part) {
     int J = static_cast<int>((sqrtf(8.0f * blockIdx.x + 1.0f) - 1.0f) * 0.5f);
