@@ -345,6 +345,12 @@ void build_scs_periodic(const AtomBufs &b, const CellGeom &c, double beta, doubl
 // damped-away part, both triangles; rows >= n padded with omega_0^2 on the diagonal.
 void build_q_periodic(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, double *Q, long long ld,
                       int n, int *status, cudaStream_t s);
+// The same with the reciprocal sums as residue products (k_qbuild.cu) through build_q_products_bytes of
+// scratch (0: not for this cell, whose image table would be too large); without the padding.
+size_t build_q_products_bytes(int N, const CellGeom &c, int nk, int maxG);
+cudaError_t build_q_products(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, double *Q, long long ld,
+                             void *work, int *status, cudaStream_t s);
+void pad_q_periodic(const AtomBufs &b, const PeriodicBufs &p, double *Q, long long ld, int n, cudaStream_t s);
 // Batched complex helpers (nk planar matrices of order ld).
 void cscale(double *Y, long long ld, int nk, double scale, cudaStream_t s);
 void cset_identity(double *Z, long long ld, int nk, cudaStream_t s);

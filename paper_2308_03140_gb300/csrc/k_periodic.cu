@@ -792,6 +792,10 @@ void build_q_periodic(const AtomBufs &b, const PeriodicBufs &p, double beta, dou
     const int ntile = cdiv(b.N, kQT);
     count_launches(1);
     k_build_q_periodic<<<dim3(ntile * (ntile + 1) / 2, p.nk), 256, 0, s>>>(b, p, beta, a, Q, ld, ntile, status);
+    pad_q_periodic(b, p, Q, ld, n, s);
+}
+
+void pad_q_periodic(const AtomBufs &b, const PeriodicBufs &p, double *Q, long long ld, int n, cudaStream_t s) {
     if (ld > n) {
         count_launches(1);
         k_pad_q_periodic<<<dim3(cdiv((ld - n) * ld, 256), p.nk), 256, 0, s>>>(Q, ld, n, b.ombar);

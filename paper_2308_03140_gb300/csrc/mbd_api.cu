@@ -145,6 +145,9 @@ struct mbd_ctx {
     // the products then run on the FP64 pipe.
     char *crt = nullptr;
     double *dPT = nullptr;
+    char *qwork = nullptr;   // cells: scratch of the Q(q) build's products (null: it runs on the FP64 pipe)
+    size_t qwork_bytes = 0;
+    bool no_scratch = false;   // the scratch of the tensor-core products did not fit the card
     double *dkq = nullptr, *dkw = nullptr, *dG = nullptr, *dcoef = nullptr, *dlzw = nullptr, *dgA = nullptr, *dgAout = nullptr,
            *dgApart = nullptr, *dgc = nullptr, *dtsg = nullptr;
     int *dglist = nullptr, *dgcount = nullptr;
@@ -469,10 +472,14 @@ int allocate(mbd_ctx *ctx) {
                                    al(sizeof(float) * grad32)
                              : 0;
     bytes += scs32;
-    const size_t crt_work =
-        fp64_path(prec) ? std::max(al(cholesky_crt_bytes(ld, static_cast<int>(nf1))),
-                                   al(ctx->periodic ? crt_cell_bytes(ctx->n, static_cast<int>(nk)) : crt_ns_bytes(ctx->n))) + matq
-                        : 0;
+    // Scratch of the tensor-core products, taken only where it fits: FP64 products and factors (and the
+    // transpose of P), and the build of Q(q), which can share theirs.
+    const size_t q_work = ctx->periodic ? al(build_q_products_bytes(ctx->N, ctx->cell, static_cast<int>(nk), ctx->maxG)) : 0;
+    const size_t crt_part =
+        fp64_path(prec) ? std::max({al(cholesky_crt_bytes(ld, static_cast<int>(nf1))),
+                                    al(ctx->periodic ? crt_cell_bytes(ctx->n, static_cast<int>(nk)) : crt_ns_bytes(ctx->n)), q_work})
+                        : q_work;
+    const size_t pt_part = fp64_path(prec) ? matq : 0, crt_work = crt_part + pt_part;
     // A slab large enough for the new size is re-carved in place (systems of varying size in
     // a batch then reuse one allocation); otherwise it is replaced.
     cudaError_t e = cudaSuccess;
@@ -492,8 +499,12 @@ int allocate(mbd_ctx *ctx) {
         ctx->slab_bytes = want;
     }
     const bool crt = crt_work && ctx->slab_bytes >= bytes + crt_work;
-    ctx->dPT = crt ? reinterpret_cast<double *>(static_cast<char *>(ctx->slab) + bytes) : nullptr;
-    ctx->crt = crt ? static_cast<char *>(ctx->slab) + bytes + matq : nullptr;
+    ctx->no_scratch = crt_work && !crt;
+    ctx->qwork_bytes = crt ? q_work : 0;
+    char *scratch = crt ? static_cast<char *>(ctx->slab) + bytes + pt_part : nullptr;
+    ctx->dPT = crt && pt_part ? reinterpret_cast<double *>(static_cast<char *>(ctx->slab) + bytes) : nullptr;
+    ctx->crt = pt_part ? scratch : nullptr;
+    ctx->qwork = q_work ? scratch : nullptr;
     char *p = static_cast<char *>(ctx->slab);
     for (auto &q : plan) {
         *q.first = reinterpret_cast<double *>(p);
@@ -1000,7 +1011,13 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
     if (rc) return rc;
     ctx->have_screening = true;
     // ---- Q(q) and the spectrum bounds ----
-    build_q_periodic(b, pb, beta, a, ctx->dQ, ld, n, ctx->dstatus, s);
+    const size_t qbytes = build_q_products_bytes(N, ctx->cell, nk, ctx->maxG);
+    if (ctx->qwork && qbytes && qbytes <= ctx->qwork_bytes) {
+        MBD_CUDA(build_q_products(b, pb, beta, a, ctx->dQ, ld, ctx->qwork, ctx->dstatus, s), "coupled_oscillator_matrix");
+        pad_q_periodic(b, pb, ctx->dQ, ld, n, s);
+    } else {
+        build_q_periodic(b, pb, beta, a, ctx->dQ, ld, n, ctx->dstatus, s);
+    }
     cmax_abs_rowsum(ctx->dQ, ld, nk, ctx->dscal + 1, s);
     double sc = 0.0;
     MBD_CUDA(cudaMemcpyAsync(&sc, ctx->dscal + 1, sizeof(double), cudaMemcpyDeviceToHost, s), "newton_schulz");
@@ -1556,7 +1573,9 @@ int mbd_set_geometry(mbd_ctx *ctx, int n_atoms, const double *coords, const doub
     }
     MBD_CUDA(cudaSetDevice(ctx->device), "mbd_set_geometry");
     const bool realloc = (n_atoms != ctx->N) || !ctx->slab || periodic != ctx->periodic ||
-                         (periodic && (ps.nk != ctx->nk || ps.nG != ctx->nG || ps.maxG != ctx->maxG));
+                         (periodic && (ps.nk != ctx->nk || ps.nG != ctx->nG || ps.maxG != ctx->maxG)) ||
+                         (periodic && !ctx->no_scratch &&   // (the image table's size depends on the lattice)
+                          build_q_products_bytes(n_atoms, ps.cell, ps.nk, ps.maxG) > ctx->qwork_bytes);
     ctx->N = n_atoms;
     ctx->n = 3 * n_atoms;
     ctx->ld = (ctx->n + 127) / 128 * 128;   // 128: the tensor-core tile (also a multiple of 64)
