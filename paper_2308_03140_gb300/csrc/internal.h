@@ -32,6 +32,7 @@ enum : int {
 // outputs: C (FP32), Ch/Cl (bf16 hi/lo), CT/CTh/CTl (transposes, mode 0 only), and
 // resid += sum over the leading nvalid x nvalid block of (delta - C)^2 (mode 0 only).
 // Timeouts set ST_TC_TIMEOUT in *err.
+constexpr int kTcSlots = 16;
 struct TcOperands {
     const void *A0, *A1, *B0, *B1;
     long long lda, ldb;
@@ -53,9 +54,15 @@ struct TcArgs {
     int chunk_stages = 0;    // K stages per TMEM accumulation (0: all of K in one)
     // Batch of independent products (blockIdx.y): A and B stacked as [batch][M][lda] and
     // [batch][N][ldb]; D and C of item b at D + b sC, C + b sC.  batch > 1 allows no other
-    // output than C.
+    // output than C, unless slots are given.
     int batch = 1;
     long long sC = 0;
+    // nslots > 0 (= batch): the items are the matrices slot[0..nslots-1] of the stacked operands (M == N),
+    // each with its own alpha and beta, and every output is allowed (sC elements from matrix to
+    // matrix, resid[slot]).
+    int nslots = 0;
+    int slot[kTcSlots] = {};
+    float alphas[kTcSlots] = {}, betas[kTcSlots] = {};
 };
 cudaError_t tc_gemm(int kind, const TcOperands &op, const TcArgs &g, cudaStream_t s);
 // The GEMM's bounded mbarrier wait on a barrier nothing arrives at, with a budget of `budget`
@@ -220,9 +227,10 @@ void lanczos_coefficients(const double *A, long long ld, int steps, double *work
                           cudaStream_t s);
 // As lanczos_coefficients, with the matrix-vector products in FP32 on an FP32 copy of A
 // written to A32 (ld x ld floats) and an FP32 copy of the Lanczos vector; the recurrence
-// (alpha, beta, orthogonalisation) stays FP64.  work: 3 ld doubles + ld floats.
+// (alpha, beta, orthogonalisation) stays FP64.  work: 3 ld doubles + ld floats, wstride (even) doubles from
+// item to item of a batch of matrices stacked in A and A32; coef: 2 steps doubles an item.
 void lanczos_coefficients_f32(const double *A, float *A32, long long ld, int steps, double *work, double *coef,
-                              cudaStream_t s);
+                              cudaStream_t s, int batch = 1, long long wstride = 0);
 // Maximum absolute row sum over rows 0..n-1 (Gershgorin bound), written to out[0].
 void max_abs_rowsum(const double *Q, long long ld, int n, double *out, cudaStream_t s);
 

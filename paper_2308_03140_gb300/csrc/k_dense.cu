@@ -252,8 +252,12 @@ __global__ void k_max_abs_rowsum(const double *Q, long long ld, int n, unsigned 
 // ---- Lanczos estimates of the extreme eigenvalues of a symmetric matrix ----
 // y = A x for an ld x ld row-major A: one warp per row, coalesced row reads.  T = double,
 // or float for an FP32 copy of A with an FP32 copy of x (products and row sums in FP32).
+// blockIdx.y: item of a batch, matrices mstride and vectors vstride (bytes) apart.
 template <typename T>
-__global__ void k_gemv(const T *A, long long ld, const T *x, double *y) {
+__global__ void k_gemv(const T *A, long long ld, const T *x, double *y, long long mstride, long long vstride) {
+    A += blockIdx.y * mstride;
+    x = reinterpret_cast<const T *>(reinterpret_cast<const char *>(x) + blockIdx.y * vstride);
+    y += blockIdx.y * (vstride / 8);
     const long long row = blockIdx.x * static_cast<long long>(blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= ld) return;
@@ -287,7 +291,12 @@ __device__ __forceinline__ double block_sum1024(double v, double *sh, bool activ
 }
 
 // v = a fixed pseudo-random unit vector, vprev = 0; v32 (if given) = (float) v.
-__global__ void __launch_bounds__(1024) k_lanczos_init(double *v, double *vprev, float *v32, long long ld) {
+// blockIdx.x: item of a batch, vectors vstride bytes apart.
+__global__ void __launch_bounds__(1024) k_lanczos_init(double *v, double *vprev, float *v32, long long ld,
+                                                       long long vstride) {
+    v += blockIdx.x * (vstride / 8);
+    vprev += blockIdx.x * (vstride / 8);
+    if (v32) v32 += blockIdx.x * (vstride / 4);
     __shared__ double sh[33];
     double ss = 0.0;
     for (long long p = threadIdx.x; p < ld; p += 1024) {
@@ -311,8 +320,13 @@ __global__ void __launch_bounds__(1024) k_lanczos_init(double *v, double *vprev,
 // from registers (20.6 us at 6016 either way).
 template <int kPer>
 __global__ void __launch_bounds__(1024) k_lanczos_update(double *w, double *v, double *vprev, float *v32, long long ld,
-                                                         double *coef, int j) {
+                                                         double *coef, int j, int steps, long long vstride) {
     __shared__ double sh[2][33];
+    w += blockIdx.x * (vstride / 8);
+    v += blockIdx.x * (vstride / 8);
+    vprev += blockIdx.x * (vstride / 8);
+    if (v32) v32 += blockIdx.x * (vstride / 4);
+    coef += blockIdx.x * 2LL * steps;
     constexpr int kHeld = kPer > 0 ? kPer : 1;
     double rw[kHeld], rv[kHeld], rp[kHeld];
     const bool active = (threadIdx.x & ~31) < ld;
@@ -376,19 +390,23 @@ __global__ void __launch_bounds__(1024) k_lanczos_update(double *w, double *v, d
 
 }  // namespace
 
-// work: 3 ld doubles (v, vprev, w), then for T = float ld floats (the FP32 copy of v).
+// work: 3 ld doubles (v, vprev, w), then for T = float ld floats (the FP32 copy of v); wstride doubles
+// apart for a batch of matrices mstride apart.
 template <typename T>
-void lanczos_run(const T *A, long long ld, int steps, double *work, double *coef, cudaStream_t s) {
+void lanczos_run(const T *A, long long ld, int steps, double *work, double *coef, cudaStream_t s, int batch = 1,
+                 long long mstride = 0, long long wstride = 0) {
     double *v = work, *vprev = work + ld, *w = work + 2 * ld;
     float *v32 = std::is_same<T, float>::value ? reinterpret_cast<float *>(work + 3 * ld) : nullptr;
     const T *x = std::is_same<T, float>::value ? reinterpret_cast<const T *>(v32) : reinterpret_cast<const T *>(v);
+    const long long vs = 8 * wstride;
+    const dim3 rows(static_cast<unsigned>((ld + 7) / 8), batch);
     count_launches(1);
-    k_lanczos_init<<<1, 1024, 0, s>>>(v, vprev, v32, ld);
+    k_lanczos_init<<<batch, 1024, 0, s>>>(v, vprev, v32, ld, vs);
     for (int j = 0; j < steps; ++j) {
         count_launches(2);
-        k_gemv<T><<<static_cast<int>((ld + 7) / 8), 256, 0, s>>>(A, ld, x, w);
-        if (ld <= 1024) k_lanczos_update<1><<<1, 1024, 0, s>>>(w, v, vprev, v32, ld, coef, j);
-        else k_lanczos_update<0><<<1, 1024, 0, s>>>(w, v, vprev, v32, ld, coef, j);
+        k_gemv<T><<<rows, 256, 0, s>>>(A, ld, x, w, mstride, vs);
+        if (ld <= 1024) k_lanczos_update<1><<<batch, 1024, 0, s>>>(w, v, vprev, v32, ld, coef, j, steps, vs);
+        else k_lanczos_update<0><<<batch, 1024, 0, s>>>(w, v, vprev, v32, ld, coef, j, steps, vs);
     }
 }
 
@@ -397,11 +415,11 @@ void lanczos_coefficients(const double *A, long long ld, int steps, double *work
 }
 
 void lanczos_coefficients_f32(const double *A, float *A32, long long ld, int steps, double *work, double *coef,
-                              cudaStream_t s) {
+                              cudaStream_t s, int batch, long long wstride) {
+    const long long total = batch * ld * ld;
     count_launches(1);
-    k_f64_to_f32<<<static_cast<int>(std::min<long long>((ld * ld + 255) / 256, 152 * 16)), 256, 0, s>>>(A, ld * ld,
-                                                                                                      A32);
-    lanczos_run<float>(A32, ld, steps, work, coef, s);
+    k_f64_to_f32<<<static_cast<int>(std::min<long long>((total + 255) / 256, 152 * 16)), 256, 0, s>>>(A, total, A32);
+    lanczos_run<float>(A32, ld, steps, work, coef, s, batch, ld * ld, wstride);
 }
 
 void gemm_f64(const GemmArgs &g, cudaStream_t s) {

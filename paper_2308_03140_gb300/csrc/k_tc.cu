@@ -109,13 +109,19 @@ struct TcCfg {
     static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 512;
 };
 
+// Batch item bz's place among the stacked matrices, and its beta.
+__device__ __forceinline__ int item_slot(const TcArgs &g, int bz) { return g.nslots ? g.slot[bz] : bz; }
+__device__ __forceinline__ float item_beta(const TcArgs &g, int bz) { return g.nslots ? g.betas[bz] : g.beta; }
+
 // Epilogue of one 128 x 128 tile for the thread owning row m: alpha/beta with D, the
 // optional outputs (FP32, split parts, FP64 accumulation, transposes, mirrored writes of the
 // symmetric products) and the residual sum.  Warp-uniform: every lane of a warp handles a row
 // of the same tile.
 template <int KIND>
 __device__ __forceinline__ void tile_epilogue(const TcArgs &g, const float (&acc)[TN], long long m, int tm, int tn,
-                                              const float *Dp, float *Cp, int lane) {
+                                              int item, int slot, int lane) {
+    const long long at = slot * g.sC;   // the item's first element in every output and in D
+    const float alpha = g.nslots ? g.alphas[item] : g.alpha, beta = g.nslots ? g.betas[item] : g.beta;
     using Cfg = TcCfg<KIND>;
     const bool mirror = (g.mode == 2) && (tm != tn);
     const bool diag = (g.mode == 2) && (tm == tn);
@@ -125,16 +131,16 @@ __device__ __forceinline__ void tile_epilogue(const TcArgs &g, const float (&acc
         const long long n0 = static_cast<long long>(tn) * TN + c0;
         float v[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = g.alpha * acc[c0 + j];
-        if (g.beta != 0.f) {   // this row of D was prefetched into L2 during the last chunks
-            const float4 *dp = reinterpret_cast<const float4 *>(Dp + m * g.ld + n0);
+        for (int j = 0; j < 16; ++j) v[j] = alpha * acc[c0 + j];
+        if (beta != 0.f) {   // this row of D was prefetched into L2 during the last chunks
+            const float4 *dp = reinterpret_cast<const float4 *>(g.D + at + m * g.ld + n0);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const float4 d = dp[q];
-                v[4 * q] += g.beta * d.x;
-                v[4 * q + 1] += g.beta * d.y;
-                v[4 * q + 2] += g.beta * d.z;
-                v[4 * q + 3] += g.beta * d.w;
+                v[4 * q] += beta * d.x;
+                v[4 * q + 1] += beta * d.y;
+                v[4 * q + 2] += beta * d.z;
+                v[4 * q + 3] += beta * d.w;
             }
         }
         if (g.resid && m < g.nvalid) {
@@ -149,8 +155,8 @@ __device__ __forceinline__ void tile_epilogue(const TcArgs &g, const float (&acc
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 if (diag && n0 + j < m) continue;
-                g.C64[m * g.ld + n0 + j] += static_cast<double>(v[j]);
-                if ((mirror || diag) && n0 + j != m) g.C64[(n0 + j) * g.ld + m] += static_cast<double>(v[j]);
+                g.C64[at + m * g.ld + n0 + j] += static_cast<double>(v[j]);
+                if ((mirror || diag) && n0 + j != m) g.C64[at + (n0 + j) * g.ld + m] += static_cast<double>(v[j]);
             }
         }
         // split of the result into the next product's operand parts: bf16 pairs
@@ -184,15 +190,15 @@ __device__ __forceinline__ void tile_epilogue(const TcArgs &g, const float (&acc
         // diagonal tiles keep their upper triangle and mirror it, so the result is
         // exactly symmetric whatever order the tensor cores summed in.
         if (!diag) {
-            if (Cp) {
-                float4 *cp = reinterpret_cast<float4 *>(Cp + m * g.ld + n0);
+            if (g.C) {
+                float4 *cp = reinterpret_cast<float4 *>(g.C + at + m * g.ld + n0);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) cp[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
             }
             if (g.Ch) {
                 constexpr int NV = KIND == 2 ? 4 : 2;   // uint4 vectors per 16 elements
-                uint4 *hp = reinterpret_cast<uint4 *>(static_cast<char *>(g.Ch) + (m * g.ld + n0) * Cfg::ELEM);
-                uint4 *lp = reinterpret_cast<uint4 *>(static_cast<char *>(g.Cl) + (m * g.ld + n0) * Cfg::ELEM);
+                uint4 *hp = reinterpret_cast<uint4 *>(static_cast<char *>(g.Ch) + (at + m * g.ld + n0) * Cfg::ELEM);
+                uint4 *lp = reinterpret_cast<uint4 *>(static_cast<char *>(g.Cl) + (at + m * g.ld + n0) * Cfg::ELEM);
 #pragma unroll
                 for (int q = 0; q < NV; ++q) {
                     hp[q] = make_uint4(hw[4 * q], hw[4 * q + 1], hw[4 * q + 2], hw[4 * q + 3]);
@@ -203,8 +209,8 @@ __device__ __forceinline__ void tile_epilogue(const TcArgs &g, const float (&acc
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 if (n0 + j < m) continue;
-                const long long off = m * g.ld + n0 + j;
-                if (Cp) Cp[off] = v[j];
+                const long long off = at + m * g.ld + n0 + j;
+                if (g.C) g.C[off] = v[j];
                 if (g.Ch) {
                     store_part<KIND>(g.Ch, off, hw, j);
                     store_part<KIND>(g.Cl, off, lw, j);
@@ -214,12 +220,12 @@ __device__ __forceinline__ void tile_epilogue(const TcArgs &g, const float (&acc
         // transposed copies (coalesced across the warp: consecutive rows m).  For a
         // mirrored tile of a symmetric product the transpose goes into C itself.
         const bool into_c = mirror || diag;
-        float *Tf = into_c ? Cp : g.CT;
+        float *Tf = into_c ? g.C : g.CT;
         void *Th = into_c ? g.Ch : g.CTh, *Tl = into_c ? g.Cl : g.CTl;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
             if (diag && n0 + j <= m) continue;
-            const long long off = (n0 + j) * g.ld + m;
+            const long long off = at + (n0 + j) * g.ld + m;
             if (Tf) Tf[off] = v[j];
             if (Th) {
                 store_part<KIND>(Th, off, hw, j);
@@ -230,7 +236,7 @@ __device__ __forceinline__ void tile_epilogue(const TcArgs &g, const float (&acc
     if (g.resid) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
-        if (lane == 0 && rs != 0.0) atomicAdd(g.resid, rs);
+        if (lane == 0 && rs != 0.0) atomicAdd(g.resid + slot, rs);
     }
 }
 
@@ -361,8 +367,6 @@ __global__ void __launch_bounds__(192, 1)
         for (int w = blockIdx.x; w < items && ok; w += gridDim.x, cg += nchunks) {
             int bz, tm, tn;
             item_tile(w, tiles, g.mode, tiles_m, tiles_n, bz, tm, tn);
-            const float *Dp = g.D ? g.D + bz * g.sC : nullptr;
-            float *Cp = g.C ? g.C + bz * g.sC : nullptr;
             float acc[TN];
 #pragma unroll
             for (int j = 0; j < TN; ++j) acc[j] = 0.f;
@@ -371,7 +375,7 @@ __global__ void __launch_bounds__(192, 1)
             for (int c = 0; c < nchunks; ++c) {
                 const int buf = (cg + c) % kBufs;
                 if (c == max(0, nchunks - 2) && g.beta != 0.f) {   // this row of D into L2 ahead of the epilogue
-                    const float *drow = Dp + m * g.ld + static_cast<long long>(tn) * TN;
+                    const float *drow = g.D + bz * g.sC + m * g.ld + static_cast<long long>(tn) * TN;
 #pragma unroll
                     for (int q = 0; q < TN / 32; ++q) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(drow + 32 * q));
                 }
@@ -394,7 +398,7 @@ __global__ void __launch_bounds__(192, 1)
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(su32(&cfree[buf])) : "memory");
             }
-            if (ok) tile_epilogue<KIND>(g, acc, m, tm, tn, Dp, Cp, lane);
+            if (ok) tile_epilogue<KIND>(g, acc, m, tm, tn, bz, bz, lane);
         }   // work items
     }
     __syncwarp();
@@ -461,7 +465,7 @@ __device__ __forceinline__ void mmaw(uint32_t tmem, uint64_t a, uint64_t b, uint
 template <int KIND>
 __global__ void __launch_bounds__(384, 1)
     k_tc_gemm_w(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
-                const __grid_constant__ CUtensorMap mB0, const __grid_constant__ CUtensorMap mB1, TcArgs g,
+                const __grid_constant__ CUtensorMap mB0, const __grid_constant__ CUtensorMap mB1, const __grid_constant__ TcArgs g,
                 int tiles_n, const int2 *tile_of) {
     using Cfg = TcCfgW<KIND>;
     extern __shared__ uint8_t smem_raw[];
@@ -508,10 +512,18 @@ __global__ void __launch_bounds__(384, 1)
 
     if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(504 - 2 * EPI_REGS));
-        if (warp == 8 && lane == 0) {
+        // Warps 8 and 9 run as whole warps and one elected lane issues (elected(), tc_ops.cuh).
+        auto warp_wait = [&](uint64_t *bar, uint32_t parity) {   // the same answer in every lane
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, g.err) && !*abort_flag);
+            if (!ok) *abort_flag = 1;
+            return ok;
+        };
+        if (warp == 8) {
             // ---- TMA producer ----
+            const bool one = elected();
+            bool ok = true;
             int issued = 0, kg = 0;
-            for (int w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
+            for (int w = blockIdx.x; w < items && ok; w += gridDim.x) {
                 const int bz = w / wtiles;
                 int tm, TPn;
                 {
@@ -519,65 +531,69 @@ __global__ void __launch_bounds__(384, 1)
                     tm = c.x;
                     TPn = c.y;
                 }
-                const int ya = bz * g.M + tm * TM, yb = bz * g.N + TPn * TNW;
-                for (int kt = 0; kt < nk && !*abort_flag; ++kt, ++kg) {
+                const int slot = item_slot(g, bz), ya = slot * g.M + tm * TM, yb = slot * g.N + TPn * TNW;
+                for (int kt = 0; kt < nk; ++kt, ++kg) {
                     const int s = kg % Cfg::STAGES;
-                    const uint32_t ph = (kg / Cfg::STAGES) & 1;
-                    if (kg >= Cfg::STAGES && !mbar_wait(&empty[s], ph ^ 1, g.err)) {
-                        *abort_flag = 1;
-                        break;
+                    if (kg >= Cfg::STAGES && !(ok = warp_wait(&empty[s], ((kg / Cfg::STAGES) & 1) ^ 1))) break;
+                    if (one) {
+                        uint8_t *st = smem + s * Cfg::STAGE_BYTES;
+                        mbar_expect_tx(&full[s], Cfg::STAGE_BYTES);
+                        const int kx = kt * KELEM;
+                        tma_load_2d(st, &mA0, kx, ya, &full[s]);
+                        tma_load_2d(st + Cfg::OFF_B0, &mB0, kx, yb, &full[s]);
+                        if (KIND != 0) {
+                            tma_load_2d(st + Cfg::OFF_A1, &mA1, kx, ya, &full[s]);
+                            tma_load_2d(st + Cfg::OFF_B1, &mB1, kx, yb, &full[s]);
+                        }
                     }
-                    uint8_t *st = smem + s * Cfg::STAGE_BYTES;
-                    mbar_expect_tx(&full[s], Cfg::STAGE_BYTES);
-                    const int kx = kt * KELEM;
-                    tma_load_2d(st, &mA0, kx, ya, &full[s]);
-                    tma_load_2d(st + Cfg::OFF_B0, &mB0, kx, yb, &full[s]);
-                    if (KIND != 0) {
-                        tma_load_2d(st + Cfg::OFF_A1, &mA1, kx, ya, &full[s]);
-                        tma_load_2d(st + Cfg::OFF_B1, &mB1, kx, yb, &full[s]);
-                    }
+                    __syncwarp();
                     issued = kg + 1;
                 }
             }
-            if (*abort_flag) {   // let this CTA's copies land before shared memory is released
+            if (!ok) {   // let this CTA's copies land before shared memory is released
                 for (int k = (issued > Cfg::STAGES ? issued - Cfg::STAGES : 0); k < issued; ++k)
                     mbar_wait(&full[k % Cfg::STAGES], (k / Cfg::STAGES) & 1, g.err);
             }
-        } else if (warp == 9 && lane == 0) {
+        } else if (warp == 9) {
             // ---- MMA issuer: chunk c accumulates afresh into buffer c % kWideBufs ----
+            const bool one = elected();
+            bool ok = true;
             int kg = 0, cg = 0;
-            for (int w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x, cg += nchunks) {
-                for (int kt = 0; kt < nk && !*abort_flag; ++kt, ++kg) {
-                    const int c = cg + kt / cs, buf = c % kWideBufs;
-                    if (kt % cs == 0 && c >= kWideBufs &&
-                        !mbar_wait(&cfree[buf], ((c / kWideBufs) - 1) & 1, g.err)) {
-                        *abort_flag = 1;
-                        break;
-                    }
-                    const int s = kg % Cfg::STAGES;
-                    if (!mbar_wait(&full[s], (kg / Cfg::STAGES) & 1, g.err)) {
-                        *abort_flag = 1;
-                        break;
-                    }
+            for (int w = blockIdx.x; w < items && ok; w += gridDim.x, cg += nchunks) {
+                int in = 0, c = cg;   // stage of the chunk, chunk
+                for (int kt = 0; kt < nk; ++kt, ++kg) {
+                    const int buf = c % kWideBufs, s = kg % Cfg::STAGES;
+                    if (in == 0 && c >= kWideBufs && !(ok = warp_wait(&cfree[buf], ((c / kWideBufs) - 1) & 1))) break;
+                    if (!(ok = warp_wait(&full[s], (kg / Cfg::STAGES) & 1))) break;
                     fence_after();
                     const uint32_t base = su32(smem + s * Cfg::STAGE_BYTES);
                     const uint32_t dt = tmem + static_cast<uint32_t>(buf * TNW);
+                    const bool end = in == cs - 1 || kt == nk - 1;
+                    if (one) {
+                        const uint64_t a0 = sdesc(base), b0 = sdesc(base + Cfg::OFF_B0);
+                        const uint64_t a1 = sdesc(base + Cfg::OFF_A1), b1 = sdesc(base + Cfg::OFF_B1);
 #pragma unroll
-                    for (int k = 0; k < KB / 32; ++k) {
-                        const uint64_t a0 = sdesc(base + k * 32), b0 = sdesc(base + Cfg::OFF_B0 + k * 32);
-                        mmaw<Cfg::TF32>(dt, a0, b0, (kt % cs != 0 || k != 0) ? 1u : 0u);
-                        if (Cfg::PAIRS == 3) {
-                            const uint64_t a1 = sdesc(base + Cfg::OFF_A1 + k * 32);
-                            const uint64_t b1 = sdesc(base + Cfg::OFF_B1 + k * 32);
-                            mmaw<Cfg::TF32>(dt, a0, b1, 1u);
-                            mmaw<Cfg::TF32>(dt, a1, b0, 1u);
+                        for (int k = 0; k < KB / 32; ++k) {   // 32 bytes of K: two 16-byte units of the descriptor
+                            mmaw<Cfg::TF32>(dt, a0 + 2 * k, b0 + 2 * k, (in | k) != 0 ? 1u : 0u);
+                            if (Cfg::PAIRS == 3) {
+                                mmaw<Cfg::TF32>(dt, a0 + 2 * k, b1 + 2 * k, 1u);
+                                mmaw<Cfg::TF32>(dt, a1 + 2 * k, b0 + 2 * k, 1u);
+                            }
                         }
+                        mma_commit(&empty[s]);
+                        if (end) mma_commit(&cfull[buf]);
                     }
-                    mma_commit(&empty[s]);
-                    if (kt % cs == cs - 1 || kt == nk - 1) mma_commit(&cfull[buf]);
+                    __syncwarp();
+                    if (end) {
+                        in = 0;
+                        ++c;
+                    } else {
+                        ++in;
+                    }
                 }
             }
-            mma_commit(done);
+            if (one) mma_commit(done);
+            __syncwarp();
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(EPI_REGS));
@@ -586,7 +602,7 @@ __global__ void __launch_bounds__(384, 1)
         bool ok = true;
         int cg = 0;
         for (int w = blockIdx.x; w < items && ok; w += gridDim.x, cg += nchunks) {
-            const int bz = w / wtiles;
+            const int bz = w / wtiles, slot = item_slot(g, bz);
             int tm, TPn;
             {
                     const int2 c = tile_of[w - bz * wtiles];   // (tm, TPn) of the item, tabulated on the host
@@ -595,8 +611,6 @@ __global__ void __launch_bounds__(384, 1)
                 }
             const int tn = 2 * TPn + h;
             const bool write = tctiles::wide_half_valid(g.mode, tiles_n, tm, TPn, h);
-            const float *Dp = g.D ? g.D + bz * g.sC : nullptr;
-            float *Cp = g.C ? g.C + bz * g.sC : nullptr;
             float acc[TN];
 #pragma unroll
             for (int j = 0; j < TN; ++j) acc[j] = 0.f;
@@ -604,8 +618,8 @@ __global__ void __launch_bounds__(384, 1)
             const long long m = static_cast<long long>(tm) * TM + row;
             for (int c = 0; c < nchunks; ++c) {
                 const int buf = (cg + c) % kWideBufs;
-                if (write && c == max(0, nchunks - 2) && g.beta != 0.f) {
-                    const float *drow = Dp + m * g.ld + static_cast<long long>(tn) * TN;
+                if (write && c == max(0, nchunks - 2) && item_beta(g, bz) != 0.f) {
+                    const float *drow = g.D + slot * g.sC + m * g.ld + static_cast<long long>(tn) * TN;
 #pragma unroll
                     for (int qq = 0; qq < TN / 32; ++qq) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(drow + 32 * qq));
                 }
@@ -629,7 +643,7 @@ __global__ void __launch_bounds__(384, 1)
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(su32(&cfree[buf])) : "memory");
             }
-            if (ok && write) tile_epilogue<KIND>(g, acc, m, tm, tn, Dp, Cp, lane);
+            if (ok && write) tile_epilogue<KIND>(g, acc, m, tm, tn, bz, slot, lane);
         }
     }
     __syncwarp();
@@ -895,8 +909,6 @@ __global__ void __launch_bounds__(192, 1)
             tctiles::pair_tile(w - bz * ptiles, g.mode, tiles_m, tiles_n, TP, tn);
             const int tm = 2 * TP + static_cast<int>(rank);
             const bool write = tctiles::pair_tile_valid(g.mode, tiles_m, TP, tn, static_cast<int>(rank));
-            const float *Dp = g.D ? g.D + bz * g.sC : nullptr;
-            float *Cp = g.C ? g.C + bz * g.sC : nullptr;
             float acc[TN];
 #pragma unroll
             for (int j = 0; j < TN; ++j) acc[j] = 0.f;
@@ -905,7 +917,7 @@ __global__ void __launch_bounds__(192, 1)
             for (int c = 0; c < nchunks; ++c) {
                 const int buf = (cg + c) % kBufs;
                 if (write && c == max(0, nchunks - 2) && g.beta != 0.f) {
-                    const float *drow = Dp + m * g.ld + static_cast<long long>(tn) * TN;
+                    const float *drow = g.D + bz * g.sC + m * g.ld + static_cast<long long>(tn) * TN;
 #pragma unroll
                     for (int q = 0; q < TN / 32; ++q) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(drow + 32 * q));
                 }
@@ -928,7 +940,7 @@ __global__ void __launch_bounds__(192, 1)
                 __syncwarp();
                 if (lane == 0) remote_arrive(cfree_pair + static_cast<uint32_t>(buf) * 8u);
             }
-            if (ok && write) tile_epilogue<KIND>(g, acc, m, tm, tn, Dp, Cp, lane);
+            if (ok && write) tile_epilogue<KIND>(g, acc, m, tm, tn, bz, bz, lane);
         }
     }
     __syncwarp();
@@ -1060,7 +1072,8 @@ cudaError_t launch_tcw(const TcOperands &op, const TcArgs &g, cudaStream_t s) {
     }
     CUtensorMap a0, a1, b0, b1;
     const long long lda = op.lda, ldb = op.ldb;
-    const long long rows_a = static_cast<long long>(g.batch) * g.M, rows_b = static_cast<long long>(g.batch) * g.N;
+    const int mats = g.nslots ? 1 + *std::max_element(g.slot, g.slot + g.nslots) : g.batch;   // stacked matrices
+    const long long rows_a = static_cast<long long>(mats) * g.M, rows_b = static_cast<long long>(mats) * g.N;
     if (!make_map(&a0, op.A0, KIND, rows_a, g.K, lda, TM) || !make_map(&b0, op.B0, KIND, rows_b, g.K, ldb, TNW))
         return cudaErrorInvalidValue;
     if (KIND != 0) {
@@ -1166,9 +1179,32 @@ cudaError_t tc_gemm(int kind, const TcOperands &op, const TcArgs &g, cudaStream_
         g.ld % 8 || op.lda % 8 || op.ldb % 8 ||
         !g.err || (g.beta != 0.f && !g.D) || (g.Ch && !g.Cl) || (g.CTh && !g.CTl) || kind < 0 || kind > 2 ||
         (kind != 0 && (!op.A1 || !op.B1)) || (kind == 0 && (g.Ch || g.CTh)) || g.batch < 1 || g.batch > 65535 ||
-        (g.batch > 1 && (g.Ch || g.CT || g.CTh || g.C64 || g.resid || g.sC < static_cast<long long>(g.M) * g.ld)))
+        (g.batch > 1 && !g.nslots && (g.Ch || g.CT || g.CTh || g.C64 || g.resid)) ||
+        ((g.batch > 1 || g.nslots) && g.sC < static_cast<long long>(g.M) * g.ld) ||
+        (g.nslots && (g.nslots > kTcSlots || g.batch != g.nslots || g.M != g.N || op.lda != op.ldb)))
         return cudaErrorInvalidValue;
+    for (int k = 0; k < g.nslots; ++k)
+        if (g.slot[k] < 0 || (g.betas[k] != 0.f && !g.D)) return cudaErrorInvalidValue;
     const int form = tc_form();
+    if (g.nslots && form != 0) {   // the other forms take the items one by one
+        for (int k = 0; k < g.nslots; ++k) {
+            const size_t es = kind == 1 ? 2 : 4, rows = static_cast<size_t>(g.slot[k]) * g.M;
+            const long long at = g.slot[k] * g.sC;
+            auto moved = [](const void *p, size_t bytes) { return p ? static_cast<const char *>(p) + bytes : nullptr; };
+            auto out = [&](void *p) { return const_cast<char *>(moved(p, at * es)); };
+            TcOperands o = op;
+            const size_t ab = rows * op.lda * es;
+            o.A0 = moved(op.A0, ab), o.A1 = moved(op.A1, ab), o.B0 = moved(op.B0, ab), o.B1 = moved(op.B1, ab);
+            TcArgs h = g;
+            h.nslots = 0, h.batch = 1, h.alpha = g.alphas[k], h.beta = g.betas[k];
+            h.D = g.D ? g.D + at : nullptr, h.C = g.C ? g.C + at : nullptr, h.CT = g.CT ? g.CT + at : nullptr;
+            h.Ch = out(g.Ch), h.Cl = out(g.Cl), h.CTh = out(g.CTh), h.CTl = out(g.CTl);
+            h.C64 = g.C64 ? g.C64 + at : nullptr, h.resid = g.resid ? g.resid + g.slot[k] : nullptr;
+            const cudaError_t e = tc_gemm(kind, o, h, s);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
     if (form == 0) {
         if (kind == 0) return launch_tcw<0>(op, g, s);
         if (kind == 1) return launch_tcw<1>(op, g, s);

@@ -88,12 +88,14 @@ void tridiag_extremes(const std::vector<double> &a, const std::vector<double> &b
     double l = g0, h = g1;
     for (int it = 0; it < 200; ++it) {   // smallest: count(x) >= 1
         const double mid = 0.5 * (l + h);
+        if (mid == l || mid == h) break;   // the interval is one rounding wide
         if (sturm_count(a, b, mid) >= 1) h = mid; else l = mid;
     }
     lo = h;
     l = g0; h = g1;
     for (int it = 0; it < 200; ++it) {   // largest: count(x) >= m
         const double mid = 0.5 * (l + h);
+        if (mid == l || mid == h) break;
         if (sturm_count(a, b, mid) >= m) h = mid; else l = mid;
     }
     hi = h;
@@ -131,6 +133,8 @@ struct mbd_ctx {
     // mixed modes on a cell: each Hermitian Q(q) as the real symmetric [[Re, -Im], [Im, Re]] of
     // order 2n (leading dimension lde), its FP64 workspaces
     long long lde = 0;
+    int mgroup = 1;   // Bloch vectors iterated on together, of which the FP32, split and e* buffers hold one matrix each
+    double *dmix = nullptr;   // per matrix of a group: |I - ZY|^2, the correction's residual, the largest row sum
     double *eM = nullptr, *eV = nullptr, *eW = nullptr, *eVT = nullptr, *eZ = nullptr;
     double *dh, *dgomb, *dgab0, *dgrb, *dgR, *dga0, *dgom, *dgrv, *dgp;
     // periodic systems: cell, Bloch vectors and reciprocal lattice (host lists, device copies)
@@ -413,8 +417,19 @@ int factorise(mbd_ctx *ctx, double *A, int batch, cudaStream_t s, const char *or
     return MBD_OK;
 }
 
+// Bloch vectors that the mixed modes iterate on together: enough for eight tiles of a symmetric product
+// on every SM, while their matrices take at most 4 GiB.  Alone, a matrix of the 256-atom cell (order 1536: 42
+// tiles) leaves most of the 152 SMs idle, and each of its launches and read-backs serves one matrix.
+int mixed_group(int nk, long long lde, int precision) {
+    const long long t = lde / 128, tiles = (t + 1) * (t + 1) / 4;   // 128 x 256 tiles of one triangle
+    const long long split = precision == MBD_PREC_BF16X3 ? 24 : (precision == MBD_PREC_TF32X3 ? 48 : 0);
+    const long long bytes = lde * lde * (6 * 4 + 5 * 8 + split);
+    const long long want = std::min<long long>((8 * 152 + tiles - 1) / tiles, (4LL << 30) / bytes);
+    return static_cast<int>(std::max<long long>(1, std::min<long long>({want, nk, kTcSlots})));
+}
+
 // Carves the workspace out of one allocation (256-byte aligned pieces).
-int allocate(mbd_ctx *ctx) {
+int allocate(mbd_ctx *ctx, bool groups = true) {
     const long long ld = ctx->ld, N = ctx->N, nf1 = ctx->nf1, nb = ctx->nb;
     const size_t mat = sizeof(double) * static_cast<size_t>(ld) * ld;
     std::vector<std::pair<double **, size_t>> plan = {
@@ -426,13 +441,14 @@ int allocate(mbd_ctx *ctx) {
         {&ctx->dB, nf1 * ld * 3},
         {&ctx->dh, nf1 * N}, {&ctx->dgomb, N}, {&ctx->dgab0, N}, {&ctx->dgrb, N}, {&ctx->dgR, 3 * N},
         {&ctx->dga0, N}, {&ctx->dgom, N}, {&ctx->dgrv, N}, {&ctx->dgp, 4 * N}, {&ctx->dscal, 8 + 2 * 64 + 1824},
+        {&ctx->dmix, 3 * kTcSlots},
     };
     const long long nk = ctx->nk;
     if (ctx->periodic) {
         plan.push_back({&ctx->dkq, 3 * nk});
         plan.push_back({&ctx->dkw, nk});
         plan.push_back({&ctx->dG, 3LL * ctx->nG});
-        plan.push_back({&ctx->dcoef, nk * 2 * kLanczosSteps});
+        plan.push_back({&ctx->dcoef, nk * (2 * kLanczosSteps + 1)});   // and the mixed modes' energies
         plan.push_back({&ctx->dlzw, 3 * nk * 2 * ld});
         plan.push_back({&ctx->dgA, 9});
         plan.push_back({&ctx->dgAout, 9});
@@ -456,10 +472,11 @@ int allocate(mbd_ctx *ctx) {
     // the mixed modes' iteration buffers: the matrix order, or the order of a cell's embedded
     // Hermitian matrices
     const long long ldm = ctx->periodic ? ctx->lde : ld;
-    const size_t mat32 = sizeof(float) * static_cast<size_t>(ldm) * ldm, mat16 = mat32 / 2;
+    ctx->mgroup = groups && ctx->periodic && !fp64_path(prec) ? mixed_group(static_cast<int>(nk), ldm, prec) : 1;
+    const size_t mat32 = sizeof(float) * static_cast<size_t>(ldm) * ldm * ctx->mgroup, mat16 = mat32 / 2;
     const size_t split_mat = prec == MBD_PREC_BF16X3 ? mat16 : (prec == MBD_PREC_TF32X3 ? mat32 : 0);
     if (!fp64_path(prec)) bytes += 6 * mat32;
-    const size_t emat = sizeof(double) * static_cast<size_t>(ctx->lde) * ctx->lde;
+    const size_t emat = sizeof(double) * static_cast<size_t>(ctx->lde) * ctx->lde * ctx->mgroup;
     const bool embed = ctx->periodic && !fp64_path(prec);
     if (embed) bytes += 5 * emat;
     bytes += 12 * split_mat;
@@ -487,6 +504,11 @@ int allocate(mbd_ctx *ctx) {
         release(ctx);
         size_t want = bytes + crt_work;
         e = cudaMalloc(&ctx->slab, want);
+        if (e != cudaSuccess && ctx->mgroup > 1) {   // one matrix at a time
+            cudaGetLastError();
+            ctx->slab = nullptr;
+            return allocate(ctx, false);
+        }
         if (e != cudaSuccess && crt_work) {   // without the tensor-core products' scratch
             cudaGetLastError();
             want = bytes;
@@ -739,26 +761,37 @@ struct MixMat {
     const void *op1(bool split) const { return split ? static_cast<const void *>(l) : static_cast<const void *>(f); }
 };
 
-// The matrix of one mixed-precision matrix function and where its results go: Q (FP64,
-// symmetric, ld x ld, valid n x n, decoupled padding), the FP64 workspaces V and W (ld^2
-// doubles each) and VT (ld^2 doubles), the FP64 output Zd ~ Q^{-1/2}, and (if tq is not NULL)
+// The matrices of a mixed-precision matrix function and where its results go: `count` of Q (FP64,
+// symmetric, ld x ld, valid n x n, decoupled padding) one after another, the FP64 workspaces V, W and VT (ld^2
+// doubles each a matrix), the FP64 outputs Zd ~ Q^{-1/2}, the energies [count], and (if tq is not NULL) for each
 // the traces of the first N diagonal 3x3 blocks of Q^{1/2}, second order in the error of Zd.
 struct MixProblem {
     const double *Q;
     long long ld;
     int n;
     double *V, *W, *VT, *Zd;
-    double *tq;
+    double *tq, *energy;
+    int count = 1;
+};
+// A matrix's scale and spectrum bounds (inputs), and how its iteration went.
+struct MixItem {
+    double sc, lbound, ubound;
+    double resid = 0.0, prev = 1e300;
+    int it = 0, code = MBD_OK;
+    bool done = false;
+    const float *Z = nullptr;   // its Z after the last step
 };
 
 // Mixed-precision coupled Newton-Schulz (same scaled steps as the FP64 loop) on the
 // tensor cores, stopped at the precision floor, then the FP64 correction:
 // Zd = Z/sqrt(s) ~ Q^{-1/2}, V = Q Zd, W = Zd V, E = (3 Tr V - sum V o W)/4 - 3/2 sum w.
-// The FP32 and split-part buffers of the context hold the iteration (ld^2 elements each).
-int newton_schulz_mixed(mbd_ctx *ctx, cudaStream_t s, const MixProblem &pr, double sc, double lbound, double ubound,
-                        double *energy_out, std::vector<Span> &spans, cudaEvent_t &e_corr) {
-    const long long ld = pr.ld;
-    const int n = pr.n, N = ctx->N, M = static_cast<int>(ld);
+// The FP32 and split-part buffers of the context hold the iteration (ld^2 elements each a matrix).
+// The matrices of a group share launches and read-backs; each takes its own steps, as if it were alone, and
+// leaves the group when it is done.
+int newton_schulz_mixed(mbd_ctx *ctx, cudaStream_t s, const MixProblem &pr, std::vector<MixItem> &items,
+                        std::vector<Span> &spans, cudaEvent_t &e_corr) {
+    const long long ld = pr.ld, mat = ld * ld;
+    const int n = pr.n, N = ctx->N, M = static_cast<int>(ld), count = pr.count;
     const int kind = ctx->opt.precision == MBD_PREC_TF32 ? 0 : (ctx->opt.precision == MBD_PREC_BF16X3 ? 1 : 2);
     const bool split = kind != 0;
     const double nd = static_cast<double>(n);
@@ -766,88 +799,124 @@ int newton_schulz_mixed(mbd_ctx *ctx, cudaStream_t s, const MixProblem &pr, doub
     MixMat Y{ctx->fY, ctx->hY[0], ctx->hY[1]}, Z{ctx->fZ, ctx->hZ[0], ctx->hZ[1]};
     MixMat Y2{ctx->fY2, ctx->hY2[0], ctx->hY2[1]}, Z2{ctx->fZ2, ctx->hZ2[0], ctx->hZ2[1]};
     MixMat P{ctx->fP, ctx->hP[0], ctx->hP[1]}, PT{ctx->fPT, ctx->hPT[0], ctx->hPT[1]};
-    mixed_init(kind, pr.Q, ld, 1.0 / sc, Y.f, split ? Y.h : nullptr, Y.l, Z.f, Z.h, Z.l, s);
+    auto at = [&](const MixMat &m, int k) {   // matrix k of the group
+        const long long part = k * mat * (kind == 1 ? 2 : 4);
+        auto moved = [&](void *p) { return split ? static_cast<void *>(static_cast<char *>(p) + part) : p; };
+        return MixMat{m.f + k * mat, moved(m.h), moved(m.l)};
+    };
+    for (int k = 0; k < count; ++k) {
+        const MixMat y = at(Y, k), z = at(Z, k);
+        mixed_init(kind, pr.Q + k * mat, ld, 1.0 / items[k].sc, y.f, split ? y.h : nullptr, y.l, z.f, z.h, z.l, s);
+    }
     // K stages per tensor-memory accumulation: the option, or the kind's default (BF16x3: 8,
     // i.e. 512 products per FP32 sum in tensor memory; TF32 and TF32x3: 2, i.e. 64 products)
     const int cstages = ctx->opt.tc_chunk_stages > 0 ? ctx->opt.tc_chunk_stages : (kind == 1 ? 8 : 2);
     // the correction's TF32x3 products keep short accumulations whatever the iteration's kind
     constexpr int kCorrectionChunk = 2;
-    auto tc = [&](const TcOperands &op, TcArgs g, double flops) -> int {
+    std::vector<int> active;   // matrices still iterated on
+    for (int k = 0; k < count; ++k) active.push_back(k);
+    // One product of every active matrix, timed; alpha and beta by matrix.
+    auto tc = [&](int tk, const TcOperands &op, TcArgs g, double flops, const char *origin, auto alpha, auto beta) -> int {
+        if (count == 1) {
+            g.alpha = static_cast<float>(alpha(0));
+            g.beta = static_cast<float>(beta(0));
+        } else {
+            g.batch = g.nslots = static_cast<int>(active.size());
+            g.sC = mat;
+            for (int j = 0; j < g.nslots; ++j) {
+                g.slot[j] = active[j];
+                g.alphas[j] = static_cast<float>(alpha(active[j]));
+                g.betas[j] = static_cast<float>(beta(active[j]));
+            }
+        }
         Span sp;
-        sp.flops = flops;
-        g.chunk_stages = cstages;
+        sp.flops = flops * static_cast<double>(active.size());
         mark(ctx, s, sp.a);
-        const cudaError_t e = tc_gemm(kind, op, g, s);
+        const cudaError_t e = tc_gemm(tk, op, g, s);
         mark(ctx, s, sp.b);
         if (ctx->profiling) spans.push_back(sp);
-        return e == cudaSuccess ? MBD_OK : cuda_fail(ctx, "newton_schulz_tc", e);
+        return e == cudaSuccess ? MBD_OK : cuda_fail(ctx, origin, e);
     };
-    double *resid_dev = ctx->dscal + 2;
-    double resid = 0.0, prev = 1e300;
-    bool floor_reached = false;
-    int it = 0;
-    for (; it < ctx->opt.ns_max_iter; ++it) {
+    auto one = [](int) { return 1.0; };
+    auto zero = [](int) { return 0.0; };
+    double *resid_dev = ctx->dmix, *corr_dev = ctx->dmix + kTcSlots;
+    std::vector<ns::Coeffs> cf(count);
+    auto c1 = [&](int k) { return cf[k].c1; };
+    auto c3 = [&](int k) { return cf[k].c3; };
+    for (int it = 0; it < ctx->opt.ns_max_iter && !active.empty(); ++it) {
         MixMat Pk = Y, PTk = Y;   // P_0 = Y_0 (symmetric)
         if (it > 0) {
-            MBD_CUDA(cudaMemsetAsync(resid_dev, 0, sizeof(double), s), "newton_schulz_tc");
+            MBD_CUDA(cudaMemsetAsync(resid_dev, 0, sizeof(double) * count, s), "newton_schulz_tc");
             TcOperands op{Z.op0(split), Z.op1(split), Y.op0(split), Y.op1(split), ld, ld};
             TcArgs g{M, M, M, 1.f, 0.f, nullptr, ld, split ? nullptr : P.f, split ? P.h : nullptr,
                      split ? P.l : nullptr, split ? nullptr : PT.f, split ? PT.h : nullptr, split ? PT.l : nullptr,
                      resid_dev, n, 0, ctx->dstatus};
-            int rc = tc(op, g, flops_full);   // P = Z Y (and its transpose), resid = |I - P|_F^2
-            if (rc) return rc;
+            g.chunk_stages = cstages;
+            // P = Z Y (and its transpose), resid = |I - P|_F^2
+            if (const int rc = tc(kind, op, g, flops_full, "newton_schulz_tc", one, zero)) return rc;
             Pk = P;
             PTk = PT;
-            double r2 = 0.0;
-            MBD_CUDA(cudaMemcpyAsync(&r2, resid_dev, sizeof(double), cudaMemcpyDeviceToHost, s), "newton_schulz_tc");
+            double r2[kTcSlots] = {};
+            MBD_CUDA(cudaMemcpyAsync(r2, resid_dev, sizeof(double) * count, cudaMemcpyDeviceToHost, s), "newton_schulz_tc");
             MBD_CUDA(cudaStreamSynchronize(s), "newton_schulz_tc");
-            resid = std::sqrt(r2);
-            if (!std::isfinite(resid) || resid > 2.0 * std::sqrt(nd) + 1.0) {
-                ctx->ns_iter = it;
-                ctx->ns_resid = resid;
-                return fail(ctx, MBD_ERR_NEG_EIGENVALUE, "newton_schulz_tc",
-                            "Q has a non-positive eigenvalue (polarization catastrophe)");
+            std::vector<int> good;
+            for (int k : active) {
+                MixItem &m = items[k];
+                m.resid = std::sqrt(r2[k]);
+                if (!std::isfinite(m.resid) || m.resid > 2.0 * std::sqrt(nd) + 1.0) {
+                    m.it = it;
+                    m.code = MBD_ERR_NEG_EIGENVALUE;
+                } else {
+                    good.push_back(k);
+                }
             }
+            active = good;
+            if (active.empty()) break;
         }
-        // The tensor-core phase ends at its precision floor (ns::mixed_last).
-        const bool last = it > 0 && ns::mixed_last(resid, prev, ctx->opt.ns_tol, kMixedFloor * std::sqrt(nd));
-        const ns::Coeffs cf = ns::step(lbound, ubound, last);
-        const double c1 = cf.c1, c3 = cf.c3;
+        for (int k : active) {
+            MixItem &m = items[k];
+            // The tensor-core phase ends at its precision floor (ns::mixed_last).
+            m.done = it > 0 && ns::mixed_last(m.resid, m.prev, ctx->opt.ns_tol, kMixedFloor * std::sqrt(nd));
+            cf[k] = ns::step(m.lbound, m.ubound, m.done);
+        }
         {   // Y' = c1 Y + c3 Y P = NT(Y, P^T): symmetric
             TcOperands op{Y.op0(split), Y.op1(split), PTk.op0(split), PTk.op1(split), ld, ld};
-            TcArgs g{M, M, M, static_cast<float>(c3), static_cast<float>(c1), Y.f, ld, Y2.f,
-                     split ? Y2.h : nullptr, split ? Y2.l : nullptr, nullptr, nullptr, nullptr, nullptr, 0, 2,
-                     ctx->dstatus};
-            int rc = tc(op, g, flops_sym);
-            if (rc) return rc;
+            TcArgs g{M, M, M, 0.f, 0.f, Y.f, ld, Y2.f, split ? Y2.h : nullptr, split ? Y2.l : nullptr, nullptr, nullptr,
+                     nullptr, nullptr, 0, 2, ctx->dstatus};
+            g.chunk_stages = cstages;
+            if (const int rc = tc(kind, op, g, flops_sym, "newton_schulz_tc", c3, c1)) return rc;
         }
         if (it == 0) {
-            mixed_axpby_identity(kind, Y.f, ld, static_cast<float>(c1), static_cast<float>(c3), Z2.f,
-                                 split ? Z2.h : nullptr, Z2.l, s);
+            for (int k : active) {
+                const MixMat z = at(Z2, k);
+                mixed_axpby_identity(kind, at(Y, k).f, ld, static_cast<float>(cf[k].c1), static_cast<float>(cf[k].c3), z.f,
+                                     split ? z.h : nullptr, z.l, s);
+            }
         } else {   // Z' = c1 Z + c3 P Z = NT(P, Z): symmetric
             TcOperands op{Pk.op0(split), Pk.op1(split), Z.op0(split), Z.op1(split), ld, ld};
-            TcArgs g{M, M, M, static_cast<float>(c3), static_cast<float>(c1), Z.f, ld, Z2.f,
-                     split ? Z2.h : nullptr, split ? Z2.l : nullptr, nullptr, nullptr, nullptr, nullptr, 0, 2,
-                     ctx->dstatus};
-            int rc = tc(op, g, flops_sym);
-            if (rc) return rc;
+            TcArgs g{M, M, M, 0.f, 0.f, Z.f, ld, Z2.f, split ? Z2.h : nullptr, split ? Z2.l : nullptr, nullptr, nullptr,
+                     nullptr, nullptr, 0, 2, ctx->dstatus};
+            g.chunk_stages = cstages;
+            if (const int rc = tc(kind, op, g, flops_sym, "newton_schulz_tc", c3, c1)) return rc;
         }
         std::swap(Y, Y2);
         std::swap(Z, Z2);
-        if (it > 0) prev = resid;
-        if (last) {
-            floor_reached = true;
-            ++it;
-            break;
+        std::vector<int> left;
+        for (int k : active) {
+            MixItem &m = items[k];
+            m.it = it + 1;
+            if (it > 0) m.prev = m.resid;
+            if (m.done) m.Z = Z.f + k * mat;
+            else left.push_back(k);
         }
+        active = left;
     }
-    ctx->ns_iter = it;
-    ctx->ns_resid = resid;
     int st = 0;
     MBD_CUDA(cudaMemcpyAsync(&st, ctx->dstatus, sizeof(int), cudaMemcpyDeviceToHost, s), "newton_schulz_tc");
     MBD_CUDA(cudaStreamSynchronize(s), "newton_schulz_tc");
     if (st & ST_TC_TIMEOUT) return fail(ctx, MBD_ERR_CUDA, "newton_schulz_tc", "tensor-core GEMM wait timed out");
-    if (!floor_reached) return fail(ctx, MBD_ERR_NOT_CONVERGED, "newton_schulz_tc", "iteration cap reached");
+    active.clear();   // the matrices before the first one that failed
+    for (int k = 0; k < count && items[k].done && items[k].code == MBD_OK; ++k) active.push_back(k);
     // ---- correction ----
     // With Zs ~ (Q/s)^{-1/2} (FP32 values of the iteration), Vs = (Q/s) Zs, Ws = Zs Vs:
     // Tr Q^{1/2} ~ sqrt(s) (3 Tr Vs - sum Vs o Ws)/2, second order in the error of Zs.
@@ -855,64 +924,69 @@ int newton_schulz_mixed(mbd_ctx *ctx, cudaStream_t s, const MixProblem &pr, doub
     // diagonal scalings and TF32x3 tensor-core products of the off-diagonal parts (no
     // accumulator mixes a dominant term with many small ones; chunk sums in FP32 with
     // round-to-nearest), each product added once into its FP64 result.
-    mark(ctx, s, e_corr);
-    {
-        // FP32 workspace: the iteration's matrices are free now.  Parts of offdiag(Q/s) and of
+    double c2[kTcSlots] = {};
+    if (!active.empty()) {
+        mark(ctx, s, e_corr);
+        // FP32 workspace: the iteration's matrices other than Z are free now.  Parts of offdiag(Q/s) and of
         // the full Zs feed the first product; offdiag(Zs) (reusing the Q parts) and Vs^T the
         // second.
         float *Qh = Y.f, *Ql = Y2.f, *Zs_h = P.f, *Zs_l = PT.f, *Zh = Qh, *Zl = Ql;
-        float *VTh = reinterpret_cast<float *>(pr.VT), *VTl = VTh + ld * ld;
-        double *V64 = pr.V, *W64 = pr.W;
-        const float *Zs = Z.f;
-        split_tf32_f64(pr.Q, ld, 1.0 / sc, 1, Qh, Ql, s);
-        split_tf32_f32(Zs, ld, 0, Zs_h, Zs_l, s);
-        diag_scale_rows_f64(pr.Q, Zs, ld, 1.0 / sc, V64, s);
-        auto tc64 = [&](const TcOperands &op, const TcArgs &g) -> int {   // timed like the iteration's products
-            Span sp;
-            sp.flops = flops_full;
-            mark(ctx, s, sp.a);
-            const cudaError_t e = tc_gemm(2, op, g, s);
-            mark(ctx, s, sp.b);
-            if (ctx->profiling) spans.push_back(sp);
-            return e == cudaSuccess ? MBD_OK : cuda_fail(ctx, "correction", e);
-        };
+        float *VTh = reinterpret_cast<float *>(pr.VT), *VTl = VTh + count * mat;
+        for (int k : active) {
+            const long long o = k * mat;
+            split_tf32_f64(pr.Q + o, ld, 1.0 / items[k].sc, 1, Qh + o, Ql + o, s);
+            split_tf32_f32(items[k].Z, ld, 0, Zs_h + o, Zs_l + o, s);
+            diag_scale_rows_f64(pr.Q + o, items[k].Z, ld, 1.0 / items[k].sc, pr.V + o, s);
+        }
         {   // Vs += offdiag(Q/s) Zs = NT(offdiag(Q/s), Zs) (Zs symmetric)
             TcOperands op{Qh, Ql, Zs_h, Zs_l, ld, ld};
             TcArgs g{M, M, M, 1.f, 0.f, nullptr, ld, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                     0, 0, ctx->dstatus, V64, kCorrectionChunk};
-            if (int rc = tc64(op, g)) return rc;
+                     0, 0, ctx->dstatus, pr.V, kCorrectionChunk};
+            if (const int rc = tc(2, op, g, flops_full, "correction", one, zero)) return rc;
         }
-        split_tf32_f64_t(V64, ld, 1.0, VTh, VTl, s);
-        split_tf32_f32(Zs, ld, 1, Zh, Zl, s);
-        diag_scale_rows_f32(Zs, V64, ld, W64, s);
+        for (int k : active) {
+            const long long o = k * mat;
+            split_tf32_f64_t(pr.V + o, ld, 1.0, VTh + o, VTl + o, s);
+            split_tf32_f32(items[k].Z, ld, 1, Zh + o, Zl + o, s);
+            diag_scale_rows_f32(items[k].Z, pr.V + o, ld, pr.W + o, s);
+        }
         {   // Ws += offdiag(Zs) Vs = NT(offdiag(Zs), Vs^T)
             TcOperands op{Zh, Zl, VTh, VTl, ld, ld};
             TcArgs g{M, M, M, 1.f, 0.f, nullptr, ld, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                     0, 0, ctx->dstatus, W64, kCorrectionChunk};
-            if (int rc = tc64(op, g)) return rc;
+                     0, 0, ctx->dstatus, pr.W, kCorrectionChunk};
+            if (const int rc = tc(2, op, g, flops_full, "correction", one, zero)) return rc;
         }
-        energy_correction(pr.Q, 1.0 / sc, Zs, V64, W64, ld, n, std::sqrt(sc), ctx->dombar, N,
-                          ctx->dscal + 8 + 2 * 64, energy_out, ctx->dscal + 3, s);
-        if (pr.tq)   // diagonal blocks of Q^{1/2}, second order in the error of Zs, for dE/d omega_bar
-            block_trace_sqrt(V64, W64, ld, N, std::sqrt(sc), pr.tq, s);
+        for (int k : active) {
+            const long long o = k * mat;
+            const double sc = items[k].sc;
+            energy_correction(pr.Q + o, 1.0 / sc, items[k].Z, pr.V + o, pr.W + o, ld, n, std::sqrt(sc), ctx->dombar, N,
+                              ctx->dscal + 8 + 2 * 64, pr.energy + k, corr_dev + k, s);
+            if (pr.tq)   // diagonal blocks of Q^{1/2}, second order in the error of Zs, for dE/d omega_bar
+                block_trace_sqrt(pr.V + o, pr.W + o, ld, N, std::sqrt(sc), pr.tq + static_cast<long long>(k) * N, s);
+            to_f64(items[k].Z, ld, 1.0 / std::sqrt(sc), pr.Zd + o, s);   // Q^{-1/2} for the gradient
+        }
+        MBD_CUDA(cudaMemcpyAsync(c2, corr_dev, sizeof(double) * count, cudaMemcpyDeviceToHost, s), "correction");
+        int st2 = 0;
+        MBD_CUDA(cudaMemcpyAsync(&st2, ctx->dstatus, sizeof(int), cudaMemcpyDeviceToHost, s), "correction");
+        MBD_CUDA(cudaStreamSynchronize(s), "correction");
+        if (st2 & ST_TC_TIMEOUT) return fail(ctx, MBD_ERR_CUDA, "correction", "tensor-core GEMM wait timed out");
     }
-    double *Zd = pr.Zd;
-    to_f64(Z.f, ld, 1.0 / std::sqrt(sc), Zd, s);   // Q^{-1/2} for the gradient
-    double c2 = 0.0;
-    MBD_CUDA(cudaMemcpyAsync(&c2, ctx->dscal + 3, sizeof(double), cudaMemcpyDeviceToHost, s), "correction");
-    MBD_CUDA(cudaStreamSynchronize(s), "correction");
-    int st2 = 0;
-    MBD_CUDA(cudaMemcpyAsync(&st2, ctx->dstatus, sizeof(int), cudaMemcpyDeviceToHost, s), "correction");
-    MBD_CUDA(cudaStreamSynchronize(s), "correction");
-    if (st2 & ST_TC_TIMEOUT) return fail(ctx, MBD_ERR_CUDA, "correction", "tensor-core GEMM wait timed out");
-    ctx->corr_resid = c2;
-    // The corrected energy is second order in the error of Zs: with Zs = (Q/s)^{-1/2} (I + F),
-    // Ws - I ~ 2F and the error of Tr Q^{1/2}/2 is about (3/4) Tr(Q^{1/2} F^2) <= (3/16) sqrt(s) r^2.
-    // The split kinds claim the 1e-6 Ha/atom bar; a Z too poor for it is reported, not used.
-    if (split && !(3.0 / 16.0 * std::sqrt(sc) * c2 * c2 / (n / 3) <= ctx->opt.mixed_max_error))
-        return fail(ctx, MBD_ERR_NOT_CONVERGED, "correction",
-                    "the tensor-core Q^{-1/2} is too inaccurate for the energy bar (mixed_max_error)");
-    ctx->Zlast = Zd;
+    for (int k = 0; k < count; ++k) {
+        const MixItem &m = items[k];
+        ctx->ns_iter = m.it;
+        ctx->ns_resid = m.resid;
+        if (m.code != MBD_OK)
+            return fail(ctx, m.code, "newton_schulz_tc", "Q has a non-positive eigenvalue (polarization catastrophe)");
+        if (!m.done) return fail(ctx, MBD_ERR_NOT_CONVERGED, "newton_schulz_tc", "iteration cap reached");
+        ctx->corr_resid = k ? std::max(ctx->corr_resid, c2[k]) : c2[k];
+        // The corrected energy is second order in the error of Zs: with Zs = (Q/s)^{-1/2} (I + F),
+        // Ws - I ~ 2F and the error of Tr Q^{1/2}/2 is about (3/4) Tr(Q^{1/2} F^2) <= (3/16) sqrt(s) r^2.
+        // The split kinds claim the 1e-6 Ha/atom bar; a Z too poor for it is reported, not used.
+        if (split && !(3.0 / 16.0 * std::sqrt(m.sc) * c2[k] * c2[k] / (n / 3) <= ctx->opt.mixed_max_error))
+            return fail(ctx, MBD_ERR_NOT_CONVERGED, "correction",
+                        "the tensor-core Q^{-1/2} is too inaccurate for the energy bar (mixed_max_error)");
+    }
+    ctx->Zlast = pr.Zd;
     ctx->zscale = 1.0;
     return MBD_OK;
 }
@@ -1035,50 +1109,65 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
         const int ne = 2 * n, lzs = std::min(kLanczosSteps, static_cast<int>(lde));
         int it_max = 0;
         double res_max = 0.0, corr_max = 0.0, sc_max = 0.0;
-        std::vector<double> lzk(2 * lzs);
-        for (int k = 0; k < nk; ++k) {
-            embed_hermitian(ctx->dQ, ld, n, k, ctx->eM, lde, s);
-            max_abs_rowsum(ctx->eM, lde, static_cast<int>(lde), ctx->dscal + 1, s);
-            double sk = 0.0;
-            MBD_CUDA(cudaMemcpyAsync(&sk, ctx->dscal + 1, sizeof(double), cudaMemcpyDeviceToHost, s), "newton_schulz");
-            lanczos_coefficients_f32(ctx->eM, ctx->fY, lde, lzs, ctx->eV, ctx->dscal + 8, s);
-            MBD_CUDA(cudaMemcpyAsync(lzk.data(), ctx->dscal + 8, sizeof(double) * 2 * lzs, cudaMemcpyDeviceToHost, s),
+        std::vector<double> lzk;
+        double *energies = ctx->dcoef + static_cast<long long>(nk) * 2 * kLanczosSteps;
+        double *rowsum = ctx->dmix + 2 * kTcSlots;
+        const long long emat = lde * lde;
+        for (int k0 = 0; k0 < nk; k0 += ctx->mgroup) {
+            const int g = std::min(ctx->mgroup, nk - k0);
+            for (int k = 0; k < g; ++k) {
+                embed_hermitian(ctx->dQ, ld, n, k0 + k, ctx->eM + k * emat, lde, s);
+                max_abs_rowsum(ctx->eM + k * emat, lde, static_cast<int>(lde), rowsum + k, s);
+            }
+            double sums[kTcSlots] = {};
+            MBD_CUDA(cudaMemcpyAsync(sums, rowsum, sizeof(double) * g, cudaMemcpyDeviceToHost, s), "newton_schulz");
+            lanczos_coefficients_f32(ctx->eM, ctx->fY, lde, lzs, ctx->eV, ctx->dcoef, s, g, emat);
+            lzk.resize(static_cast<size_t>(g) * 2 * lzs);
+            MBD_CUDA(cudaMemcpyAsync(lzk.data(), ctx->dcoef, sizeof(double) * lzk.size(), cudaMemcpyDeviceToHost, s),
                      "newton_schulz");
             MBD_CUDA(cudaStreamSynchronize(s), "newton_schulz");
-            if (!(sk > 0.0) || !std::isfinite(sk)) return fail(ctx, MBD_ERR_INPUT, "newton_schulz", "invalid Q scale");
-            double lo = 0.0, hi = sk;
-            {
+            std::vector<MixItem> items(g);
+            for (int k = 0; k < g; ++k) {
+                double sk = sums[k];
+                if (!(sk > 0.0) || !std::isfinite(sk))
+                    return fail(ctx, MBD_ERR_INPUT, "newton_schulz", "invalid Q scale");
+                double lo = 0.0, hi = sk;
+                const double *lz = lzk.data() + static_cast<size_t>(k) * 2 * lzs;
                 std::vector<double> da, db;
                 for (int j = 0; j < lzs; ++j) {
-                    da.push_back(lzk[2 * j]);
-                    if (j + 1 < lzs) db.push_back(lzk[2 * j + 1]);
-                    if (!(lzk[2 * j + 1] > 1e-14 * sk)) break;
+                    da.push_back(lz[2 * j]);
+                    if (j + 1 < lzs) db.push_back(lz[2 * j + 1]);
+                    if (!(lz[2 * j + 1] > 1e-14 * sk)) break;
                 }
                 db.resize(da.empty() ? 0 : da.size() - 1);
                 if (!da.empty()) tridiag_extremes(da, db, lo, hi);
+                double ub = 1.0;
+                if (std::isfinite(hi) && hi > 0.0 && 1.05 * hi < sk) {
+                    sk = 1.05 * hi;
+                    ub = 1.05;
+                }
+                items[k].sc = sk;
+                items[k].lbound = ns::lower_estimate(lo, sk);   // an estimate (ns_schedule.h)
+                items[k].ubound = ub;
             }
-            double ub = 1.0;
-            if (std::isfinite(hi) && hi > 0.0 && 1.05 * hi < sk) {
-                sk = 1.05 * hi;
-                ub = 1.05;
-            }
-            double lb = ns::lower_estimate(lo, sk);   // an estimate (ns_schedule.h)
             // Re Tr (Q(q_k)^{1/2})_ii: the first N diagonal blocks of M_k^{1/2}, into row k of dlzw
             const MixProblem pr{ctx->eM, lde, ne, ctx->eV, ctx->eW, ctx->eVT, ctx->eZ,
-                                ctx->dlzw + static_cast<long long>(k) * N};
-            const int rk = newton_schulz_mixed(ctx, s, pr, sk, lb, ub, ctx->dcoef + k, tc_spans, e_corr);
+                                ctx->dlzw + static_cast<long long>(k0) * N, energies + k0, g};
+            const int rk = newton_schulz_mixed(ctx, s, pr, items, tc_spans, e_corr);
             if (rk) return rk;
-            extract_hermitian(ctx->eZ, lde, n, ctx->dZ, ld, k, s);
-            it_max = std::max(it_max, ctx->ns_iter);
-            res_max = std::max(res_max, ctx->ns_resid);
+            for (int k = 0; k < g; ++k) extract_hermitian(ctx->eZ + k * emat, lde, n, ctx->dZ, ld, k0 + k, s);
+            for (const MixItem &m : items) {
+                it_max = std::max(it_max, m.it);
+                res_max = std::max(res_max, m.resid);
+                sc_max = std::max(sc_max, m.sc);
+            }
             corr_max = std::max(corr_max, ctx->corr_resid);
-            sc_max = std::max(sc_max, sk);
         }
         ctx->ns_iter = it_max;
         ctx->ns_resid = res_max;
         ctx->corr_resid = corr_max;
         ctx->ns_scale = sc_max;
-        periodic_mixed_energy(ctx->dcoef, nk, ctx->dombar, N, energy_out, s);
+        periodic_mixed_energy(energies, nk, ctx->dombar, N, energy_out, s);
         mean_rows(ctx->dlzw, nk, N, ctx->dtq, s);   // (1/nk) sum_q Re Tr (Q(q)^{1/2})_ii
         ctx->tq_valid = true;
         ctx->Zlast = ctx->dZ;
@@ -1406,8 +1495,10 @@ int run(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &out, bool
         ctx->Zlast = Z;
         ctx->zscale = 1.0 / ss;
     } else {
-        const MixProblem pr{ctx->dQ, ld, n, ctx->dP, ctx->dZ2, ctx->dY2, ctx->dZ, ctx->dtq};
-        rc = newton_schulz_mixed(ctx, s, pr, sc, lbound, ubound, energy_out, tc_spans, e_corr);
+        const MixProblem pr{ctx->dQ, ld, n, ctx->dP, ctx->dZ2, ctx->dY2, ctx->dZ, ctx->dtq, energy_out};
+        std::vector<MixItem> items(1);
+        items[0].sc = sc, items[0].lbound = lbound, items[0].ubound = ubound;
+        rc = newton_schulz_mixed(ctx, s, pr, items, tc_spans, e_corr);
         if (rc) return rc;
         ctx->tq_valid = true;
     }
