@@ -442,7 +442,8 @@ struct TcCfgW {
     static constexpr int STAGES = KIND == 0 ? 4 : 2;
     static constexpr int ELEM = KIND == 1 ? 2 : 4;
     static constexpr bool TF32 = KIND != 1;
-    static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 512;
+    static constexpr int EPI_BYTES = 8 * 32 * 16 * 4;   // a block of 32 x 16 results per epilogue warp
+    static constexpr int SMEM = STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 512;
 };
 __host__ __device__ constexpr uint32_t idescw(uint32_t fmt) {
     return (1u << 4) | (fmt << 7) | (fmt << 10) | (static_cast<uint32_t>(TNW >> 3) << 17) |
@@ -462,6 +463,195 @@ __device__ __forceinline__ void mmaw(uint32_t tmem, uint64_t a, uint64_t b, uint
             "l"(a), "l"(b), "r"(idescw(1)), "r"(acc));
 }
 
+// ---- epilogue of the wide form -----------------------------------------------------------
+// A warp takes its 32 rows of a 128 x 128 tile 16 columns at a time through 2 KB of shared memory, in a loop that is
+// not unrolled: the sums leave the registers a row per lane, come back four lanes to a row for D, the outputs
+// and the residual, and eight lanes to a column for the transposes and mirrored writes, so that every store
+// writes whole 32-byte sectors.  Unrolled over the 128 columns with a row per lane (tile_epilogue: 240 KB of code, each
+// instruction fetched for one use a tile), instruction fetches and 16-byte stores bound it.  A symmetric product
+// with D and split parts: order 896 72 -> 47 us, order 4608 BF16x3 366 -> 294 and TF32x3 648 -> 547 us (with
+// K = 64, that is little but the epilogue, 149 -> 92 us).  Element (r, c) of the 32 x 16 block lies at stage_at(r, c): the
+// swizzle of four-column groups keeps the row accesses free of bank conflicts and the column accesses two-way.
+constexpr int STAGE_F = 32 * 16;   // floats of a warp's block
+__device__ __forceinline__ int stage_at(int r, int c) {
+    const int s = (((r >> 1) ^ (r >> 3)) & 1) | (((r >> 2) & 1) << 1);
+    return r * 16 + (((c >> 2) ^ s) << 2) + (c & 3);
+}
+// Four values as the next product's operand parts: BF16 pairs (two words each), or TF32 hi and remainder.
+template <int KIND>
+__device__ __forceinline__ void split4(const float (&v)[4], uint32_t (&h)[4], uint32_t (&l)[4]) {
+    if (KIND == 2) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(h[j]) : "f"(v[j]));
+            asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(l[j]) : "f"(v[j] - __uint_as_float(h[j])));
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * q]), h1 = __float2bfloat16_rn(v[2 * q + 1]);
+            const __nv_bfloat16 l0 = __float2bfloat16_rn(v[2 * q] - __bfloat162float(h0));
+            const __nv_bfloat16 l1 = __float2bfloat16_rn(v[2 * q + 1] - __bfloat162float(h1));
+            h[q] = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
+            l[q] = static_cast<uint32_t>(__bfloat16_as_ushort(l0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(l1)) << 16);
+        }
+    }
+}
+// Four neighbouring elements of an operand part at element off (a multiple of four).
+template <int KIND>
+__device__ __forceinline__ void store_part4(void *base, long long off, const uint32_t (&w)[4]) {
+    if (KIND == 2) *reinterpret_cast<uint4 *>(static_cast<uint32_t *>(base) + off) = make_uint4(w[0], w[1], w[2], w[3]);
+    else *reinterpret_cast<uint2 *>(static_cast<unsigned short *>(base) + off) = make_uint2(w[0], w[1]);
+}
+// Four neighbouring results: FP32, FP64 sums and split parts.
+template <int KIND>
+__device__ __forceinline__ void store4(float *C, double *C64, void *H, void *L, long long off, const float (&v)[4]) {
+    if (C) *reinterpret_cast<float4 *>(C + off) = make_float4(v[0], v[1], v[2], v[3]);
+    if (H) {
+        uint32_t h[4], l[4];
+        split4<KIND>(v, h, l);
+        store_part4<KIND>(H, off, h);
+        store_part4<KIND>(L, off, l);
+    }
+    if (C64) {
+        double2 *p = reinterpret_cast<double2 *>(C64 + off);
+        double2 a = p[0], b = p[1];
+        a.x += static_cast<double>(v[0]);
+        a.y += static_cast<double>(v[1]);
+        b.x += static_cast<double>(v[2]);
+        b.y += static_cast<double>(v[3]);
+        p[0] = a;
+        p[1] = b;
+    }
+}
+template <int KIND>
+__device__ __forceinline__ void store1(float *C, double *C64, void *H, void *L, long long off, float v) {
+    if (C) C[off] = v;
+    if (C64) C64[off] += static_cast<double>(v);
+    if (H) {
+        const float x[4] = {v, 0.f, 0.f, 0.f};
+        uint32_t h[4], l[4];
+        split4<KIND>(x, h, l);
+        store_part<KIND>(H, off, h, 0);
+        store_part<KIND>(L, off, l, 0);
+    }
+}
+
+template <int KIND>
+__device__ __forceinline__ void wide_epilogue(const TcArgs &g, const float (&acc)[TN], float *stage, int tm, int tn, int q,
+                                              int item, int slot, int lane) {
+    const long long at = slot * g.sC;
+    const float alpha = g.nslots ? g.alphas[item] : g.alpha, beta = item_beta(g, item);
+    // Symmetric products (mode 2): upper tiles are mirrored into the lower half; diagonal tiles keep their
+    // upper triangle and mirror it, so the result is exactly symmetric whatever order the tensor
+    // cores summed in.
+    const bool diag = g.mode == 2 && tm == tn, into_c = g.mode == 2;
+    float *Tf = into_c ? g.C : g.CT;
+    double *T64 = into_c ? g.C64 : nullptr;
+    void *Th = into_c ? g.Ch : g.CTh, *Tl = into_c ? g.Cl : g.CTl;
+    const bool transposed = Tf || T64 || Th;
+    const int m0 = tm * TM + q * 32, n0 = tn * TN;
+    const int rr = lane >> 2, rc = (lane & 3) * 4;   // row phase: row 8 i + rr, columns rc ..
+    const int cr = (lane & 7) * 4, cc = lane >> 3;   // column phase: rows cr .., column 4 i + cc
+    const float *dp = beta != 0.f ? g.D + at + static_cast<long long>(m0 + rr) * g.ld + n0 + rc : nullptr;
+    float4 d[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) d[i] = dp ? *reinterpret_cast<const float4 *>(dp + 8LL * i * g.ld) : make_float4(0.f, 0.f, 0.f, 0.f);
+    // |delta - C|^2 as compensated FP32 sums (differences, squares and sums with their rounding errors: as good as
+    // FP64 to a few 2^-46), as the FP64 pipe would take 25 us a tile.
+    float rs = 0.f, rcomp = 0.f;
+#pragma unroll 1
+    for (int c16 = 0; c16 < TN / 16; ++c16) {
+#pragma unroll
+        for (int u = 0; u < TN / 16; ++u)
+            if (u == c16) {
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+                    *reinterpret_cast<float4 *>(stage + stage_at(lane, 4 * p)) =
+                        make_float4(alpha * acc[16 * u + 4 * p], alpha * acc[16 * u + 4 * p + 1], alpha * acc[16 * u + 4 * p + 2],
+                                    alpha * acc[16 * u + 4 * p + 3]);
+            }
+        __syncwarp();
+        const int n16 = n0 + 16 * c16;
+        const bool crossing = diag && n16 < m0 + 32 && n16 + 16 > m0;   // the diagonal passes through the block
+        // (every load of the block before the first store: the compiler keeps their order)
+        float v[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 x = *reinterpret_cast<const float4 *>(stage + stage_at(8 * i + rr, rc));
+            v[i][0] = x.x, v[i][1] = x.y, v[i][2] = x.z, v[i][3] = x.w;
+        }
+        if (beta != 0.f) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                v[i][0] += beta * d[i].x;
+                v[i][1] += beta * d[i].y;
+                v[i][2] += beta * d[i].z;
+                v[i][3] += beta * d[i].w;
+                if (transposed)
+                    *reinterpret_cast<float4 *>(stage + stage_at(8 * i + rr, rc)) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+            }
+            if (c16 + 1 < TN / 16) {   // the next columns of D
+                dp += 16;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) d[i] = *reinterpret_cast<const float4 *>(dp + 8LL * i * g.ld);
+            }
+        }
+        if (g.resid) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int m = m0 + 8 * i + rr, n = n16 + rc;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float one = m == n + j ? 1.f : 0.f, e = one - v[i][j], lost = (one - e) - v[i][j];
+                    const bool in = m < g.nvalid && n + j < g.nvalid;
+                    const float p = in ? e * e : 0.f, pe = in ? fmaf(e, e, -p) + 2.f * e * lost : 0.f;
+                    const float t = rs + p, b = t - rs;
+                    rcomp += ((rs - (t - b)) + (p - b)) + pe;
+                    rs = t;
+                }
+            }
+        }
+        const long long at_row = at + static_cast<long long>(m0 + rr) * g.ld + n16 + rc;
+        if (!crossing) {
+            if (!diag || n16 > m0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) store4<KIND>(g.C, g.C64, g.Ch, g.Cl, at_row + 8LL * i * g.ld, v[i]);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)   // (what is on or above the diagonal, from shared memory)
+                *reinterpret_cast<float4 *>(stage + stage_at(8 * i + rr, rc)) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+            __syncwarp();
+#pragma unroll 1
+            for (int c = 0; c < 16; ++c) {
+                const int m = m0 + lane, n = n16 + c;
+                if (n < m) continue;
+                const float x = stage[stage_at(lane, c)];
+                store1<KIND>(g.C, g.C64, g.Ch, g.Cl, at + static_cast<long long>(m) * g.ld + n, x);
+                if (n > m) store1<KIND>(g.C, g.C64, g.Ch, g.Cl, at + static_cast<long long>(n) * g.ld + m, x);
+            }
+        }
+        __syncwarp();
+        if (transposed && !crossing && (!diag || n16 > m0)) {   // rows n of the transpose, 32 entries m0 .. of each
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[i][j] = stage[stage_at(cr + j, 4 * i + cc)];
+            const long long at_col = at + static_cast<long long>(n16 + cc) * g.ld + m0 + cr;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) store4<KIND>(Tf, T64, Th, Tl, at_col + 4LL * i * g.ld, v[i]);
+            __syncwarp();
+        }
+    }
+    if (g.resid) {
+        double t = static_cast<double>(rs) + static_cast<double>(rcomp);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0 && t != 0.0) atomicAdd(g.resid + slot, t);
+    }
+}
+
 template <int KIND>
 __global__ void __launch_bounds__(384, 1)
     k_tc_gemm_w(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
@@ -470,7 +660,7 @@ __global__ void __launch_bounds__(384, 1)
     using Cfg = TcCfgW<KIND>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + Cfg::STAGES * Cfg::STAGE_BYTES);
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + Cfg::STAGES * Cfg::STAGE_BYTES + Cfg::EPI_BYTES);
     uint64_t *empty = full + Cfg::STAGES;
     uint64_t *cfull = empty + Cfg::STAGES;
     uint64_t *cfree = cfull + kWideBufs;
@@ -599,6 +789,7 @@ __global__ void __launch_bounds__(384, 1)
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(EPI_REGS));
         // ---- epilogue warps 0-7: lane quarter q, column half h; thread = row of the tile ----
         const int q = warp & 3, h = warp >> 2;
+        float *stage = reinterpret_cast<float *>(smem + Cfg::STAGES * Cfg::STAGE_BYTES) + warp * STAGE_F;
         bool ok = true;
         int cg = 0;
         for (int w = blockIdx.x; w < items && ok; w += gridDim.x, cg += nchunks) {
@@ -643,7 +834,7 @@ __global__ void __launch_bounds__(384, 1)
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(su32(&cfree[buf])) : "memory");
             }
-            if (ok && write) tile_epilogue<KIND>(g, acc, m, tm, tn, bz, slot, lane);
+            if (ok && write) wide_epilogue<KIND>(g, acc, stage, tm, tn, q, bz, slot, lane);
         }
     }
     __syncwarp();
@@ -1185,7 +1376,11 @@ cudaError_t tc_gemm(int kind, const TcOperands &op, const TcArgs &g, cudaStream_
         return cudaErrorInvalidValue;
     for (int k = 0; k < g.nslots; ++k)
         if (g.slot[k] < 0 || (g.betas[k] != 0.f && !g.D)) return cudaErrorInvalidValue;
-    const int form = tc_form();
+    // The wide form stores four elements at a time, also of the transposes and the FP64 sums.
+    const bool aligned = ((reinterpret_cast<uintptr_t>(g.CT) | reinterpret_cast<uintptr_t>(g.CTh) |
+                           reinterpret_cast<uintptr_t>(g.CTl) | reinterpret_cast<uintptr_t>(g.C64)) & 15) == 0 &&
+                         g.sC % 4 == 0;
+    const int form = tc_form() == 0 && !aligned ? 1 : tc_form();
     if (g.nslots && form != 0) {   // the other forms take the items one by one
         for (int k = 0; k < g.nslots; ++k) {
             const size_t es = kind == 1 ? 2 : 4, rows = static_cast<size_t>(g.slot[k]) * g.M;
