@@ -283,10 +283,11 @@ void chain_screen(const AtomBufs &b, const MbdGradOut &o, double *h, double *g_a
 // -1/3 sum dM_pq (V X^T)_pq to dE/d alpha0, dE/d omega, dE/d R_vdW (g_a0, g_om, g_rv)
 // and dE/dR (gR, accumulated).  With work32 (2 nf1 (xstride + N) floats) the per-pair
 // arithmetic runs in single precision on FP32 copies of X, V, sigma(iu) and alpha(iu) (sums
-// FP64), for the reduced-precision modes; with work32 = NULL, in FP64.
+// FP64), for the reduced-precision modes; with work32 = NULL, in FP64 through work: at most
+// 128 N ceil(N / 32) doubles, 80 for up to 16 frequencies (a matrix of order 3 N padded to 128 holds them).
 void scs_grad_pass(const AtomBufs &b, double beta, double a, const double *X, const double *V,
                    long long xstride, double *g_a0, double *g_om, double *g_rv, double *gR, float *work32,
-                   cudaStream_t s);
+                   double *work, cudaStream_t s);
 
 // MBD-NL (Sec. 2.7, Eqs. mbd-nl-scaling, mbd-nl-rvdw): the oscillators from the inputs
 // alpha0_ref, C6_ref, ra (in rref) and rw (in ratio), written to abar0, ombar, rbar, c6bar,

@@ -354,24 +354,11 @@ __global__ void k_chain(AtomBufs b, MbdGradOut o, double *h, double *g_a0, doubl
 //   dE/d alpha_i(u) += -1/3 <Ws, dB/d alpha_i>,  dE/dR_vdW,i += -1/3 <Ws, dB/dS>,
 //   dE/dR_i += +1/3 <Ws, dB/dr>  (r = R_j - R_i),  B = (1 - f) T^GG,
 // plus the diagonal block: dE/d alpha_i(u) += -1/3 sum_x (V X^T)_{ix,ix} (-1/alpha_i^2).
-// The per-pair arithmetic runs in T (double, or float in the reduced-precision modes);
-// the per-thread and block sums are FP64.
+// The per-pair arithmetic runs in float, for the reduced-precision modes; the per-thread and block sums
+// are FP64.  X, V ([nf1][xstride]), sig and al ([nf1][N], sigma_i(iu) and alpha_i(iu)) are FP32 copies.
 // Dynamic shared memory: nf1 * 128 doubles of per-thread accumulators.
-template <typename T> struct PairMath;
-template <> struct PairMath<double> {
-    static __device__ __forceinline__ Fermi fermi(double r, double S, double b, double a) { return pairs::fermi(r, S, b, a); }
-    static __device__ __forceinline__ Radial radial(double r, double s) { return pairs::tgg_radial(r, s); }
-};
-template <> struct PairMath<float> {
-    static __device__ __forceinline__ FermiF fermi(float r, float S, float b, float a) { return pairs::fermi_f(r, S, b, a); }
-    static __device__ __forceinline__ RadialF radial(float r, float s) { return pairs::tgg_radial_f(r, s); }
-};
-
-// X, V ([nf1][xstride]), sig and al ([nf1][N], sigma_i(iu) and alpha_i(iu)) are read in T:
-// the FP64 arrays, or FP32 copies of them in the reduced-precision modes.
-template <typename T>
-__global__ void __launch_bounds__(128) k_scs_grad(AtomBufs b, double beta, double a, const T *X, const T *V,
-                                                  const T *sig, const T *al, long long xstride, double *g_a0,
+__global__ void __launch_bounds__(128) k_scs_grad(AtomBufs b, double beta, double a, const float *X, const float *V,
+                                                  const float *sig, const float *al, long long xstride, double *g_a0,
                                                   double *g_om, double *g_rv, double *gR) {
     extern __shared__ double gal_s[];   // [nf1][128]
     const int i = blockIdx.x, t = threadIdx.x;
@@ -380,44 +367,44 @@ __global__ void __launch_bounds__(128) k_scs_grad(AtomBufs b, double beta, doubl
     double acc[4] = {0, 0, 0, 0};   // g_rv, gR x3
     for (int j = t; j < b.N; j += 128) {
         if (j == i) continue;
-        const T r[3] = {static_cast<T>(b.R[3 * j] - Ri[0]), static_cast<T>(b.R[3 * j + 1] - Ri[1]),
-                        static_cast<T>(b.R[3 * j + 2] - Ri[2])};
-        const T rho = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]), ir = T(1) / rho;
-        const auto f = PairMath<T>::fermi(rho, static_cast<T>(b.rv[i] + b.rv[j]), static_cast<T>(beta), static_cast<T>(a));
-        const T sr = T(1) - f.f;
+        const float r[3] = {static_cast<float>(b.R[3 * j] - Ri[0]), static_cast<float>(b.R[3 * j + 1] - Ri[1]),
+                        static_cast<float>(b.R[3 * j + 2] - Ri[2])};
+        const float rho = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]), ir = 1.0f / rho;
+        const auto f = fermi_f(rho, static_cast<float>(b.rv[i] + b.rv[j]), static_cast<float>(beta), static_cast<float>(a));
+        const float sr = 1.0f - f.f;
         // Far pairs whose damping has rounded to f = 1 (1 - f = 0 and both derivatives 0)
         // contribute exact zeros at every frequency: beyond ~3.8 beta (R_i + R_j) in FP32,
         // ~7.1 in FP64.
-        if (sr == T(0) && f.df_drho == T(0) && f.df_dS == T(0)) continue;
-        T pacc[4] = {0, 0, 0, 0};
+        if (sr == 0.0f && f.df_drho == 0.0f && f.df_dS == 0.0f) continue;
+        float pacc[4] = {0, 0, 0, 0};
         for (int k = 0; k < b.nf1; ++k) {
-            const T *Vk = V + k * xstride, *Xk = X + k * xstride;
-            T Ws[9];
+            const float *Vk = V + k * xstride, *Xk = X + k * xstride;
+            float Ws[9];
             for (int x = 0; x < 3; ++x)
                 for (int y = 0; y < 3; ++y) {
-                    T w = 0;
+                    float w = 0;
                     for (int c = 0; c < 3; ++c)
                         w += Vk[9LL * i + 3 * x + c] * Xk[9LL * j + 3 * y + c] + Xk[9LL * i + 3 * x + c] * Vk[9LL * j + 3 * y + c];
                     Ws[3 * x + y] = w;
                 }
-            const T tr = Ws[0] + Ws[4] + Ws[8];
-            T Wr[3], Wtr[3];
+            const float tr = Ws[0] + Ws[4] + Ws[8];
+            float Wr[3], Wtr[3];
             for (int x = 0; x < 3; ++x) {
                 Wr[x] = Ws[3 * x] * r[0] + Ws[3 * x + 1] * r[1] + Ws[3 * x + 2] * r[2];
                 Wtr[x] = Ws[x] * r[0] + Ws[3 + x] * r[1] + Ws[6 + x] * r[2];
             }
-            const T rWr = r[0] * Wr[0] + r[1] * Wr[1] + r[2] * Wr[2];
-            const T si = sig[k * b.N + i], sj = sig[k * b.N + j];
-            const T s = sqrt(si * si + sj * sj);
-            const auto q = PairMath<T>::radial(rho, s);
-            const T WT = q.P * tr + q.W * rWr;            // <Ws, T^GG>
-            const T WTs = q.dPs * tr + q.dWs * rWr;       // <Ws, dT^GG/ds>
+            const float rWr = r[0] * Wr[0] + r[1] * Wr[1] + r[2] * Wr[2];
+            const float si = sig[k * b.N + i], sj = sig[k * b.N + j];
+            const float s = sqrt(si * si + sj * sj);
+            const auto q = tgg_radial_f(rho, s);
+            const float WT = q.P * tr + q.W * rWr;            // <Ws, T^GG>
+            const float WTs = q.dPs * tr + q.dWs * rWr;       // <Ws, dT^GG/ds>
             // ds/d alpha_i = (sigma_i / s) * sigma_i / (3 alpha_i)
-            const T dsda = si * si / (T(3) * s * al[k * b.N + i]);
+            const float dsda = si * si / (3.0f * s * al[k * b.N + i]);
             gal_s[k * 128 + t] += -1.0 / 3.0 * static_cast<double>(sr * WTs * dsda);
             pacc[0] += -f.df_dS * WT;
             for (int c = 0; c < 3; ++c) {
-                const T WdT = (q.dP * tr + q.dW * rWr) * r[c] * ir + q.W * (Wr[c] + Wtr[c]);
+                const float WdT = (q.dP * tr + q.dW * rWr) * r[c] * ir + q.W * (Wr[c] + Wtr[c]);
                 pacc[1 + c] += sr * WdT - f.df_drho * r[c] * ir * WT;
             }
         }
@@ -432,7 +419,7 @@ __global__ void __launch_bounds__(128) k_scs_grad(AtomBufs b, double beta, doubl
         const int k = t;
         double sacc = 0.0;
         for (int e = 0; e < 128; ++e) sacc += gal_s[k * 128 + e];
-        const T *Vk = V + k * xstride, *Xk = X + k * xstride;
+        const float *Vk = V + k * xstride, *Xk = X + k * xstride;
         double wd = 0.0;
         for (int e = 0; e < 9; ++e) wd += static_cast<double>(Vk[9LL * i + e]) * static_cast<double>(Xk[9LL * i + e]);
         const double alk = b.al_u[k * b.N + i];
@@ -456,6 +443,171 @@ __global__ void __launch_bounds__(128) k_scs_grad(AtomBufs b, double beta, doubl
         gR[3 * i + 1] += acc[2];
         gR[3 * i + 2] += acc[3];
     }
+}
+
+// The SCS adjoint pass in FP64: every unordered pair once, for tiles of 32 x 32 atoms (I <= J, blockIdx.x) and KF
+// frequencies (blockIdx.y).  Lane = atom j, a warp takes four atoms i one after another; sums over j by shuffles,
+// sums over i in registers and then over the warps, into part[tile of the partner][component][atom]
+// (components: dE/d alpha(u_k), then for each group of frequencies g_rv and gR), each written once.
+// The FP64 pipe bounds it (two multiply-adds a cycle and SM): with one row of ordered pairs a CTA, and a division wherever the
+// formulas have one, it took 8.76 ms for 1000 atoms, 0.64 for 251 and 0.18 for 32; so 3.71, 0.33 and 0.10.
+template <int KF>
+__global__ void __launch_bounds__(256) k_scs_grad_tiles(AtomBufs b, double beta, double a, const double *X, const double *V,
+                                                        long long xstride, int ntile, int comps, double *part) {
+    constexpr int C = KF + 4;
+    __shared__ double row[C][32], col[8][C][32], ca[2][KF][32];   // ca: sigma^2 / (3 alpha) of the tile's atoms
+    int I = 0, J = blockIdx.x;
+    while (J >= ntile - I) J -= ntile - I, ++I;
+    J += I;
+    const int k0 = blockIdx.y * KF, nk = min(KF, b.nf1 - k0), lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int j = J * 32 + lane;
+    for (int e = threadIdx.x; e < 2 * KF * 32; e += 256) {
+        const int side = e / (KF * 32), kk = e / 32 % KF, at = (side ? J : I) * 32 + e % 32;
+        if (kk >= nk || at >= b.N) continue;
+        const double sg = b.sig_u[(k0 + kk) * b.N + at];
+        ca[side][kk][e % 32] = sg * sg / (3.0 * b.al_u[(k0 + kk) * b.N + at]);
+    }
+    __syncthreads();
+    double cs[C];   // sums over this warp's atoms i, for atom j
+#pragma unroll
+    for (int c = 0; c < C; ++c) cs[c] = 0.0;
+    double Rj[3] = {0, 0, 0}, rvj = 0.0;
+    if (j < b.N) {
+        for (int e = 0; e < 3; ++e) Rj[e] = b.R[3 * j + e];
+        rvj = b.rv[j];
+    }
+#pragma unroll 1
+    for (int m = 0; m < 4; ++m) {
+        const int il = 4 * w + m, i = I * 32 + il;
+        double rs[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) rs[c] = 0.0;
+        bool active = i < b.N && j < b.N && i < j;
+        double r[3] = {1, 0, 0}, rho = 1.0, ir = 1.0, sr = 0.0;
+        Fermi f{1.0, 0.0, 0.0};
+        if (active) {
+            for (int e = 0; e < 3; ++e) r[e] = Rj[e] - b.R[3 * i + e];
+            rho = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
+            ir = 1.0 / rho;
+            f = fermi(rho, b.rv[i] + rvj, beta, a);
+            sr = 1.0 - f.f;
+            // far pairs whose damping has rounded to f = 1 contribute exact zeros
+            active = !(sr == 0.0 && f.df_drho == 0.0 && f.df_dS == 0.0);
+        }
+        if (__any_sync(0xffffffffu, active)) {
+            if (active) {
+                const double ir2 = ir * ir, ir3 = ir2 * ir, ir5 = ir3 * ir2;
+#pragma unroll
+                for (int kk = 0; kk < KF; ++kk) {
+                    if (kk >= nk) break;
+                    const int k = k0 + kk;
+                    const double *Vi = V + k * xstride + 9LL * i, *Xi = X + k * xstride + 9LL * i;
+                    const double *Vj = V + k * xstride + 9LL * j, *Xj = X + k * xstride + 9LL * j;
+                    double Ws[9];
+#pragma unroll
+                    for (int x = 0; x < 3; ++x)
+#pragma unroll
+                        for (int y = 0; y < 3; ++y) {
+                            double t = 0.0;
+#pragma unroll
+                            for (int c = 0; c < 3; ++c) t += Vi[3 * x + c] * Xj[3 * y + c] + Xi[3 * x + c] * Vj[3 * y + c];
+                            Ws[3 * x + y] = t;
+                        }
+                    const double tr = Ws[0] + Ws[4] + Ws[8];
+                    double Wb[3];   // (Ws + Ws^T) r
+                    Wb[0] = 2.0 * Ws[0] * r[0] + (Ws[1] + Ws[3]) * r[1] + (Ws[2] + Ws[6]) * r[2];
+                    Wb[1] = (Ws[1] + Ws[3]) * r[0] + 2.0 * Ws[4] * r[1] + (Ws[5] + Ws[7]) * r[2];
+                    Wb[2] = (Ws[2] + Ws[6]) * r[0] + (Ws[5] + Ws[7]) * r[1] + 2.0 * Ws[8] * r[2];
+                    const double rWr = 0.5 * (r[0] * Wb[0] + r[1] * Wb[1] + r[2] * Wb[2]);
+                    const double si = b.sig_u[k * b.N + i], sj = b.sig_u[k * b.N + j];
+                    // radial parts of T^GG as tgg_radial has them, with 1/s in place of its divisions
+                    const double is = rsqrt(si * si + sj * sj), z = rho * is;
+                    double P = ir3, W = -3.0 * ir5, dP = -3.0 * ir3 * ir, dW = 15.0 * ir5 * ir, WTs = 0.0;
+                    if (!(z > kGaussFar)) {
+                        const double z2 = z * z, th = kTwoOverSqrtPi * z * exp(-z2);
+                        const double F1 = erf(z) - th, t = 2.0 * z * th * is;
+                        P = F1 * ir3;
+                        W = (2.0 * z2 * th - 3.0 * F1) * ir5;
+                        dP = t * ir3 - 3.0 * P * ir;
+                        dW = -2.0 * z2 * t * ir5 - 5.0 * W * ir;
+                        WTs = z * t * (2.0 * z2 * ir5 * rWr - ir3 * tr);   // <Ws, dT^GG/ds>
+                    }
+                    const double WT = P * tr + W * rWr, g = -1.0 / 3.0 * sr * WTs * is;
+                    rs[kk] = g * ca[0][kk][il];
+                    cs[kk] += g * ca[1][kk][lane];
+                    rs[KF] += f.df_dS * WT;
+                    const double rad = (sr * (dP * tr + dW * rWr) - f.df_drho * WT) * ir, srW = sr * W;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) rs[KF + 1 + c] += rad * r[c] + srW * Wb[c];
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) rs[KF + c] *= 1.0 / 3.0;
+                cs[KF] += rs[KF];
+#pragma unroll
+                for (int c = 1; c < 4; ++c) cs[KF + c] -= rs[KF + c];
+            }
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < C; ++c) rs[c] = warp_sum(rs[c]);
+        }
+        if (lane == 0)
+#pragma unroll
+            for (int c = 0; c < C; ++c) row[c][il] = rs[c];
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) col[w][c][lane] = cs[c];
+    __syncthreads();
+    for (int e = threadIdx.x; e < C * 32; e += 256) {
+        const int c = e >> 5, at = e & 31;
+        if (c < KF && c >= nk) continue;
+        const int comp = c < KF ? k0 + c : b.nf1 + 4 * static_cast<int>(blockIdx.y) + c - KF;
+        double v = 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v += col[u][c][at];
+        const double rw = row[c][at];
+        const int ai = I * 32 + at, aj = J * 32 + at;
+        if (I == J) {
+            if (ai < b.N) part[(static_cast<long long>(I) * comps + comp) * b.N + ai] = rw + v;
+        } else {
+            if (ai < b.N) part[(static_cast<long long>(J) * comps + comp) * b.N + ai] = rw;
+            if (aj < b.N) part[(static_cast<long long>(I) * comps + comp) * b.N + aj] = v;
+        }
+    }
+}
+
+// Sums of part over the tiles, the diagonal blocks, and the chain to alpha0 and omega; 32 atoms a CTA.
+__global__ void __launch_bounds__(256) k_scs_grad_sum(AtomBufs b, const double *X, const double *V, long long xstride,
+                                                      int ntile, int comps, const double *part, double *g_a0,
+                                                      double *g_om, double *g_rv, double *gR) {
+    extern __shared__ double sum[];   // [comps][32], then dE/d omega's terms [nf1][32]
+    const int lane = threadIdx.x & 31, i = blockIdx.x * 32 + lane;
+    if (i < b.N)
+        for (int c = threadIdx.x >> 5; c < comps; c += 8) {
+            double v = 0.0;
+            for (int t = 0; t < ntile; ++t) v += part[(static_cast<long long>(t) * comps + c) * b.N + i];
+            if (c < b.nf1) {
+                const double *Vk = V + c * xstride + 9LL * i, *Xk = X + c * xstride + 9LL * i;
+                double wd = 0.0;
+                for (int e = 0; e < 9; ++e) wd += Vk[e] * Xk[e];
+                const double alk = b.al_u[c * b.N + i], om = b.om[i], u = b.u[c], q = 1.0 + u * u / (om * om);
+                v = (v + 1.0 / 3.0 * wd / (alk * alk)) / q;   // its term of dE/d alpha0
+                sum[(comps + c) * 32 + lane] = v * b.a0[i] * 2.0 * u * u / (om * om * om * q);
+            }
+            sum[c * 32 + lane] = v;
+        }
+    __syncthreads();
+    if (threadIdx.x >= 32 || i >= b.N) return;
+    double ga0 = 0.0, gom = 0.0;
+    for (int k = 0; k < b.nf1; ++k) {
+        ga0 += sum[k * 32 + lane];
+        gom += sum[(comps + k) * 32 + lane];
+    }
+    double x[4] = {0, 0, 0, 0};
+    for (int c = b.nf1; c < comps; ++c) x[(c - b.nf1) & 3] += sum[c * 32 + lane];
+    g_a0[i] += ga0;
+    g_om[i] += gom;
+    g_rv[i] += x[0];
+    for (int c = 0; c < 3; ++c) gR[3 * i + c] += x[1 + c];
 }
 
 // FP32 copies of X, V ([nf1][xstride] each) and of sigma(iu), alpha(iu) ([nf1][N] each),
@@ -656,19 +808,28 @@ void chain_screen(const AtomBufs &b, const MbdGradOut &o, double *h, double *g_a
 
 void scs_grad_pass(const AtomBufs &b, double beta, double a, const double *X, const double *V,
                    long long xstride, double *g_a0, double *g_om, double *g_rv, double *gR, float *work32,
-                   cudaStream_t s) {
-    const size_t smem = sizeof(double) * b.nf1 * 128;
+                   double *work, cudaStream_t s) {
     if (work32) {
+        const size_t smem = sizeof(double) * b.nf1 * 128;
         const long long nx = xstride * b.nf1, na = static_cast<long long>(b.nf1) * b.N;
         float *X32 = work32, *V32 = work32 + nx, *sig32 = work32 + 2 * nx, *al32 = sig32 + na;
         count_launches(2);
         k_scs_grad_inputs_f32<<<cdiv(2 * nx + 2 * na, 256), 256, 0, s>>>(X, V, b.sig_u, b.al_u, nx, na, work32);
-        k_scs_grad<float><<<b.N, 128, smem, s>>>(b, beta, a, X32, V32, sig32, al32, xstride, g_a0, g_om, g_rv, gR);
-    } else {
-        count_launches(1);
-        k_scs_grad<double><<<b.N, 128, smem, s>>>(b, beta, a, X, V, b.sig_u, b.al_u, xstride, g_a0, g_om, g_rv,
-                                                 gR);
+        k_scs_grad<<<b.N, 128, smem, s>>>(b, beta, a, X32, V32, sig32, al32, xstride, g_a0, g_om, g_rv, gR);
+        return;
     }
+    // Frequencies a CTA: four where the tiles alone nearly fill the chip twice with four groups of them, else fewer (a group
+    // repeats the pairs' damping, a quarter of a frequency's work: four at 1000 atoms, two at 251, one at 32).  Four
+    // for grids of more than 16 frequencies, which bounds the workspace.
+    const int ntile = cdiv(b.N, 32), tiles = ntile * (ntile + 1) / 2;
+    const int kf = b.nf1 > 16 || tiles >= 64 ? 4 : (tiles >= 24 ? 2 : 1);
+    const int groups = cdiv(b.nf1, kf), comps = b.nf1 + 4 * groups;
+    const dim3 grid(tiles, groups);
+    count_launches(2);
+    if (kf == 4) k_scs_grad_tiles<4><<<grid, 256, 0, s>>>(b, beta, a, X, V, xstride, ntile, comps, work);
+    else if (kf == 2) k_scs_grad_tiles<2><<<grid, 256, 0, s>>>(b, beta, a, X, V, xstride, ntile, comps, work);
+    else k_scs_grad_tiles<1><<<grid, 256, 0, s>>>(b, beta, a, X, V, xstride, ntile, comps, work);
+    k_scs_grad_sum<<<ntile, 256, sizeof(double) * (comps + b.nf1) * 32, s>>>(b, X, V, xstride, ntile, comps, work, g_a0, g_om, g_rv, gR);
 }
 
 void nl_params(const AtomBufs &b, int *status, cudaStream_t s) {
