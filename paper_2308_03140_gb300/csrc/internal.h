@@ -390,9 +390,17 @@ void energy_trace_periodic(const double *Y, long long ld, int n, const PeriodicB
 // Z), or NULL to take it from Z.
 // f32_recip: the reciprocal-space sum in FP32 (chunk sums added in FP64), for the mixed
 // modes, whose Z ~ Q^{-1/2} is accurate to far less than FP32 rounding.
-void periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, const double *Z,
-                       long long ld, double zscale, const MbdGradOut &o, double *work, double *gA, cudaStream_t s,
-                       const double *tq = nullptr, bool f32_recip = false);
+// products (or null): scratch of grad_products_bytes, for the sums as products on the tensor cores (k_qgrad.cu), whose
+// timeouts set ST_TC_TIMEOUT in *status.
+cudaError_t periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, const double *Z,
+                              long long ld, double zscale, const MbdGradOut &o, double *work, double *gA, cudaStream_t s,
+                              const double *tq, bool f32_recip, void *products, int *status);
+// Its real-space and, with recip, reciprocal sums through products (0 bytes: not for this cell), added to g_c, g_rbar,
+// gR and gA.
+size_t grad_products_bytes(int N, const CellGeom &c, int nk, int maxG);
+cudaError_t grad_products(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, const double *Z, long long ld,
+                          double zscale, double *g_c, double *g_rbar, double *gR, double *gA, bool recip, void *work,
+                          int *status, cudaStream_t s);
 // out[i] = (1/rows) sum_r x[r][i] for a rows x N array (compensated).
 void mean_rows(const double *x, int rows, int N, double *out, cudaStream_t s);
 // SCS adjoint pair pass over lattice images (as scs_grad_pass), with the lattice part

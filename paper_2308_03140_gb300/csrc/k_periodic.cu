@@ -470,11 +470,12 @@ __global__ void __launch_bounds__(256) k_energy_periodic(const double *Y, long l
 // gR[i] -= c_i c_j zx, gA += c_i c_j zA (c_i = omega_bar_i sqrt(abar0_i)).
 // Real-space sums in FP64; the reciprocal sum in R (double, or float for the mixed modes,
 // whose Z carries errors far above FP32 rounding), each chunk of kGC vectors summed in R and
-// added into FP64 totals.
+// added into FP64 totals.  images: with the real-space part and the self term (k_qgrad.cu has them otherwise, and in
+// FP64 the reciprocal part too).
 template <typename R>
 __global__ void __launch_bounds__(256) k_mbd_grad_periodic(AtomBufs b, PeriodicBufs p, double beta, double a,
                                                            const double *Z, long long ld, double zscale, int ntile,
-                                                           double *g_c, double *g_rbar, double *gR, double *gA) {
+                                                           bool images, double *g_c, double *g_rbar, double *gR, double *gA) {
     const int kq = blockIdx.y;
     int I, J;
     tile_pair(blockIdx.x, ntile, I, J);
@@ -501,6 +502,7 @@ __global__ void __launch_bounds__(256) k_mbd_grad_periodic(AtomBufs b, PeriodicB
         const double S = b.rbar[i] + b.rbar[j];
         int lo[3], hi[3];
         image_box(c, x, lo, hi);
+        if (!images) hi[0] = lo[0] - 1;
         for (int n0 = lo[0]; n0 <= hi[0]; ++n0)
             for (int n1 = lo[1]; n1 <= hi[1]; ++n1)
                 for (int n2 = lo[2]; n2 <= hi[2]; ++n2) {
@@ -590,7 +592,7 @@ __global__ void __launch_bounds__(256) k_mbd_grad_periodic(AtomBufs b, PeriodicB
     }
     if (!valid) return;
     zT += su;
-    if (i == j) zT -= 4.0 * c.gamma * c.gamma * c.gamma / (3.0 * sqrt(kPi)) * (zr[0] + zr[1] + zr[2]);   // self term
+    if (i == j && images) zT -= 4.0 * c.gamma * c.gamma * c.gamma / (3.0 * sqrt(kPi)) * (zr[0] + zr[1] + zr[2]);   // self term
     for (int d = 0; d < 3; ++d) zx[d] -= M1[d];
     for (int k = 0; k < 3; ++k)
         for (int d = 0; d < 3; ++d) {
@@ -935,9 +937,9 @@ void mean_rows(const double *x, int rows, int N, double *out, cudaStream_t s) {
     k_mean_rows<<<cdiv(N, 128), 128, 0, s>>>(x, rows, N, out);
 }
 
-void periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, const double *Z,
-                       long long ld, double zscale, const MbdGradOut &o, double *work, double *gA, cudaStream_t s,
-                       const double *tq, bool f32_recip) {
+cudaError_t periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, const double *Z,
+                              long long ld, double zscale, const MbdGradOut &o, double *work, double *gA, cudaStream_t s,
+                              const double *tq, bool f32_recip, void *products, int *status) {
     double *g_c = work;
     cudaMemsetAsync(g_c, 0, sizeof(double) * b.N, s);
     cudaMemsetAsync(o.g_rbar, 0, sizeof(double) * b.N, s);
@@ -946,11 +948,14 @@ void periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double beta, do
     const int ntile = cdiv(b.N, kQT);
     count_launches(2);
     const dim3 grid(ntile * (ntile + 1) / 2, p.nk);
+    cudaError_t e = cudaSuccess;
+    if (products) e = grad_products(b, p, beta, a, Z, ld, zscale, g_c, o.g_rbar, o.gR, gA, !f32_recip, products, status, s);
     if (f32_recip)
-        k_mbd_grad_periodic<float><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, g_c, o.g_rbar, o.gR, gA);
-    else
-        k_mbd_grad_periodic<double><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, g_c, o.g_rbar, o.gR, gA);
+        k_mbd_grad_periodic<float><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, !products, g_c, o.g_rbar, o.gR, gA);
+    else if (!products)
+        k_mbd_grad_periodic<double><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, true, g_c, o.g_rbar, o.gR, gA);
     k_mbd_grad_periodic_finalize<<<cdiv(b.N, 128), 128, 0, s>>>(b, Z, ld, p.nk, p.kw, zscale / p.nkt, g_c, o, tq);
+    return e;
 }
 
 long long scs_grad_periodic_words(int N, int nf1) {

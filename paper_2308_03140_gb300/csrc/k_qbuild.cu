@@ -12,6 +12,7 @@
 // Together 10.2 ms for that cell.
 #include <algorithm>
 
+#include "cell_pairs.cuh"
 #include "internal.h"
 #include "pair_math.cuh"
 
@@ -19,42 +20,7 @@ namespace mbdgb {
 namespace {
 
 using namespace pairs;
-
-constexpr int kQT = 16;   // atom tile edge: 16 x 16 threads, tile pairs I <= J
-
-__device__ __forceinline__ void tile_pair(int t, int ntile, int &I, int &J) {
-    I = 0;
-    while (t >= ntile - I) { t -= ntile - I; ++I; }
-    J = I + t;
-}
-
-// First image index of each direction for separation x: r = x + n A within the cutoff needs
-// n_c in [-L_c - f_c, L_c - f_c] (f = fractional x, L_c = rc |b_c| / 2 pi).
-__device__ __forceinline__ void first_image(const CellGeom &c, const double *x, int *lo, int *hi) {
-    for (int k = 0; k < 3; ++k) {
-        const double bn = sqrt(c.B[3 * k] * c.B[3 * k] + c.B[3 * k + 1] * c.B[3 * k + 1] + c.B[3 * k + 2] * c.B[3 * k + 2]);
-        const double L = c.rc * bn / (2.0 * kPi) + 1e-9, f = x[0] * c.Ainv[k] + x[1] * c.Ainv[3 + k] + x[2] * c.Ainv[6 + k];
-        lo[k] = static_cast<int>(ceil(-L - f));
-        hi[k] = static_cast<int>(floor(L - f));
-    }
-}
-
-struct Pair {
-    int i, j;
-    bool valid;
-    double x[3];
-};
-__device__ __forceinline__ Pair pair_of(const AtomBufs &b, int ntile) {
-    int I, J;
-    tile_pair(blockIdx.x, ntile, I, J);
-    const int ty = threadIdx.x / kQT, tx = threadIdx.x % kQT;
-    Pair p;
-    p.i = I * kQT + ty;
-    p.j = J * kQT + tx;
-    p.valid = p.i < b.N && p.j < b.N && (I < J || ty <= tx);
-    for (int e = 0; e < 3; ++e) p.x[e] = p.valid ? b.R[3 * p.j + e] - b.R[3 * p.i + e] : 0.0;
-    return p;
-}
+using namespace cellpairs;
 
 // F of one pair at blockIdx.y's image offset (o0, o1, o2) from its first image: T^erfc - (1 - g) T as
 // xx, yy, zz, xy, xz, yz, zero beyond the cutoff; F[(offset 6 + e)][pair].

@@ -428,6 +428,11 @@ int mixed_group(int nk, long long lde, int precision) {
     return static_cast<int>(std::max<long long>(1, std::min<long long>({want, nk, kTcSlots})));
 }
 
+// Scratch of a cell's products, the build of Q(q) and the gradient.
+size_t cell_products_bytes(int N, const CellGeom &c, int nk, int maxG) {
+    return std::max(build_q_products_bytes(N, c, nk, maxG), grad_products_bytes(N, c, nk, maxG));
+}
+
 // Carves the workspace out of one allocation (256-byte aligned pieces).
 int allocate(mbd_ctx *ctx, bool groups = true) {
     const long long ld = ctx->ld, N = ctx->N, nf1 = ctx->nf1, nb = ctx->nb;
@@ -491,7 +496,7 @@ int allocate(mbd_ctx *ctx, bool groups = true) {
     bytes += scs32;
     // Scratch of the tensor-core products, taken only where it fits: FP64 products and factors (and the
     // transpose of P), and the build of Q(q), which can share theirs.
-    const size_t q_work = ctx->periodic ? al(build_q_products_bytes(ctx->N, ctx->cell, static_cast<int>(nk), ctx->maxG)) : 0;
+    const size_t q_work = ctx->periodic ? al(cell_products_bytes(ctx->N, ctx->cell, static_cast<int>(nk), ctx->maxG)) : 0;
     const size_t crt_part =
         fp64_path(prec) ? std::max({al(cholesky_crt_bytes(ld, static_cast<int>(nf1))),
                                     al(ctx->periodic ? crt_cell_bytes(ctx->n, static_cast<int>(nk)) : crt_ns_bytes(ctx->n)), q_work})
@@ -994,21 +999,27 @@ int newton_schulz_mixed(mbd_ctx *ctx, cudaStream_t s, const MixProblem &pr, std:
 // Gradient passes of a periodic system: the MBD pair pass over Bloch vectors (atoms,
 // screened parameters, lattice), the chain through the screened parameters, the adjoint
 // solves on the Gamma-point factors and the SCS pass over lattice images.
-void backward_periodic(mbd_ctx *ctx, cudaStream_t s, const AtomBufs &b, const double *grad_energy,
-                       double *grad_coords, double *grad_params) {
+int backward_periodic(mbd_ctx *ctx, cudaStream_t s, const AtomBufs &b, const double *grad_energy,
+                      double *grad_coords, double *grad_params) {
     const long long ld = ctx->ld, mat = ld * ld, xs = 3 * ld;
     const double beta = ctx->opt.beta, a = ctx->opt.a;
     const PeriodicBufs pb = periodic_bufs(ctx);
     MbdGradOut go{ctx->dgomb, ctx->dgab0, ctx->dgrb, ctx->dgR};
     const bool mixed = ctx->opt.precision != MBD_PREC_FP64 && ctx->opt.precision != MBD_PREC_FP64_SPLIT;
-    periodic_mbd_grad(b, pb, beta, a, ctx->Zlast, ld, ctx->zscale, go, ctx->dgc, ctx->dgA, s,
-                      ctx->tq_valid ? ctx->dtq : nullptr, mixed);
+    const size_t bytes = grad_products_bytes(ctx->N, ctx->cell, ctx->nk, ctx->maxG);
+    char *products = ctx->qwork && bytes && bytes <= ctx->qwork_bytes ? ctx->qwork : nullptr;
+    if (products) MBD_CUDA(cudaMemsetAsync(ctx->dstatus, 0, sizeof(int), s), "gradient");
+    MBD_CUDA(periodic_mbd_grad(b, pb, beta, a, ctx->Zlast, ld, ctx->zscale, go, ctx->dgc, ctx->dgA, s,
+                               ctx->tq_valid ? ctx->dtq : nullptr, mixed, products, ctx->dstatus), "gradient");
     if (ctx->opt.scs_mode == MBD_SCS_NL) {   // MBD-NL: no screening to differentiate
         if (grad_params) nl_chain(b, go, grad_energy, grad_params, s);
         if (grad_coords) scale_copy(ctx->dgR, 3 * ctx->N, grad_energy, grad_coords, s);
         scale_copy(ctx->dgA, 9, grad_energy, ctx->dgAout, s);
+        if (products) {   // its tensor-core waits are bounded: check them
+            if (const int rc = read_status(ctx, s, "gradient")) return rc;
+        }
         ctx->have_lattice_grad = true;
-        return;
+        return MBD_OK;
     }
     chain_screen(b, go, ctx->dh, ctx->dga0, ctx->dgrv, ctx->dV, ld, xs, s);
     cudaMemsetAsync(ctx->dgom, 0, sizeof(double) * ctx->N, s);
@@ -1018,7 +1029,11 @@ void backward_periodic(mbd_ctx *ctx, cudaStream_t s, const AtomBufs &b, const do
     if (grad_params) ts_chain(b, ctx->dga0, ctx->dgom, ctx->dgrv, grad_energy, grad_params, s);
     if (grad_coords) scale_copy(ctx->dgR, 3 * ctx->N, grad_energy, grad_coords, s);
     scale_copy(ctx->dgA, 9, grad_energy, ctx->dgAout, s);
+    if (products) {
+        if (const int rc = read_status(ctx, s, "gradient")) return rc;
+    }
     ctx->have_lattice_grad = true;
+    return MBD_OK;
 }
 
 // Periodic evaluation (Secs. 2.2 and 2.3): Gamma-point screening, Q(q) for every Bloch vector of
@@ -1259,7 +1274,9 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
     }
     mark(ctx, s, e_ns);
     nv.next("mbd gradient");
-    if (want_grad) backward_periodic(ctx, s, b, nullptr, out.grad_coords, out.grad_params);
+    if (want_grad) {
+        if (const int rg = backward_periodic(ctx, s, b, nullptr, out.grad_coords, out.grad_params)) return rg;
+    }
     if (out.alpha_scs)
         MBD_CUDA(cudaMemcpyAsync(out.alpha_scs, ctx->dabar0, sizeof(double) * N, cudaMemcpyDeviceToDevice, s),
                  "outputs");
@@ -1666,7 +1683,7 @@ int mbd_set_geometry(mbd_ctx *ctx, int n_atoms, const double *coords, const doub
     const bool realloc = (n_atoms != ctx->N) || !ctx->slab || periodic != ctx->periodic ||
                          (periodic && (ps.nk != ctx->nk || ps.nG != ctx->nG || ps.maxG != ctx->maxG)) ||
                          (periodic && !ctx->no_scratch &&   // (the image table's size depends on the lattice)
-                          build_q_products_bytes(n_atoms, ps.cell, ps.nk, ps.maxG) > ctx->qwork_bytes);
+                          cell_products_bytes(n_atoms, ps.cell, ps.nk, ps.maxG) > ctx->qwork_bytes);
     ctx->N = n_atoms;
     ctx->n = 3 * n_atoms;
     ctx->ld = (ctx->n + 127) / 128 * 128;   // 128: the tensor-core tile (also a multiple of 64)
@@ -1798,8 +1815,9 @@ int mbd_backward_dev(mbd_ctx *ctx, void *stream, long long evaluation, int n_ato
     MBD_CUDA(cudaSetDevice(ctx->device), "mbd_backward_dev");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Inputs in{coords, alpha0_ref, c6_ref, rvdw_ref, volume_ratio};
-    if (ctx->periodic) backward_periodic(ctx, s, atom_bufs(ctx, in), grad_energy, grad_coords, grad_params);
-    else backward_passes(ctx, s, atom_bufs(ctx, in), grad_energy, grad_coords, grad_params);
+    if (ctx->periodic) {
+        if (const int rc = backward_periodic(ctx, s, atom_bufs(ctx, in), grad_energy, grad_coords, grad_params)) return rc;
+    } else backward_passes(ctx, s, atom_bufs(ctx, in), grad_energy, grad_coords, grad_params);
     MBD_CUDA(cudaStreamSynchronize(s), "mbd_backward_dev");
     MBD_CUDA(cudaGetLastError(), "mbd_backward_dev");
     return MBD_OK;
