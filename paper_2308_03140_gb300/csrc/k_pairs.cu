@@ -496,7 +496,6 @@ __global__ void __launch_bounds__(256) k_scs_grad_tiles(AtomBufs b, double beta,
         }
         if (__any_sync(0xffffffffu, active)) {
             if (active) {
-                const double ir2 = ir * ir, ir3 = ir2 * ir, ir5 = ir3 * ir2;
 #pragma unroll
                 for (int kk = 0; kk < KF; ++kk) {
                     if (kk >= nk) break;
@@ -520,23 +519,14 @@ __global__ void __launch_bounds__(256) k_scs_grad_tiles(AtomBufs b, double beta,
                     Wb[2] = (Ws[2] + Ws[6]) * r[0] + (Ws[5] + Ws[7]) * r[1] + 2.0 * Ws[8] * r[2];
                     const double rWr = 0.5 * (r[0] * Wb[0] + r[1] * Wb[1] + r[2] * Wb[2]);
                     const double si = b.sig_u[k * b.N + i], sj = b.sig_u[k * b.N + j];
-                    // radial parts of T^GG as tgg_radial has them, with 1/s in place of its divisions
-                    const double is = rsqrt(si * si + sj * sj), z = rho * is;
-                    double P = ir3, W = -3.0 * ir5, dP = -3.0 * ir3 * ir, dW = 15.0 * ir5 * ir, WTs = 0.0;
-                    if (!(z > kGaussFar)) {
-                        const double z2 = z * z, th = kTwoOverSqrtPi * z * exp(-z2);
-                        const double F1 = erf(z) - th, t = 2.0 * z * th * is;
-                        P = F1 * ir3;
-                        W = (2.0 * z2 * th - 3.0 * F1) * ir5;
-                        dP = t * ir3 - 3.0 * P * ir;
-                        dW = -2.0 * z2 * t * ir5 - 5.0 * W * ir;
-                        WTs = z * t * (2.0 * z2 * ir5 * rWr - ir3 * tr);   // <Ws, dT^GG/ds>
-                    }
-                    const double WT = P * tr + W * rWr, g = -1.0 / 3.0 * sr * WTs * is;
+                    const double is = rsqrt(si * si + sj * sj);
+                    const Radial T = tgg_radial_inv(rho, ir, is);
+                    const double WT = T.P * tr + T.W * rWr;
+                    const double g = -1.0 / 3.0 * sr * (T.dPs * tr + T.dWs * rWr) * is;   // <Ws, dT^GG/ds> / s
                     rs[kk] = g * ca[0][kk][il];
                     cs[kk] += g * ca[1][kk][lane];
                     rs[KF] += f.df_dS * WT;
-                    const double rad = (sr * (dP * tr + dW * rWr) - f.df_drho * WT) * ir, srW = sr * W;
+                    const double rad = (sr * (T.dP * tr + T.dW * rWr) - f.df_drho * WT) * ir, srW = sr * T.W;
 #pragma unroll
                     for (int c = 0; c < 3; ++c) rs[KF + 1 + c] += rad * r[c] + srW * Wb[c];
                 }

@@ -470,12 +470,12 @@ __global__ void __launch_bounds__(256) k_energy_periodic(const double *Y, long l
 // gR[i] -= c_i c_j zx, gA += c_i c_j zA (c_i = omega_bar_i sqrt(abar0_i)).
 // Real-space sums in FP64; the reciprocal sum in R (double, or float for the mixed modes,
 // whose Z carries errors far above FP32 rounding), each chunk of kGC vectors summed in R and
-// added into FP64 totals.  images: with the real-space part and the self term (k_qgrad.cu has them otherwise, and in
+// added into FP64 totals.  kImages: with the real-space part and the self term (k_qgrad.cu has them otherwise, and in
 // FP64 the reciprocal part too).
-template <typename R>
+template <typename R, bool kImages>
 __global__ void __launch_bounds__(256) k_mbd_grad_periodic(AtomBufs b, PeriodicBufs p, double beta, double a,
                                                            const double *Z, long long ld, double zscale, int ntile,
-                                                           bool images, double *g_c, double *g_rbar, double *gR, double *gA) {
+                                                           double *g_c, double *g_rbar, double *gR, double *gA) {
     const int kq = blockIdx.y;
     int I, J;
     tile_pair(blockIdx.x, ntile, I, J);
@@ -502,7 +502,7 @@ __global__ void __launch_bounds__(256) k_mbd_grad_periodic(AtomBufs b, PeriodicB
         const double S = b.rbar[i] + b.rbar[j];
         int lo[3], hi[3];
         image_box(c, x, lo, hi);
-        if (!images) hi[0] = lo[0] - 1;
+        if (!kImages) hi[0] = lo[0] - 1;
         for (int n0 = lo[0]; n0 <= hi[0]; ++n0)
             for (int n1 = lo[1]; n1 <= hi[1]; ++n1)
                 for (int n2 = lo[2]; n2 <= hi[2]; ++n2) {
@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(256) k_mbd_grad_periodic(AtomBufs b, PeriodicB
     }
     if (!valid) return;
     zT += su;
-    if (i == j && images) zT -= 4.0 * c.gamma * c.gamma * c.gamma / (3.0 * sqrt(kPi)) * (zr[0] + zr[1] + zr[2]);   // self term
+    if (i == j && kImages) zT -= 4.0 * c.gamma * c.gamma * c.gamma / (3.0 * sqrt(kPi)) * (zr[0] + zr[1] + zr[2]);   // self term
     for (int d = 0; d < 3; ++d) zx[d] -= M1[d];
     for (int k = 0; k < 3; ++k)
         for (int d = 0; d < 3; ++d) {
@@ -652,7 +652,7 @@ __global__ void k_mean_rows(const double *x, int rows, int N, double *out) {
 // One CTA (128 threads) per atom i and kGradFreq frequencies; its units are partners j = 0..N-1 including
 // j = i (its images), each partner's images dealt out to kScsSplit units.  Bound by FP64 arithmetic as the
 // matrix build; one CTA per atom with all frequencies left two thirds of the chip idle with 96
-// atoms (11.2 ms, 5.8 so).  Partial sums per CTA: part[group][atom] = (g_rv, gR, gA), gal[k][atom].
+// atoms (11.2 ms, 5.6 so; 4.5 with the symmetric part of Ws alone and without divisions).  Partial sums per CTA: part[group][atom] = (g_rv, gR, gA), gal[k][atom].
 constexpr int kGradFreq = 2, kScsSplit = 4, kScsPart = 13;
 __global__ void __launch_bounds__(128) k_scs_grad_periodic(AtomBufs b, CellGeom c, double beta, double a,
                                                            const double *X, const double *V, long long xstride,
@@ -668,22 +668,26 @@ __global__ void __launch_bounds__(128) k_scs_grad_periodic(AtomBufs b, CellGeom 
         image_box(c, x, lo, hi);
         const int d1 = hi[1] - lo[1] + 1, d2 = hi[2] - lo[2] + 1, boxes = (hi[0] - lo[0] + 1) * d1 * d2;
         const double S = b.rv[i] + b.rv[j];
-        double Ws[kGradFreq][9], s[kGradFreq], dsda[kGradFreq];
+        double Ws[kGradFreq][6], is[kGradFreq], dsda[kGradFreq];   // Ws: its symmetric part, which is all that counts
 #pragma unroll
         for (int f = 0; f < kGradFreq; ++f) {
             const int k = min(k0 + f, b.nf1 - 1);
             const double *Vk = V + k * xstride, *Xk = X + k * xstride;
-            for (int xx = 0; xx < 3; ++xx)
-                for (int y = 0; y < 3; ++y) {
-                    double w = 0.0;
-                    for (int cc = 0; cc < 3; ++cc)
-                        w += Vk[9LL * i + 3 * xx + cc] * Xk[9LL * j + 3 * y + cc] +
-                             Xk[9LL * i + 3 * xx + cc] * Vk[9LL * j + 3 * y + cc];
-                    Ws[f][3 * xx + y] = k0 + f < b.nf1 ? w : 0.0;
-                }
+            auto block = [&](int xx, int y) {
+                double w = 0.0;
+                for (int cc = 0; cc < 3; ++cc)
+                    w += Vk[9LL * i + 3 * xx + cc] * Xk[9LL * j + 3 * y + cc] + Xk[9LL * i + 3 * xx + cc] * Vk[9LL * j + 3 * y + cc];
+                return w;
+            };
+            for (int xx = 0; xx < 3; ++xx) Ws[f][xx] = block(xx, xx);
+            Ws[f][3] = 0.5 * (block(0, 1) + block(1, 0));
+            Ws[f][4] = 0.5 * (block(0, 2) + block(2, 0));
+            Ws[f][5] = 0.5 * (block(1, 2) + block(2, 1));
+            if (k0 + f >= b.nf1)
+                for (int e = 0; e < 6; ++e) Ws[f][e] = 0.0;
             const double si = b.sig_u[k * b.N + i], sj = b.sig_u[k * b.N + j];
-            s[f] = sqrt(si * si + sj * sj);
-            dsda[f] = si * si / (3.0 * s[f] * b.al_u[k * b.N + i]);
+            is[f] = rsqrt(si * si + sj * sj);
+            dsda[f] = si * si * is[f] / (3.0 * b.al_u[k * b.N + i]);
         }
         for (int box = part_of; box < boxes; box += kScsSplit) {
             const int nn[3] = {lo[0] + box / (d1 * d2), lo[1] + box / d2 % d1, lo[2] + box % d2};
@@ -698,22 +702,15 @@ __global__ void __launch_bounds__(128) k_scs_grad_periodic(AtomBufs b, CellGeom 
             double dBs[3] = {0.0, 0.0, 0.0}, wts = 0.0;
 #pragma unroll
             for (int q = 0; q < kGradFreq; ++q) {
-                double Wr[3], Wtr[3];
-                for (int xx = 0; xx < 3; ++xx) {
-                    Wr[xx] = Ws[q][3 * xx] * r[0] + Ws[q][3 * xx + 1] * r[1] + Ws[q][3 * xx + 2] * r[2];
-                    Wtr[xx] = Ws[q][xx] * r[0] + Ws[q][3 + xx] * r[1] + Ws[q][6 + xx] * r[2];
-                }
-                const double tr = Ws[q][0] + Ws[q][4] + Ws[q][8];
-                const double rWr = r[0] * Wr[0] + r[1] * Wr[1] + r[2] * Wr[2];
-                const Radial qd = tgg_radial(rho, s[q]);
+                double Wr[3];
+                sym_mv(Ws[q], r, Wr);
+                const double tr = sym_tr(Ws[q]), rWr = r[0] * Wr[0] + r[1] * Wr[1] + r[2] * Wr[2];
+                const Radial qd = tgg_radial_inv(rho, ir, is[q]);
                 const double WT = qd.P * tr + qd.W * rWr;
-                const double WTs = qd.dPs * tr + qd.dWs * rWr;
-                acc[kScsPart + q] += -1.0 / 3.0 * sr * WTs * dsda[q];
+                acc[kScsPart + q] += -1.0 / 3.0 * sr * (qd.dPs * tr + qd.dWs * rWr) * dsda[q];
                 wts += WT;
-                for (int cc = 0; cc < 3; ++cc) {
-                    const double WdT = (qd.dP * tr + qd.dW * rWr) * r[cc] * ir + qd.W * (Wr[cc] + Wtr[cc]);
-                    dBs[cc] += sr * WdT - f.df_drho * r[cc] * ir * WT;   // <Ws, dB/dr_cc>
-                }
+                const double rad = (sr * (qd.dP * tr + qd.dW * rWr) - f.df_drho * WT) * ir, srW = 2.0 * sr * qd.W;
+                for (int cc = 0; cc < 3; ++cc) dBs[cc] += rad * r[cc] + srW * Wr[cc];   // <Ws, dB/dr_cc>
             }
             acc[0] += 1.0 / 3.0 * f.df_dS * wts;
             for (int cc = 0; cc < 3; ++cc) {
@@ -950,10 +947,12 @@ cudaError_t periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double b
     const dim3 grid(ntile * (ntile + 1) / 2, p.nk);
     cudaError_t e = cudaSuccess;
     if (products) e = grad_products(b, p, beta, a, Z, ld, zscale, g_c, o.g_rbar, o.gR, gA, !f32_recip, products, status, s);
-    if (f32_recip)
-        k_mbd_grad_periodic<float><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, !products, g_c, o.g_rbar, o.gR, gA);
+    if (f32_recip && products)
+        k_mbd_grad_periodic<float, false><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, g_c, o.g_rbar, o.gR, gA);
+    else if (f32_recip)
+        k_mbd_grad_periodic<float, true><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, g_c, o.g_rbar, o.gR, gA);
     else if (!products)
-        k_mbd_grad_periodic<double><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, true, g_c, o.g_rbar, o.gR, gA);
+        k_mbd_grad_periodic<double, true><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, g_c, o.g_rbar, o.gR, gA);
     k_mbd_grad_periodic_finalize<<<cdiv(b.N, 128), 128, 0, s>>>(b, Z, ld, p.nk, p.kw, zscale / p.nkt, g_c, o, tq);
     return e;
 }

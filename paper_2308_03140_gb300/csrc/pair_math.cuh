@@ -78,6 +78,16 @@ __host__ __device__ __forceinline__ Radial tgg_radial(double rho, double s) {
     return o;
 }
 
+// The same from 1/rho and 1/s, without tgg_radial's divisions (FP64 division costs ten operations or so of the pipe that
+// bounds the pair passes).
+__device__ __forceinline__ Radial tgg_radial_inv(double rho, double ir, double is) {
+    const double z = rho * is, ir2 = ir * ir, ir3 = ir2 * ir, ir5 = ir3 * ir2;
+    if (z > kGaussFar) return {ir3, -3.0 * ir5, -3.0 * ir3 * ir, 15.0 * ir5 * ir, 0.0, 0.0};
+    const double z2 = z * z, th = kTwoOverSqrtPi * z * exp(-z2), F1 = erf(z) - th, t = 2.0 * z * th * is;
+    const double P = F1 * ir3, W = (2.0 * z2 * th - 3.0 * F1) * ir5;
+    return {P, W, t * ir3 - 3.0 * P * ir, -2.0 * z2 * t * ir5 - 5.0 * W * ir, -z * t * ir3, 2.0 * z2 * z * t * ir5};
+}
+
 // Bare dipole tensor T = -grad grad 1/r, Eq. (dipole): P = 1/r^3, W = -3/r^5, and d/dr.
 struct RadialT { double P, W, dP, dW; };
 __host__ __device__ __forceinline__ RadialT bare_radial(double rho) {
