@@ -100,8 +100,7 @@ __global__ void k_nl_chain(AtomBufs b, const double *g_ab0, const double *g_om, 
 // tile, so that those rows too are written in contiguous runs.  Thread (i, i) writes the
 // diagonal block 1/alpha_i(u) I.  The factorisations read the lower triangle, the residuals
 // of the refined solves the full matrix.  Rows >= n: identity (k_pad_identity).  kf frequencies a CTA (blockIdx.z).
-// FP64 arithmetic bounds it; with divisions by s, and all frequencies in one CTA, it took 145 us for 32
-// atoms, 243 for 251 and 4.23 ms for 2000; so 15, 123 and 3.96 ms.
+// FP64 arithmetic bounds it; with all frequencies in one CTA it took 145 us for 32 atoms (four CTAs).
 __global__ void __launch_bounds__(256) k_build_scs(AtomBufs b, double beta, double a, double *M, long long ld,
                                                    long long mstride, int kf, int *status) {
     const int j0 = blockIdx.x * 32, i0 = blockIdx.y * 8;
@@ -110,7 +109,7 @@ __global__ void __launch_bounds__(256) k_build_scs(AtomBufs b, double beta, doub
     const int j = j0 + tx, i = i0 + ty;
     const bool pair = i < b.N && j < i, diag = i < b.N && j == i;
     __shared__ double T[24][97];
-    double r[3] = {0.0, 0.0, 0.0}, rho = 1.0, ir = 1.0, sr = 0.0, far_P = 0.0, far_W = 0.0, far2 = 0.0;
+    double r[3] = {0.0, 0.0, 0.0}, rho = 1.0, sr = 0.0, far_P = 0.0, far_W = 0.0, far2 = 0.0;
     if (pair) {
         r[0] = b.R[3 * j] - b.R[3 * i];
         r[1] = b.R[3 * j + 1] - b.R[3 * i + 1];
@@ -120,8 +119,7 @@ __global__ void __launch_bounds__(256) k_build_scs(AtomBufs b, double beta, doub
         sr = 1.0 - fermi(rho, b.rv[i] + b.rv[j], beta, a).f;
         // the bare tensor's radial parts, which T^GG equals beyond rho/s = kGaussFar (the far
         // branch of tgg_radial), once per pair for every frequency
-        ir = 1.0 / rho;
-        const double ir2 = ir * ir, ir3 = ir2 * ir, ir5 = ir3 * ir2;
+        const double ir = 1.0 / rho, ir2 = ir * ir, ir3 = ir2 * ir, ir5 = ir3 * ir2;
         far_P = ir3;
         far_W = -3.0 * ir5;
         far2 = rho * rho / (kGaussFar * kGaussFar);   // s^2 below this: the far branch
@@ -135,7 +133,7 @@ __global__ void __launch_bounds__(256) k_build_scs(AtomBufs b, double beta, doub
             const double s2 = si * si + sj * sj;
             double P = far_P, W = far_W;
             if (!(s2 < far2)) {
-                const Radial tg = tgg_radial_inv(rho, ir, rsqrt(s2));
+                const Radial tg = tgg_radial(rho, sqrt(s2));   // (to the bit: the mixed modes round these to FP32)
                 P = tg.P;
                 W = tg.W;
             }
