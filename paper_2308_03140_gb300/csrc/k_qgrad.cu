@@ -331,6 +331,7 @@ Layout layout(int N, const CellGeom &c, int nk, int maxG) {
         if (p <= kPartBytes || l.chunk == 256) break;
     }
     l.total = std::max(l.total, p);
+    if (l.total > 8 * kPartBytes) l.total = 0;   // (thousands of atoms, or grids of tens of thousands of vectors)
     return l;
 }
 

@@ -428,9 +428,12 @@ int mixed_group(int nk, long long lde, int precision) {
     return static_cast<int>(std::max<long long>(1, std::min<long long>({want, nk, kTcSlots})));
 }
 
-// Scratch of a cell's products, the build of Q(q) and the gradient.
-size_t cell_products_bytes(int N, const CellGeom &c, int nk, int maxG) {
-    return std::max(build_q_products_bytes(N, c, nk, maxG), grad_products_bytes(N, c, nk, maxG));
+// Scratch of a cell's products: the gradient's and, in FP64, those that build Q(q).  (The mixed modes round Q to FP32 and
+// bf16 parts, where a last-place difference of the FP64 entries now and then turns a rounding, and keep the direct build:
+// through products their 256-atom cell takes 150 ms less, but one in five seeds comes out 5e-9 off.)
+size_t cell_products_bytes(int N, const CellGeom &c, int nk, int maxG, int precision) {
+    const size_t grad = grad_products_bytes(N, c, nk, maxG);
+    return fp64_path(precision) ? std::max(build_q_products_bytes(N, c, nk, maxG), grad) : grad;
 }
 
 // Carves the workspace out of one allocation (256-byte aligned pieces).
@@ -496,7 +499,7 @@ int allocate(mbd_ctx *ctx, bool groups = true) {
     bytes += scs32;
     // Scratch of the tensor-core products, taken only where it fits: FP64 products and factors (and the
     // transpose of P), and the build of Q(q), which can share theirs.
-    const size_t q_work = ctx->periodic ? al(cell_products_bytes(ctx->N, ctx->cell, static_cast<int>(nk), ctx->maxG)) : 0;
+    const size_t q_work = ctx->periodic ? al(cell_products_bytes(ctx->N, ctx->cell, static_cast<int>(nk), ctx->maxG, prec)) : 0;
     const size_t crt_part =
         fp64_path(prec) ? std::max({al(cholesky_crt_bytes(ld, static_cast<int>(nf1))),
                                     al(ctx->periodic ? crt_cell_bytes(ctx->n, static_cast<int>(nk)) : crt_ns_bytes(ctx->n)), q_work})
@@ -1101,7 +1104,7 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
     ctx->have_screening = true;
     // ---- Q(q) and the spectrum bounds ----
     const size_t qbytes = build_q_products_bytes(N, ctx->cell, nk, ctx->maxG);
-    if (ctx->qwork && qbytes && qbytes <= ctx->qwork_bytes) {
+    if (fp64_path(ctx->opt.precision) && ctx->qwork && qbytes && qbytes <= ctx->qwork_bytes) {
         MBD_CUDA(build_q_products(b, pb, beta, a, ctx->dQ, ld, ctx->qwork, ctx->dstatus, s), "coupled_oscillator_matrix");
         pad_q_periodic(b, pb, ctx->dQ, ld, n, s);
     } else {
@@ -1683,7 +1686,7 @@ int mbd_set_geometry(mbd_ctx *ctx, int n_atoms, const double *coords, const doub
     const bool realloc = (n_atoms != ctx->N) || !ctx->slab || periodic != ctx->periodic ||
                          (periodic && (ps.nk != ctx->nk || ps.nG != ctx->nG || ps.maxG != ctx->maxG)) ||
                          (periodic && !ctx->no_scratch &&   // (the image table's size depends on the lattice)
-                          cell_products_bytes(n_atoms, ps.cell, ps.nk, ps.maxG) > ctx->qwork_bytes);
+                          cell_products_bytes(n_atoms, ps.cell, ps.nk, ps.maxG, ctx->opt.precision) > ctx->qwork_bytes);
     ctx->N = n_atoms;
     ctx->n = 3 * n_atoms;
     ctx->ld = (ctx->n + 127) / 128 * 128;   // 128: the tensor-core tile (also a multiple of 64)
