@@ -9,7 +9,8 @@
 // and 1644 vectors G each.  The real-space part is F(r) e^{-i q.r} over images r = x + n A with F real
 // and the same for every q: F is tabulated per pair and image offset once (about 150 operations each), and a
 // Bloch vector adds F times a phase that depends on the offset alone, times e^{-i q.(x + lo A)} at the end.
-// Together 10.2 ms for that cell.
+// Together 10.2 ms for that cell.  For the FP64 path: the mixed modes round Q further and keep the direct
+// build (mbd_api.cu).
 #include <algorithm>
 
 #include "cell_pairs.cuh"
