@@ -163,7 +163,9 @@ int mbdk_mlp_forward(void *stream, int n_atoms, int n_members, const float *X, c
  * features; grad (optional) [n_members][MBD_LEARNED_PARAMS] FP32 is ACCUMULATED with the
  * gradient with respect to the parameters (clear it first for a fresh gradient).  Without grad
  * the products run on the tensor cores (TF32 hi/lo parts against the exact FP16 weights, as
- * the forward), with grad in FP32 on the CUDA cores. */
+ * the forward), with grad in FP32 on the CUDA cores; its sums over atoms have one order, so that the
+ * same inputs give the same bits, and the call then takes up to 21 MB of stream-ordered device memory, of
+ * which the library keeps up to 32 MB a device until the next mbd_destroy there. */
 int mbdk_mlp_backward(void *stream, int n_atoms, int n_members, const float *X, const float *mean,
                       const float *std, const void *params_fp16, const float *zcache, const float *dY,
                       float *dX, float *grad);

@@ -438,6 +438,7 @@ cudaError_t mlp_forward(int B, int members, const float *X, const float *mean, c
 cudaError_t mlp_backward(int B, int members, const float *X, const float *mean, const float *stdv,
                          const void *params16, const float *zcache, const float *dY, float *dX, float *grad,
                          cudaStream_t s, const float *packed = nullptr);
+void scratch_trim(int device);   // gives back the memory that mlp_backward keeps for its next call
 void mse_grad(long long n, const float *y, const float *t, float *dy, double *loss, cudaStream_t s);
 void adam_step(long long n, float *p, const float *g, float *m, float *v, int step, float lr, void *p16,
                cudaStream_t s);

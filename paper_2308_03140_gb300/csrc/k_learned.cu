@@ -21,6 +21,8 @@
 // b2 [128], W3 [128][16], b3 [16] (W[in][out], row-major), kParams halves in all.
 #include <cuda_fp16.h>
 
+#include <mutex>
+
 #include "freq_grid.h"
 #include "internal.h"
 #include "pair_math.cuh"
@@ -884,19 +886,20 @@ __device__ __forceinline__ void atom_axpy(const float *row, float w, float (&acc
     }
 }
 
-// Backward of sum(dY * Y): grid (ceil(B / 32), members), 128 threads.  Needs the cache of the
-// forward pass.  dX (optional) [member][B][122]: gradient with respect to the raw features.
-// grad (optional) [member][kParams] FP32, accumulated (atomic adds of per-CTA sums).
+// Backward of sum(dY * Y), 128 threads, a CTA per item0 + blockIdx.x: 32 atoms of a member (ceil(B / 32) items a
+// member).  Needs the cache of the forward pass.  dX (optional) [member][B][122]: gradient with respect to the raw features.
+// part [blockIdx.x][kParams]: the parameter gradient of the item's atoms, which k_mlp_grad_sum adds up.
 // Bound by shared-memory reads: thread t holds one unit's 32 atoms in registers, and a read of four atoms
 // of another unit, the same for the whole warp, feeds four multiply-adds; a weight is read once for all
 // atoms.  (One word per multiply-add, and a row of weights per thread with all threads on one bank:
-// 169 us for 4096 atoms of a member, 98 so.)
+// 169 us for 4096 atoms of a member.)
 __global__ void __launch_bounds__(128) k_mlp_backward(int B, const float *X, const float *mean, const float *stdv,
                                                       const __half *params, const float *zcache, const float *dY,
-                                                      float *dX, float *grad) {
+                                                      float *dX, long long item0, float *part) {
     extern __shared__ __align__(16) char smem[];
     const MlpSmem m = mlp_smem(smem);
-    const int member = blockIdx.y, a0 = blockIdx.x * kTA, t = threadIdx.x;
+    const long long blocks = (static_cast<long long>(B) + kTA - 1) / kTA, item = item0 + blockIdx.x;
+    const int member = static_cast<int>(item / blocks), a0 = static_cast<int>(item - member * blocks) * kTA, t = threadIdx.x;
     const __half *P = params + static_cast<long long>(member) * kParams;
     if (aligned16(P)) {
 #pragma unroll 8
@@ -922,21 +925,19 @@ __global__ void __launch_bounds__(128) k_mlp_backward(int B, const float *X, con
         m.h2[t * kTS + a] = ok ? silu(z2[row * kH + t]) : 0.0f;
     }
     __syncthreads();
-    float *g = grad ? grad + static_cast<long long>(member) * kParams : nullptr;
-    const int first = static_cast<int>(blockIdx.x * 37u) & (kH - 1);   // the CTAs' atomics start at different rows
-    if (g) {   // output layer: gW3[k][o] = sum_a h2[a][k] dy[a][o], gb3[o] = sum_a dy[a][o]
-        for (int e = t; e < kH * kO; e += 128) {
-            const int k = e / kO, o = e % kO;
-            float s = 0.0f;
+    float *g = part + static_cast<long long>(blockIdx.x) * kParams;
+    // output layer: gW3[k][o] = sum_a h2[a][k] dy[a][o], gb3[o] = sum_a dy[a][o]
+    for (int e = t; e < kH * kO; e += 128) {
+        const int k = e / kO, o = e % kO;
+        float s = 0.0f;
 #pragma unroll
-            for (int a = 0; a < kTA; ++a) s += m.h2[k * kTS + a] * dy_s[a * kO + o];
-            atomicAdd(&g[oW3 + e], s);
-        }
-        if (t < kO) {
-            float s = 0.0f;
-            for (int a = 0; a < kTA; ++a) s += dy_s[a * kO + t];
-            atomicAdd(&g[ob3 + t], s);
-        }
+        for (int a = 0; a < kTA; ++a) s += m.h2[k * kTS + a] * dy_s[a * kO + o];
+        g[oW3 + e] = s;
+    }
+    if (t < kO) {
+        float s = 0.0f;
+        for (int a = 0; a < kTA; ++a) s += dy_s[a * kO + t];
+        g[ob3 + t] = s;
     }
     // dz2[a][t] = (sum_o dy[a][o] W3[t][o]) dsilu(z2[a][t]); kept in registers
     float dz[kTA], w3[kO];
@@ -949,17 +950,13 @@ __global__ void __launch_bounds__(128) k_mlp_backward(int B, const float *X, con
         for (int o = 0; o < kO; ++o) s += dy_s[a * kO + o] * w3[o];
         dz[a] = a0 + a < B ? s * dsilu(z2[static_cast<long long>(a0 + a) * kH + t]) : 0.0f;
     }
-    if (g) {   // gW2[k][t] = sum_a h1[a][k] dz2[a][t]; gb2[t]
-        float sb = 0.0f;
+    // gW2[k][t] = sum_a h1[a][k] dz2[a][t]; gb2[t]
+    float sb = 0.0f;
 #pragma unroll
-        for (int a = 0; a < kTA; ++a) sb += dz[a];
-        atomicAdd(&g[ob2 + t], sb);
+    for (int a = 0; a < kTA; ++a) sb += dz[a];
+    g[ob2 + t] = sb;
 #pragma unroll 4
-        for (int u = 0; u < kH; ++u) {
-            const int k = (u + first) & (kH - 1);
-            atomicAdd(&g[oW2 + k * kH + t], atom_dot(m.h1 + k * kTS, dz));
-        }
-    }
+    for (int k = 0; k < kH; ++k) g[oW2 + k * kH + t] = atom_dot(m.h1 + k * kTS, dz);
     __syncthreads();   // h2 is no longer needed: reuse it for dz2
 #pragma unroll
     for (int a = 0; a < kTA; ++a) {
@@ -977,17 +974,13 @@ __global__ void __launch_bounds__(128) k_mlp_backward(int B, const float *X, con
     }
 #pragma unroll
     for (int a = 0; a < kTA; ++a) dz[a] = a0 + a < B ? dz[a] * dsilu(z1[static_cast<long long>(a0 + a) * kH + t]) : 0.0f;
-    if (g) {   // gW1[k][t] = sum_a Xs[a][k] dz1[a][t]; gb1[t]
-        float sb = 0.0f;
+    // gW1[k][t] = sum_a Xs[a][k] dz1[a][t]; gb1[t]
+    sb = 0.0f;
 #pragma unroll
-        for (int a = 0; a < kTA; ++a) sb += dz[a];
-        atomicAdd(&g[ob1 + t], sb);
+    for (int a = 0; a < kTA; ++a) sb += dz[a];
+    g[ob1 + t] = sb;
 #pragma unroll 4
-        for (int u = 0; u < kH; ++u) {
-            const int k = (u + first) & (kH - 1);
-            if (k < kF) atomicAdd(&g[oW1 + k * kH + t], atom_dot(m.Xs + k * kTS, dz));
-        }
-    }
+    for (int k = 0; k < kF; ++k) g[oW1 + k * kH + t] = atom_dot(m.Xs + k * kTS, dz);
     if (dX) {
         __syncthreads();
 #pragma unroll
@@ -1009,6 +1002,44 @@ __global__ void __launch_bounds__(128) k_mlp_backward(int B, const float *X, con
                 if (a0 + a < B) dX[(static_cast<long long>(member) * B + a0 + a) * kF + t] = dz[a] / sd;
         }
     }
+}
+
+// grad += the parts of items item0 .. item0 + items - 1, those of a member (blockIdx.y counts from the first item's) as
+// four compensated sums of a quarter each, one after another: every sum has one order, and the same step gives the
+// same bits.  (FP32 atomics by the CTAs of k_mlp_backward left the order to the moment: gradients 1e-7 apart from run to
+// run, and now and then another FP16 weight after the step.)  Latency bounds it: 6.7 us for the 128 parts of 4096 atoms,
+// beside 89 us that form them; a training step of four members 576 us with the atomics, 588 so.
+constexpr int kSumParams = 64, kSumGroups = 4;
+struct SumF {
+    float s = 0.0f, lost = 0.0f;
+    __device__ __forceinline__ void add(float x) {
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+        lost = __fadd_rn(lost, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+        s = t;
+    }
+};
+__global__ void __launch_bounds__(kSumParams * kSumGroups)
+    k_mlp_grad_sum(long long blocks, long long item0, int items, const float *part, float *grad) {
+    __shared__ SumF sh[kSumGroups][kSumParams];
+    const int c = threadIdx.x % kSumParams, g = threadIdx.x / kSumParams, p = blockIdx.x * kSumParams + c;
+    const long long member = item0 / blocks + blockIdx.y;
+    const int from = static_cast<int>(max(member * blocks - item0, 0LL)),
+              to = static_cast<int>(min((member + 1) * blocks - item0, static_cast<long long>(items)));
+    const int each = (to - from + kSumGroups - 1) / kSumGroups, k1 = min(to, from + (g + 1) * each);
+    SumF v;
+    if (p < kParams) {
+#pragma unroll 16
+        for (int k = from + g * each; k < k1; ++k) v.add(part[static_cast<long long>(k) * kParams + p]);
+    }
+    sh[g][c] = v;
+    __syncthreads();
+    if (g || p >= kParams) return;
+#pragma unroll
+    for (int q = 1; q < kSumGroups; ++q) {
+        v.add(sh[q][c].s);
+        v.lost += sh[q][c].lost;
+    }
+    atomicAdd(grad + member * kParams + p, v.s + v.lost);   // (calls on other streams may add to it too)
 }
 
 __global__ void k_mse_grad(long long n, const float *y, const float *t, float *dy, double *loss) {
@@ -1329,6 +1360,45 @@ cudaError_t mlp_forward(int B, int members, const float *X, const float *mean, c
     return cudaGetLastError();
 }
 
+namespace {
+// Stream-ordered scratch of the parameter gradient, from a pool of its own for each device that keeps at most
+// kScratchKept bytes between calls (the default pool gives its memory back whenever the stream is waited for, and a
+// call after that took 300 us more).  scratch_trim gives that back too.
+constexpr size_t kScratchKept = size_t{32} << 20;
+constexpr int kScratchDevices = 64;
+std::mutex g_pool_mutex;
+cudaMemPool_t g_pool[kScratchDevices] = {};
+
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool = nullptr;
+    if (dev < kScratchDevices) {
+        std::lock_guard<std::mutex> lock(g_pool_mutex);
+        if (!g_pool[dev]) {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            uint64_t kept = kScratchKept;
+            if (cudaMemPoolCreate(&pool, &props) == cudaSuccess &&
+                cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &kept) == cudaSuccess)
+                g_pool[dev] = pool;
+            else cudaGetLastError();
+        }
+        pool = g_pool[dev];
+    }
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+}
+}  // namespace
+
+void scratch_trim(int device) {
+    if (device < 0 || device >= kScratchDevices) return;
+    std::lock_guard<std::mutex> lock(g_pool_mutex);
+    if (g_pool[device]) cudaMemPoolTrimTo(g_pool[device], 0);
+}
+
 cudaError_t mlp_backward(int B, int members, const float *X, const float *mean, const float *stdv,
                          const void *params16, const float *zcache, const float *dY, float *dX, float *grad,
                          cudaStream_t s, const float *packed) {
@@ -1351,10 +1421,27 @@ cudaError_t mlp_backward(int B, int members, const float *X, const float *mean, 
     cudaError_t e = cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(kMlpSmem));
     if (e != cudaSuccess) return e;
-    count_launches(1);
-    k_mlp_backward<<<dim3(cdiv(B, kTA), members), 128, kMlpSmem, s>>>(
-        B, X, mean, stdv, static_cast<const __half *>(params16), zcache, dY, dX, grad);
-    return cudaGetLastError();
+    // The parts of a wave of CTAs (one an SM, 21 MB) at a time, in stream-ordered memory; fewer where that much is not
+    // to be had.
+    const long long blocks = cdiv(B, kTA), items = members * blocks;
+    long long wave = std::min<long long>(items, 152);
+    float *part = nullptr;
+    for (;; wave = (wave + 1) / 2) {
+        e = scratch_alloc(reinterpret_cast<void **>(&part), sizeof(float) * kParams * wave, s);
+        if (e == cudaSuccess) break;
+        if (e != cudaErrorMemoryAllocation || wave == 1) return e;
+        cudaGetLastError();
+    }
+    for (long long i = 0; i < items; i += wave) {
+        const int n = static_cast<int>(std::min(wave, items - i));
+        count_launches(2);
+        k_mlp_backward<<<n, 128, kMlpSmem, s>>>(B, X, mean, stdv, static_cast<const __half *>(params16), zcache, dY, dX, i, part);
+        k_mlp_grad_sum<<<dim3(cdiv(kParams, kSumParams), static_cast<unsigned>((i + n - 1) / blocks - i / blocks + 1)),
+                         kSumParams * kSumGroups, 0, s>>>(blocks, i, n, part, grad);
+    }
+    e = cudaGetLastError();
+    const cudaError_t freed = cudaFreeAsync(part, s);
+    return e != cudaSuccess ? e : freed;
 }
 
 void mse_grad(long long n, const float *y, const float *t, float *dy, double *loss, cudaStream_t s) {

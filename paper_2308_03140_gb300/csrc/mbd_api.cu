@@ -1661,6 +1661,7 @@ int mbd_destroy(mbd_ctx *ctx) {
     if (ctx->lslab) cudaFree(ctx->lslab);
     for (cudaEvent_t e : ctx->events) cudaEventDestroy(e);
     if (ctx->stream) cudaStreamDestroy(ctx->stream);
+    scratch_trim(ctx->device);
     delete ctx;
     return MBD_OK;
 }
