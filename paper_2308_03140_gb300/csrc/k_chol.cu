@@ -2,9 +2,11 @@
 // of Eq. (scs) and the log-formula route: the 64-column blocks and the trailing updates are residue
 // products (k_crt.cu), only the 64 x 64 diagonal blocks are factored on the FP64 pipe.
 //
-// Every row r of the factor has |L_r|^2 = A_rr, so its scaling exponent is known before the
-// factorisation starts and each column block of L becomes residue planes once, for all products
-// that read it.  Panels of kPanel columns; inside a panel, for each block of 64 columns (all launches
+// A row r of the factor of a positive definite matrix has |L_r|^2 = A_rr, so its scaling exponent is known before
+// the factorisation starts and each column block of L becomes residue planes once, for all products
+// that read it.  The row of a matrix that is not may be longer, and its products would come back modulo P with any
+// pivot: k_solve counts the squares of a row's entries against A_rr and raises ST_SCS_NOT_PD when they
+// exceed it by 0.1 % (P leaves 1.6 %; below that the products are exact and the pivot tells).  Panels of kPanel columns; inside a panel, for each block of 64 columns (all launches
 // take the whole batch):
 //   products   C = A[j:, j] - L[j:, p:j] L[j, p:j]^T          (narrow tiles; not for the first block)
 //   k_column   FP64 values of the diagonal block, residues of the rows below
@@ -24,13 +26,16 @@ namespace {
 
 using crt::kMod;
 
-// exps[b][r] of the rows of the factor, from the diagonal.
-__global__ void k_factor_exponents(const double *A, long long ld, long long mstride, int *exps) {
+// exps[b][r] of the rows of the factor, from the diagonal, and left[b][r]: the sum of squares that the row's scaled
+// entries may reach (negative for a bad row).
+__global__ void k_factor_exponents(const double *A, long long ld, long long mstride, int *exps, float *left) {
     const long long r = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x, b = blockIdx.y;
     if (r >= ld) return;
     const double d = A[b * mstride + r * ld + r];
     const int e = crt::row_exponent(sqrt(d) * (1.0 + 1e-6));   // (the root of a negative diagonal is NaN: a bad row)
     exps[b * ld + r] = e == crt::kBadRow ? e : min(e, 1000);
+    const double root = e == crt::kBadRow ? 0.0 : sqrt(d) * crt::pow2(min(e, 1000));   // below 2^59
+    left[b * ld + r] = e == crt::kBadRow ? -1.0f : static_cast<float>(1.001 * root * root);
 }
 
 // Two neighbouring entries' residues, bf16 pairs into the planes at `out`.
@@ -95,8 +100,8 @@ __global__ void __launch_bounds__(256) k_column(double *A, long long ld, long lo
     if (ss > 1e-280 && ss < 1e280) {
         e = crt::row_exponent(sqrt(ss));
     } else {   // an upper bound of the norm serves: 8 times the largest entry
-        double mx = fmax(fabs(v[0]), fabs(v[1]));
-        if (!(mx <= crt::kMaxDouble / 16)) mx = CUDART_INF;
+        double mx = fmax(fabs(v[0]), fabs(v[1]));   // (drops a NaN beside a number)
+        if (!(mx <= crt::kMaxDouble / 16) || isnan(v[0]) || isnan(v[1])) mx = CUDART_INF;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         e = crt::row_exponent(8.0 * mx);
@@ -109,10 +114,13 @@ __global__ void __launch_bounds__(256) k_column(double *A, long long ld, long lo
 }
 
 // Row r = j0 + 64 + rr of the solved block, a warp per row: FP64 values from the product's bytes, and
-// residues at the row's exponent in the panel's planes ([b][kMod][ld][pitch], columns from kcol).
+// residues at the row's exponent in the panel's planes ([b][kMod][ld][pitch], columns from kcol).  The squares of the scaled
+// entries are taken from left[b][r], which this launch alone touches: in FP32, whose 1e-7 a block of columns is far
+// inside the 0.1 % and whose sums over the warp cost a sixteenth of FP64's.
 __global__ void __launch_bounds__(256) k_solve(double *A, long long ld, long long mstride, int j0, int m,
                                                const uint8_t *Y, const int *rexps, long long rstride, const int *dexps,
-                                               const int *fexps, __nv_bfloat16 *planes, int pitch, int kcol) {
+                                               const int *fexps, __nv_bfloat16 *planes, int pitch, int kcol, float *left,
+                                               int *status) {
     const int rr = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (rr >= m) return;
     const long long b = blockIdx.y, r = j0 + 64 + rr, plane = 64LL * m;
@@ -124,10 +132,20 @@ __global__ void __launch_bounds__(256) k_solve(double *A, long long ld, long lon
     v[1] = crt::scaled_down(v[1], er, ec.y);
     *reinterpret_cast<double2 *>(A + b * mstride + r * ld + j0 + 2 * lane) = make_double2(v[0], v[1]);
     const int e = fexps[b * ld + r];
+    const double scale = row_scale(e);
+    const float x0 = static_cast<float>(v[0] * scale), x1 = static_cast<float>(v[1] * scale);
+    float used = x0 * x0 + x1 * x1;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) used += __shfl_xor_sync(0xffffffffu, used, o);
+    if (lane == 0) {
+        const float rest = left[b * ld + r] - used;
+        left[b * ld + r] = rest;
+        if (!(rest >= 0.0f)) atomicOr(status, ST_SCS_NOT_PD);
+    }
     if (e == crt::kBadRow || !(fabs(v[0]) <= crt::kMaxDouble)) v[0] = 0.0;   // (a factorisation that has failed)
     if (e == crt::kBadRow || !(fabs(v[1]) <= crt::kMaxDouble)) v[1] = 0.0;
     const long long pp = ld * pitch;
-    put2(v[0], v[1], row_scale(e), pp, planes + b * kMod * pp + r * pitch + kcol + 2 * lane);
+    put2(v[0], v[1], scale, pp, planes + b * kMod * pp + r * pitch + kcol + 2 * lane);
 }
 
 // 1 / d to about an ulp, d a normal number: two Newton steps from the hardware's approximation.
@@ -325,7 +343,7 @@ constexpr size_t kTrailingBytes = size_t{1} << 30;
 inline size_t al(size_t b) { return (b + 255) / 256 * 256; }
 
 struct Layout {
-    long long panel, rows, inverse, exps, rexps, dexps, bytes, total;   // offsets
+    long long panel, rows, inverse, exps, rexps, dexps, left, bytes, total;   // offsets
 };
 Layout layout(long long ld, int batch) {
     Layout l;
@@ -342,6 +360,7 @@ Layout layout(long long ld, int batch) {
     l.exps = take(4 * static_cast<size_t>(batch) * ld);
     l.rexps = take(4 * static_cast<size_t>(batch) * ld);
     l.dexps = take(4 * static_cast<size_t>(batch) * 64);
+    l.left = take(4 * static_cast<size_t>(batch) * ld);
     const size_t m = ld > kPanel ? static_cast<size_t>(ld) - kPanel : 0, whole = kMod * m * m;
     const size_t strip = kMod * m * std::min<size_t>(m, 2048);   // at least a strip of 2048 columns
     l.bytes = take(std::max<size_t>(z * ld * 64, std::min<size_t>(whole * batch, std::max<size_t>(kTrailingBytes, strip))));
@@ -361,6 +380,7 @@ cudaError_t cholesky_crt(double *A, long long ld, long long mstride, int batch, 
          *inverse = reinterpret_cast<__nv_bfloat16 *>(w + l.inverse);
     int *exps = reinterpret_cast<int *>(w + l.exps), *rexps = reinterpret_cast<int *>(w + l.rexps),
         *dexps = reinterpret_cast<int *>(w + l.dexps);
+    float *left = reinterpret_cast<float *>(w + l.left);
     uint8_t *Y = reinterpret_cast<uint8_t *>(w + l.bytes);
     const size_t ybytes = static_cast<size_t>(l.total - l.bytes);
     const int nb = static_cast<int>(ld / kTile), pitch = static_cast<int>(std::min<long long>(kPanel, ld));
@@ -391,7 +411,7 @@ cudaError_t cholesky_crt(double *A, long long ld, long long mstride, int batch, 
         return o;
     };
     count_launches(1);
-    k_factor_exponents<<<dim3(static_cast<unsigned>((ld + 255) / 256), batch), 256, 0, s>>>(A, ld, mstride, exps);
+    k_factor_exponents<<<dim3(static_cast<unsigned>((ld + 255) / 256), batch), 256, 0, s>>>(A, ld, mstride, exps, left);
     cudaError_t e = cudaSuccess;
     for (long long p0 = 0; p0 < ld; p0 += kPanel) {
         const long long p1 = std::min<long long>(ld, p0 + kPanel);
@@ -416,7 +436,7 @@ cudaError_t cholesky_crt(double *A, long long ld, long long mstride, int batch, 
             if (e != cudaSuccess) return e;
             count_launches(1);
             k_solve<<<dim3((below + 7) / 8, batch), 256, 0, s>>>(A, ld, mstride, static_cast<int>(j0), below, Y, rexps + 64,
-                                                                m, dexps, exps, panel, pitch, kc);
+                                                                m, dexps, exps, panel, pitch, kc, left, status);
         }
         const long long m = ld - p1;
         if (m <= 0) continue;

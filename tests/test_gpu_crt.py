@@ -265,3 +265,87 @@ def test_cholesky_flags_what_is_not_positive_definite(dev):
     A = np.stack([good, good])
     A[0, 630, 10] = A[0, 10, 630] = 1e6      # positive diagonal, negative eigenvalue
     assert _factor(dev, A)[2] == 2
+
+
+def _sunk(rng, ld, row, ratio):
+    # positive definite but for one row: L's entries left of the diagonal carry `ratio` times the
+    # row's diagonal element, so that its pivot is (1 - ratio) A_rr (the rows below are apart from it)
+    X = rng.normal(size=(ld, ld)) / np.sqrt(ld)
+    A = X @ X.T + np.diag(rng.uniform(0.1, 1.0, ld))
+    L = np.linalg.cholesky(A)
+    A[row, row] = (L[row, :row] ** 2).sum() / ratio
+    A[row + 1:, :row + 1] = A[:row + 1, row + 1:] = 0.0
+    return A
+
+
+@pytest.mark.parametrize("ld", [128, 256, 512, 640])
+def test_cholesky_flags_every_row_longer_than_its_diagonal(dev, ld):
+    # a row's scale comes from its diagonal element, which bounds the row of the factor only if the
+    # matrix is positive definite: a longer row's product would come back modulo P
+    dev.crt_cholesky_bytes.restype = C.c_size_t
+    A = np.eye(128)
+    A[100, :64] = A[:64, 100] = np.sqrt(2.0 / 64)   # lowest eigenvalue 1 - sqrt(2)
+    assert _factor(dev, A[None])[2] == 2
+    rng = np.random.default_rng(ld)
+    passed = []
+    for ratio in np.exp(np.linspace(np.log(1.0 + 1e-6), np.log(10.0), 60)):
+        row = int(rng.integers(64, ld))
+        A = _sunk(rng, ld, row, ratio)
+        if _factor(dev, A[None])[2] != 2:
+            passed.append((row, ratio))
+    assert not passed
+
+
+@pytest.mark.parametrize("ld,row", [(128, 64), (128, 127), (640, 600)])
+def test_cholesky_keeps_what_is_barely_positive_definite(dev, ld, row):
+    dev.crt_cholesky_bytes.restype = C.c_size_t
+    A = _sunk(np.random.default_rng(row), ld, row, 1.0 - 1e-9)
+    assert np.linalg.cholesky(A)[row, row] > 0.0 and _factor(dev, A[None])[2] == 0
+
+
+@pytest.mark.parametrize("row,col", [(70, 10), (70, 11), (600, 10), (600, 63), (639, 598)])
+def test_cholesky_flags_a_nan_beside_finite_entries(dev, row, col):
+    dev.crt_cholesky_bytes.restype = C.c_size_t
+    rng = np.random.default_rng(row + col)
+    X = rng.normal(size=(640, 640))
+    A = X @ X.T + np.eye(640)
+    A[row, col] = A[col, row] = np.nan
+    assert _factor(dev, A[None])[2] == 2
+
+
+def _lowest(R, a0, c6, ra, rw, u):
+    """Lowest eigenvalue of I + alpha(iu)^(1/2) T^lr alpha(iu)^(1/2) of MBD-NL oscillators."""
+    a, om, rad = a0 * ra, 4.0 * c6 / (3.0 * a0 ** 2) * rw, 2.5 * a0 ** (1.0 / 7.0) * ra ** (1.0 / 3.0)
+    r = R[None] - R[:, None]
+    d = np.sqrt((r ** 2).sum(-1) + np.eye(len(R)))
+    f = 1.0 / (1.0 + np.exp(-6.0 * (d / (0.83 * (rad[:, None] + rad[None])) - 1.0)))
+    T = np.eye(3) / d[..., None, None] ** 3 - 3.0 * r[..., :, None] * r[..., None, :] / d[..., None, None] ** 5
+    al = np.sqrt(a / (1.0 + (u / om) ** 2))
+    B = (f * al[:, None] * al[None] * (1.0 - np.eye(len(R))))[..., None, None] * T
+    return np.linalg.eigvalsh(np.eye(3 * len(R)) + B.transpose(0, 2, 1, 3).reshape(3 * len(R), -1))[0]
+
+
+def test_log_energy_refuses_dense_random_oscillators(dev):
+    # random positions without a least distance: some I + A_k are not positive definite
+    from paper_2308_03140_gb300 import synthetic as syn
+    x = np.polynomial.legendre.leggauss(15)[0]
+    nodes, seen = 0.6 * (1 + x) / (1 - x), set()
+    base = syn.sphere_cluster(74, seed=1)
+    with binding.MBD(0, scs_mode=binding.MBD_SCS_NL) as m:
+        for seed in range(40):
+            rng = np.random.default_rng(seed)
+            R = rng.uniform(0, rng.uniform(9.0, 16.0), (74, 3))
+            ra, rw = syn.nl_ratios(74, seed)
+            m.set_geometry(R)
+            m.set_nl_params(base.alpha0_ref, base.c6_ref, ra, rw)
+            code = 0
+            for call in (lambda: m.evaluate(False), lambda: m.log_energy(1)):
+                try:
+                    call()
+                    code = 0
+                except binding.MBDError as e:   # (the energy itself may have no square root)
+                    code = e.code
+            low = min(_lowest(R, base.alpha0_ref, base.c6_ref, ra, rw, u) for u in nodes)
+            assert abs(low) > 1e-9 and code == (0 if low > 0 else 4), (seed, low, code)
+            seen.add(code)
+    assert seen == {0, 4}
