@@ -6,7 +6,7 @@
 // the factorisation starts and each column block of L becomes residue planes once, for all products
 // that read it.  The row of a matrix that is not may be longer, and its products would come back modulo P with any
 // pivot: k_solve counts the squares of a row's entries against A_rr and raises ST_SCS_NOT_PD when they
-// exceed it by 0.1 % (P leaves 1.6 %; below that the products are exact and the pivot tells).  Panels of kPanel columns; inside a panel, for each block of 64 columns (all launches
+// exceed it by 0.1 % (P leaves 1.8 %; below that the products are exact and the pivot tells).  Panels of kPanel columns; inside a panel, for each block of 64 columns (all launches
 // take the whole batch):
 //   products   C = A[j:, j] - L[j:, p:j] L[j, p:j]^T          (narrow tiles; not for the first block)
 //   k_column   FP64 values of the diagonal block, residues of the rows below
