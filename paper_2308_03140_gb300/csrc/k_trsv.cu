@@ -63,7 +63,9 @@ __global__ void __launch_bounds__(256) k_trsv_first(const T *dinv, long long dst
     diag_solve<T, BWD>(D, s, out + b * xstride + 192LL * I);
 }
 
-template <typename T>
+// kWide: L in 16-byte loads, for an L that starts on 16 bytes (its rows are multiples of 64 entries); callers may
+// also pass one that does not, which is read entry by entry.
+template <typename T, bool kWide>
 __global__ void __launch_bounds__(256) k_trsv_fwd_block(const T *L, long long ld, long long mstride, const T *dinv,
                                                         long long dstride, T *X, T *W, long long xstride, int I) {
     const long long b = blockIdx.x;   // (the batch first: the CTAs of the next blocks start first)
@@ -78,10 +80,12 @@ __global__ void __launch_bounds__(256) k_trsv_fwd_block(const T *L, long long ld
     const long long r0 = I0 + 64 + static_cast<long long>(blockIdx.y) * 64;
     const int rr = threadIdx.x >> 2, q = threadIdx.x & 3;
     const T *Lq = Lb + (r0 + rr) * ld + I0 + 16 * q;
-    T l[16];
+    alignas(16) T l[16];
 #pragma unroll
-    for (int c = 0; c < 16; c += 16 / sizeof(T))   // 16 bytes at a time
-        *reinterpret_cast<int4 *>(l + c) = *reinterpret_cast<const int4 *>(Lq + c);
+    for (int c = 0; c < 16; c += kWide ? 16 / sizeof(T) : 1) {
+        if constexpr (kWide) *reinterpret_cast<int4 *>(l + c) = *reinterpret_cast<const int4 *>(Lq + c);
+        else l[c] = Lq[c];
+    }
     if (next) load_inverse(dinv + b * dstride + static_cast<long long>(I + 1) * 4096, D);
     wait_for_previous();
     if (threadIdx.x < 192) x[threadIdx.x / 3][threadIdx.x % 3] = Wb[3 * I0 + threadIdx.x];
@@ -181,9 +185,11 @@ void trsv_blocked(const T *L, long long ld, long long mstride, int batch, const 
     count_launches(2 * nb);
     cudaLaunchKernelEx(&cfg, k_trsv_first<T, false>, dinv, dstride, static_cast<const T *>(X), W, xstride, 0);
     cfg.numAttrs = 1;
+    const bool wide = (reinterpret_cast<uintptr_t>(L) & 15) == 0 && mstride * sizeof(T) % 16 == 0;
     for (int I = 0; I + 1 < nb; ++I) {
         cfg.gridDim = dim3(batch, nb - 1 - I);   // 64-row slices below block I
-        cudaLaunchKernelEx(&cfg, k_trsv_fwd_block<T>, L, ld, mstride, dinv, dstride, X, W, xstride, I);
+        if (wide) cudaLaunchKernelEx(&cfg, k_trsv_fwd_block<T, true>, L, ld, mstride, dinv, dstride, X, W, xstride, I);
+        else cudaLaunchKernelEx(&cfg, k_trsv_fwd_block<T, false>, L, ld, mstride, dinv, dstride, X, W, xstride, I);
     }
     cfg.gridDim = dim3(batch);
     cudaLaunchKernelEx(&cfg, k_trsv_first<T, true>, dinv, dstride, static_cast<const T *>(W), X, xstride, nb - 1);
