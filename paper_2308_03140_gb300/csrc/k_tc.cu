@@ -1376,9 +1376,10 @@ cudaError_t tc_gemm(int kind, const TcOperands &op, const TcArgs &g, cudaStream_
         return cudaErrorInvalidValue;
     for (int k = 0; k < g.nslots; ++k)
         if (g.slot[k] < 0 || (g.betas[k] != 0.f && !g.D)) return cudaErrorInvalidValue;
-    // The wide form stores four elements at a time, also of the transposes and the FP64 sums.
-    const bool aligned = ((reinterpret_cast<uintptr_t>(g.CT) | reinterpret_cast<uintptr_t>(g.CTh) |
-                           reinterpret_cast<uintptr_t>(g.CTl) | reinterpret_cast<uintptr_t>(g.C64)) & 15) == 0 &&
+    // The wide form stores four elements at a time, also of the transposes, the FP64 sums and the tiles on the diagonal of a
+    // symmetric product; the single form stores these one by one, at any address.
+    auto bits = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
+    const bool aligned = ((bits(g.C) | bits(g.Ch) | bits(g.Cl) | bits(g.CT) | bits(g.CTh) | bits(g.CTl) | bits(g.C64)) & 15) == 0 &&
                          g.sC % 4 == 0;
     const int form = tc_form() == 0 && !aligned ? 1 : tc_form();
     if (g.nslots && form != 0) {   // the other forms take the items one by one

@@ -87,3 +87,25 @@ def test_lower_tiles_in_place():
     assert torch.equal(C[~low], upper[~low])
     d = (C.double() - ref).abs()[low].max().item()
     assert d <= TOL[2] * (A.double().abs() @ A.double().abs().T).max().item()
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+@pytest.mark.parametrize("kind", [0, 1, 2])
+def test_one_symmetric_tile_at_any_address(kind, shift):
+    # a tile on the diagonal is stored entry by entry where its outputs do not start on 16 bytes
+    import torch
+    n, k = 128, 192
+    A, hi, lo = _operands(n, k, kind, 21)
+    part = torch.bfloat16 if kind == 1 else torch.float32
+    at = lambda dtype: torch.zeros(n * n + 4, dtype=dtype, device="cuda")[shift:shift + n * n].view(n, n)
+    C, H, L = at(torch.float32), at(part), at(part)
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rc = binding.mbdk_gemm_tc(kind, hi, hi, C, A1=lo, B1=lo, C_hi=H if kind else None, C_lo=L if kind else None, mode=2, err=err,
+                              chunk_stages=1)
+    torch.cuda.synchronize()
+    assert rc == 0 and err.item() == 0 and torch.equal(C, C.T)
+    ref = A.double() @ A.double().T
+    assert (C.double() - ref).abs().max().item() <= TOL[kind] * (A.double().abs() @ A.double().abs().T).max().item()
+    if kind:
+        h, l = _parts(C, kind)
+        assert torch.equal(H, h) and torch.equal(L, l)
