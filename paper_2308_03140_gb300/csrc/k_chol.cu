@@ -27,25 +27,28 @@ namespace {
 using crt::kMod;
 
 // exps[b][r] of the rows of the factor, from the diagonal, and left[b][r]: the sum of squares that the row's scaled
-// entries may reach (negative for a bad row).
+// entries may reach, in units of 2^64 (negative for a bad row).
 __global__ void k_factor_exponents(const double *A, long long ld, long long mstride, int *exps, float *left) {
     const long long r = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x, b = blockIdx.y;
     if (r >= ld) return;
     const double d = A[b * mstride + r * ld + r];
     const int e = crt::row_exponent(sqrt(d) * (1.0 + 1e-6));   // (the root of a negative diagonal is NaN: a bad row)
     exps[b * ld + r] = e == crt::kBadRow ? e : min(e, 1000);
-    const double root = e == crt::kBadRow ? 0.0 : sqrt(d) * crt::pow2(min(e, 1000));   // below 2^59
+    const double root = e == crt::kBadRow ? 0.0 : sqrt(d) * crt::pow2(min(e, 1000) - 32);   // below 2^27
     left[b * ld + r] = e == crt::kBadRow ? -1.0f : static_cast<float>(1.001 * root * root);
 }
 
-// Two neighbouring entries' residues, bf16 pairs into the planes at `out`.
-__device__ __forceinline__ void put2(double v0, double v1, double scale, long long plane, __nv_bfloat16 *out) {
+// Two neighbouring entries' residues, bf16 pairs into the planes at `out`.  Returns the sum of their scaled squares in units
+// of 2^64, from the upper limbs: to 2^-26 of what a row may reach.
+__device__ __forceinline__ float put2(double v0, double v1, double scale, long long plane, __nv_bfloat16 *out) {
     const crt::Limbs l0 = crt::limbs(__double2ll_rn(v0 * scale)), l1 = crt::limbs(__double2ll_rn(v1 * scale));
     crt::each_modulus([&](auto I) {
         constexpr int k = decltype(I)::value;
         const uint32_t f0 = __float_as_uint(crt::residue<k>(l0)), f1 = __float_as_uint(crt::residue<k>(l1));
         *reinterpret_cast<uint32_t *>(out + k * plane) = __byte_perm(f0, f1, 0x7632);
     });
+    const float x0 = 65536.0f * l0.l3 + l0.l2, x1 = 65536.0f * l1.l3 + l1.l2;
+    return x0 * x0 + x1 * x1;
 }
 // 2^e (exponents are kept at most 1000: rows below 1e-283 keep fewer bits); zero for bad rows.
 __device__ __forceinline__ double row_scale(int e) { return e == crt::kBadRow ? 0.0 : crt::pow2(e); }
@@ -116,7 +119,7 @@ __global__ void __launch_bounds__(256) k_column(double *A, long long ld, long lo
 // Row r = j0 + 64 + rr of the solved block, a warp per row: FP64 values from the product's bytes, and
 // residues at the row's exponent in the panel's planes ([b][kMod][ld][pitch], columns from kcol).  The squares of the scaled
 // entries are taken from left[b][r], which this launch alone touches: in FP32, whose 1e-7 a block of columns is far
-// inside the 0.1 % and whose sums over the warp cost a sixteenth of FP64's.
+// inside the 0.1 %, as FP64 sums over the warp would take the pipe that bounds this kernel.
 __global__ void __launch_bounds__(256) k_solve(double *A, long long ld, long long mstride, int j0, int m,
                                                const uint8_t *Y, const int *rexps, long long rstride, const int *dexps,
                                                const int *fexps, __nv_bfloat16 *planes, int pitch, int kcol, float *left,
@@ -132,9 +135,11 @@ __global__ void __launch_bounds__(256) k_solve(double *A, long long ld, long lon
     v[1] = crt::scaled_down(v[1], er, ec.y);
     *reinterpret_cast<double2 *>(A + b * mstride + r * ld + j0 + 2 * lane) = make_double2(v[0], v[1]);
     const int e = fexps[b * ld + r];
-    const double scale = row_scale(e);
-    const float x0 = static_cast<float>(v[0] * scale), x1 = static_cast<float>(v[1] * scale);
-    float used = x0 * x0 + x1 * x1;
+    const bool fine = fabs(v[0]) <= crt::kMaxDouble && fabs(v[1]) <= crt::kMaxDouble;
+    if (e == crt::kBadRow || !fine) v[0] = v[1] = 0.0;   // (a factorisation that has failed)
+    const long long pp = ld * pitch;
+    float used = put2(v[0], v[1], row_scale(e), pp, planes + b * kMod * pp + r * pitch + kcol + 2 * lane);
+    if (!fine) used = CUDART_INF_F;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) used += __shfl_xor_sync(0xffffffffu, used, o);
     if (lane == 0) {
@@ -142,10 +147,6 @@ __global__ void __launch_bounds__(256) k_solve(double *A, long long ld, long lon
         left[b * ld + r] = rest;
         if (!(rest >= 0.0f)) atomicOr(status, ST_SCS_NOT_PD);
     }
-    if (e == crt::kBadRow || !(fabs(v[0]) <= crt::kMaxDouble)) v[0] = 0.0;   // (a factorisation that has failed)
-    if (e == crt::kBadRow || !(fabs(v[1]) <= crt::kMaxDouble)) v[1] = 0.0;
-    const long long pp = ld * pitch;
-    put2(v[0], v[1], scale, pp, planes + b * kMod * pp + r * pitch + kcol + 2 * lane);
 }
 
 // 1 / d to about an ulp, d a normal number: two Newton steps from the hardware's approximation.
