@@ -151,6 +151,7 @@ struct mbd_ctx {
     double *dPT = nullptr;
     char *qwork = nullptr;   // cells: scratch of the Q(q) build's products (null: it runs on the FP64 pipe)
     size_t qwork_bytes = 0;
+    void *qslab = nullptr;   // qwork's own memory, once a changed lattice needed more than the slab's
     bool no_scratch = false;   // the scratch of the tensor-core products did not fit the card
     double *dkq = nullptr, *dkw = nullptr, *dG = nullptr, *dcoef = nullptr, *dlzw = nullptr, *dgA = nullptr, *dgAout = nullptr,
            *dgApart = nullptr, *dgc = nullptr, *dtsg = nullptr;
@@ -258,6 +259,8 @@ double span_ms(cudaEvent_t a, cudaEvent_t b) {
 void release(mbd_ctx *ctx) {
     if (ctx->slab) cudaFree(ctx->slab);
     ctx->slab = nullptr;
+    if (ctx->qslab) cudaFree(ctx->qslab);
+    ctx->qslab = nullptr;
     ctx->slab_bytes = 0;
 }
 
@@ -531,6 +534,8 @@ int allocate(mbd_ctx *ctx, bool groups = true) {
     const bool crt = crt_work && ctx->slab_bytes >= bytes + crt_work;
     ctx->no_scratch = crt_work && !crt;
     ctx->qwork_bytes = crt ? q_work : 0;
+    if (ctx->qslab) cudaFree(ctx->qslab);
+    ctx->qslab = nullptr;
     char *scratch = crt ? static_cast<char *>(ctx->slab) + bytes + pt_part : nullptr;
     ctx->dPT = crt && pt_part ? reinterpret_cast<double *>(static_cast<char *>(ctx->slab) + bytes) : nullptr;
     ctx->crt = pt_part ? scratch : nullptr;
@@ -1685,9 +1690,7 @@ int mbd_set_geometry(mbd_ctx *ctx, int n_atoms, const double *coords, const doub
     }
     MBD_CUDA(cudaSetDevice(ctx->device), "mbd_set_geometry");
     const bool realloc = (n_atoms != ctx->N) || !ctx->slab || periodic != ctx->periodic ||
-                         (periodic && (ps.nk != ctx->nk || ps.nG != ctx->nG || ps.maxG != ctx->maxG)) ||
-                         (periodic && !ctx->no_scratch &&   // (the image table's size depends on the lattice)
-                          cell_products_bytes(n_atoms, ps.cell, ps.nk, ps.maxG, ctx->opt.precision) > ctx->qwork_bytes);
+                         (periodic && (ps.nk != ctx->nk || ps.nG != ctx->nG || ps.maxG != ctx->maxG));
     ctx->N = n_atoms;
     ctx->n = 3 * n_atoms;
     ctx->ld = (ctx->n + 127) / 128 * 128;   // 128: the tensor-core tile (also a multiple of 64)
@@ -1718,6 +1721,20 @@ int mbd_set_geometry(mbd_ctx *ctx, int n_atoms, const double *coords, const doub
         if (rc) { ctx->have_geom = false; return rc; }
     }
     if (periodic) {
+        // The image tables' size depends on the lattice.  More scratch for a changed one comes beside the slab, whose
+        // parameters and last evaluation stay; where it does not fit, the cell takes the direct kernels.
+        const size_t need = ctx->no_scratch ? 0 : cell_products_bytes(n_atoms, ps.cell, ps.nk, ps.maxG, ctx->opt.precision);
+        void *more = nullptr;
+        if (need > ctx->qwork_bytes) {
+            if (cudaMalloc(&more, need) == cudaSuccess) {
+                if (ctx->qslab) cudaFree(ctx->qslab);
+                ctx->qslab = more;
+                ctx->qwork = static_cast<char *>(more);
+                ctx->qwork_bytes = need;
+            } else {
+                cudaGetLastError();
+            }
+        }
         const int rc = upload_periodic(ctx);
         if (rc) { ctx->have_geom = false; return rc; }
     }
