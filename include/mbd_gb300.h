@@ -261,6 +261,12 @@ int mbd_ts_energy(mbd_ctx *ctx, double s_r, double *energy, double *grad_coords,
 int mbd_get_stats(mbd_ctx *ctx, int *ns_iterations, double *ns_scale, double *ns_residual,
                   double *correction_residual);
 
+/* What mbd_set_geometry found room for on the device.  tensor_products: 1 if the FP64 products and factorisations (and a
+ * cell's Q(q) and gradient sums) have the scratch they need on the tensor cores, 0 if it did not fit and they run
+ * on the FP64 pipe with the same accuracy, up to 30 times slower; matrices_together: Bloch vectors that the mixed modes
+ * iterate on at a time.  Either may be NULL.  MBD_ERR_STATE before mbd_set_geometry. */
+int mbd_get_workspace(const mbd_ctx *ctx, int *tensor_products, int *matrices_together);
+
 /* Device-time profile of the last evaluation, gathered with CUDA events on the stream
  * the work was launched on when profiling is enabled (mbd_set_profiling).  Times in
  * milliseconds; flops are the algorithmic counts of the listed kernels (2 m n k for a

@@ -28,7 +28,7 @@ EXPORTS = ("mbd_default_options", "mbd_create", "mbd_destroy", "mbd_set_geometry
            "mbd_get_evaluation_count",
            "mbd_get_lattice_gradient", "mbd_set_scs_model", "mbd_get_learned_stats", "mbd_screen",
            "mbd_get_scs_detail", "mbd_log_energy", "mbd_ts_energy",
-           "mbd_get_stats", "mbd_get_exception", "mbd_set_profiling", "mbd_get_profile",
+           "mbd_get_stats", "mbd_get_workspace", "mbd_get_exception", "mbd_set_profiling", "mbd_get_profile",
            "mbdk_gemm_f64", "mbdk_gemm_tc", "mbdk_tc_wait_check", "mbdk_gemm_f64_split", "mbdk_gemm_f64_split_work_bytes", "mbdk_cholesky_f64", "mbdk_chol_solve3_f64",
            "mbdk_cholesky_solve3_f64_noalloc", "mbdk_scs_features", "mbdk_mlp_forward", "mbdk_mlp_backward",
            "mbdk_mse_grad", "mbdk_adam_step", "mbdk_learned_targets", "mbdk_gather_rows")
@@ -87,6 +87,7 @@ def load(path: str | None = None):
     L.mbd_get_learned_stats.argtypes = [vp, _P, C.POINTER(C.c_int)]
     L.mbd_screen.argtypes = [vp, _P, _P, _P, _P, _P]
     L.mbd_get_stats.argtypes = [vp, C.POINTER(C.c_int), _P, _P, _P]
+    L.mbd_get_workspace.argtypes = [vp, C.POINTER(C.c_int), C.POINTER(C.c_int)]
     L.mbd_log_energy.argtypes = [vp, C.c_int, _P, _P]
     L.mbd_ts_energy.argtypes = [vp, C.c_double, _P, _P, _P, _P]
     L.mbd_get_exception.argtypes = [vp, C.POINTER(C.c_int), C.c_char_p, C.c_char_p, sz]
@@ -331,6 +332,13 @@ class MBD:
         self._check(self.lib.mbd_get_stats(self.h, C.byref(it), C.byref(sc), C.byref(res), C.byref(cr)))
         return dict(ns_iterations=it.value, ns_scale=sc.value, ns_residual=res.value,
                     correction_residual=cr.value)
+
+    def workspace(self):
+        """What set_geometry found room for (mbd_get_workspace): whether the FP64 products run on the tensor cores, and
+        how many Bloch vectors the mixed modes iterate on together."""
+        tc, group = C.c_int(), C.c_int()
+        self._check(self.lib.mbd_get_workspace(self.h, C.byref(tc), C.byref(group)))
+        return dict(tensor_products=bool(tc.value), matrices_together=group.value)
 
 
 def _stream(t, stream):

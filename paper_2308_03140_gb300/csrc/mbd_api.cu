@@ -2041,6 +2041,14 @@ int mbd_get_stats(mbd_ctx *ctx, int *ns_iterations, double *ns_scale, double *ns
     return MBD_OK;
 }
 
+int mbd_get_workspace(const mbd_ctx *ctx, int *tensor_products, int *matrices_together) {
+    if (!ctx) return MBD_ERR_INPUT;
+    if (!ctx->have_geom) return MBD_ERR_STATE;
+    if (tensor_products) *tensor_products = ctx->no_scratch ? 0 : 1;
+    if (matrices_together) *matrices_together = ctx->mgroup;
+    return MBD_OK;
+}
+
 int mbd_set_profiling(mbd_ctx *ctx, int enable) {
     if (!ctx) return MBD_ERR_INPUT;
     ctx->profiling = enable != 0;
