@@ -5,6 +5,8 @@
 #include <cstddef>
 #include <cstdint>
 
+struct mbd_ctx;
+
 namespace mbdgb {
 
 constexpr int kTile = 64;          // dense tile edge; leading dimensions are multiples of it
@@ -77,6 +79,19 @@ size_t gemm_f64_split_work_bytes(int M, int N, int K);
 cudaError_t gemm_f64_split(int trans_b, int mode, int M, int N, int K, double alpha, const double *A, long long lda,
                            const double *B, long long ldb, double beta, const double *D, long long ldd, double *C,
                            long long ldc, void *work, int *err, cudaStream_t s);
+// Bounds on the scratch of the products on the tensor cores.  A context has these; the tests give one others before
+// mbd_set_geometry, so that small systems take the groups, strips, panels and kernels of large ones or of a full card.
+struct ScratchLimits {
+    bool none = false;                         // as where the scratch does not fit: the FP64 pipe, one Bloch vector at a time
+    int panel = 8192;                          // columns and K of a panel of a real product: the planes of a matrix of order n
+                                               // then take at most 30 n panel bytes, and all of the scratch 17 GB at
+                                               // n = 41000, the largest order that fits the card
+    size_t trailing = size_t{1} << 30;         // bytes of a trailing product of the Cholesky factorisation (a group of
+    int strip = 2048;                          // whole matrices, or strips of columns of one, of at least as many)
+    size_t cell_products = size_t{2} << 30;    // of a group of Bloch vectors' Newton-Schulz products: at order 768 16, which are
+                                               // 48 times the chip in tiles (the full grid gains nothing and costs 7 GB)
+    size_t cell_sums = size_t{1} << 30;        // of a group of the Q(q) build, or of either part of the cell gradient
+};
 // FP64-accurate products on the bf16 tensor cores by residues (k_crt.cu, crt64.cuh).  An operand
 // is an array of rows along K: A's rows, or the columns of B (the rows of B^T).  crt_rows turns it into
 // residue planes in caller memory of crt_operand_bytes; crt_multiply forms
@@ -118,13 +133,10 @@ cudaError_t crt_products(const CrtOperand &A, const CrtOperand &B, int M, int ha
 cudaError_t crt_multiply(const CrtOperand &A, const CrtOperand &B, const CrtResult &r, void *bytes, int *err,
                          cudaStream_t st);
 // C = alpha A B + beta D for real operands of any size through crt_gemm_bytes of scratch, in panels
-// of columns and of K when they are long.  Bt: the rows of B^T.
-// Columns and K of one panel: the planes of a matrix of order n then take at most 30 n kCrtBlock
-// bytes, and all of the scratch 17 GB at n = 41000, the largest order that fits the card.
-constexpr int kCrtBlock = 8192;
-size_t crt_gemm_bytes(int M, int N, int K);
+// of columns and of K when they are long.  Bt: the rows of B^T.  panel: an even number.
+size_t crt_gemm_bytes(int M, int N, int K, int panel = ScratchLimits{}.panel);
 cudaError_t crt_gemm(const double *A, long long lda, const double *Bt, long long ldb, int M, int N, int K,
-                     const CrtResult &r, void *work, int *err, cudaStream_t st);
+                     const CrtResult &r, void *work, int *err, cudaStream_t st, int panel = ScratchLimits{}.panel);
 
 // Mixed-precision helpers: Y = scale Q (FP32 and, if Yh, bf16 hi/lo) and Z = I;
 // Z = a I + b P; Zd = scale Zf in FP64.
@@ -180,9 +192,9 @@ void cholesky_f64(double *A, long long ld, long long mstride, int batch, double 
 
 // The same factorisation with its products on the tensor cores (k_chol.cu), through
 // cholesky_crt_bytes of scratch; tensor-core timeouts set ST_TC_TIMEOUT in *status.  ld a multiple of 128.
-size_t cholesky_crt_bytes(long long ld, int batch);
+size_t cholesky_crt_bytes(long long ld, int batch, const ScratchLimits &lim = {});
 cudaError_t cholesky_crt(double *A, long long ld, long long mstride, int batch, double *dinv, void *work, int *status,
-                         cudaStream_t s);
+                         cudaStream_t s, const ScratchLimits &lim = {});
 
 // Batched triangular solves with 3 right-hand sides, in place on X [b][ld][3]:
 // forward L y = x, then backward L^T z = y (L from cholesky_f64).  work: same shape
@@ -356,9 +368,9 @@ void build_q_periodic(const AtomBufs &b, const PeriodicBufs &p, double beta, dou
                       int n, int *status, cudaStream_t s);
 // The same with the reciprocal sums as residue products (k_qbuild.cu) through build_q_products_bytes of
 // scratch (0: not for this cell, whose image table would be too large); without the padding.
-size_t build_q_products_bytes(int N, const CellGeom &c, int nk, int maxG);
+size_t build_q_products_bytes(int N, const CellGeom &c, int nk, int maxG, const ScratchLimits &lim = {});
 cudaError_t build_q_products(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, double *Q, long long ld,
-                             void *work, int *status, cudaStream_t s);
+                             void *work, int *status, cudaStream_t s, const ScratchLimits &lim = {});
 void pad_q_periodic(const AtomBufs &b, const PeriodicBufs &p, double *Q, long long ld, int n, cudaStream_t s);
 // Batched complex helpers (nk planar matrices of order ld).
 void cscale(double *Y, long long ld, int nk, double scale, cudaStream_t s);
@@ -394,13 +406,14 @@ void energy_trace_periodic(const double *Y, long long ld, int n, const PeriodicB
 // timeouts set ST_TC_TIMEOUT in *status.
 cudaError_t periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, const double *Z,
                               long long ld, double zscale, const MbdGradOut &o, double *work, double *gA, cudaStream_t s,
-                              const double *tq, bool f32_recip, void *products, int *status);
+                              const double *tq, bool f32_recip, void *products, int *status,
+                              const ScratchLimits &lim = {});
 // Its real-space and, with recip, reciprocal sums through products (0 bytes: not for this cell), added to g_c, g_rbar,
 // gR and gA.
-size_t grad_products_bytes(int N, const CellGeom &c, int nk, int maxG);
+size_t grad_products_bytes(int N, const CellGeom &c, int nk, int maxG, const ScratchLimits &lim = {});
 cudaError_t grad_products(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, const double *Z, long long ld,
                           double zscale, double *g_c, double *g_rbar, double *gR, double *gA, bool recip, void *work,
-                          int *status, cudaStream_t s);
+                          int *status, cudaStream_t s, const ScratchLimits &lim = {});
 // out[i] = (1/rows) sum_r x[r][i] for a rows x N array (compensated).
 void mean_rows(const double *x, int rows, int N, double *out, cudaStream_t s);
 // SCS adjoint pair pass over lattice images (as scs_grad_pass), with the lattice part
@@ -459,5 +472,8 @@ void learned_forces(int N, const int *offsets, const double *R, const double *a0
 // the members): the energy-error estimate per atom from the members' first-order energies.
 void learned_estimate(int N, int nf1, int members, double scale, const double *h, const double *al_u,
                       const float *Y, double *out, cudaStream_t s);
+
+// The limits of a context's scratch from its next mbd_set_geometry on (mbd_api.cu).
+void set_scratch_limits(mbd_ctx *ctx, const ScratchLimits &lim);
 
 }  // namespace mbdgb

@@ -338,15 +338,13 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256)
 // Columns of a panel.  Its planes take 480 ld kPanel bytes for 16 matrices; each panel passes the
 // trailing matrix through memory once.
 constexpr int kPanel = 512;
-// Bytes of a trailing product at most (a group of whole matrices, or strips of columns of one).
-constexpr size_t kTrailingBytes = size_t{1} << 30;
 
 inline size_t al(size_t b) { return (b + 255) / 256 * 256; }
 
 struct Layout {
     long long panel, rows, inverse, exps, rexps, dexps, left, bytes, total;   // offsets
 };
-Layout layout(long long ld, int batch) {
+Layout layout(long long ld, int batch, const ScratchLimits &lim) {
     Layout l;
     size_t p = 0;
     auto take = [&](size_t n) {
@@ -363,19 +361,21 @@ Layout layout(long long ld, int batch) {
     l.dexps = take(4 * static_cast<size_t>(batch) * 64);
     l.left = take(4 * static_cast<size_t>(batch) * ld);
     const size_t m = ld > kPanel ? static_cast<size_t>(ld) - kPanel : 0, whole = kMod * m * m;
-    const size_t strip = kMod * m * std::min<size_t>(m, 2048);   // at least a strip of 2048 columns
-    l.bytes = take(std::max<size_t>(z * ld * 64, std::min<size_t>(whole * batch, std::max<size_t>(kTrailingBytes, strip))));
+    const size_t strip = kMod * m * std::min<size_t>(m, lim.strip);
+    l.bytes = take(std::max<size_t>(z * ld * 64, std::min<size_t>(whole * batch, std::max<size_t>(lim.trailing, strip))));
     l.total = static_cast<long long>(p);
     return l;
 }
 
 }  // namespace
 
-size_t cholesky_crt_bytes(long long ld, int batch) { return static_cast<size_t>(layout(ld, batch).total); }
+size_t cholesky_crt_bytes(long long ld, int batch, const ScratchLimits &lim) {
+    return static_cast<size_t>(layout(ld, batch, lim).total);
+}
 
 cudaError_t cholesky_crt(double *A, long long ld, long long mstride, int batch, double *dinv, void *work, int *status,
-                         cudaStream_t s) {
-    const Layout l = layout(ld, batch);
+                         cudaStream_t s, const ScratchLimits &lim) {
+    const Layout l = layout(ld, batch, lim);
     char *w = static_cast<char *>(work);
     auto *panel = reinterpret_cast<__nv_bfloat16 *>(w + l.panel), *rows = reinterpret_cast<__nv_bfloat16 *>(w + l.rows),
          *inverse = reinterpret_cast<__nv_bfloat16 *>(w + l.inverse);

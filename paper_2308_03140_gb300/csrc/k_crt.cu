@@ -737,22 +737,22 @@ cudaError_t crt_multiply(const CrtOperand &A, const CrtOperand &B, const CrtResu
     return cudaGetLastError();
 }
 
-size_t crt_gemm_bytes(int M, int N, int K) {
-    const int kb = std::min(K, kCrtBlock), nb = std::min(N, kCrtBlock);
+size_t crt_gemm_bytes(int M, int N, int K, int panel) {
+    const int kb = std::min(K, panel), nb = std::min(N, panel);
     return crt_operand_bytes(crt_shape(M, kb, 1, false, false)) + crt_operand_bytes(crt_shape(nb, kb, 1, false, true)) +
            crt_bytes_bytes(M, nb, 1);
 }
 
 cudaError_t crt_gemm(const double *A, long long lda, const double *Bt, long long ldb, int M, int N, int K,
-                     const CrtResult &r, void *work, int *err, cudaStream_t st) {
-    for (int k0 = 0; k0 < K; k0 += kCrtBlock) {
-        const int kb = std::min(K - k0, kCrtBlock);
+                     const CrtResult &r, void *work, int *err, cudaStream_t st, int panel) {
+    for (int k0 = 0; k0 < K; k0 += panel) {
+        const int kb = std::min(K - k0, panel);
         char *p = static_cast<char *>(work);
         const CrtShape sa = crt_shape(M, kb, 1, false, false);
         const CrtOperand a = crt_rows(sa, A + k0, nullptr, lda, 0, false, p, st);
         p += crt_operand_bytes(sa);
-        for (int n0 = 0; n0 < N; n0 += kCrtBlock) {
-            const int nb = std::min(N - n0, kCrtBlock);
+        for (int n0 = 0; n0 < N; n0 += panel) {
+            const int nb = std::min(N - n0, panel);
             const CrtShape sb = crt_shape(nb, kb, 1, false, true);
             const CrtOperand b = crt_rows(sb, Bt + n0 * ldb + k0, nullptr, ldb, 0, false, p, st);
             CrtResult rp = r;

@@ -936,7 +936,7 @@ void mean_rows(const double *x, int rows, int N, double *out, cudaStream_t s) {
 
 cudaError_t periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, const double *Z,
                               long long ld, double zscale, const MbdGradOut &o, double *work, double *gA, cudaStream_t s,
-                              const double *tq, bool f32_recip, void *products, int *status) {
+                              const double *tq, bool f32_recip, void *products, int *status, const ScratchLimits &lim) {
     double *g_c = work;
     cudaMemsetAsync(g_c, 0, sizeof(double) * b.N, s);
     cudaMemsetAsync(o.g_rbar, 0, sizeof(double) * b.N, s);
@@ -946,7 +946,7 @@ cudaError_t periodic_mbd_grad(const AtomBufs &b, const PeriodicBufs &p, double b
     count_launches(2);
     const dim3 grid(ntile * (ntile + 1) / 2, p.nk);
     cudaError_t e = cudaSuccess;
-    if (products) e = grad_products(b, p, beta, a, Z, ld, zscale, g_c, o.g_rbar, o.gR, gA, !f32_recip, products, status, s);
+    if (products) e = grad_products(b, p, beta, a, Z, ld, zscale, g_c, o.g_rbar, o.gR, gA, !f32_recip, products, status, s, lim);
     if (f32_recip && products)
         k_mbd_grad_periodic<float, false><<<grid, 256, 0, s>>>(b, p, beta, a, Z, ld, zscale, ntile, g_c, o.g_rbar, o.gR, gA);
     else if (f32_recip)

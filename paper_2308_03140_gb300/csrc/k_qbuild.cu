@@ -172,10 +172,9 @@ struct Layout {
     CrtShape left, right;
     size_t images, weights, lrows, rrows, lplanes, rplanes, bytes, rec, total;   // offsets
 };
-constexpr size_t kGroupBytes = size_t{1} << 30;    // of the product's arrays: 4 Bloch vectors of the 256-atom cell,
-                                                   // nine times the chip in tiles
 constexpr size_t kImageBytes = size_t{512} << 20;  // of the image table at most
-Layout layout(int N, const CellGeom &c, int nk, int maxG) {
+// Groups of lim.cell_sums bytes of the product's arrays: 4 Bloch vectors of the 256-atom cell, nine times the chip in tiles.
+Layout layout(int N, const CellGeom &c, int nk, int maxG, const ScratchLimits &lim) {
     Layout l{};
     l.slots = 1;
     double slots = 1.0;
@@ -207,7 +206,7 @@ Layout layout(int N, const CellGeom &c, int nk, int maxG) {
         l.rplanes = take(crt_operand_bytes(l.right));
         l.bytes = take(crt_bytes_bytes(6 * N, l.right.out_rows, l.group));
         l.rec = take(8 * z * 12 * n * l.ldr);
-        if (p <= kGroupBytes || l.group == 1) {
+        if (p <= lim.cell_sums || l.group == 1) {
             l.images = p;
             l.total = p + al(static_cast<size_t>(48.0 * pairs) * l.slots);
             return l;
@@ -217,11 +216,13 @@ Layout layout(int N, const CellGeom &c, int nk, int maxG) {
 
 }  // namespace
 
-size_t build_q_products_bytes(int N, const CellGeom &c, int nk, int maxG) { return layout(N, c, nk, maxG).total; }
+size_t build_q_products_bytes(int N, const CellGeom &c, int nk, int maxG, const ScratchLimits &lim) {
+    return layout(N, c, nk, maxG, lim).total;
+}
 
 cudaError_t build_q_products(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, double *Q, long long ld,
-                             void *work, int *status, cudaStream_t s) {
-    const Layout l = layout(b.N, p.cell, p.nk, p.maxG);
+                             void *work, int *status, cudaStream_t s, const ScratchLimits &lim) {
+    const Layout l = layout(b.N, p.cell, p.nk, p.maxG, lim);
     char *w = static_cast<char *>(work);
     auto at = [&](size_t o) { return reinterpret_cast<double *>(w + o); };
     const int ntile = cdiv(b.N, kQT), tiles = ntile * (ntile + 1) / 2;

@@ -283,8 +283,9 @@ struct Layout {
     size_t table, tplanes, rows, yplanes, ybytes, ab;              // offsets, real part
     size_t total;
 };
-constexpr size_t kPartBytes = size_t{1} << 30;   // of either part where a smaller group of vectors or pairs allows it
-Layout layout(int N, const CellGeom &c, int nk, int maxG) {
+constexpr size_t kMostBytes = size_t{8} << 30;
+// Groups of vectors and chunks of pairs of lim.cell_sums bytes each.
+Layout layout(int N, const CellGeom &c, int nk, int maxG, const ScratchLimits &lim) {
     Layout l{};
     double slots = 1.0;
     for (int k = 0; k < 3; ++k) {
@@ -314,7 +315,7 @@ Layout layout(int N, const CellGeom &c, int nk, int maxG) {
         l.rplanes = take(crt_operand_bytes(right));
         l.bytes = take(crt_bytes_bytes(6 * N, right.out_rows, l.group));
         l.out = take(8 * z * 12 * n * l.ldg);
-        if (p <= kPartBytes || l.group == 1) break;
+        if (p <= lim.cell_sums || l.group == 1) break;
     }
     l.total = p;
     const int ntile = cdiv(N, kQT);
@@ -328,21 +329,23 @@ Layout layout(int N, const CellGeom &c, int nk, int maxG) {
         l.yplanes = take(crt_operand_bytes(crt_shape(rows, 2 * nk, 1, false, false)));
         l.ybytes = take(crt_bytes_bytes(rows, l.ldab, 1));
         l.ab = take(8 * static_cast<size_t>(rows) * l.ldab);
-        if (p <= kPartBytes || l.chunk == 256) break;
+        if (p <= lim.cell_sums || l.chunk == 256) break;
     }
     l.total = std::max(l.total, p);
-    if (l.total > 8 * kPartBytes) l.total = 0;   // (thousands of atoms, or grids of tens of thousands of vectors)
+    if (l.total > kMostBytes) l.total = 0;   // (thousands of atoms, or grids of tens of thousands of vectors)
     return l;
 }
 
 }  // namespace
 
-size_t grad_products_bytes(int N, const CellGeom &c, int nk, int maxG) { return layout(N, c, nk, maxG).total; }
+size_t grad_products_bytes(int N, const CellGeom &c, int nk, int maxG, const ScratchLimits &lim) {
+    return layout(N, c, nk, maxG, lim).total;
+}
 
 cudaError_t grad_products(const AtomBufs &b, const PeriodicBufs &p, double beta, double a, const double *Z, long long ld,
                           double zscale, double *g_c, double *g_rbar, double *gR, double *gA, bool recip, void *work,
-                          int *status, cudaStream_t s) {
-    const Layout l = layout(b.N, p.cell, p.nk, p.maxG);
+                          int *status, cudaStream_t s, const ScratchLimits &lim) {
+    const Layout l = layout(b.N, p.cell, p.nk, p.maxG, lim);
     char *w = static_cast<char *>(work);
     auto at = [&](size_t o) { return reinterpret_cast<double *>(w + o); };
     for (int k0 = 0; recip && k0 < p.nk; k0 += l.group) {

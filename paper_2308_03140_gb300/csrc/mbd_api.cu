@@ -116,6 +116,7 @@ struct mbd_ctx {
     // device memory: one slab, carved
     void *slab = nullptr;
     size_t slab_bytes = 0;
+    ScratchLimits lim;
     double *dR, *da0ref, *dc6ref, *drref, *dratio;
     double *da0, *dom, *drv, *dalu, *dsigu, *dabar, *dabar0, *dc6bar, *dombar, *drbar, *du, *dwu;
     double *dM, *ddinv, *dX, *dV, *dB;
@@ -319,8 +320,8 @@ int ensure_learned(mbd_ctx *ctx) {
 
 // Scratch of the FP64 path's products for matrices of order n: three operands' residue planes and a
 // product's bytes while a matrix is one panel, else that of products in panels.
-size_t crt_ns_bytes(int n) {
-    if (n > kCrtBlock) return crt_gemm_bytes(n, n, n);
+size_t crt_ns_bytes(int n, const ScratchLimits &lim) {
+    if (n > lim.panel) return crt_gemm_bytes(n, n, n, lim.panel);
     return 3 * crt_operand_bytes(crt_shape(n, n, 1, false, false)) + crt_bytes_bytes(n, n, 1);
 }
 
@@ -338,14 +339,14 @@ struct CrtProducts {
         for (int k = 0; k < 3; ++k) slot[k] = c->crt + k * b;
         bytes = c->crt + 3 * b;
     }
-    bool panels() const { return ctx->n > kCrtBlock; }
+    bool panels() const { return ctx->n > ctx->lim.panel; }
     CrtOperand rows(const double *X, int k) { return crt_rows(shape, X, nullptr, ctx->ld, 0, false, slot[k], s); }
     CrtResult result(double *C, double *T, double alpha, double beta, const double *D, bool sym) const {
         const long long ld = ctx->ld;
         return CrtResult{alpha, beta, D, C, T, ld, ld, ld, 0, 0, 0, 0, 0, sym ? 1 : 0};
     }
     cudaError_t whole(const double *A, const double *Bt, const CrtResult &r) {
-        return crt_gemm(A, ctx->ld, Bt, ctx->ld, ctx->n, ctx->n, ctx->n, r, ctx->crt, ctx->dstatus, s);
+        return crt_gemm(A, ctx->ld, Bt, ctx->ld, ctx->n, ctx->n, ctx->n, r, ctx->crt, ctx->dstatus, s, ctx->lim.panel);
     }
     // P = Z Y and its transpose
     cudaError_t product(const double *Z, const double *Y, double *P, double *PT) {
@@ -375,16 +376,15 @@ struct CrtProducts {
     }
 };
 
-// Bloch vectors per complex product, and its scratch: as many as 2 GiB hold, which at order 768 is
-// 16, 48 times the chip in tiles (the full grid at once gains nothing and costs 7 GB).
-int crt_cell_group(int n, int nk) {
+// Bloch vectors per complex product, and its scratch.
+int crt_cell_group(int n, int nk, const ScratchLimits &lim) {
     const size_t one = crt_operand_bytes(crt_shape(n, n, 1, true, false)) +
                        crt_operand_bytes(crt_shape(n, n, 1, true, true)) +
                        crt_bytes_bytes(n, crt_shape(n, n, 1, true, true).out_rows, 1);
-    return static_cast<int>(std::min<size_t>(nk, std::max<size_t>(1, (size_t{2} << 30) / one)));
+    return static_cast<int>(std::min<size_t>(nk, std::max<size_t>(1, lim.cell_products / one)));
 }
-size_t crt_cell_bytes(int n, int nk) {
-    const int g = crt_cell_group(n, nk);
+size_t crt_cell_bytes(int n, int nk, const ScratchLimits &lim) {
+    const int g = crt_cell_group(n, nk, lim);
     return crt_operand_bytes(crt_shape(n, n, g, true, false)) + crt_operand_bytes(crt_shape(n, n, g, true, true)) +
            crt_bytes_bytes(n, crt_shape(n, n, g, true, true).out_rows, g);
 }
@@ -393,7 +393,7 @@ size_t crt_cell_bytes(int n, int nk) {
 // (conj: from the rows of a Hermitian B); T: also the transpose; sym: Hermitian results.
 cudaError_t crt_cell_product(mbd_ctx *ctx, const double *A, const double *Bt, bool conj, const double *D, double *C,
                              double *T, double alpha, double beta, bool sym, cudaStream_t s) {
-    const int n = ctx->n, group = crt_cell_group(n, ctx->nk);
+    const int n = ctx->n, group = crt_cell_group(n, ctx->nk, ctx->lim);
     const long long ld = ctx->ld, m2 = ld * ld, st = 2 * m2;
     for (int k0 = 0; k0 < ctx->nk; k0 += group) {
         const int g = std::min(group, ctx->nk - k0);
@@ -416,7 +416,7 @@ int factorise(mbd_ctx *ctx, double *A, int batch, cudaStream_t s, const char *or
         cholesky_f64(A, ld, ld * ld, batch, ctx->ddinv, ctx->dstatus, s);
         return MBD_OK;
     }
-    MBD_CUDA(cholesky_crt(A, ld, ld * ld, batch, ctx->ddinv, ctx->crt, ctx->dstatus, s), origin);
+    MBD_CUDA(cholesky_crt(A, ld, ld * ld, batch, ctx->ddinv, ctx->crt, ctx->dstatus, s, ctx->lim), origin);
     return MBD_OK;
 }
 
@@ -434,9 +434,9 @@ int mixed_group(int nk, long long lde, int precision) {
 // Scratch of a cell's products: the gradient's and, in FP64, those that build Q(q).  (The mixed modes round Q to FP32 and
 // bf16 parts, where a last-place difference of the FP64 entries now and then turns a rounding, and keep the direct build:
 // through products their 256-atom cell takes 150 ms less, but one in five seeds comes out 5e-9 off.)
-size_t cell_products_bytes(int N, const CellGeom &c, int nk, int maxG, int precision) {
-    const size_t grad = grad_products_bytes(N, c, nk, maxG);
-    return fp64_path(precision) ? std::max(build_q_products_bytes(N, c, nk, maxG), grad) : grad;
+size_t cell_products_bytes(int N, const CellGeom &c, int nk, int maxG, int precision, const ScratchLimits &lim) {
+    const size_t grad = grad_products_bytes(N, c, nk, maxG, lim);
+    return fp64_path(precision) ? std::max(build_q_products_bytes(N, c, nk, maxG, lim), grad) : grad;
 }
 
 // Carves the workspace out of one allocation (256-byte aligned pieces).
@@ -483,7 +483,7 @@ int allocate(mbd_ctx *ctx, bool groups = true) {
     // the mixed modes' iteration buffers: the matrix order, or the order of a cell's embedded
     // Hermitian matrices
     const long long ldm = ctx->periodic ? ctx->lde : ld;
-    ctx->mgroup = groups && ctx->periodic && !fp64_path(prec) ? mixed_group(static_cast<int>(nk), ldm, prec) : 1;
+    ctx->mgroup = groups && !ctx->lim.none && ctx->periodic && !fp64_path(prec) ? mixed_group(static_cast<int>(nk), ldm, prec) : 1;
     const size_t mat32 = sizeof(float) * static_cast<size_t>(ldm) * ldm * ctx->mgroup, mat16 = mat32 / 2;
     const size_t split_mat = prec == MBD_PREC_BF16X3 ? mat16 : (prec == MBD_PREC_TF32X3 ? mat32 : 0);
     if (!fp64_path(prec)) bytes += 6 * mat32;
@@ -502,12 +502,13 @@ int allocate(mbd_ctx *ctx, bool groups = true) {
     bytes += scs32;
     // Scratch of the tensor-core products, taken only where it fits: FP64 products and factors (and the
     // transpose of P), and the build of Q(q), which can share theirs.
-    const size_t q_work = ctx->periodic ? al(cell_products_bytes(ctx->N, ctx->cell, static_cast<int>(nk), ctx->maxG, prec)) : 0;
+    const size_t q_work = ctx->periodic ? al(cell_products_bytes(ctx->N, ctx->cell, static_cast<int>(nk), ctx->maxG, prec, ctx->lim)) : 0;
     const size_t crt_part =
-        fp64_path(prec) ? std::max({al(cholesky_crt_bytes(ld, static_cast<int>(nf1))),
-                                    al(ctx->periodic ? crt_cell_bytes(ctx->n, static_cast<int>(nk)) : crt_ns_bytes(ctx->n)), q_work})
+        fp64_path(prec) ? std::max({al(cholesky_crt_bytes(ld, static_cast<int>(nf1), ctx->lim)),
+                                    al(ctx->periodic ? crt_cell_bytes(ctx->n, static_cast<int>(nk), ctx->lim) : crt_ns_bytes(ctx->n, ctx->lim)), q_work})
                         : q_work;
-    const size_t pt_part = fp64_path(prec) ? matq : 0, crt_work = crt_part + pt_part;
+    const size_t pt_part = fp64_path(prec) ? matq : 0, crt_wanted = crt_part + pt_part;
+    const size_t crt_work = ctx->lim.none ? 0 : crt_wanted;
     // A slab large enough for the new size is re-carved in place (systems of varying size in
     // a batch then reuse one allocation); otherwise it is replaced.
     cudaError_t e = cudaSuccess;
@@ -532,7 +533,7 @@ int allocate(mbd_ctx *ctx, bool groups = true) {
         ctx->slab_bytes = want;
     }
     const bool crt = crt_work && ctx->slab_bytes >= bytes + crt_work;
-    ctx->no_scratch = crt_work && !crt;
+    ctx->no_scratch = crt_wanted && !crt;
     ctx->qwork_bytes = crt ? q_work : 0;
     if (ctx->qslab) cudaFree(ctx->qslab);
     ctx->qslab = nullptr;
@@ -1014,11 +1015,11 @@ int backward_periodic(mbd_ctx *ctx, cudaStream_t s, const AtomBufs &b, const dou
     const PeriodicBufs pb = periodic_bufs(ctx);
     MbdGradOut go{ctx->dgomb, ctx->dgab0, ctx->dgrb, ctx->dgR};
     const bool mixed = ctx->opt.precision != MBD_PREC_FP64 && ctx->opt.precision != MBD_PREC_FP64_SPLIT;
-    const size_t bytes = grad_products_bytes(ctx->N, ctx->cell, ctx->nk, ctx->maxG);
+    const size_t bytes = grad_products_bytes(ctx->N, ctx->cell, ctx->nk, ctx->maxG, ctx->lim);
     char *products = ctx->qwork && bytes && bytes <= ctx->qwork_bytes ? ctx->qwork : nullptr;
     if (products) MBD_CUDA(cudaMemsetAsync(ctx->dstatus, 0, sizeof(int), s), "gradient");
     MBD_CUDA(periodic_mbd_grad(b, pb, beta, a, ctx->Zlast, ld, ctx->zscale, go, ctx->dgc, ctx->dgA, s,
-                               ctx->tq_valid ? ctx->dtq : nullptr, mixed, products, ctx->dstatus), "gradient");
+                               ctx->tq_valid ? ctx->dtq : nullptr, mixed, products, ctx->dstatus, ctx->lim), "gradient");
     if (ctx->opt.scs_mode == MBD_SCS_NL) {   // MBD-NL: no screening to differentiate
         if (grad_params) nl_chain(b, go, grad_energy, grad_params, s);
         if (grad_coords) scale_copy(ctx->dgR, 3 * ctx->N, grad_energy, grad_coords, s);
@@ -1108,9 +1109,9 @@ int run_periodic(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &
     if (rc) return rc;
     ctx->have_screening = true;
     // ---- Q(q) and the spectrum bounds ----
-    const size_t qbytes = build_q_products_bytes(N, ctx->cell, nk, ctx->maxG);
+    const size_t qbytes = build_q_products_bytes(N, ctx->cell, nk, ctx->maxG, ctx->lim);
     if (fp64_path(ctx->opt.precision) && ctx->qwork && qbytes && qbytes <= ctx->qwork_bytes) {
-        MBD_CUDA(build_q_products(b, pb, beta, a, ctx->dQ, ld, ctx->qwork, ctx->dstatus, s), "coupled_oscillator_matrix");
+        MBD_CUDA(build_q_products(b, pb, beta, a, ctx->dQ, ld, ctx->qwork, ctx->dstatus, s, ctx->lim), "coupled_oscillator_matrix");
         pad_q_periodic(b, pb, ctx->dQ, ld, n, s);
     } else {
         build_q_periodic(b, pb, beta, a, ctx->dQ, ld, n, ctx->dstatus, s);
@@ -1610,6 +1611,12 @@ int run(mbd_ctx *ctx, cudaStream_t s, const Inputs &in, const Outputs &out, bool
 
 }  // namespace
 
+void mbdgb::set_scratch_limits(mbd_ctx *ctx, const ScratchLimits &lim) {
+    ctx->lim = lim;
+    release(ctx);   // the next mbd_set_geometry carves anew
+    ctx->have_geom = ctx->have_params = ctx->have_forward = ctx->have_result = false;
+}
+
 extern "C" {
 
 int mbd_default_options(mbd_options *opt) {
@@ -1723,7 +1730,7 @@ int mbd_set_geometry(mbd_ctx *ctx, int n_atoms, const double *coords, const doub
     if (periodic) {
         // The image tables' size depends on the lattice.  More scratch for a changed one comes beside the slab, whose
         // parameters and last evaluation stay; where it does not fit, the cell takes the direct kernels.
-        const size_t need = ctx->no_scratch ? 0 : cell_products_bytes(n_atoms, ps.cell, ps.nk, ps.maxG, ctx->opt.precision);
+        const size_t need = ctx->no_scratch ? 0 : cell_products_bytes(n_atoms, ps.cell, ps.nk, ps.maxG, ctx->opt.precision, ctx->lim);
         void *more = nullptr;
         if (need > ctx->qwork_bytes) {
             if (cudaMalloc(&more, need) == cudaSuccess) {
