@@ -622,8 +622,13 @@ __global__ void k_scs_grad_inputs_f32(const double *X, const double *V, const do
 // once (i in tile I, j in tile J, i < j), and writes both ends' sums of the tile pair to
 // part[other tile][7][atom]; k_ts_sum adds them up in a fixed order.  Bound by FP64 arithmetic: four
 // divisions, a square root and an exponential a pair of about 150 operations (each ordered pair for itself with a
-// division wherever the formula has one, 250 operations: 1.36 ms for 2000 atoms, 0.61 so).
+// division wherever the formula has one, 250 operations: 1.36 ms for 2000 atoms, 0.62 so).
 constexpr int kTsTile = 32, kTsVals = 7;   // e, gR x3, ga0, gom, grv
+// a / b as the division rounds it (but for a tie now and then), from the rounded 1 / b.
+__device__ __forceinline__ double quotient(double a, double b, double ib) {
+    const double q = a * ib;
+    return fma(fma(-q, b, a), ib, q);
+}
 __global__ void __launch_bounds__(256) k_ts_pairs(AtomBufs b, double s_r, int tiles, double *part) {
     int J = static_cast<int>((sqrtf(8.0f * blockIdx.x + 1.0f) - 1.0f) * 0.5f);
     while ((J + 1) * (J + 2) / 2 <= static_cast<int>(blockIdx.x)) ++J;
@@ -645,16 +650,18 @@ __global__ void __launch_bounds__(256) k_ts_pairs(AtomBufs b, double s_r, int ti
         const int i = I * kTsTile + ty + 8 * u;
         if (i >= b.N) continue;   // the same for the whole warp
         double acc[kTsVals] = {0, 0, 0, 0, 0, 0, 0};
+        const double iwi = 1.0 / b.om[i];
         if (j < b.N && i < j) {
             const double ai = b.a0[i], wi = b.om[i];
             const double r[3] = {Rj[0] - b.R[3 * i], Rj[1] - b.R[3 * i + 1], Rj[2] - b.R[3 * i + 2]};
-            const double rho = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]), ir = 1.0 / rho, ir2 = ir * ir;
-            const double iw = 1.0 / (wi + wj), c6 = 1.5 * ai * aj * wi * wj * iw;
-            // Fermi damping of steepness 20 and its derivatives (pair_math.cuh)
-            const double iS = 1.0 / (s_r * (b.rv[i] + rvj)), x = rho * iS;
+            const double rho2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2], rho = sqrt(rho2), ir2 = 1.0 / rho2, ir = rho * ir2;
+            const double w = wi + wj, iw = 1.0 / w, c6 = quotient(1.5 * ai * aj * wi * wj, w, iw);
+            // Fermi damping of steepness 20, which its exponent multiplies rho / S's rounding by, and its derivatives
+            // (pair_math.cuh)
+            const double S = s_r * (b.rv[i] + rvj), iS = 1.0 / S, x = quotient(rho, S, iS);
             const double f = 1.0 / (1.0 + exp(-20.0 * (x - 1.0))), df = 20.0 * f * (1.0 - f);
             const double ir6 = ir2 * ir2 * ir2, h = f * ir6, hc = h * c6;
-            const double dh = (df * iS * ir6 - 6.0 * h * ir) * c6 * ir;
+            const double dh = (df * iS * ir6 * ir - 6.0 * h * ir2) * c6;   // over rho
             acc[0] = -0.5 * hc;
             for (int c = 0; c < 3; ++c) acc[1 + c] = dh * r[c];
             acc[6] = c6 * ir6 * df * x * s_r * iS;   // -c6 dh/dS
@@ -663,15 +670,13 @@ __global__ void __launch_bounds__(256) k_ts_pairs(AtomBufs b, double s_r, int ti
             accj[4] -= hc * iaj;
             accj[5] -= hc * (iwj - iw);
             accj[6] += acc[6];
-            acc[4] = -hc;             // over alpha_i and with 1/omega_i below
-            acc[5] = hc * iw;
+            acc[4] = -hc;             // over alpha_i below
+            acc[5] = -hc * (iwi - iw);
         }
 #pragma unroll
         for (int e = 0; e < kTsVals; ++e) acc[e] = warp_sum(acc[e]);
         if (tx == 0) {
-            const double hc = -acc[4];
-            acc[5] -= hc / b.om[i];
-            acc[4] = -hc / b.a0[i];
+            acc[4] /= b.a0[i];
             double *p = part + static_cast<long long>(J) * kTsVals * b.N + i;
             // (the diagonal tile's other ends are added below)
             for (int e = 0; e < kTsVals; ++e) p[static_cast<long long>(e) * b.N] = acc[e];
@@ -688,14 +693,18 @@ __global__ void __launch_bounds__(256) k_ts_pairs(AtomBufs b, double s_r, int ti
     }
 }
 
-// Sums over the partner tiles, a warp per atom and value.
+// Sums over the partner tiles, a thread per atom and value: eight sums side by side, then those in pairs, so that 2000 atoms
+// round 11 times on the way and not 63.
 __global__ void __launch_bounds__(256) k_ts_sum(int N, int tiles, const double *part, double *eatom, double *gR,
                                                 double *ga0, double *gom, double *grv) {
     const int i = blockIdx.x * 32 + (threadIdx.x & 31), e = threadIdx.x >> 5;
     if (i >= N || e >= kTsVals) return;
-    double s = 0.0;
-#pragma unroll 8
-    for (int t = 0; t < tiles; ++t) s += part[(static_cast<long long>(t) * kTsVals + e) * N + i];
+    double q[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int t0 = 0; t0 < tiles; t0 += 8)
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (t0 + u < tiles) q[u] += part[(static_cast<long long>(t0 + u) * kTsVals + e) * N + i];
+    const double s = ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
     if (e == 0) eatom[i] = s;
     else if (e < 4) gR[3 * i + e - 1] = s;
     else if (e == 4) ga0[i] = s;
