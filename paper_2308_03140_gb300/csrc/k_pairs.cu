@@ -651,10 +651,11 @@ __global__ void __launch_bounds__(256) k_ts_pairs(AtomBufs b, double s_r, int ti
         if (i >= b.N) continue;   // the same for the whole warp
         double acc[kTsVals] = {0, 0, 0, 0, 0, 0, 0};
         const double iwi = 1.0 / b.om[i];
-        if (j < b.N && i < j) {
+        const double r[3] = {Rj[0] - b.R[3 * i], Rj[1] - b.R[3 * i + 1], Rj[2] - b.R[3 * i + 2]};
+        const double rho2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
+        if (j < b.N && i < j && !(rho2 > 1e300)) {   // (beyond, every term is zero)
             const double ai = b.a0[i], wi = b.om[i];
-            const double r[3] = {Rj[0] - b.R[3 * i], Rj[1] - b.R[3 * i + 1], Rj[2] - b.R[3 * i + 2]};
-            const double rho2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2], rho = sqrt(rho2), ir2 = 1.0 / rho2, ir = rho * ir2;
+            const double rho = sqrt(rho2), ir2 = 1.0 / rho2, ir = rho * ir2;
             const double w = wi + wj, iw = 1.0 / w, c6 = quotient(1.5 * ai * aj * wi * wj, w, iw);
             // Fermi damping of steepness 20, which its exponent multiplies rho / S's rounding by, and its derivatives
             // (pair_math.cuh)
