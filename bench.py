@@ -396,7 +396,7 @@ def time_arm(binding, dev, stream, sysm, p3, p4, precision, scs_mode, steps, war
     m.set_profiling(False)
     out = {"ms": ms, "steps": steps, "warmup": warmup, "energy": energy.item(), "gR": gR.cpu().numpy().copy(),
            "gp": gp.cpu().numpy().copy() if gp is not None else None, "profs": profs, "stats": m.stats(),
-           "clocks": clk, "ctx": m,
+           "clocks": clk, "ctx": m, "tensor": m.workspace()["tensor_products"],
            "gA": m.lattice_gradient() if periodic else None}
     return out
 
@@ -417,8 +417,9 @@ def errors_vs(arm, ref, N):
                if arm.get("gA") is not None and ref.get("gA") is not None else {})}
 
 
-def roofline_of(binding, args_precision, precision, profs, ms, steps, workload):
-    """Roofline of the dominant kernel of an arm from the library's CUDA-event profile."""
+def roofline_of(binding, args_precision, precision, profs, ms, steps, workload, tensor=False):
+    """Roofline of the dominant kernel of an arm from the library's CUDA-event profile.  tensor: the FP64 products ran
+    on the tensor cores (workspace()); else on the FP64 pipe."""
     gemm_ms = sum(p["gemm_ms"] for p in profs)
     gemm_flops = sum(p["gemm_flops"] for p in profs)
     gemm_launches = sum(p["gemm_launches"] for p in profs)
@@ -426,14 +427,13 @@ def roofline_of(binding, args_precision, precision, profs, ms, steps, workload):
     bf16_sus = peaks.get("bf16_tflops_sustained") if peaks else None
     src = "of measured" if bf16_sus else "of fallback"
     bf16_sus = bf16_sus or 1700.0
-    if precision == binding.MBD_PREC_FP64_SPLIT:
-        kernel = "k_tc_gemm<TF32> slice products of the split FP64 GEMM (Newton-Schulz products)"
+    if precision in (binding.MBD_PREC_FP64, binding.MBD_PREC_FP64_SPLIT) and tensor:
+        kernel = "k_crt_gemm with k_crt_rows and k_crt_result (FP64 Newton-Schulz products by bf16 residues, tcgen05)"
         k_ms, k_flops, k_launches = gemm_ms, gemm_flops, gemm_launches
-        peak = bf16_sus * 0.5 / 53
-        peak_src = (f"{src}: bf16_tflops_sustained x nominal TF32/BF16 rate (0.5) / 53 slice products per "
-                    "algorithmic product")
+        peak = bf16_sus / 15
+        peak_src = f"{src}: bf16_tflops_sustained / 15 residue products per algorithmic product"
         traffic, tsrc = None, None
-    elif precision == binding.MBD_PREC_FP64:
+    elif precision in (binding.MBD_PREC_FP64, binding.MBD_PREC_FP64_SPLIT):
         kernel = "k_gemm_nn (FP64 mma.sync m8n8k4, Newton-Schulz products)"
         k_ms, k_flops, k_launches = gemm_ms, gemm_flops, gemm_launches
         peak = bf16_sus * FP64_OVER_BF16
@@ -544,7 +544,7 @@ def run_ours(args):
     line["tflops_algorithmic_min"] = (None if periodic else
                                       ((0.0 if nl else 16.0 * (n ** 3 / 3.0 + 12.0 * n ** 2)) + 9.0 * n ** 3)
                                       / (ms / args.steps / 1e3) / 1e12)
-    line["roofline"] = roofline_of(binding, args.precision, precision, profs, ms, args.steps, args.workload)
+    line["roofline"] = roofline_of(binding, args.precision, precision, profs, ms, args.steps, args.workload, main["tensor"])
     line["e2e"] = e2e
     line["clocks"] = main["clocks"]
     line["gpu_launches"] = sum(p["launches"] for p in profs)
@@ -578,7 +578,7 @@ def run_ours(args):
                 "energy_ha": f["energy"], "ns_iterations": f["stats"]["ns_iterations"],
                 "stage_ms": stage_means(f["profs"]),
                 "roofline": roofline_of(binding, "fp64", binding.MBD_PREC_FP64, f["profs"], f["ms"],
-                                        args.fp64_steps, args.workload),
+                                        args.fp64_steps, args.workload, f["tensor"]),
                 "errors_of": {args.precision: errors_vs(main, f, N),
                               **{k: errors_vs(a, f, N) for k, a in arms.items()}}}
     line["fp64_path"] = fp64
@@ -587,7 +587,7 @@ def run_ours(args):
                                     "energy_ha": a["energy"], "ns_iterations": a["stats"]["ns_iterations"],
                                     "stage_ms": stage_means(a["profs"]),
                                     "roofline": roofline_of(binding, k, precision_code(binding, k), a["profs"],
-                                                            a["ms"], a["steps"], args.workload)}
+                                                            a["ms"], a["steps"], args.workload, a["tensor"])}
                                 for k, a in arms.items()}
     # further workloads (the 2000-atom cluster, the 256-atom cell), each measured the same way
     # with fewer steps, and the varlen cluster batch with the learned screening beside plain
@@ -616,7 +616,7 @@ def run_ours(args):
                          "energy_ha": a["energy"], "ns_iterations": a["stats"]["ns_iterations"],
                          "stage_ms": stage_means(a["profs"]),
                          "roofline": roofline_of(binding, name, precision_code(binding, name), a["profs"], a["ms"],
-                                                 xk, xw)}
+                                                 xk, xw, a["tensor"])}
         if not xper and not nl and args.learned_arm:   # the learned screening (no fallback) with the same matrix function
             model = np.load(os.path.join(ROOT, "paper_2308_03140_gb300", "learned_scs_model.npz"))
             a = time_arm(binding, dev, stream, xs, xp3, xp4, precision_code(binding, args.precision), scs_mode, xk, 1,
@@ -636,7 +636,7 @@ def run_ours(args):
                                 "warmup": 1, "energy_ha": f["energy"], "ns_iterations": f["stats"]["ns_iterations"],
                                 "stage_ms": stage_means(f["profs"]),
                                 "roofline": roofline_of(binding, "fp64", binding.MBD_PREC_FP64, f["profs"], f["ms"],
-                                                        args.extra_fp64_steps, xw),
+                                                        args.extra_fp64_steps, xw, f["tensor"]),
                                 "errors_of": {k: errors_vs(a, f, xs.n_atoms) for k, a in xarms.items()}}
         torch.cuda.empty_cache()
         line[xw] = sec
