@@ -48,12 +48,18 @@ extern "C" {
  * iterations on the 5th-generation tensor cores with FP32 accumulation, then one FP64
  * correction: with Z ~ Q^{-1/2}, V = Q Z and W = Z V (FP64), Tr Q^{1/2} is taken as
  * (3 Tr V - sum V o W)/2, whose error is second order in the error of Z; the energy
- * subtraction and all sums stay in FP64 with compensation.  Gradients use Z.  In the same
+ * subtraction and the sums stay in FP64, chains of four products each added into compensated
+ * sums.  Gradients use Z.  In the same
  * modes the screening matrices are factored in FP32 (tensor-core TF32x3 updates) and each
  * solution is refined once against the FP64 matrix. */
-#define MBD_PREC_FP64 0           /* FP64 throughout; the Newton-Schulz products are formed on the
-                                     bf16 tensor cores from exact residues, with less rounding
-                                     than an FP64 sum                                 */
+#define MBD_PREC_FP64 0           /* FP64 throughout.  The Newton-Schulz products, the screening's (and the
+                                     log formula's) Cholesky factors, a cell's Q(q) and its gradient
+                                     sums are formed on the bf16 tensor cores from exact residues of
+                                     58-bit rows: a product errs by some 2^-59 of its row's times its
+                                     column's 2-norm, less than an FP64 sum of terms of like size, more than one
+                                     whose terms are all far below the two norms.  Where the scratch of
+                                     these products does not fit the device (mbd_get_workspace), they run
+                                     on the FP64 pipe                                 */
 #define MBD_PREC_TF32 1           /* TF32 tensor-core products, FP64 correction      */
 #define MBD_PREC_BF16X3 2         /* bf16 hi/lo split products (3 per GEMM), FP64 correction */
 #define MBD_PREC_TF32X3 3         /* TF32 hi/lo split products (3 per GEMM), FP64 correction */
@@ -274,8 +280,10 @@ int mbd_get_workspace(const mbd_ctx *ctx, int *tensor_products, int *matrices_to
  * triangle, n^3/3 per Cholesky factorisation). */
 typedef struct {
     int launches;            /* CUDA kernels launched by the evaluation                  */
-    int gemm_launches;       /* FP64 tensor-path GEMM launches of the Newton-Schulz stage */
-    double gemm_ms;          /* summed device time of those launches                      */
+    int gemm_launches;       /* timed FP64 products of the Newton-Schulz stage: launches on the FP64
+                                pipe; on the tensor cores a product with its conversions, or both products
+                                of a step together                                        */
+    double gemm_ms;          /* their summed device time                                  */
     double gemm_flops;       /* their summed algorithmic flops                            */
     double screening_ms;     /* build + factorise + solve, all frequency points           */
     double screening_flops;  /* (n_freq + 1) n^3 / 3                                      */

@@ -9,7 +9,11 @@
 // sum products of residues in [-128, 128] (exact in bf16: 8 bits), 1024 of them at a time, so that
 // every partial sum is an integer of at most 2^24 and exact in FP32.  What is lost is only the rounding of x
 // and y: an error of about 0.4 2^-kRowBits |a| |b| in a.b, against about 0.2 2^-52 |a| |b| for an
-// FP64 sum of random terms, whose roundings grow with their number.
+// FP64 sum of random terms, whose roundings grow with their number.  That is relative to the rows' norms: where one
+// entry dominates a row and meets a small one, so that |a.b| is far below |a| |b|, an FP64 sum keeps more
+// bits of a.b (entries 1e-8 of their rows: 2e-16 against 2e-11).  The matrices here are summed into traces and
+// contracted with rows of their own size, and over the sizes the library is timed on the results' errors against
+// 64-bit eigenvalues are what they were on the FP64 pipe.
 #pragma once
 #include <cmath>
 #include <cstdint>

@@ -149,7 +149,9 @@ __global__ void __launch_bounds__(256) k_solve(double *A, long long ld, long lon
     }
 }
 
-// 1 / d to about an ulp, d a normal number: two Newton steps from the hardware's approximation.
+// 1 / d, d a normal number: two Newton steps from the hardware's approximation (2^-20 or better), after which only the last
+// rounding is left, so that all but a few quotients are the division's.  (Diagonals beyond 1e+-280, the inverses of
+// polarizabilities in bohr^3, are not served, here and in the exponents.)
 __device__ __forceinline__ double reciprocal(double d) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(d));
