@@ -1,4 +1,4 @@
-// Pairs of a cell's atoms by tiles, and their lattice images (k_qbuild.cu, k_qgrad.cu).
+// Pairs of a cell's atoms by tiles, and their lattice images (k_periodic.cu, k_qbuild.cu, k_qgrad.cu).
 #pragma once
 #include "internal.h"
 #include "pair_math.cuh"
@@ -16,12 +16,16 @@ __device__ __forceinline__ void tile_pair(int t, int ntile, int &I, int &J) {
     J = I + t;
 }
 
+__device__ __forceinline__ double frac_coord(const CellGeom &c, const double *v, int k) {
+    return v[0] * c.Ainv[k] + v[1] * c.Ainv[3 + k] + v[2] * c.Ainv[6 + k];
+}
+
 // First and last image index of each direction for separation x: r = x + n A within the cutoff needs
 // n_c in [-L_c - f_c, L_c - f_c] (f = fractional x, L_c = rc |b_c| / 2 pi).
-__device__ __forceinline__ void first_image(const CellGeom &c, const double *x, int *lo, int *hi) {
+__device__ __forceinline__ void image_box(const CellGeom &c, const double *x, int *lo, int *hi) {
     for (int k = 0; k < 3; ++k) {
         const double bn = sqrt(c.B[3 * k] * c.B[3 * k] + c.B[3 * k + 1] * c.B[3 * k + 1] + c.B[3 * k + 2] * c.B[3 * k + 2]);
-        const double L = c.rc * bn / (2.0 * kPi) + 1e-9, f = x[0] * c.Ainv[k] + x[1] * c.Ainv[3 + k] + x[2] * c.Ainv[6 + k];
+        const double L = c.rc * bn / (2.0 * kPi) + 1e-9, f = frac_coord(c, x, k);
         lo[k] = static_cast<int>(ceil(-L - f));
         hi[k] = static_cast<int>(floor(L - f));
     }

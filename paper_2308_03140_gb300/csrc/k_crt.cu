@@ -220,41 +220,12 @@ struct GemmCrt {
     int *err;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t peer_addr(uint32_t local, uint32_t rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(local), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ bool mbar_wait_cl(uint64_t *b, uint32_t parity, int *err, long long budget = kSpinCycles) {
-    const long long t0 = clock64();
-    for (;;) {
-        uint32_t ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(ok)
-            : "r"(su32(b)), "r"(parity)
-            : "memory");
-        if (ok) return true;
-        if (clock64() - t0 > budget) {
-            atomicOr(err, ST_TC_TIMEOUT);
-            return false;
-        }
-    }
-}
 __device__ __forceinline__ void tma_load_3d_pair(void *dst, const CUtensorMap *map, int x, int y, int z, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n" ::"r"(
             su32(dst)),
         "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
         : "memory");
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 // bf16 operands, FP32 accumulator, both K-major, M = 256 (two CTAs), N = kN.
 template <int kN>
@@ -559,18 +530,6 @@ __global__ void __launch_bounds__(256) k_crt_result(ResultArgs g, int tiles_c) {
         const int cc = g.col0 + c0 + k;
         if (r < g.M && c0 + k < g.n && (!g.sym || r < cc)) out[cc * ldo + r] = sign * tile[i][k];
     }
-}
-
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        const bool ok = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                            cudaSuccess &&
-                        q == cudaDriverEntryPointSuccess;
-        return ok ? reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p) : nullptr;
-    }();
-    return fn;
 }
 
 // Planes [z][rows][pitch] of bf16, boxes of box_rows rows by 64 entries of one plane, 128-byte swizzle.

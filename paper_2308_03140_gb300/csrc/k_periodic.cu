@@ -16,6 +16,7 @@
 // The reciprocal phase e^{+i G.(R_j - R_i)} with k = G + q follows from Poisson summation of
 // sum_n T(r) e^{-i q.r}; the erfc numerator is the -grad grad of erfc(gamma r)/r; the
 // damped-away part (1 - g) T is removed in real space because it decays exponentially.
+#include "cell_pairs.cuh"
 #include "comp_sum.cuh"
 #include "internal.h"
 #include "pair_math.cuh"
@@ -24,24 +25,9 @@ namespace mbdgb {
 namespace {
 
 using namespace pairs;
+using namespace cellpairs;
 
-constexpr int kQT = 16;   // atom tile edge of the pair-tile kernels (16 x 16 threads)
 constexpr int kGC = 64;   // reciprocal vectors staged per chunk
-
-__device__ __forceinline__ double frac_coord(const CellGeom &c, const double *v, int k) {
-    return v[0] * c.Ainv[k] + v[1] * c.Ainv[3 + k] + v[2] * c.Ainv[6 + k];
-}
-
-// Lattice translations n with |x + n A| < rc: n_c in [-L_c - f_c(x), L_c - f_c(x)],
-// L_c = rc |b_c| / (2 pi) (|f_c(r)| <= |r| |b_c| / 2 pi for any r).
-__device__ __forceinline__ void image_box(const CellGeom &c, const double *x, int *lo, int *hi) {
-    for (int k = 0; k < 3; ++k) {
-        const double bn = sqrt(c.B[3 * k] * c.B[3 * k] + c.B[3 * k + 1] * c.B[3 * k + 1] + c.B[3 * k + 2] * c.B[3 * k + 2]);
-        const double L = c.rc * bn / (2.0 * kPi) + 1e-9, f = frac_coord(c, x, k);
-        lo[k] = static_cast<int>(ceil(-L - f));
-        hi[k] = static_cast<int>(floor(L - f));
-    }
-}
 
 // Symmetric 3x3 stored as xx, yy, zz, xy, xz, yz; contractions with P delta + W r r.
 struct Sym6 { double v[6]; };
@@ -140,12 +126,6 @@ __global__ void __launch_bounds__(128) k_build_scs_periodic(AtomBufs b, CellGeom
 // grid (upper-triangle tile pairs, nk); thread (ty, tx) of tile (I, J) owns the atom pair
 // (i, j) = (16 I + ty, 16 J + tx) when i <= j, and writes block (i, j) and its Hermitian
 // mirror (j, i) = conj(block)^T (the 3x3 blocks are complex symmetric).
-__device__ __forceinline__ void tile_pair(int t, int ntile, int &I, int &J) {
-    I = 0;
-    while (t >= ntile - I) { t -= ntile - I; ++I; }
-    J = I + t;
-}
-
 // The reduced-precision staging of the gradient's reciprocal sum (F32: the mixed modes).
 template <typename R> struct Vec2;
 template <> struct Vec2<double> { using T = double2; };

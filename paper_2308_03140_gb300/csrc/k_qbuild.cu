@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(256) k_q_images(AtomBufs b, CellGeom c, double
     if (p.valid) {
         const int o = blockIdx.y, off[3] = {o / (d1 * d2), o / d2 % d1, o % d2};
         int lo[3], hi[3];
-        first_image(c, p.x, lo, hi);
+        image_box(c, p.x, lo, hi);
         bool in = true;
         for (int e = 0; e < 3; ++e) in = in && lo[e] + off[e] <= hi[e];
         if (in) {
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(256) k_q_assemble(AtomBufs b, PeriodicBufs p, 
         }
     }
     int lo[3], hi[3];
-    first_image(c, pr.x, lo, hi);
+    image_box(c, pr.x, lo, hi);
     double t = 0.0;
     for (int e = 0; e < 3; ++e) t += q[e] * (pr.x[e] + lo[0] * c.A[e] + lo[1] * c.A[3 + e] + lo[2] * c.A[6 + e]);
     double sn, cs;

@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(256) k_grad_rows(AtomBufs b, PeriodicBufs p, c
     }
     const CellGeom &c = p.cell;
     int lo[3], hi[3];
-    first_image(c, pr.x, lo, hi);
+    image_box(c, pr.x, lo, hi);
     double t = 0.0;
     for (int e = 0; e < 3; ++e)
         t += p.kq[3 * kq + e] * (pr.x[e] + lo[0] * c.A[e] + lo[1] * c.A[3 + e] + lo[2] * c.A[6 + e]);
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(256) k_grad_images(AtomBufs b, CellGeom c, dou
         const Pair p = pair_at(b, ntile, pair0 + at);
         if (!p.valid) continue;
         int lo[3], hi[3];
-        first_image(c, p.x, lo, hi);
+        image_box(c, p.x, lo, hi);
         double fx[3];
         for (int k = 0; k < 3; ++k) fx[k] = p.x[0] * c.Ainv[k] + p.x[1] * c.Ainv[3 + k] + p.x[2] * c.Ainv[6 + k];
         const double S = b.rbar[p.i] + b.rbar[p.j];

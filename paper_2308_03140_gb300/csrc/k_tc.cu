@@ -879,39 +879,8 @@ struct TcCfg2 {
     static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 512;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
-    return r;
-}
-// Address in the shared::cluster window of the same shared-memory object in CTA `rank`.
-__device__ __forceinline__ uint32_t peer_addr(uint32_t local, uint32_t rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(local), "r"(rank));
-    return a;
-}
 __device__ __forceinline__ void remote_arrive(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(cluster_addr) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_cl(uint64_t *b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(su32(b)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait (cluster-scope acquire: arrivals may come from the peer CTA).
-__device__ __forceinline__ bool mbar_wait_cl(uint64_t *b, uint32_t parity, int *err) {
-    const long long t0 = clock64();
-    while (!mbar_try_cl(b, parity)) {
-        if (clock64() - t0 > kSpinCycles) {
-            atomicOr(err, ST_TC_TIMEOUT);
-            return false;
-        }
-    }
-    return true;
 }
 // TMA load into this CTA's shared memory whose completion is counted on an mbarrier of either
 // CTA of the pair (shared::cluster address).
@@ -921,9 +890,6 @@ __device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *m
             su32(dst)),
         "l"(map), "r"(x), "r"(y), "r"(bar)
         : "memory");
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 // Instruction descriptor of the pair MMA: M = 256 (two CTAs), N = TN.
 __host__ __device__ constexpr uint32_t idesc2(uint32_t fmt) {
@@ -1157,19 +1123,6 @@ __global__ void k_wait_probe(long long budget, int *err) {
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         mbar_wait(&bar, 0, err, budget);
     }
-}
-
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
 }
 
 // Tensor map of a row-major rows x cols matrix (row pitch ld elements), box of 128 rows

@@ -1,10 +1,11 @@
 // tcgen05 / TMA / mbarrier building blocks of the tensor-core kernels (sm_103a), shared by the
-// GEMM (k_tc.cu) and the learned model's MLP (k_learned.cu).
+// GEMM (k_tc.cu), the residue products (k_crt.cu) and the learned model's MLP (k_learned.cu).
 //
 // Every wait is bounded (clock64 budget); on a timeout it raises ST_TC_TIMEOUT in the caller's
 // error flag and returns false.
 #pragma once
 #include <cuda.h>
+#include <cudaTypedefs.h>
 
 #include "internal.h"
 
@@ -12,6 +13,19 @@ namespace mbdgb {
 namespace tcops {
 
 constexpr long long kSpinCycles = 4000000000LL;   // ~2 s at 2 GHz
+
+// The driver's tensor-map encoder, null where it has none.
+inline PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
+    static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                            cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        return ok ? reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p) : nullptr;
+    }();
+    return fn;
+}
 
 __device__ __forceinline__ uint32_t su32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -41,6 +55,41 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, int *err
         }
     }
     return true;
+}
+// ---- clusters ----
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+    return r;
+}
+// Address in the shared::cluster window of the same shared-memory object in CTA `rank`.
+__device__ __forceinline__ uint32_t peer_addr(uint32_t local, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(local), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ bool mbar_try_cl(uint64_t *b, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(su32(b)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Bounded wait (cluster-scope acquire: arrivals may come from the peer CTA).
+__device__ __forceinline__ bool mbar_wait_cl(uint64_t *b, uint32_t parity, int *err, long long budget = kSpinCycles) {
+    const long long t0 = clock64();
+    while (!mbar_try_cl(b, parity)) {
+        if (clock64() - t0 > budget) {
+            atomicOr(err, ST_TC_TIMEOUT);
+            return false;
+        }
+    }
+    return true;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
     asm volatile(
