@@ -1445,16 +1445,21 @@ __global__ void k_split_panel_tf32(const float *A, long long ld, long long mstri
 }
 
 // tq[i] = sqrt_s (3 Tr V_ii - Tr (V W)_ii) / 2 over the 3x3 diagonal block of atom i; one
-// warp per atom, (V W)_pp = sum_k V[p][k] W[k][p] with the rows of V read coalesced.
+// warp per atom, (V W)_pp = sum_k V[p][k] W[k][p] with the rows of V read coalesced.  Row after row: these traces end, after a
+// subtraction that leaves a hundredth of them, as right-hand sides of FP32 solves, where a last-place
+// difference turns a rounding now and then (the forces of 5000 atoms moved by up to 6e-9 when the three rows
+// were summed together, in one pass over W).
 __global__ void __launch_bounds__(128) k_block_trace_sqrt(const double *V, const double *W, long long ld, int N,
                                                          double sqrt_s, double *tq) {
     const int i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= N) return;
-    const double *v0 = V + 3LL * i * ld, *v1 = v0 + ld, *v2 = v1 + ld, *w = W + 3LL * i;
     double acc = 0.0;
-#pragma unroll 4
-    for (long long k = lane; k < ld; k += 32)   // three neighbouring columns of W: one sector of a row or two
-        acc += v0[k] * w[k * ld] + v1[k] * w[k * ld + 1] + v2[k] * w[k * ld + 2];
+    for (int x = 0; x < 3; ++x) {
+        const long long p = 3LL * i + x;
+        const double *vp = V + p * ld;
+#pragma unroll 8
+        for (long long k = lane; k < ld; k += 32) acc += vp[k] * W[k * ld + p];
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) {
