@@ -48,8 +48,8 @@ extern "C" {
  * iterations on the 5th-generation tensor cores with FP32 accumulation, then one FP64
  * correction: with Z ~ Q^{-1/2}, V = Q Z and W = Z V (FP64), Tr Q^{1/2} is taken as
  * (3 Tr V - sum V o W)/2, whose error is second order in the error of Z; the energy
- * subtraction and the sums stay in FP64, chains of four products each added into compensated
- * sums.  Gradients use Z.  In the same
+ * subtraction and the sums stay in FP64 with compensation (the off-diagonal products in chains of
+ * four).  Gradients use Z.  In the same
  * modes the screening matrices are factored in FP32 (tensor-core TF32x3 updates) and each
  * solution is refined once against the FP64 matrix. */
 #define MBD_PREC_FP64 0           /* FP64 throughout.  The Newton-Schulz products, the screening's (and the

@@ -557,9 +557,15 @@ __device__ __forceinline__ void wide_epilogue(const TcArgs &g, const float (&acc
     float4 d[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) d[i] = dp ? *reinterpret_cast<const float4 *>(dp + 8LL * i * g.ld) : make_float4(0.f, 0.f, 0.f, 0.f);
-    // |delta - C|^2 as compensated FP32 sums (differences, squares and sums with their rounding errors: as good as
-    // FP64 to a few 2^-46), as the FP64 pipe would take 25 us a tile.
-    float rs = 0.f, rcomp = 0.f;
+    // |delta - C|^2 as FP32 sums with what they lose and what those lose (squares and differences with their rounding
+    // errors): to 2^-60 a tile, where FP64 sums have 2^-50 and would take the FP64 pipe 25 us a tile, and sums compensated
+    // once 2^-45.
+    float rs = 0.f, rcomp = 0.f, rlast = 0.f;
+    auto two_sum = [](float &sum, float x) {   // sum += x; returns what that lost
+        const float t = __fadd_rn(sum, x), b = __fsub_rn(t, sum), lost = __fadd_rn(__fsub_rn(sum, __fsub_rn(t, b)), __fsub_rn(x, b));
+        sum = t;
+        return lost;
+    };
 #pragma unroll 1
     for (int c16 = 0; c16 < TN / 16; ++c16) {
 #pragma unroll
@@ -605,10 +611,11 @@ __device__ __forceinline__ void wide_epilogue(const TcArgs &g, const float (&acc
                 for (int j = 0; j < 4; ++j) {
                     const float one = m == n + j ? 1.f : 0.f, e = one - v[i][j], lost = (one - e) - v[i][j];
                     const bool in = m < g.nvalid && n + j < g.nvalid;
-                    const float p = in ? e * e : 0.f, pe = in ? fmaf(e, e, -p) + 2.f * e * lost : 0.f;
-                    const float t = rs + p, b = t - rs;
-                    rcomp += ((rs - (t - b)) + (p - b)) + pe;
-                    rs = t;
+                    const float p = in ? __fmul_rn(e, e) : 0.f, pe = in ? fmaf(e, e, -p) : 0.f;
+                    const float pl = in ? 2.f * e * lost : 0.f;   // (zero off the diagonal)
+                    rlast += two_sum(rcomp, two_sum(rs, p));
+                    rlast += two_sum(rcomp, pe);
+                    rlast += pl;
                 }
             }
         }
@@ -645,7 +652,7 @@ __device__ __forceinline__ void wide_epilogue(const TcArgs &g, const float (&acc
         }
     }
     if (g.resid) {
-        double t = static_cast<double>(rs) + static_cast<double>(rcomp);
+        double t = static_cast<double>(rs) + (static_cast<double>(rcomp) + static_cast<double>(rlast));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (lane == 0 && t != 0.0) atomicAdd(g.resid + slot, t);
@@ -1516,7 +1523,8 @@ __global__ void k_to_f64(const float *Zf, long long total, double scale, double 
 
 // Per-block partial sums over the leading n x n block of T1 = sum Q o Z (FP64 x FP32, i.e.
 // Tr(Q Z) for symmetric Z), T2 = sum V o W and R = sum (delta - W)^2.  A thread adds the products
-// of kRun entries of a row in one chain of multiply-adds and then the chain to its compensated sum:
+// of kRun entries of a row in one chain of multiply-adds and then the chain to its compensated sum (but the diagonal's,
+// nearly all of T1 and T2, go there directly, rounded once):
 // the chain rounds as often as the products themselves would, and the FP64 pipe, which bounds the pass,
 // spends 7 operations an entry instead of 21 (order 6000: 1.33 -> 0.74 ms; the entries' 28 bytes
 // would take 0.15).
@@ -1534,10 +1542,16 @@ __global__ void __launch_bounds__(256) k_correction_partials(const double *Q, co
             for (int u = 0; u < kRun; ++u) {
                 const int j = j0 + 32 * u + lane;
                 if (j < n) {
-                    const double w = W[row + j], d = i == j ? 1.0 - w : w;
-                    a += Q[row + j] * static_cast<double>(Z[row + j]);
-                    b += V[row + j] * w;
-                    c += d * d;
+                    const double w = W[row + j], q = Q[row + j], z = static_cast<double>(Z[row + j]), v = V[row + j];
+                    if (i == j) {   // by itself: in a chain every addition would round at its size
+                        t1.add(q * z);
+                        t2.add(v * w);
+                        c += (1.0 - w) * (1.0 - w);
+                    } else {
+                        a += q * z;
+                        b += v * w;
+                        c += w * w;
+                    }
                 }
             }
             t1.add(a);
